@@ -163,11 +163,10 @@ sr_status sr_graph_set_node_bias(sr_graph* g, int node, const float* bias_host);
 /* Options.  key 0 "engine": 0 = tensor cores where a node qualifies (default), 1 = CUDA-core kernels only.
  *           key 1 "frames per CUDA graph" used by sr_rollout_run: 0 = plain launches, n >= 1 = graphs
  *                  of n frames (default 0).
- *           key 2 "weight ring": weight boxes the tensor-core kernel keeps in flight in shared memory
+ *           key 2 "weight ring": weight slots (one K-block of 64 channels each) the tensor-core kernel keeps in shared memory
  *                  (2..8; 0 = default); the rest of the shared memory holds activation boxes.
- *           key 3 "tile width": width in pixels (8, 16 or 32; 0 = default) of the 128-pixel output tiles of
- *                  nodes that have a stride-1 k x k incoming edge (narrow tiles reload less halo, wide
- *                  tiles read longer contiguous runs).
+ *           key 3 "tile width": width in pixels (8, 16 or 32; 0 = default) of the output tiles of the tensor-core kernel
+ *                  (for nodes with an edge whose taps share activation boxes).
  *           key 4 "overlap": 1 (default) runs independent launches of a frame on a second, library-owned
  *                  stream (the CUDA-core and the tensor-core kernel of a group; the next frame's input
  *                  copy when no input edge has R = 0), joined before the frame ends; 0 = one stream.
@@ -189,13 +188,9 @@ sr_status sr_graph_set_node_bias(sr_graph* g, int node, const float* bias_host);
  *                  for its own copies in flight, frees its tensor memory and returns, and sr_graph_sync_status
  *                  reports SR_ERR_TIMEOUT.  0 is a test hook: every tensor-core launch reports the error at once and
  *                  returns before it touches a barrier, a copy or an MMA.  May be set at any time.
- *           key 11 "tile pairs": the tensor-core kernel's work item is a pair of neighbouring pixel tiles that share every
- *                  weight box (half the weight traffic, twice the work per item).  0 (default) and 1 = single tiles,
- *                  2 = pairs wherever the geometry allows.
- *           key 12 "staged boxes in the weight ring": the activation box of a staged few-channel input edge (two MMAs'
- *                  worth of work) is fetched into the tensor-core kernel's weight ring together with its weights, so
- *                  that it does not hold one of the few large activation slots.  1 (default) = in launch groups whose
- *                  weight ring has at least four slots, 2 = wherever the box fits a weight slot, 0 = never.
+ *           key 11 "tile pairs" (0, 1, 2) and key 12 "staged boxes in the weight ring" (0, 1, 2): accepted for the callers
+ *                  that set them, without effect any more: the library chooses the columns of a tile that share their
+ *                  weights, and the activation ring takes boxes of any size.
  *           key 13 "work lists": how the tensor-core kernel's persistent CTAs get their work items.  1 = one list per
  *                  CTA, balanced on the host by estimated cost; 0 (default) = the same for the larger items, while
  *                  the smallest ones (a fifth of the work of a launch with many items) form one shared list that

@@ -109,6 +109,7 @@ SrRegion take(size_t& off, size_t bytes)
 sr_status plan(sr_graph* g)
 {
     if (g->batch <= 0) return SR_ERR_STATE;
+    if (g->planned) return SR_OK;                                // asking for the size and binding share one plan
     const int n_nodes = (int)g->nodes.size(), n_edges = (int)g->edges.size();
     for (int v = 0; v < n_nodes; ++v) {
         SrHostNode& n = g->nodes[v];
@@ -195,6 +196,7 @@ sr_status plan(sr_graph* g)
         sr_dn_describe(g, &g->info.resident_cluster, &g->info.resident_smem_bytes);
         g->info.resident_heads_on_chip = 1;
     }
+    g->planned = true;
     return SR_OK;
 }
 
@@ -355,6 +357,7 @@ sr_status sr_graph_levels(const sr_graph* g, int32_t* level)
 sr_status sr_graph_set_option(sr_graph* g, int key, int value)
 {
     if (!g) return SR_ERR_INVALID_ARG;
+    if (!g->ws) g->planned = false;
     if (key == 0) {
         if (g->ws) return SR_ERR_STATE;
         if (value != 0 && value != 1) return SR_ERR_INVALID_ARG;
