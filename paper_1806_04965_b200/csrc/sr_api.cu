@@ -143,6 +143,7 @@ sr_status plan(sr_graph* g)
     g->items.clear();
     g->group_item_offset.clear();
     g->group_item_count.clear();
+    g->group_head_nodes.assign(g->groups.size(), {});
     const int px = sr_direct_conv_pixels_per_block(), dco = sr_direct_dense_outputs_per_block(),
               dsb = sr_direct_dense_samples_per_block();
     for (size_t gi = 0; gi < g->groups.size(); ++gi) {
@@ -151,20 +152,8 @@ sr_status plan(sr_graph* g)
             const SrHostNode& n = g->nodes[v];
             if (n.use_tc) continue;
             if (n.dense_target) {
-                // one sample and a chunk of outputs per block, unless a mean-dense source has more channels
-                // than the block's mean buffer holds (then: one warp per output and 8 samples)
-                bool fast = true;
-                for (int e : n.in_edges)
-                    if (g->edges[e].d.kind == SR_EDGE_MEAN_DENSE && g->nodes[g->edges[e].d.src].d.c > sr_direct_head_max_channels())
-                        fast = false;
-                if (fast) {
-                    // a block takes up to 16 outputs of one sample; with a long reduction (thousands of inputs per
-                    // output) only 4, so that a small batch still gives every SM several blocks' worth of loads in flight
-                    long long k_in = 0;
-                    for (int e : n.in_edges) k_in += g->edges[e].K;
-                    const int hco = k_in >= 4096 ? 4 : sr_direct_head_outputs_per_block();
-                    for (int b0 = 0; b0 < g->batch; ++b0)
-                        for (int c0 = 0; c0 < n.d.c; c0 += hco) g->items.push_back(SrDirectItem{v, b0, c0, 1 | (hco << 8)});
+                if (sr_head_takes(g, v)) {
+                    g->group_head_nodes[gi].push_back(v);
                 } else {
                     for (int b0 = 0; b0 < g->batch; b0 += dsb)
                         for (int c0 = 0; c0 < n.d.c; c0 += dco) g->items.push_back(SrDirectItem{v, b0, c0, 0});
@@ -248,16 +237,12 @@ int enqueue_frames(sr_graph* g, int first_off, int frames, cudaStream_t s)
         ++launches;
         launches += sr_tc_stage_inputs(g, f, in_stream);
         for (int gi = 0; gi < (int)g->groups.size(); ++gi) {
-            const bool has_direct = g->group_item_count[gi] > 0, has_tc = sr_tc_group_has_work(g, gi);
-            if (has_direct) {
-                cudaStream_t ds = s;
-                if (side && has_tc) {
-                    fork();
-                    ds = side->stream;
-                }
-                sr_launch_direct_group(g, gi, f, ds);
-                ++launches;
-            }
+            // up to three independent launches: the heads go beside whatever else the group has, the other CUDA-core nodes
+            // beside the tensor-core kernel
+            const bool has_heads = !g->group_heads[gi].empty(), has_items = g->group_item_count[gi] > 0, has_tc = sr_tc_group_has_work(g, gi);
+            if (side && ((has_heads && (has_items || has_tc)) || (has_items && has_tc))) fork();
+            if (has_heads) launches += sr_launch_heads(g, gi, f, side && (has_items || has_tc) ? side->stream : s);
+            if (has_items) launches += sr_launch_direct_group(g, gi, f, side && has_tc ? side->stream : s);
             launches += sr_tc_launch_group(g, gi, f, s);
             if (gi + 1 < (int)g->groups.size()) join();       // the next group reads what this one wrote
         }
@@ -520,6 +505,28 @@ sr_status sr_graph_bind_workspace(sr_graph* g, void* workspace_dev, size_t bytes
     if (!cuda_ok(cudaMemcpy(ws + g->r_ctl.offset + sizeof(SrFrameCtl), il.data(), sizeof(int) * SR_MAX_INPUTS,
                             cudaMemcpyHostToDevice)))
         return SR_ERR_CUDA;
+    g->group_heads.assign(g->groups.size(), {});
+    for (size_t gi = 0; gi < g->groups.size(); ++gi)
+        for (int v : g->group_head_nodes[gi]) {
+            const SrHostNode& n = g->nodes[v];
+            SrHeadNode h{};
+            h.state[0] = ws + n.state[0].offset;
+            h.state[1] = ws + n.state[1].offset;
+            h.bias = reinterpret_cast<const float*>(ws + n.bias.offset);
+            h.C = n.d.c; h.act = n.d.act;
+            h.is_output = v == g->info.output_node;
+            for (int e : n.in_edges) {
+                const SrHostEdge& he = g->edges[e];
+                const SrHostNode& s = g->nodes[he.d.src];
+                SrHeadEdge& x = h.edges[h.n_edges++];
+                x.src[0] = ws + s.state[0].offset;
+                x.src[1] = ws + s.state[1].offset;
+                x.w = reinterpret_cast<const float*>(ws + he.w_direct.offset);
+                x.HW = s.d.h * s.d.w; x.Cs = s.d.c; x.kind = he.d.kind; x.R = he.R; x.K = he.K;
+                h.has_mean |= he.d.kind == SR_EDGE_MEAN_DENSE;
+            }
+            g->group_heads[gi].push_back(h);
+        }
     g->ws = ws;
     st = sr_tc_bind(g);
     if (st == SR_OK) st = sr_rs_bind(g);

@@ -114,7 +114,7 @@ __device__ void conv_item(const SrDevNode& nd, const SrDevEdge* edges, const SrD
     }
 }
 
-// Dense node: one warp per output channel and chunk of kDenseB samples; lanes stride over the
+// Dense node outside the limits of the head kernels: one warp per output channel and chunk of kDenseB samples; lanes stride over the
 // reduction index (coalesced weight and state reads), partial sums meet in a shuffle reduction.
 // A mean-dense edge is the dense edge whose weight index is k mod C_in, scaled by 1/(H*W).
 template <typename T>
@@ -166,115 +166,187 @@ __device__ void dense_item(const SrDevNode& nd, const SrDevEdge* edges, const Sr
 }
 
 
-constexpr int kHeadCo = 16;        // outputs per block (dense nodes, one sample per block)
-constexpr int kHeadMaxC = 1024;    // channels the mean buffer holds
+// Dense and mean-dense heads.  Bound by the latency of their loads, so as many as possible are in flight together, and
+// everything a block needs to know arrives as a kernel parameter (tables in global memory cost a dependent round trip each:
+// item, node, edge).
+// Measured on B200, us per launch, before (one sample and up to 16 outputs per block of 128 threads, tables in global memory)
+// -> now: 784 -> 128 fp32 at one sample 6.9 -> 2.5; 8192 -> 10 bf16 at one sample 18.3 -> 4.2, at 128 samples beside the
+// tensor-core kernel 41 -> 20; mean of 8 x 8 x 256, then 256 -> 43, at 128 samples beside that kernel 71 -> 19.5.
+constexpr int kHeadThreads = 256, kHeadWarps = kHeadThreads / 32;
+constexpr int kHeadMaxC = 1024;    // channels of a node's mean-dense sources together
 
-// Dense node, one sample and kHeadCo outputs per block.  Every thread keeps a partial sum for each of
-// the block's outputs over its own slice of the reduction index, so the weight loads of all outputs
-// are independent and in flight together (the kernel is bound by load latency, not by arithmetic);
-// a shuffle reduction and one pass through shared memory combine the slices.  A mean-dense edge first
-// reduces the source over its pixels into shared memory (threads run over channels: coalesced NHWC
-// reads).  Source and weight rows are read with 16-byte loads where the length allows it.
-template <typename T>
-__device__ void head_item(const SrDevNode& nd, const SrDevEdge* edges, const SrDirectItem& it, int prev, int cur,
-                          float* out_f32)
+struct HeadParams {
+    int32_t n_nodes, B, t_off, pad_;
+    int32_t first_block[SR_HEAD_NODES + 1];
+    const SrFrameCtl* ctl;
+    SrHeadNode nodes[SR_HEAD_NODES];
+};
+static_assert(sizeof(HeadParams) <= 4000, "kernel parameters");
+
+// Nodes with dense edges only: a block takes CO outputs of S samples; its threads stride over the reduction index in vectors
+// of four, every thread keeps S x CO partial sums (a weight vector serves S samples).  The sums of a warp meet by halving,
+// those of the warps in shared memory in a fixed order.
+template <typename T, int S, int CO>
+__global__ void __launch_bounds__(kHeadThreads) sr_head_kernel(const __grid_constant__ HeadParams P)
 {
-    __shared__ float mean[kHeadMaxC];
-    __shared__ float part[4 * kWarps * 32];
-    __shared__ float red[kWarps][kHeadCo];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
-    const int b = it.b0, co0 = it.p0;
-    const int nco = min(it.pad_ >> 8, nd.C - co0);      // outputs of this block (at most kHeadCo)
-    float acc[kHeadCo];
+    __shared__ float red[kHeadWarps][32];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const long long t = P.ctl->t + P.t_off, run_t = P.ctl->run_t + P.t_off;      // this launch computes frame t+1 from frame t
+    float* const out_base = P.ctl->out_base;
+    const long long out_stride = P.ctl->out_stride;
+    int ni = 0;
+    while (ni + 1 < P.n_nodes && (int)blockIdx.x >= P.first_block[ni + 1]) ++ni;
+    const SrHeadNode& nd = P.nodes[ni];
+    const int co_blocks = (nd.C + CO - 1) / CO, bi = (int)blockIdx.x - P.first_block[ni], b0 = (bi / co_blocks) * S, co0 = (bi % co_blocks) * CO;
+    const int nco = min(CO, nd.C - co0), prev = (int)(t & 1), cur = prev ^ 1;
+    float acc[S][CO];
 #pragma unroll
-    for (int o = 0; o < kHeadCo; ++o) acc[o] = 0.f;
+    for (int s = 0; s < S; ++s)
+#pragma unroll
+        for (int o = 0; o < CO; ++o) acc[s][o] = 0.f;
     for (int ei = 0; ei < nd.n_edges; ++ei) {
-        const SrDevEdge& e = edges[nd.first_edge + ei];
-        const int HW = e.Hs * e.Ws, Kx = HW * e.Cs;
-        const T* src = static_cast<const T*>(e.src[e.R ? prev : cur]) + (size_t)b * Kx;
-        const float* w0 = e.w + (size_t)co0 * e.K;
-        if (e.kind == SR_EDGE_MEAN_DENSE) {
-            // the sums run in a fixed order (no atomics), so a frame update is bit-reproducible
-            __syncthreads();
-            if ((e.Cs & 3) == 0 && e.Cs / 4 <= (int)blockDim.x) {
-                // groups of Cs/4 threads share the pixels; a group's partial sums take one row of part[][Cs]
-                // (groups * Cs <= 4 * blockDim.x floats), the rows are then added in group order
-                const int vc = e.Cs / 4, groups = blockDim.x / vc;
-                const int col = tid % vc, grp = tid / vc;
-                if (grp < groups) {
-                    float s4[4] = {0.f, 0.f, 0.f, 0.f};
-                    for (int p = grp; p < HW; p += groups) {
-                        float x[4];
-                        load4(src + (size_t)p * e.Cs + 4 * col, x);
+        const SrHeadEdge& e = nd.edges[ei];
+        const int K = e.K;
+        const T* x[S];
+        const float* w[CO];
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) s4[q] += x[q];
+        for (int s = 0; s < S; ++s) x[s] = static_cast<const T*>(e.src[e.R ? prev : cur]) + (size_t)min(b0 + s, P.B - 1) * K;   // samples and rows beyond
+#pragma unroll
+        for (int o = 0; o < CO; ++o) w[o] = e.w + (size_t)(co0 + min(o, nco - 1)) * K;                                          // the last repeat it
+        if ((K & 3) == 0) {
+#pragma unroll(S == 1 ? 4 : 1)
+            for (int k = 4 * tid; k < K; k += 4 * kHeadThreads) {
+                float4 wv[CO];
+                float xv[S][4];
+#pragma unroll
+                for (int s = 0; s < S; ++s) load4(x[s] + k, xv[s]);
+#pragma unroll
+                for (int o = 0; o < CO; ++o) wv[o] = __ldg(reinterpret_cast<const float4*>(w[o] + k));
+#pragma unroll
+                for (int o = 0; o < CO; ++o)
+#pragma unroll
+                    for (int s = 0; s < S; ++s) {
+                        acc[s][o] = fmaf(wv[o].x, xv[s][0], acc[s][o]); acc[s][o] = fmaf(wv[o].y, xv[s][1], acc[s][o]);
+                        acc[s][o] = fmaf(wv[o].z, xv[s][2], acc[s][o]); acc[s][o] = fmaf(wv[o].w, xv[s][3], acc[s][o]);
                     }
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) part[grp * e.Cs + 4 * col + q] = s4[q];
-                }
-                __syncthreads();
-                for (int c = tid; c < e.Cs; c += blockDim.x) {
-                    float m = 0.f;
-                    for (int gq = 0; gq < groups; ++gq) m += part[gq * e.Cs + c];
-                    mean[c] = m;
-                }
-            } else {
-                for (int c = tid; c < e.Cs; c += blockDim.x) {
-                    float m = 0.f;
-                    for (int p = 0; p < HW; ++p) m += to_f(src[(size_t)p * e.Cs + c]);
-                    mean[c] = m;
-                }
-            }
-            __syncthreads();
-            const float inv = 1.f / (float)HW;
-            for (int c = tid; c < e.Cs; c += blockDim.x) {
-                const float m = mean[c] * inv;
-#pragma unroll
-                for (int o = 0; o < kHeadCo; ++o)
-                    if (o < nco) acc[o] = fmaf(w0[(size_t)o * e.K + c], m, acc[o]);
-            }
-        } else if ((Kx & 3) == 0) {
-            // all blocks of a launch walk the same weight rows: every block starts at another step (its sample index),
-            // so that they do not all ask the same L2 lines at the same moment
-            const int stride = 4 * (int)blockDim.x, steps = (Kx + stride - 1) / stride;
-            for (int s = 0; s < steps; ++s) {
-                const int k = 4 * tid + ((s + b) % steps) * stride;
-                if (k >= Kx) continue;
-                float x[4];
-                load4(src + k, x);
-#pragma unroll
-                for (int o = 0; o < kHeadCo; ++o) {
-                    if (o < nco) {
-                        const float4 w = *reinterpret_cast<const float4*>(w0 + (size_t)o * e.K + k);
-                        acc[o] = fmaf(w.x, x[0], acc[o]); acc[o] = fmaf(w.y, x[1], acc[o]);
-                        acc[o] = fmaf(w.z, x[2], acc[o]); acc[o] = fmaf(w.w, x[3], acc[o]);
-                    }
-                }
             }
         } else {
-            for (int k = tid; k < Kx; k += blockDim.x) {
-                const float x = to_f(src[k]);
+            for (int k = tid; k < K; k += kHeadThreads)
 #pragma unroll
-                for (int o = 0; o < kHeadCo; ++o)
-                    if (o < nco) acc[o] = fmaf(w0[(size_t)o * e.K + k], x, acc[o]);
-            }
+                for (int o = 0; o < CO; ++o) {
+                    const float wk = __ldg(w[o] + k);
+#pragma unroll
+                    for (int s = 0; s < S; ++s) acc[s][o] = fmaf(wk, to_f(x[s][k]), acc[s][o]);
+                }
         }
     }
+    // sums over the lanes: while more than one value is left, the step with distance d keeps the half that matches the lane's
+    // bit d; then plain butterflies.  Lane l ends with value l / (32 / (S * CO)).
+    constexpr int N = S * CO;
+    static_assert(N <= 32 && (N & (N - 1)) == 0, "lane layout");
+    float v[N];
 #pragma unroll
-    for (int o = 0; o < kHeadCo; ++o) {
-        float v = acc[o];
+    for (int i = 0; i < N; ++i) v[i] = acc[i / CO][i % CO];
 #pragma unroll
-        for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-        if (lane == 0) red[warp][o] = v;
+    for (int d = 16, n = N; d > 0; d >>= 1) {
+        if (n > 1) {
+            n >>= 1;
+            const bool up = (lane & d) != 0;
+#pragma unroll
+            for (int i = 0; i < N / 2; ++i)
+                if (i < n) {
+                    const float keep = up ? v[i + n] : v[i], send = up ? v[i] : v[i + n];
+                    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, d);
+                }
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], d);
+        }
     }
+    if (lane % (32 / N) == 0) red[warp][lane / (32 / N)] = v[0];
     __syncthreads();
-    if (tid < nco) {
-        float z = nd.bias[co0 + tid];
+    if (tid < N) {
+        const int b = b0 + tid / CO, o = tid % CO;
+        if (o < nco && b < P.B) {
+            float z = nd.bias[co0 + o];
 #pragma unroll
-        for (int w = 0; w < kWarps; ++w) z += red[w][tid];
-        if (nd.act == 1) z = fmaxf(z, 0.f);
-        from_f(static_cast<T*>(nd.state[cur]) + (size_t)b * nd.C + co0 + tid, z);
-        if (out_f32) out_f32[(size_t)b * nd.C + co0 + tid] = z;
+            for (int q = 0; q < kHeadWarps; ++q) z += red[q][tid];
+            if (nd.act == 1) z = fmaxf(z, 0.f);
+            from_f(static_cast<T*>(nd.state[cur]) + (size_t)b * nd.C + co0 + o, z);
+            if (nd.is_output && out_base) out_base[run_t * out_stride + (size_t)b * nd.C + co0 + o] = z;
+        }
+    }
+}
+
+// Nodes with a mean-dense edge: a block takes one sample.  First the means of the sources (groups of Cs / 4 threads share the
+// pixels, the groups' sums are added in group order), then every warp takes outputs by itself.
+template <typename T>
+__global__ void __launch_bounds__(kHeadThreads) sr_mean_head_kernel(const __grid_constant__ HeadParams P)
+{
+    __shared__ __align__(16) float mean[kHeadMaxC];
+    __shared__ float part[4 * kHeadThreads];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const long long t = P.ctl->t + P.t_off, run_t = P.ctl->run_t + P.t_off;
+    float* const out_base = P.ctl->out_base;
+    const long long out_stride = P.ctl->out_stride;
+    int ni = 0;
+    while (ni + 1 < P.n_nodes && (int)blockIdx.x >= P.first_block[ni + 1]) ++ni;
+    const SrHeadNode& nd = P.nodes[ni];
+    const int b = (int)blockIdx.x - P.first_block[ni], prev = (int)(t & 1), cur = prev ^ 1;
+    int m_off = 0;
+    for (int ei = 0; ei < nd.n_edges; ++ei) {
+        const SrHeadEdge& e = nd.edges[ei];
+        if (e.kind != SR_EDGE_MEAN_DENSE) continue;
+        const int vc = e.Cs / 4, groups = kHeadThreads / vc, col = tid % vc, grp = tid / vc;
+        if (grp < groups) {
+            const T* xs = static_cast<const T*>(e.src[e.R ? prev : cur]) + (size_t)b * e.HW * e.Cs + 4 * col;
+            float s4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+            for (int px = grp; px < e.HW; px += groups) {
+                float x[4];
+                load4(xs + (size_t)px * e.Cs, x);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) s4[q] += x[q];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) part[grp * e.Cs + 4 * col + q] = s4[q];
+        }
+        __syncthreads();
+        const float inv = 1.f / (float)e.HW;
+        for (int c = tid; c < e.Cs; c += kHeadThreads) {
+            float m = 0.f;
+            for (int gq = 0; gq < groups; ++gq) m += part[gq * e.Cs + c];
+            mean[m_off + c] = m * inv;
+        }
+        __syncthreads();
+        m_off += e.Cs;
+    }
+    for (int o = warp; o < nd.C; o += kHeadWarps) {
+        float a = 0.f;
+        m_off = 0;
+        for (int ei = 0; ei < nd.n_edges; ++ei) {
+            const SrHeadEdge& e = nd.edges[ei];
+            const float* w = e.w + (size_t)o * e.K;
+            if (e.kind == SR_EDGE_MEAN_DENSE) {
+#pragma unroll 2
+                for (int c = 4 * lane; c < e.Cs; c += 128) {
+                    const float4 q = __ldg(reinterpret_cast<const float4*>(w + c)), m = *reinterpret_cast<const float4*>(mean + m_off + c);
+                    a = fmaf(q.x, m.x, a); a = fmaf(q.y, m.y, a); a = fmaf(q.z, m.z, a); a = fmaf(q.w, m.w, a);
+                }
+                m_off += e.Cs;
+            } else {
+                const T* x = static_cast<const T*>(e.src[e.R ? prev : cur]) + (size_t)b * e.K;
+#pragma unroll 4
+                for (int k = lane; k < e.K; k += 32) a = fmaf(__ldg(w + k), to_f(x[k]), a);
+            }
+        }
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) a += __shfl_xor_sync(0xffffffffu, a, d);
+        if (lane == 0) {
+            float z = a + nd.bias[o];
+            if (nd.act == 1) z = fmaxf(z, 0.f);
+            from_f(static_cast<T*>(nd.state[cur]) + (size_t)b * nd.C + o, z);
+            if (nd.is_output && out_base) out_base[run_t * out_stride + (size_t)b * nd.C + o] = z;
+        }
     }
 }
 
@@ -289,12 +361,8 @@ sr_direct_group_kernel(const SrDevNode* __restrict__ nodes, const SrDevEdge* __r
     const int prev = (int)(t & 1), cur = prev ^ 1;
     float* out = nullptr;
     if (nd.is_output && ctl->out_base) out = ctl->out_base + (ctl->run_t + t_off) * ctl->out_stride;
-    if (nd.H == 1 && nd.W == 1 && edges[nd.first_edge].kind != SR_EDGE_CONV) {
-        if ((it.pad_ & 0xFF) == 1) head_item<T>(nd, edges, it, prev, cur, out);
-        else dense_item<T>(nd, edges, it, prev, cur, B, out);
-    }
-    else
-        conv_item<T>(nd, edges, it, prev, cur, out);
+    if (nd.H == 1 && nd.W == 1 && edges[nd.first_edge].kind != SR_EDGE_CONV) dense_item<T>(nd, edges, it, prev, cur, B, out);
+    else conv_item<T>(nd, edges, it, prev, cur, out);
 }
 
 // Frame input: the input nodes' frame-(t+1) state is the caller's frame.
@@ -335,10 +403,10 @@ __global__ void sr_advance_kernel(SrFrameCtl* ctl, int n)
 
 }  // namespace
 
-void sr_launch_direct_group(const sr_graph* g, int group, int t_off, cudaStream_t s)
+int sr_launch_direct_group(const sr_graph* g, int group, int t_off, cudaStream_t s)
 {
     const int n = g->group_item_count[group];
-    if (n == 0) return;
+    if (n == 0) return 0;
     const SrDevNode* nodes = reinterpret_cast<const SrDevNode*>(g->ws + g->r_nodes.offset);
     const SrDevEdge* edges = reinterpret_cast<const SrDevEdge*>(g->ws + g->r_edges.offset);
     const SrDirectItem* items = reinterpret_cast<const SrDirectItem*>(g->ws + g->r_items.offset) + g->group_item_offset[group];
@@ -347,6 +415,52 @@ void sr_launch_direct_group(const sr_graph* g, int group, int t_off, cudaStream_
         sr_direct_group_kernel<__nv_bfloat16><<<n, kWarps * 32, 0, s>>>(nodes, edges, items, ctl, t_off, g->batch);
     else
         sr_direct_group_kernel<float><<<n, kWarps * 32, 0, s>>>(nodes, edges, items, ctl, t_off, g->batch);
+    return 1;
+}
+
+int sr_launch_heads(const sr_graph* g, int group, int t_off, cudaStream_t s)
+{
+    int launches = 0;
+    for (int cls = 0; cls < 2; ++cls) {                                      // 0: nodes with a mean-dense edge, 1: without
+        // Dense nodes: with 16 samples or more a block takes 4 x 8 (samples x outputs), with fewer 1 x 2, which spreads a small
+        // batch over more blocks and keeps four steps of the reduction in flight.
+        const bool wide = g->batch >= 16;
+        const int S = cls == 0 ? 1 : (wide ? 4 : 1), CO = cls == 0 ? 1 << 30 : (wide ? 8 : 2);
+        HeadParams P;
+        P.B = g->batch;
+        P.t_off = t_off;
+        P.pad_ = 0;
+        P.ctl = reinterpret_cast<const SrFrameCtl*>(g->ws + g->r_ctl.offset);
+        P.n_nodes = 0;
+        int blocks = 0;
+        auto flush = [&]() {
+            if (P.n_nodes == 0) return;
+            const bool bf = g->dtype == SR_DTYPE_BF16;
+            if (cls == 0) {
+                if (bf) sr_mean_head_kernel<__nv_bfloat16><<<blocks, kHeadThreads, 0, s>>>(P);
+                else sr_mean_head_kernel<float><<<blocks, kHeadThreads, 0, s>>>(P);
+            } else if (wide) {
+                if (bf) sr_head_kernel<__nv_bfloat16, 4, 8><<<blocks, kHeadThreads, 0, s>>>(P);
+                else sr_head_kernel<float, 4, 8><<<blocks, kHeadThreads, 0, s>>>(P);
+            } else {
+                if (bf) sr_head_kernel<__nv_bfloat16, 1, 2><<<blocks, kHeadThreads, 0, s>>>(P);
+                else sr_head_kernel<float, 1, 2><<<blocks, kHeadThreads, 0, s>>>(P);
+            }
+            ++launches;
+            P.n_nodes = 0;
+            blocks = 0;
+        };
+        for (const SrHeadNode& h : g->group_heads[group]) {
+            if ((h.has_mean ? 0 : 1) != cls) continue;
+            P.nodes[P.n_nodes] = h;
+            P.first_block[P.n_nodes++] = blocks;
+            blocks += (g->batch + S - 1) / S * (cls == 0 ? 1 : (h.C + CO - 1) / CO);
+            P.first_block[P.n_nodes] = blocks;
+            if (P.n_nodes == SR_HEAD_NODES) flush();
+        }
+        flush();
+    }
+    return launches;
 }
 
 void sr_launch_input(const sr_graph* g, const int* input_nodes_dev, int t_off, cudaStream_t s)
@@ -376,5 +490,19 @@ void sr_launch_advance(const sr_graph* g, int n, cudaStream_t s)
 int sr_direct_conv_pixels_per_block() { return kWarps * kPix; }
 int sr_direct_dense_outputs_per_block() { return kWarps; }
 int sr_direct_dense_samples_per_block() { return kDenseB; }
-int sr_direct_head_outputs_per_block() { return kHeadCo; }
-int sr_direct_head_max_channels() { return kHeadMaxC; }
+
+// Can the head kernels take the node?
+bool sr_head_takes(const sr_graph* g, int v)
+{
+    const SrHostNode& n = g->nodes[v];
+    if (n.in_edges.size() > SR_HEAD_EDGES) return false;
+    int channels = 0;
+    for (int e : n.in_edges) {
+        const SrHostEdge& he = g->edges[e];
+        if (he.d.kind != SR_EDGE_MEAN_DENSE) continue;
+        const int cs = g->nodes[he.d.src].d.c;
+        if (cs % 4 != 0) return false;
+        channels += cs;
+    }
+    return channels <= kHeadMaxC;
+}

@@ -40,6 +40,22 @@ struct SrDirectItem {
     int32_t pad_;
 };
 
+// Dense / mean-dense nodes as the head kernels see them: passed as kernel parameters.
+#define SR_HEAD_EDGES 6
+#define SR_HEAD_NODES 8
+struct SrHeadEdge {
+    const void* src[2];
+    const float* w;              // [C_out][K]
+    int32_t HW, Cs, kind, R, K, pad_;
+};
+struct SrHeadNode {
+    void* state[2];
+    const float* bias;
+    int32_t C, act, is_output, n_edges;
+    int32_t has_mean, pad_[3];
+    SrHeadEdge edges[SR_HEAD_EDGES];
+};
+
 // Frame control block in device memory: lets a recorded launch sequence be replayed for later frames.
 struct SrFrameCtl {
     int64_t t;                            // frame updates completed since reset
@@ -100,6 +116,8 @@ struct sr_graph {
     std::vector<int> group_item_count;
     std::vector<SrDirectItem> items;
     std::vector<int> group_item_offset;
+    std::vector<std::vector<int>> group_head_nodes;       // per group: nodes of the head kernels
+    std::vector<std::vector<SrHeadNode>> group_heads;     // and what they need to know about them (filled when a workspace is bound)
     // dynamic state
     int64_t t = 0;
     int64_t launches = 0;

@@ -429,8 +429,8 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
         }
     } else if (warp == 0) {
         // ---------------------------------------------------------------- weight producer
-        // (One elected thread per producer: what a ring slot costs between its release and its next copy is the latency of
-        // this loop, and the loop is a third shorter without the warp-wide votes.)
+        // (One elected thread per producer, no warp-wide votes: what a ring slot costs between its release and its next copy is
+        // the latency of this loop.)
         if (elect_one()) {
             uint32_t n = 0, s = 0, ph = 1;                        // copies started; next slot, parity of its release
             const uint32_t n_w = (uint32_t)P.n_w, w_slot = (uint32_t)P.w_slot;

@@ -217,3 +217,21 @@ def test_edges_that_bridge_several_frames_run_as_chains_of_copy_nodes(dtype):
     assert parity.rel_err(out.cpu().numpy().reshape(want[o][1:].shape), want[o][1:]) <= tol
     for v in range(len(g.nodes)):
         assert parity.rel_err(G.get_state(v).float().cpu().numpy(), want[v][g.frames]) <= tol, g.nodes[v].name
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("batch", [1, 15, 16, 19])
+@pytest.mark.parametrize("c_mid,c_out", [(9, 1), (32, 17)])
+def test_heads_at_the_edges_of_their_blocks(batch, c_mid, c_out, dtype):
+    # dense nodes take 4 samples x 8 outputs per block from 16 samples on, 1 x 2 below; reductions of 4 x 4 x 12 = 192, of 1100
+    # (more than one step of 256 threads) and of c_mid (not a multiple of four: scalar loads); a node with a mean-dense
+    # edge sums two means and a dense edge.  Tolerance: that of the element type, as everywhere.
+    from workloads.graphs import CONV, DENSE, GAP_DENSE, IDENTITY, Edge, GraphSpec, Node, check_shapes
+    nodes = [Node("in", 4, 4, 12, IDENTITY), Node("flat", 1, 1, 1100, IDENTITY), Node("a", 1, 1, c_mid), Node("m", 1, 1, 6), Node("o", 1, 1, c_out, IDENTITY)]
+    edges = [Edge(0, 2, DENSE), Edge(1, 2, DENSE), Edge(2, 2, DENSE), Edge(0, 3, GAP_DENSE), Edge(1, 3, DENSE), Edge(0, 3, GAP_DENSE),
+             Edge(2, 4, DENSE), Edge(3, 4, DENSE)]
+    g = GraphSpec("heads", nodes, edges, batch=batch, frames=3, dtype=dtype, seed=88)
+    check_shapes(g)
+    g.patterns = {"p": [1] * 8, "q": [0, 1, 1, 0, 0, 1, 0, 0]}
+    for p in g.patterns:
+        parity.check_stepwise(g, p, zero_bias=False, resident=False)
