@@ -124,12 +124,21 @@ sr_status plan(sr_graph* g)
     if ((int)g->input_nodes.size() > SR_MAX_INPUTS) return SR_ERR_UNSUPPORTED;
     if (g->opt_engine == 0 && g->dtype == SR_DTYPE_BF16) sr_tc_select_nodes(g);
     size_t off = 0;
+    // what a reset zeroes comes first, in one piece
+    g->r_clear.offset = off;
+    g->r_flags = take(off, 256);
+    for (int v = 0; v < n_nodes; ++v)
+        if (!g->nodes[v].is_input) g->nodes[v].state[0] = take(off, node_elems(g, v) * g->elem);
+    g->r_clear.bytes = off - g->r_clear.offset;
     for (int v = 0; v < n_nodes; ++v) {
         SrHostNode& n = g->nodes[v];
-        n.state[0] = take(off, node_elems(g, v) * g->elem);
+        if (n.is_input) n.state[0] = take(off, node_elems(g, v) * g->elem);
         n.state[1] = take(off, node_elems(g, v) * g->elem);
         n.bias = take(off, (size_t)n.d.c * sizeof(float));
     }
+    g->input_read = 0;
+    for (int e = 0; e < n_edges; ++e)
+        if (g->nodes[g->edges[e].d.src].is_input && !sr_tc_stages(g, e)) g->input_read |= 1u << g->nodes[g->edges[e].d.src].input_slot;
     for (int e = 0; e < n_edges; ++e) {
         SrHostEdge& he = g->edges[e];
         const SrHostNode& t = g->nodes[he.d.tgt];
@@ -138,7 +147,7 @@ sr_status plan(sr_graph* g)
     }
     g->r_nodes = take(off, sizeof(SrDevNode) * n_nodes);
     g->r_edges = take(off, sizeof(SrDevEdge) * n_edges);
-    g->r_ctl = take(off, sizeof(SrFrameCtl) + sizeof(int) * SR_MAX_INPUTS);
+    g->r_ctl = take(off, sizeof(SrFrameCtl));
     // work lists of the direct kernels, one contiguous range per group
     g->items.clear();
     g->group_item_offset.clear();
@@ -201,17 +210,14 @@ sr_status ready(const sr_graph* g)
     return SR_OK;
 }
 
-const int* input_list_dev(const sr_graph* g)
-{
-    return reinterpret_cast<const int*>(g->ws + g->r_ctl.offset + sizeof(SrFrameCtl));
-}
-
-// Queue the kernels of `frames` consecutive frame updates; returns the number of launches.
-int enqueue_frames(sr_graph* g, int first_off, int frames, cudaStream_t s)
+// Queue the kernels of `frames` consecutive frame updates, the first of them the one `fr` describes; returns the number of
+// launches.  copies, stems_R: what sr_launch_input does for every frame.
+int enqueue_frames(sr_graph* g, const SrFrameArgs& fr, int frames, cudaStream_t s, unsigned copies = ~0u, unsigned stems_R = 3u)
 {
     int launches = 0;
     SideStream* side = g->opt_overlap ? side_of(g) : nullptr;
-    for (int f = first_off; f < first_off + frames; ++f) {
+    g->frame = fr;
+    for (int f = 0; f < frames; ++f, ++g->frame.off) {
         bool forked = false;
         auto fork = [&]() {
             if (!forked) {
@@ -227,23 +233,20 @@ int enqueue_frames(sr_graph* g, int first_off, int frames, cudaStream_t s)
                 forked = false;
             }
         };
-        // frame input: on the side stream if this frame's update does not read it
-        cudaStream_t in_stream = s;
-        if (side && !g->input_feeds_same_frame) {
-            fork();
-            in_stream = side->stream;
-        }
-        sr_launch_input(g, input_list_dev(g), f, in_stream);
-        ++launches;
-        launches += sr_tc_stage_inputs(g, f, in_stream);
+        // frame input: on the side stream if this frame's update does not read it, queued behind the first group's tensor-core
+        // kernel (whose CTAs each need most of an SM)
+        const bool input_beside = side && !g->input_feeds_same_frame;
+        if (input_beside) fork();
+        else launches += sr_launch_input(g, g->frame, copies, stems_R, false, s);
         for (int gi = 0; gi < (int)g->groups.size(); ++gi) {
             // up to three independent launches: the heads go beside whatever else the group has, the other CUDA-core nodes
             // beside the tensor-core kernel
             const bool has_heads = !g->group_heads[gi].empty(), has_items = g->group_item_count[gi] > 0, has_tc = sr_tc_group_has_work(g, gi);
             if (side && ((has_heads && (has_items || has_tc)) || (has_items && has_tc))) fork();
-            if (has_heads) launches += sr_launch_heads(g, gi, f, side && (has_items || has_tc) ? side->stream : s);
-            if (has_items) launches += sr_launch_direct_group(g, gi, f, side && has_tc ? side->stream : s);
-            launches += sr_tc_launch_group(g, gi, f, s);
+            launches += sr_tc_launch_group(g, gi, s);
+            if (gi == 0 && input_beside) launches += sr_launch_input(g, g->frame, copies, stems_R, true, side->stream);
+            if (has_heads) launches += sr_launch_heads(g, gi, side && (has_items || has_tc) ? side->stream : s);
+            if (has_items) launches += sr_launch_direct_group(g, gi, side && has_tc ? side->stream : s);
             if (gi + 1 < (int)g->groups.size()) join();       // the next group reads what this one wrote
         }
         join();
@@ -265,15 +268,27 @@ SrFrameCtl make_ctl(const sr_graph* g, const void* const* in, bool sequence, flo
     return c;
 }
 
-// What the launch path derives from the input nodes' current state (staged few-channel edges) is brought up to
-// date after a resident run.
+SrFrameArgs by_value(const SrFrameCtl& c) { return SrFrameArgs{nullptr, 0, c}; }
+
+// The staged copies of the input nodes' current state that the next update reads (edges with R = 1), from the state itself.
+void stage_current(sr_graph* g, cudaStream_t s)
+{
+    SrFrameCtl c{};
+    c.t = g->t - 1;                                              // "the input of frame t"
+    for (size_t i = 0; i < g->input_nodes.size(); ++i) c.in_base[i] = g->ws + g->nodes[g->input_nodes[i]].state[g->t & 1].offset;
+    g->launches += sr_launch_input(g, by_value(c), 0u, 2u, false, s);
+}
+
+// After a resident run they are brought up to date when the launch path is used next.
 void refresh_staging(sr_graph* g, cudaStream_t s)
 {
-    if (g->stage_dirty) {
-        g->launches += sr_tc_after_state_change(g, s);
-        g->stage_dirty = false;
-    }
+    if (g->stage_dirty) stage_current(g, s);
+    g->stage_dirty = false;
 }
+
+// The states of the last window are the current ones of this graph; an update of all nodes supersedes them.  (It does not read
+// them: windows exist only for patterns in which every edge that bridges a frame leaves an input node.)
+void leave_window(sr_graph* g) { g->in_window.assign(g->in_window.size(), 0); }
 
 }  // namespace
 
@@ -500,11 +515,6 @@ sr_status sr_graph_bind_workspace(sr_graph* g, void* workspace_dev, size_t bytes
         !cuda_ok(cudaMemcpy(ws + g->r_items.offset, g->items.data(), sizeof(SrDirectItem) * g->items.size(),
                             cudaMemcpyHostToDevice)))
         return SR_ERR_CUDA;
-    std::vector<int> il(SR_MAX_INPUTS, 0);
-    for (size_t i = 0; i < g->input_nodes.size(); ++i) il[i] = g->input_nodes[i];
-    if (!cuda_ok(cudaMemcpy(ws + g->r_ctl.offset + sizeof(SrFrameCtl), il.data(), sizeof(int) * SR_MAX_INPUTS,
-                            cudaMemcpyHostToDevice)))
-        return SR_ERR_CUDA;
     g->group_heads.assign(g->groups.size(), {});
     for (size_t gi = 0; gi < g->groups.size(); ++gi)
         for (int v : g->group_head_nodes[gi]) {
@@ -527,8 +537,10 @@ sr_status sr_graph_bind_workspace(sr_graph* g, void* workspace_dev, size_t bytes
             }
             g->group_heads[gi].push_back(h);
         }
+    g->stems.clear();
     g->ws = ws;
     st = sr_tc_bind(g);
+    if (st == SR_OK && g->info.n_tensor_core_nodes > 0 && (!sr_input_share_sm() || !sr_direct_share_sm())) st = SR_ERR_CUDA;
     if (st == SR_OK) st = sr_rs_bind(g);
     if (st == SR_OK) st = sr_dn_bind(g);
     if (st != SR_OK) {
@@ -536,6 +548,7 @@ sr_status sr_graph_bind_workspace(sr_graph* g, void* workspace_dev, size_t bytes
         return st;
     }
     g->t = 0;
+    g->in_window.assign(g->nodes.size(), 0);
     return SR_OK;
 }
 
@@ -644,25 +657,22 @@ sr_status sr_graph_reset(sr_graph* g, const void* const* in0_dev, void* stream)
     if (!g || !in0_dev) return SR_ERR_INVALID_ARG;
     if (g->batch <= 0 || !g->ws) return SR_ERR_STATE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    for (int v = 0; v < (int)g->nodes.size(); ++v) {
-        const SrHostNode& n = g->nodes[v];
-        const size_t bytes = node_elems(g, v) * g->elem;
-        if (n.is_input) {
-            if (!in0_dev[n.input_slot]) return SR_ERR_INVALID_ARG;
-            if (!cuda_ok(cudaMemcpyAsync(g->ws + n.state[0].offset, in0_dev[n.input_slot], bytes,
-                                         cudaMemcpyDeviceToDevice, s)))
-                return SR_ERR_CUDA;
-            if (!cuda_ok(cudaMemsetAsync(g->ws + n.state[1].offset, 0, bytes, s))) return SR_ERR_CUDA;
-        } else {
-            if (!cuda_ok(cudaMemsetAsync(g->ws + n.state[0].offset, 0, bytes, s))) return SR_ERR_CUDA;
-            if (!cuda_ok(cudaMemsetAsync(g->ws + n.state[1].offset, 0, bytes, s))) return SR_ERR_CUDA;
-        }
-    }
-    // a reported device-side error (an expired wait) is cleared here: the rollout starts over
-    if (!cuda_ok(cudaMemsetAsync(g->ws + g->r_ctl.offset + offsetof(SrFrameCtl, error), 0, sizeof(int32_t), s))) return SR_ERR_CUDA;
+    for (size_t i = 0; i < g->input_nodes.size(); ++i)
+        if (!in0_dev[i]) return SR_ERR_INVALID_ARG;
+    // One memset: the non-input states of frame 0 (those of the other parity are written before they are read), a reported
+    // device-side error (an expired wait: the rollout starts over) and the shared work list's counters (every launch leaves
+    // them at zero; this covers a launch cut short).
+    if (!cuda_ok(cudaMemsetAsync(g->ws + g->r_clear.offset, 0, g->r_clear.bytes, s))) return SR_ERR_CUDA;
+    if (g->window && g->window->ws && !cuda_ok(cudaMemsetAsync(g->window->ws + g->window->r_flags.offset, 0, g->window->r_flags.bytes, s)))
+        return SR_ERR_CUDA;
     g->t = 0;
-    g->stage_dirty = false;
-    g->launches += sr_tc_after_state_change(g, s);
+    leave_window(g);
+    SrFrameCtl c{};
+    c.t = -1;                                                    // "the input of frame 0"
+    for (size_t i = 0; i < g->input_nodes.size(); ++i) c.in_base[i] = in0_dev[i];
+    const bool resident = sr_rs_available(g);                    // a resident run does not read staged edges
+    g->launches += sr_launch_input(g, by_value(c), ~0u, resident ? 0u : 2u, false, s);
+    g->stage_dirty = resident;
     return cuda_ok(cudaGetLastError()) ? SR_OK : SR_ERR_CUDA;
 }
 
@@ -675,9 +685,9 @@ sr_status sr_rollout_step(sr_graph* g, const void* const* in_next_dev, float* ou
         if (!in_next_dev[i]) return SR_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     refresh_staging(g, s);
-    sr_launch_set_ctl(g, make_ctl(g, in_next_dev, false, out_dev), s);
-    g->launches += 1 + enqueue_frames(g, 0, 1, s);
+    g->launches += enqueue_frames(g, by_value(make_ctl(g, in_next_dev, false, out_dev)), 1, s);
     g->t += 1;
+    leave_window(g);
     return cuda_ok(cudaGetLastError()) ? SR_OK : SR_ERR_CUDA;
 }
 
@@ -690,6 +700,7 @@ sr_status sr_rollout_run(sr_graph* g, const void* const* in_seq_dev, int T, floa
     for (size_t i = 0; i < g->input_nodes.size(); ++i)
         if (!in_seq_dev[i]) return SR_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
+    leave_window(g);
     if (sr_rs_available(g)) {
         bool aligned = true;                                     // the resident kernel fetches input rows in 4-byte words
         for (size_t i = 0; i < g->input_nodes.size(); ++i)
@@ -718,8 +729,7 @@ sr_status sr_rollout_run(sr_graph* g, const void* const* in_seq_dev, int T, floa
         }
     }
     refresh_staging(g, s);
-    sr_launch_set_ctl(g, make_ctl(g, in_seq_dev, true, out_seq_dev), s);
-    g->launches += 1;
+    SrFrameArgs fr = by_value(make_ctl(g, in_seq_dev, true, out_seq_dev));
     int done = 0;
     const int gf = g->opt_graph_frames;
     if (gf > 0 && T >= gf) {
@@ -737,7 +747,9 @@ sr_status sr_rollout_run(sr_graph* g, const void* const* in_seq_dev, int T, floa
                 return SR_ERR_CUDA;
             cudaGraph_t graph = nullptr;
             if (!cuda_ok(cudaStreamBeginCapture(c->capture_stream, cudaStreamCaptureModeThreadLocal))) return SR_ERR_CUDA;
-            int k = enqueue_frames(g, 0, gf, c->capture_stream);
+            SrFrameArgs rec{};
+            rec.ctl = reinterpret_cast<const SrFrameCtl*>(g->ws + g->r_ctl.offset);
+            int k = enqueue_frames(g, rec, gf, c->capture_stream);
             sr_launch_advance(g, gf, c->capture_stream);
             ++k;
             // a capture that has begun is always ended, also when a launch inside it failed: a stream left in
@@ -758,6 +770,8 @@ sr_status sr_rollout_run(sr_graph* g, const void* const* in_seq_dev, int T, floa
             c->frames = gf;
             c->kernels = k;
         }
+        sr_launch_set_ctl(g, fr.v, s);
+        g->launches += 1;
         while (T - done >= gf) {
             if (!cuda_ok(cudaGraphLaunch(c->exec, s))) return SR_ERR_CUDA;
             g->launches += c->kernels;
@@ -765,10 +779,8 @@ sr_status sr_rollout_run(sr_graph* g, const void* const* in_seq_dev, int T, floa
         }
     }
     if (done < T) {
-        // ctl.t / ctl.run_t already stand at `done` (each graph advanced them); offsets are relative to that
-        g->launches += enqueue_frames(g, 0, T - done, s);
-        sr_launch_advance(g, T - done, s);
-        g->launches += 1;
+        fr.off = done;
+        g->launches += enqueue_frames(g, fr, T - done, s);
     }
     g->t += T;
     return cuda_ok(cudaGetLastError()) ? SR_OK : SR_ERR_CUDA;
@@ -862,7 +874,11 @@ sr_status sr_rollout_window(sr_graph* g, const void* const* in_seq_dev, int W, f
         if (!in_seq_dev[i]) return SR_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     // frames t .. t+W-1 of the input nodes side by side: what edges that bridge a frame read (Eq. 2: frame i - R(e))
+    unsigned bridging = 0;
+    for (const SrHostEdge& e : g->edges)
+        if (e.R == 1) bridging |= 1u << g->nodes[e.d.src].input_slot;
     for (size_t i = 0; i < g->input_nodes.size(); ++i) {
+        if (!((bridging >> i) & 1u)) continue;
         const int v = g->input_nodes[i];
         const size_t frame = node_elems(g, v) * g->elem;
         char* dst = w->ws + w->nodes[v].state[0].offset;
@@ -871,21 +887,19 @@ sr_status sr_rollout_window(sr_graph* g, const void* const* in_seq_dev, int W, f
             return SR_ERR_CUDA;
     }
     w->t = 0;
-    w->stage_dirty = false;
-    w->launches += sr_tc_after_state_change(w, s);
-    // ONE update of the window graph computes all W frames: its batch is [W][B], which is how in_seq and out_seq lie in memory
-    st = sr_rollout_step(w, in_seq_dev, out_seq_dev, stream);
-    if (st != SR_OK) return st;
-    // the last frame of the window becomes the current frame of this graph (Sec. 4: windows chain)
+    if (bridging) stage_current(w, s);
+    // ONE update of the window graph computes all W frames: its batch is [W][B], which is how in_seq and out_seq lie in memory.
+    // Of its input it needs what is read within the frame only.
+    w->launches += enqueue_frames(w, by_value(make_ctl(w, in_seq_dev, false, out_seq_dev)), 1, s, w->input_read, 1u);
+    // the last frame of the window becomes the current frame of this graph (Sec. 4: windows chain); the non-input states stay
+    // where they are (see leave_window)
     const int64_t t_new = g->t + W;
-    for (size_t v = 0; v < g->nodes.size(); ++v) {
-        const size_t frame = node_elems(g, (int)v) * g->elem;
-        char* dst = g->ws + g->nodes[v].state[t_new & 1].offset;
-        const char* src = g->nodes[v].is_input
-                              ? static_cast<const char*>(in_seq_dev[g->nodes[v].input_slot]) + frame * (size_t)(W - 1)
-                              : w->ws + w->nodes[v].state[1].offset + frame * (size_t)(W - 1);
-        if (!cuda_ok(cudaMemcpyAsync(dst, src, frame, cudaMemcpyDeviceToDevice, s))) return SR_ERR_CUDA;
-    }
+    SrFrameCtl c{};
+    c.t = t_new - 1;
+    for (size_t i = 0; i < g->input_nodes.size(); ++i)
+        c.in_base[i] = static_cast<const char*>(in_seq_dev[i]) + node_elems(g, g->input_nodes[i]) * g->elem * (size_t)(W - 1);
+    w->launches += sr_launch_input(g, by_value(c), ~0u, 0u, false, s);
+    for (size_t v = 0; v < g->nodes.size(); ++v) g->in_window[v] = !g->nodes[v].is_input;
     g->t = t_new;
     g->stage_dirty = true;
     g->launches += w->launches;
@@ -897,10 +911,10 @@ sr_status sr_graph_get_state(const sr_graph* g, int node, void* dst_dev, void* s
 {
     if (!g || !dst_dev || node < 0 || node >= (int)g->nodes.size()) return SR_ERR_INVALID_ARG;
     if (g->batch <= 0 || !g->ws) return SR_ERR_STATE;
-    const SrHostNode& n = g->nodes[node];
-    return cuda_ok(cudaMemcpyAsync(dst_dev, g->ws + n.state[g->t & 1].offset, node_elems(g, node) * g->elem,
-                                   cudaMemcpyDeviceToDevice, static_cast<cudaStream_t>(stream)))
-               ? SR_OK : SR_ERR_CUDA;
+    const size_t bytes = node_elems(g, node) * g->elem;
+    const char* src = g->ws + g->nodes[node].state[g->t & 1].offset;
+    if (g->in_window[node]) src = g->window->ws + g->window->nodes[node].state[1].offset + bytes * (size_t)(g->window_frames - 1);
+    return cuda_ok(cudaMemcpyAsync(dst_dev, src, bytes, cudaMemcpyDeviceToDevice, static_cast<cudaStream_t>(stream))) ? SR_OK : SR_ERR_CUDA;
 }
 
 sr_status sr_graph_set_state(sr_graph* g, int node, const void* src_dev, void* stream)
@@ -912,7 +926,8 @@ sr_status sr_graph_set_state(sr_graph* g, int node, const void* src_dev, void* s
     if (!cuda_ok(cudaMemcpyAsync(g->ws + n.state[g->t & 1].offset, src_dev, node_elems(g, node) * g->elem,
                                  cudaMemcpyDeviceToDevice, s)))
         return SR_ERR_CUDA;
-    if (n.is_input) g->launches += sr_tc_after_state_change(g, s);
+    g->in_window[node] = 0;
+    if (n.is_input && !g->stage_dirty) stage_current(g, s);
     return SR_OK;
 }
 
@@ -951,9 +966,9 @@ sr_status sr_graph_sync_status(sr_graph* g, void* stream)
     if (!g) return SR_ERR_INVALID_ARG;
     if (g->batch <= 0 || !g->ws) return SR_ERR_STATE;
     if (!cuda_ok(cudaStreamSynchronize(static_cast<cudaStream_t>(stream)))) return SR_ERR_CUDA;
-    SrFrameCtl c;
-    if (!cuda_ok(cudaMemcpy(&c, g->ws + g->r_ctl.offset, sizeof(c), cudaMemcpyDeviceToHost))) return SR_ERR_CUDA;
-    if (c.error != 0) return SR_ERR_TIMEOUT;
+    int error = 0;
+    if (!cuda_ok(cudaMemcpy(&error, g->ws + g->r_flags.offset, sizeof(error), cudaMemcpyDeviceToHost))) return SR_ERR_CUDA;
+    if (error != 0) return SR_ERR_TIMEOUT;
     return SR_OK;
 }
 

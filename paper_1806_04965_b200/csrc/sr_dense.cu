@@ -248,7 +248,7 @@ __device__ __forceinline__ void dn_unit(const DnBlobHdr* H, const DnUnit& un, fl
 
 template <int CL>
 __global__ void __launch_bounds__(kDnWarps * 32, 1)
-sr_dense_kernel(const DnParams P, SrFrameCtl* __restrict__ ctl_out, const SrFrameCtl init, int T)
+sr_dense_kernel(const DnParams P, const SrFrameCtl init, int T)
 {
     extern __shared__ __align__(16) float dn_smem[];
     // the input nodes as the fetching warps need them: first float of this cluster's sequences in the caller's frame 0
@@ -325,13 +325,6 @@ sr_dense_kernel(const DnParams P, SrFrameCtl* __restrict__ ctl_out, const SrFram
         }
     }
 
-    if (blockIdx.x == 0 && tid == 0) {
-        SrFrameCtl c = init;
-        c.t += T;
-        c.run_t += T;
-        c.error = ctl_out->error;
-        *ctl_out = c;
-    }
     // relative frame T back to the state buffers in global memory (parity of t + T); every rank holds a full copy and
     // writes its share of it
     {
@@ -366,7 +359,7 @@ struct DnEngine {
 
 DnEngine* dn_of(const sr_graph* g) { return static_cast<DnEngine*>(g->dn); }
 
-typedef void (*DnKernel)(const DnParams, SrFrameCtl*, const SrFrameCtl, int);
+typedef void (*DnKernel)(const DnParams, const SrFrameCtl, int);
 
 bool dn_prepare(DnKernel kernel, int cluster, int smem_bytes)
 {
@@ -670,7 +663,6 @@ sr_status sr_dn_launch(sr_graph* g, int T, const SrFrameCtl& init, cudaStream_t 
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    SrFrameCtl* ctl = reinterpret_cast<SrFrameCtl*>(g->ws + g->r_ctl.offset);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     bool timed = g->opt_time_tc != 0 && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
     if (timed && E->ev_used + 2 > E->ev.size()) {
@@ -683,7 +675,7 @@ sr_status sr_dn_launch(sr_graph* g, int T, const SrFrameCtl& init, cudaStream_t 
         if (E->ev_used + 2 > E->ev.size()) timed = false;
     }
     if (timed) cudaEventRecord(E->ev[E->ev_used], s);
-    if (cudaLaunchKernelEx(&cfg, kernel, E->P, ctl, init, T) != cudaSuccess) return SR_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, kernel, E->P, init, T) != cudaSuccess) return SR_ERR_CUDA;
     if (timed) {
         cudaEventRecord(E->ev[E->ev_used + 1], s);
         E->ev_used += 2;

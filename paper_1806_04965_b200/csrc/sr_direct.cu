@@ -176,9 +176,9 @@ constexpr int kHeadThreads = 256, kHeadWarps = kHeadThreads / 32;
 constexpr int kHeadMaxC = 1024;    // channels of a node's mean-dense sources together
 
 struct HeadParams {
-    int32_t n_nodes, B, t_off, pad_;
+    SrFrameArgs fr;
+    int32_t n_nodes, B;
     int32_t first_block[SR_HEAD_NODES + 1];
-    const SrFrameCtl* ctl;
     SrHeadNode nodes[SR_HEAD_NODES];
 };
 static_assert(sizeof(HeadParams) <= 4000, "kernel parameters");
@@ -191,14 +191,13 @@ __global__ void __launch_bounds__(kHeadThreads) sr_head_kernel(const __grid_cons
 {
     __shared__ float red[kHeadWarps][32];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const long long t = P.ctl->t + P.t_off, run_t = P.ctl->run_t + P.t_off;      // this launch computes frame t+1 from frame t
-    float* const out_base = P.ctl->out_base;
-    const long long out_stride = P.ctl->out_stride;
+    const SrFrame F = sr_frame(P.fr);
     int ni = 0;
     while (ni + 1 < P.n_nodes && (int)blockIdx.x >= P.first_block[ni + 1]) ++ni;
     const SrHeadNode& nd = P.nodes[ni];
     const int co_blocks = (nd.C + CO - 1) / CO, bi = (int)blockIdx.x - P.first_block[ni], b0 = (bi / co_blocks) * S, co0 = (bi % co_blocks) * CO;
-    const int nco = min(CO, nd.C - co0), prev = (int)(t & 1), cur = prev ^ 1;
+    const int nco = min(CO, nd.C - co0), prev = (int)(F.t & 1), cur = prev ^ 1;
+    float* const out = nd.is_output ? sr_frame_output(P.fr, F) : nullptr;
     float acc[S][CO];
 #pragma unroll
     for (int s = 0; s < S; ++s)
@@ -272,7 +271,7 @@ __global__ void __launch_bounds__(kHeadThreads) sr_head_kernel(const __grid_cons
             for (int q = 0; q < kHeadWarps; ++q) z += red[q][tid];
             if (nd.act == 1) z = fmaxf(z, 0.f);
             from_f(static_cast<T*>(nd.state[cur]) + (size_t)b * nd.C + co0 + o, z);
-            if (nd.is_output && out_base) out_base[run_t * out_stride + (size_t)b * nd.C + co0 + o] = z;
+            if (out) out[(size_t)b * nd.C + co0 + o] = z;
         }
     }
 }
@@ -285,13 +284,12 @@ __global__ void __launch_bounds__(kHeadThreads) sr_mean_head_kernel(const __grid
     __shared__ __align__(16) float mean[kHeadMaxC];
     __shared__ float part[4 * kHeadThreads];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const long long t = P.ctl->t + P.t_off, run_t = P.ctl->run_t + P.t_off;
-    float* const out_base = P.ctl->out_base;
-    const long long out_stride = P.ctl->out_stride;
+    const SrFrame F = sr_frame(P.fr);
     int ni = 0;
     while (ni + 1 < P.n_nodes && (int)blockIdx.x >= P.first_block[ni + 1]) ++ni;
     const SrHeadNode& nd = P.nodes[ni];
-    const int b = (int)blockIdx.x - P.first_block[ni], prev = (int)(t & 1), cur = prev ^ 1;
+    const int b = (int)blockIdx.x - P.first_block[ni], prev = (int)(F.t & 1), cur = prev ^ 1;
+    float* const out = nd.is_output ? sr_frame_output(P.fr, F) : nullptr;
     int m_off = 0;
     for (int ei = 0; ei < nd.n_edges; ++ei) {
         const SrHeadEdge& e = nd.edges[ei];
@@ -345,7 +343,7 @@ __global__ void __launch_bounds__(kHeadThreads) sr_mean_head_kernel(const __grid
             float z = a + nd.bias[o];
             if (nd.act == 1) z = fmaxf(z, 0.f);
             from_f(static_cast<T*>(nd.state[cur]) + (size_t)b * nd.C + o, z);
-            if (nd.is_output && out_base) out_base[run_t * out_stride + (size_t)b * nd.C + o] = z;
+            if (out) out[(size_t)b * nd.C + o] = z;
         }
     }
 }
@@ -353,72 +351,34 @@ __global__ void __launch_bounds__(kHeadThreads) sr_mean_head_kernel(const __grid
 template <typename T>
 __global__ void __launch_bounds__(kWarps * 32)
 sr_direct_group_kernel(const SrDevNode* __restrict__ nodes, const SrDevEdge* __restrict__ edges,
-                       const SrDirectItem* __restrict__ items, const SrFrameCtl* __restrict__ ctl, int t_off, int B)
+                       const SrDirectItem* __restrict__ items, const __grid_constant__ SrFrameArgs fr, int B)
 {
     const SrDirectItem it = items[blockIdx.x];
     const SrDevNode& nd = nodes[it.node];
-    const long long t = ctl->t + t_off;                   // this launch computes frame t+1 from frame t
-    const int prev = (int)(t & 1), cur = prev ^ 1;
-    float* out = nullptr;
-    if (nd.is_output && ctl->out_base) out = ctl->out_base + (ctl->run_t + t_off) * ctl->out_stride;
+    const SrFrame F = sr_frame(fr);
+    const int prev = (int)(F.t & 1), cur = prev ^ 1;
+    float* out = nd.is_output ? sr_frame_output(fr, F) : nullptr;
     if (nd.H == 1 && nd.W == 1 && edges[nd.first_edge].kind != SR_EDGE_CONV) dense_item<T>(nd, edges, it, prev, cur, B, out);
     else conv_item<T>(nd, edges, it, prev, cur, out);
 }
 
-// Frame input: the input nodes' frame-(t+1) state is the caller's frame.
-__global__ void sr_input_kernel(const SrDevNode* __restrict__ nodes, const int* __restrict__ input_nodes, int n_inputs,
-                                const SrFrameCtl* __restrict__ ctl, int t_off, size_t elem_bytes, int B)
-{
-    const long long t = ctl->t + t_off;
-    const int cur = (int)((t + 1) & 1);
-    for (int i = 0; i < n_inputs; ++i) {
-        const SrDevNode& nd = nodes[input_nodes[i]];
-        const size_t bytes = (size_t)B * nd.H * nd.W * nd.C * elem_bytes;
-        const char* src = static_cast<const char*>(ctl->in_base[i]) + (ctl->run_t + t_off) * ctl->in_stride_bytes[i];
-        char* dst = static_cast<char*>(nd.state[cur]);
-        const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x, nth = (size_t)gridDim.x * blockDim.x;
-        if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0) {
-            const size_t nv = bytes / 16;
-            for (size_t j = tid; j < nv; j += nth)
-                reinterpret_cast<uint4*>(dst)[j] = reinterpret_cast<const uint4*>(src)[j];
-            for (size_t j = nv * 16 + tid; j < bytes; j += nth) dst[j] = src[j];
-        } else {
-            for (size_t j = tid; j < bytes; j += nth) dst[j] = src[j];
-        }
-    }
-}
-
-__global__ void sr_set_ctl_kernel(SrFrameCtl* ctl, SrFrameCtl v)
-{
-    const int err = ctl->error;
-    *ctl = v;
-    ctl->error = err;
-}
-
-__global__ void sr_advance_kernel(SrFrameCtl* ctl, int n)
-{
-    ctl->t += n;
-    ctl->run_t += n;
-}
-
 }  // namespace
 
-int sr_launch_direct_group(const sr_graph* g, int group, int t_off, cudaStream_t s)
+int sr_launch_direct_group(const sr_graph* g, int group, cudaStream_t s)
 {
     const int n = g->group_item_count[group];
     if (n == 0) return 0;
     const SrDevNode* nodes = reinterpret_cast<const SrDevNode*>(g->ws + g->r_nodes.offset);
     const SrDevEdge* edges = reinterpret_cast<const SrDevEdge*>(g->ws + g->r_edges.offset);
     const SrDirectItem* items = reinterpret_cast<const SrDirectItem*>(g->ws + g->r_items.offset) + g->group_item_offset[group];
-    const SrFrameCtl* ctl = reinterpret_cast<const SrFrameCtl*>(g->ws + g->r_ctl.offset);
     if (g->dtype == SR_DTYPE_BF16)
-        sr_direct_group_kernel<__nv_bfloat16><<<n, kWarps * 32, 0, s>>>(nodes, edges, items, ctl, t_off, g->batch);
+        sr_direct_group_kernel<__nv_bfloat16><<<n, kWarps * 32, 0, s>>>(nodes, edges, items, g->frame, g->batch);
     else
-        sr_direct_group_kernel<float><<<n, kWarps * 32, 0, s>>>(nodes, edges, items, ctl, t_off, g->batch);
+        sr_direct_group_kernel<float><<<n, kWarps * 32, 0, s>>>(nodes, edges, items, g->frame, g->batch);
     return 1;
 }
 
-int sr_launch_heads(const sr_graph* g, int group, int t_off, cudaStream_t s)
+int sr_launch_heads(const sr_graph* g, int group, cudaStream_t s)
 {
     int launches = 0;
     for (int cls = 0; cls < 2; ++cls) {                                      // 0: nodes with a mean-dense edge, 1: without
@@ -428,9 +388,7 @@ int sr_launch_heads(const sr_graph* g, int group, int t_off, cudaStream_t s)
         const int S = cls == 0 ? 1 : (wide ? 4 : 1), CO = cls == 0 ? 1 << 30 : (wide ? 8 : 2);
         HeadParams P;
         P.B = g->batch;
-        P.t_off = t_off;
-        P.pad_ = 0;
-        P.ctl = reinterpret_cast<const SrFrameCtl*>(g->ws + g->r_ctl.offset);
+        P.fr = g->frame;
         P.n_nodes = 0;
         int blocks = 0;
         auto flush = [&]() {
@@ -463,30 +421,6 @@ int sr_launch_heads(const sr_graph* g, int group, int t_off, cudaStream_t s)
     return launches;
 }
 
-void sr_launch_input(const sr_graph* g, const int* input_nodes_dev, int t_off, cudaStream_t s)
-{
-    const SrDevNode* nodes = reinterpret_cast<const SrDevNode*>(g->ws + g->r_nodes.offset);
-    const SrFrameCtl* ctl = reinterpret_cast<const SrFrameCtl*>(g->ws + g->r_ctl.offset);
-    size_t most = 0;
-    for (int v : g->input_nodes) {
-        const sr_node_desc& d = g->nodes[v].d;
-        most = std::max(most, (size_t)g->batch * d.h * d.w * d.c * g->elem);
-    }
-    int blocks = (int)std::min<size_t>(296, (most / 16 + 255) / 256 + 1);
-    sr_input_kernel<<<blocks, 256, 0, s>>>(nodes, input_nodes_dev, (int)g->input_nodes.size(), ctl, t_off,
-                                           (size_t)g->elem, g->batch);
-}
-
-void sr_launch_set_ctl(const sr_graph* g, const SrFrameCtl& v, cudaStream_t s)
-{
-    sr_set_ctl_kernel<<<1, 1, 0, s>>>(reinterpret_cast<SrFrameCtl*>(g->ws + g->r_ctl.offset), v);
-}
-
-void sr_launch_advance(const sr_graph* g, int n, cudaStream_t s)
-{
-    sr_advance_kernel<<<1, 1, 0, s>>>(reinterpret_cast<SrFrameCtl*>(g->ws + g->r_ctl.offset), n);
-}
-
 int sr_direct_conv_pixels_per_block() { return kWarps * kPix; }
 int sr_direct_dense_outputs_per_block() { return kWarps; }
 int sr_direct_dense_samples_per_block() { return kDenseB; }
@@ -505,4 +439,11 @@ bool sr_head_takes(const sr_graph* g, int v)
         channels += cs;
     }
     return channels <= kHeadMaxC;
+}
+
+bool sr_direct_share_sm()
+{
+    auto ask = [](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess; };
+    return ask(sr_head_kernel<__nv_bfloat16, 4, 8>) && ask(sr_head_kernel<__nv_bfloat16, 1, 2>) && ask(sr_mean_head_kernel<__nv_bfloat16>) &&
+           ask(sr_direct_group_kernel<__nv_bfloat16>);
 }

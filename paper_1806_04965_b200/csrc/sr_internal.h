@@ -56,7 +56,8 @@ struct SrHeadNode {
     SrHeadEdge edges[SR_HEAD_EDGES];
 };
 
-// Frame control block in device memory: lets a recorded launch sequence be replayed for later frames.
+// What a launch needs to know about its frame.  Plain launches carry it by value; launches recorded in a CUDA graph read it
+// from a control block in device memory, which lets the recorded sequence be replayed for later frames.
 struct SrFrameCtl {
     int64_t t;                            // frame updates completed since reset
     int64_t run_t;                        // frame updates completed inside the current step / run call
@@ -64,9 +65,35 @@ struct SrFrameCtl {
     int64_t in_stride_bytes[SR_MAX_INPUTS];
     float* out_base;                      // output of update run_t goes to out_base + run_t * out_stride (floats); may be null
     int64_t out_stride;
-    int32_t error;                        // first device-side error code (0 = none)
-    int32_t pad_;
 };
+
+struct SrFrameArgs {
+    const SrFrameCtl* ctl;                // null: the values are in v
+    int64_t off;                          // frames to add to t and run_t
+    SrFrameCtl v;
+};
+
+#ifdef __CUDACC__
+struct SrFrame { long long t, run_t; };   // this launch computes frame t+1 from frame t
+__device__ __forceinline__ SrFrame sr_frame(const SrFrameArgs& a)
+{
+    SrFrame f;
+    f.t = (a.ctl ? a.ctl->t : a.v.t) + a.off;
+    f.run_t = (a.ctl ? a.ctl->run_t : a.v.run_t) + a.off;
+    return f;
+}
+__device__ __forceinline__ const char* sr_frame_input(const SrFrameArgs& a, const SrFrame& f, int slot)
+{
+    const char* base = static_cast<const char*>(a.ctl ? a.ctl->in_base[slot] : a.v.in_base[slot]);
+    return base + f.run_t * (a.ctl ? a.ctl->in_stride_bytes[slot] : a.v.in_stride_bytes[slot]);
+}
+// The caller's output buffer for this frame, or null.
+__device__ __forceinline__ float* sr_frame_output(const SrFrameArgs& a, const SrFrame& f)
+{
+    float* base = a.ctl ? a.ctl->out_base : a.v.out_base;
+    return base ? base + f.run_t * (a.ctl ? a.ctl->out_stride : a.v.out_stride) : nullptr;
+}
+#endif
 
 // ------------------------------------------------------------------ host-side graph
 struct SrRegion { size_t offset = 0, bytes = 0; };
@@ -92,6 +119,13 @@ struct SrHostEdge {
     bool w_set = false;
 };
 
+// A few-channel input edge staged as im2col rows (see sr_input.cu).
+struct SrStem {
+    void* dst[2];                  // by frame parity
+    int slot, R;                   // input node (index among the inputs); the edge's R
+    int Hs, Ws, Cs, Ho, Wo, k, stride, pad, Kp, K;
+};
+
 struct sr_graph {
     std::vector<SrHostNode> nodes;
     std::vector<SrHostEdge> edges;
@@ -112,6 +146,10 @@ struct sr_graph {
     bool planned = false;                          // the workspace layout stands for the current options
     char* ws = nullptr;
     SrRegion r_nodes, r_edges, r_ctl, r_items;
+    SrRegion r_clear;                              // what a reset zeroes: the flags, then the non-input nodes' parity-0 states
+    SrRegion r_flags;                              // int 0: device-side error code (0 = none); ints 16, 17: the shared work list's counters
+    std::vector<SrStem> stems;                     // filled when a workspace is bound
+    unsigned input_read = 0;                       // bit i: some edge reads input node i's state itself (not a staged copy)
     std::vector<SrRegion> r_group_items;           // per group
     std::vector<int> group_item_count;
     std::vector<SrDirectItem> items;
@@ -119,6 +157,7 @@ struct sr_graph {
     std::vector<std::vector<int>> group_head_nodes;       // per group: nodes of the head kernels
     std::vector<std::vector<SrHeadNode>> group_heads;     // and what they need to know about them (filled when a workspace is bound)
     // dynamic state
+    SrFrameArgs frame{};                           // of the launches being queued
     int64_t t = 0;
     int64_t launches = 0;
     void* tc = nullptr;                            // tensor-core engine state (opaque here)
@@ -131,6 +170,7 @@ struct sr_graph {
     // deep-window mode: a second graph of the same network whose batch holds the W frames of a window side by side
     sr_graph* window = nullptr;
     int window_frames = 0;
+    std::vector<char> in_window;                   // per node: its current state is the last frame of the window's states
     std::vector<std::vector<float>> kept_weights;  // the parameters as the caller set them (host copies), for that graph
     std::vector<std::vector<float>> kept_bias;
     int static_device = -1;                        // >= 0: bound to the built-in workspace of that device

@@ -502,7 +502,7 @@ __device__ __forceinline__ void rs_dense_unit(const RsCtx& cx, const RsNode& nd,
 
 // The kernel body.  It is instantiated for 16, 24 and 32 warps per CTA (128, 80 and 64 registers per thread: the
 // code needs about 80, the compiler uses whatever the bound leaves), see the wrappers below.
-__device__ __forceinline__ void rs_kernel_body(const unsigned char* __restrict__ blobs, int blob_stride, SrFrameCtl* __restrict__ ctl_out,
+__device__ __forceinline__ void rs_kernel_body(const unsigned char* __restrict__ blobs, int blob_stride,
                                                const SrFrameCtl& init, int T, int cs)
 {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -553,8 +553,7 @@ __device__ __forceinline__ void rs_kernel_body(const unsigned char* __restrict__
         }
     }
     // frame t of every node (relative frame 0), and the first input frame of the run (relative frame 1)
-    // `init` is the frame control block of this run (frame counter, the caller's input sequences and output);
-    // the block in global memory is brought up to date at the end, for the launches that follow
+    // `init` describes this run (frame counter, the caller's input sequences and output)
     const SrFrameCtl* const ctl = &init;
     const long long t0 = ctl->t, run0 = ctl->run_t, out_stride = ctl->out_stride;
     float* const out_base = ctl->out_base;
@@ -635,13 +634,6 @@ __device__ __forceinline__ void rs_kernel_body(const unsigned char* __restrict__
         }
     }
 
-    if (blockIdx.x == 0 && tid == 0) {
-        SrFrameCtl c = init;
-        c.t += T;
-        c.run_t += T;
-        c.error = ctl_out->error;
-        *ctl_out = c;
-    }
     // relative frame T back to the state buffers in global memory (parity of t + T)
     const int parT = (int)((t0 + T) & 1);
     for (int v = 0; v < H.n_nodes; ++v) {
@@ -672,10 +664,10 @@ __device__ __forceinline__ void rs_kernel_body(const unsigned char* __restrict__
 
 template <int MAXT>
 __global__ void __launch_bounds__(MAXT, 1)
-sr_resident_kernel(const unsigned char* __restrict__ blobs, int blob_stride, SrFrameCtl* __restrict__ ctl_out,
+sr_resident_kernel(const unsigned char* __restrict__ blobs, int blob_stride,
                    const __grid_constant__ SrFrameCtl init, int T, int cs)
 {
-    rs_kernel_body(blobs, blob_stride, ctl_out, init, T, cs);
+    rs_kernel_body(blobs, blob_stride, init, T, cs);
 }
 
 // ------------------------------------------------------------------------------------------------ host side
@@ -1420,7 +1412,6 @@ sr_status sr_rs_launch(sr_graph* g, int T, const SrFrameCtl& init, cudaStream_t 
     cfg.attrs = at;
     cfg.numAttrs = E->cs > 1 ? 1 : 0;
     const unsigned char* blobs = reinterpret_cast<const unsigned char*>(g->ws + E->r_blobs.offset);
-    SrFrameCtl* ctl = reinterpret_cast<SrFrameCtl*>(g->ws + g->r_ctl.offset);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     bool timed = g->opt_time_tc != 0 && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
     if (timed && E->ev_used + 2 > E->ev.size()) {
@@ -1434,9 +1425,9 @@ sr_status sr_rs_launch(sr_graph* g, int T, const SrFrameCtl& init, cudaStream_t 
     }
     if (timed) cudaEventRecord(E->ev[E->ev_used], s);
     cudaError_t le;
-    if (E->warps <= 16) le = cudaLaunchKernelEx(&cfg, sr_resident_kernel<512>, blobs, E->blob_bytes, ctl, init, T, E->cs);
-    else if (E->warps <= 24) le = cudaLaunchKernelEx(&cfg, sr_resident_kernel<768>, blobs, E->blob_bytes, ctl, init, T, E->cs);
-    else le = cudaLaunchKernelEx(&cfg, sr_resident_kernel<1024>, blobs, E->blob_bytes, ctl, init, T, E->cs);
+    if (E->warps <= 16) le = cudaLaunchKernelEx(&cfg, sr_resident_kernel<512>, blobs, E->blob_bytes, init, T, E->cs);
+    else if (E->warps <= 24) le = cudaLaunchKernelEx(&cfg, sr_resident_kernel<768>, blobs, E->blob_bytes, init, T, E->cs);
+    else le = cudaLaunchKernelEx(&cfg, sr_resident_kernel<1024>, blobs, E->blob_bytes, init, T, E->cs);
     if (le != cudaSuccess) return SR_ERR_CUDA;
     if (timed) {
         cudaEventRecord(E->ev[E->ev_used + 1], s);

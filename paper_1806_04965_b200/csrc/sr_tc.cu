@@ -137,20 +137,15 @@ struct TcParams {
     const TcNode* nodes;
     const uint4* tables;
     const TcTile* tiles;
-    SrFrameCtl* ctl;
+    SrFrameArgs fr;
+    int* error;                     // device-side error code
     int* sched;                     // counters of the shared list, or null
     long long wait_limit;
     int n_tiles, n_own;             // items in all; those of the matrix
-    int t_off, B;
+    int B;
     int table_bytes;                // shared memory of one node table
     int n_w, w_slot;                // weight ring: slots and their size
     int ring_kb;                    // activation ring in KiB
-};
-
-struct TcStem {             // a few-channel input edge staged as im2col rows
-    const void* src[2];
-    void* dst[2];
-    int32_t Hs, Ws, Cs, Ho, Wo, k, stride, pad, Kp, K;
 };
 
 // ------------------------------------------------------------------------------------------ PTX helpers
@@ -312,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
     // A wait limit of zero (a host-side test hook) means "every wait has already expired": report it and return
     // before any barrier, tensor memory, copy or MMA is touched.
     if (wait_limit <= 0) {
-        if (threadIdx.x == 0) atomicExch(&P.ctl->error, 1);
+        if (threadIdx.x == 0) atomicExch(P.error, 1);
         return;
     }
     // weight ring first: an M = 128 instruction on a node with fewer than 128 output channels reads
@@ -354,8 +349,8 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
     const uint32_t tmem_base = tmem_slot;
     volatile int* abortp = &abort_flag;
 
-    const long long t = P.ctl->t + P.t_off;                 // this launch computes frame t+1 from frame t
-    const int prev = (int)(t & 1), cur = prev ^ 1;
+    const SrFrame F = sr_frame(P.fr);
+    const int prev = (int)(F.t & 1), cur = prev ^ 1;
     auto table_of = [&](const TcTile& it) { return reinterpret_cast<const TcNode*>(smem_raw + tab_off + (uint32_t)(it.slot * P.table_bytes)); };
 
     if (warp == 2) {
@@ -746,7 +741,7 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
     __syncwarp();
     tc_fence_before();
     __syncthreads();
-    if (threadIdx.x == 0 && abort_flag) atomicExch(&P.ctl->error, 1);
+    if (threadIdx.x == 0 && abort_flag) atomicExch(P.error, 1);
     if (threadIdx.x == 0 && P.sched && P.n_own < P.n_tiles) {
         // the CTA that leaves last (none takes an item any more) puts the counters back for the next launch
         __threadfence();
@@ -759,56 +754,6 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem_base) : "memory");
-    }
-}
-
-// Few-channel input edges: row (b, oy, ox) of the staged tensor holds the k*k*C_in receptive field
-// of that output pixel (zero outside the image, zero padded to Kp), so the edge becomes a K-block.
-__global__ void sr_tc_stage_kernel(const TcStem* __restrict__ stems, int n_stems, const SrFrameCtl* __restrict__ ctl,
-                                   int t_off, int fixed_parity, int B)
-{
-    __shared__ int tap_off[128];    // offset of element kk relative to the (unpadded) window origin, -1 = padding
-    __shared__ short tap_dy[128], tap_dx[128];
-    const int cur = fixed_parity >= 0 ? fixed_parity : (int)((ctl->t + t_off + 1) & 1);
-    for (int si = 0; si < n_stems; ++si) {
-        const TcStem st = stems[si];
-        __syncthreads();
-        if (threadIdx.x < 128) {
-            const int kk = threadIdx.x;
-            if (kk < st.K) {
-                const int ci = kk % st.Cs, tap = kk / st.Cs, kx = tap % st.k, ky = tap / st.k;
-                tap_dy[kk] = (short)(ky - st.pad);
-                tap_dx[kk] = (short)(kx - st.pad);
-                tap_off[kk] = ((ky - st.pad) * st.Ws + (kx - st.pad)) * st.Cs + ci;
-            } else {
-                tap_dy[kk] = tap_dx[kk] = 0;
-                tap_off[kk] = -1;
-            }
-        }
-        __syncthreads();
-        const __nv_bfloat16* src = static_cast<const __nv_bfloat16*>(st.src[cur]);
-        __nv_bfloat16* dst = static_cast<__nv_bfloat16*>(st.dst[cur]);
-        const int chunks = st.Kp / 8;
-        const size_t n_pix = (size_t)B * st.Ho * st.Wo;
-        for (size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x; p < n_pix; p += (size_t)gridDim.x * blockDim.x) {
-            const int ox = (int)(p % st.Wo);
-            const size_t r = p / st.Wo;
-            const int oy = (int)(r % st.Ho);
-            const int b = (int)(r / st.Ho);
-            const int y0 = oy * st.stride, x0 = ox * st.stride;
-            const __nv_bfloat16* base = src + (((size_t)b * st.Hs + y0) * st.Ws + x0) * st.Cs;
-            for (int c = 0; c < chunks; ++c) {
-                __align__(16) __nv_bfloat16 v[8];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int kk = c * 8 + j;
-                    const int iy = y0 + tap_dy[kk], ix = x0 + tap_dx[kk];
-                    const bool ok = kk < st.K && iy >= 0 && iy < st.Hs && ix >= 0 && ix < st.Ws;
-                    v[j] = ok ? base[tap_off[kk]] : __float2bfloat16_rn(0.f);
-                }
-                reinterpret_cast<uint4*>(dst)[p * chunks + c] = *reinterpret_cast<const uint4*>(v);
-            }
-        }
     }
 }
 
@@ -866,7 +811,7 @@ struct TcEngine {
     std::vector<int> stem_of_edge;
     std::vector<std::vector<TcTile>> group_tiles;
     std::vector<int> group_tile_offset, group_grid, group_n_own, group_n_w, group_w_slot, group_ring_kb, group_table_bytes;
-    SrRegion r_maps, r_nodes, r_tables, r_tiles, r_stems, r_sched;
+    SrRegion r_maps, r_nodes, r_tables, r_tiles;
     int n_maps = 0, n_kbs = 0, n_tiles = 0;
     int sm_count = 148;
     // optional timing of the group launches with CUDA events on the launching stream
@@ -1365,8 +1310,6 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
     E->r_nodes = take(sizeof(TcNode) * E->nodes.size());
     E->r_tables = take(48 * (size_t)std::max(1, n_kbs));
     E->r_tiles = take(sizeof(TcTile) * (size_t)std::max(1, n_tiles));
-    E->r_stems = take(sizeof(TcStem) * std::max<size_t>(1, E->stems.size()));
-    E->r_sched = take(256);                          // the shared list's counters: next item, CTAs that have left
     return SR_OK;
 }
 
@@ -1543,26 +1486,26 @@ sr_status sr_tc_bind(sr_graph* g)
     E->n_maps = (int)maps.size();
     std::vector<TcTile> tiles;
     for (auto& v : E->group_tiles) tiles.insert(tiles.end(), v.begin(), v.end());
-    std::vector<TcStem> stems;
+    g->stems.clear();
     for (const StemPlan& S : E->stems) {
         const SrHostEdge& he = g->edges[S.edge];
         const SrHostNode& s = g->nodes[he.d.src];
         const SrHostNode& t = g->nodes[he.d.tgt];
-        TcStem d{};
-        for (int par = 0; par < 2; ++par) {
-            d.src[par] = ws + s.state[par].offset;
-            d.dst[par] = ws + S.buf[par].offset;
-        }
+        SrStem d{};
+        d.dst[0] = ws + S.buf[0].offset;
+        d.dst[1] = ws + S.buf[1].offset;
+        d.slot = s.input_slot;
+        d.R = he.R;
         d.Hs = s.d.h; d.Ws = s.d.w; d.Cs = s.d.c; d.Ho = t.d.h; d.Wo = t.d.w;
         d.k = he.k_eff; d.stride = he.stride_eff; d.pad = he.pad_eff; d.Kp = S.Kp; d.K = he.K;
-        stems.push_back(d);
+        g->stems.push_back(d);
     }
     auto up = [&](const SrRegion& r, const void* p, size_t bytes) {
         return bytes == 0 || cudaMemcpy(ws + r.offset, p, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
     };
     if (!up(E->r_maps, maps.data(), maps.size() * sizeof(CUtensorMap)) || !up(E->r_nodes, dn.data(), dn.size() * sizeof(TcNode)) ||
         !up(E->r_tables, dt.data(), dt.size() * sizeof(uint4)) ||
-        !up(E->r_tiles, tiles.data(), tiles.size() * sizeof(TcTile)) || !up(E->r_stems, stems.data(), stems.size() * sizeof(TcStem)))
+        !up(E->r_tiles, tiles.data(), tiles.size() * sizeof(TcTile)))
         return SR_ERR_CUDA;
     return SR_OK;
 }
@@ -1609,33 +1552,12 @@ sr_status sr_tc_set_weights(sr_graph* g, int edge, const float* w_eff)
     return SR_OK;
 }
 
-static int launch_stage(sr_graph* g, int t_off, int fixed_parity, cudaStream_t s)
+bool sr_tc_stages(const sr_graph* g, int edge)
 {
-    TcEngine* E = eng(g);
-    if (!E || E->stems.empty()) return 0;
-    size_t most = 0;
-    for (const StemPlan& S : E->stems) {
-        const SrHostNode& t = g->nodes[g->edges[S.edge].d.tgt];
-        most = std::max(most, (size_t)g->batch * t.d.h * t.d.w);
-    }
-    const int blocks = (int)std::min<size_t>((size_t)E->sm_count * 8, (most + 255) / 256);
-    sr_tc_stage_kernel<<<blocks, 256, 0, s>>>(reinterpret_cast<const TcStem*>(g->ws + E->r_stems.offset), (int)E->stems.size(),
-                                              reinterpret_cast<const SrFrameCtl*>(g->ws + g->r_ctl.offset), t_off,
-                                              fixed_parity, g->batch);
-    return 1;
+    return g->nodes[g->edges[edge].d.tgt].use_tc && is_stem(g, g->edges[edge]);
 }
 
-int sr_tc_stage_inputs(sr_graph* g, int t_off, cudaStream_t s) { return launch_stage(g, t_off, -1, s); }
-
-int sr_tc_after_state_change(sr_graph* g, cudaStream_t s)
-{
-    // the shared work list's counters start from zero (every launch leaves them there; this covers a launch cut short)
-    if (TcEngine* E = eng(g))
-        if (g->ws) cudaMemsetAsync(g->ws + E->r_sched.offset, 0, 256, s);
-    return launch_stage(g, 0, (int)(g->t & 1), s);
-}
-
-int sr_tc_launch_group(sr_graph* g, int group, int t_off, cudaStream_t s)
+int sr_tc_launch_group(sr_graph* g, int group, cudaStream_t s)
 {
     TcEngine* E = eng(g);
     if (!E || E->group_tiles[group].empty()) return 0;
@@ -1660,12 +1582,12 @@ int sr_tc_launch_group(sr_graph* g, int group, int t_off, cudaStream_t s)
     P.nodes = reinterpret_cast<const TcNode*>(g->ws + E->r_nodes.offset);
     P.tables = reinterpret_cast<const uint4*>(g->ws + E->r_tables.offset);
     P.tiles = reinterpret_cast<const TcTile*>(g->ws + E->r_tiles.offset) + E->group_tile_offset[group];
-    P.ctl = reinterpret_cast<SrFrameCtl*>(g->ws + g->r_ctl.offset);
-    P.sched = g->opt_tc_lists == 0 ? reinterpret_cast<int*>(g->ws + E->r_sched.offset) : nullptr;
+    P.fr = g->frame;
+    P.error = reinterpret_cast<int*>(g->ws + g->r_flags.offset);
+    P.sched = g->opt_tc_lists == 0 ? P.error + 16 : nullptr;
     P.wait_limit = (long long)g->opt_wait_ms * 2000000LL;
     P.n_tiles = (int)E->group_tiles[group].size();
     P.n_own = E->group_n_own[group];
-    P.t_off = t_off;
     P.B = g->batch;
     P.table_bytes = E->group_table_bytes[group];
     P.n_w = E->group_n_w[group];

@@ -235,3 +235,50 @@ def test_heads_at_the_edges_of_their_blocks(batch, c_mid, c_out, dtype):
     g.patterns = {"p": [1] * 8, "q": [0, 1, 1, 0, 0, 1, 0, 0]}
     for p in g.patterns:
         parity.check_stepwise(g, p, zero_bias=False, resident=False)
+
+
+def test_states_after_a_deep_window():
+    # the states a window leaves behind can be read, replaced one by one, and are superseded by the next update
+    import torch
+    from oracle import frame_update as fu
+    g = graphs.dsr(2, batch=2, frames=5, h1_recurrence=False)
+    X, Wt, Bi = data.make_inputs(g), data.make_weights(g), data.make_biases(g, zero=False)
+    want = fu.rollout_spec(g, "sequential", X, Wt, Bi)
+    G = parity.make_graph(g, "sequential", "auto", 0, Wt, Bi)
+    G.bind_window(2)
+    x = parity.to_device(g, X[0])
+    G.reset([x[0]])
+
+    def check(t, skip=-1):
+        for v in range(len(g.nodes)):
+            if v != skip:
+                assert parity.rel_err(G.get_state(v).float().cpu().numpy(), want[v][t]) <= parity.TOL[g.dtype], (t, g.nodes[v].name)
+
+    for t in (0, 2):
+        G.rollout_window([x[t + 1:t + 3]])
+        check(t + 2)
+    mark = torch.full_like(G.get_state(2), 3.0)
+    G.set_state(2, mark)
+    assert torch.equal(G.get_state(2), mark)
+    check(4, skip=2)
+    G.step([x[5]])
+    check(5)
+    G.reset([x[0]])
+    assert float(G.get_state(2).abs().max()) == 0.0
+
+
+@pytest.mark.parametrize("cin,k,stride,size", [(1, 1, 1, 9), (5, 5, 1, 11), (3, 3, 2, 10), (3, 3, 4, 32), (2, 7, 1, 8), (14, 3, 3, 13)])
+def test_staged_input_edges(cin, k, stride, size):
+    # receptive fields of 1 .. 126 values (filters are odd) (partial and full 16-byte chunks), windows that leave the image on every side,
+    # odd sizes, strides; nine staged edges are more than one launch takes.  Half of them read the input inside the frame.
+    from workloads.graphs import CONV, GAP_DENSE, IDENTITY, Edge, GraphSpec, Node, check_shapes
+    pad = (k - 1) // 2
+    out = (size + 2 * pad - k) // stride + 1
+    n = 9 if (cin, k) == (3, 3) else 2
+    nodes = [Node("in", size, size, cin, IDENTITY)] + [Node("n%d" % i, out, out, 16) for i in range(n)] + [Node("o", 1, 1, 4, IDENTITY)]
+    edges = [Edge(0, 1 + i, CONV, k, stride) for i in range(n)] + [Edge(1 + i, n + 1, GAP_DENSE) for i in range(min(n, 6))]
+    g = GraphSpec("stems", nodes, edges, batch=3, frames=3, dtype="bf16", seed=91)
+    check_shapes(g)
+    g.patterns = {"p": [i % 2 for i in range(n)] + [1] * (len(edges) - n)}
+    parity.check_stepwise(g, "p", zero_bias=False)
+    parity.check_run(g, "p", graph_frames=2, resident=False)
