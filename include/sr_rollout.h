@@ -134,8 +134,8 @@ sr_status sr_graph_bind_workspace(sr_graph* g, void* workspace_dev, size_t bytes
  * Behaviour
  *   - allocates no device memory (no cudaMalloc / cudaFree, no allocating library call); inputs and
  *     outputs are still the caller's buffers, passed to reset / step / run as before.  Host-side objects are
- *     still created later, as for any graph: the first step / run creates a stream and two events, and
- *     sr_rollout_run with CUDA graphs enabled instantiates a graph;
+ *     still created later, as for any graph: sr_rollout_run with CUDA graphs enabled creates a stream and
+ *     instantiates a graph;
  *   - the first call on a device looks the array's address up for that device (the device must be
  *     current) and remembers it; make that first call before any stream capture begins;
  *   - a graph whose sr_graph_workspace_bytes exceeds SR_STATIC_WORKSPACE_BYTES is refused with
@@ -167,9 +167,9 @@ sr_status sr_graph_set_node_bias(sr_graph* g, int node, const float* bias_host);
  *                  (2..8; 0 = default); the rest of the shared memory holds activation boxes.
  *           key 3 "tile width": width in pixels (8, 16 or 32; 0 = default) of the output tiles of the tensor-core kernel
  *                  (for nodes with an edge whose taps share activation boxes).
- *           key 4 "overlap": 1 (default) runs independent launches of a frame on a second, library-owned
- *                  stream (the CUDA-core and the tensor-core kernel of a group; the next frame's input
- *                  copy when no input edge has R = 0), joined before the frame ends; 0 = one stream.
+ *           key 4 "overlap": 1 (default) lets independent launches of a frame run beside each other (the CUDA-core and the
+ *                  tensor-core kernel of a group; the next frame's input copy when no input edge has R = 0); 0 = one after
+ *                  the other.  All launches go to the caller's stream either way.
  *           key 5 "kernel timing": 1 brackets every tensor-core group launch and every resident launch with CUDA
  *                  events on the launching stream (plain launches only, not inside CUDA graphs); read with
  *                  sr_graph_kernel_time.

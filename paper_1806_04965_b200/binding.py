@@ -132,6 +132,8 @@ class Graph:
             if not torch.cuda.is_available():
                 raise RuntimeError("a CUDA device is required for a graph with batch > 0")
             self._torch = torch
+            # the current stream's handle without a Stream object around it (a step's host time is a few microseconds)
+            self._raw_stream, self._current_device = torch._C._cuda_getCurrentRawStream, torch.cuda.current_device
             self.tdtype = torch.bfloat16 if dtype == "bf16" else torch.float32
             _check(self._lib.sr_graph_set_option(self._h, 0, {"auto": 0, "direct": 1}[engine]), "sr_graph_set_option")
             _check(self._lib.sr_graph_set_option(self._h, 1, int(graph_frames)), "sr_graph_set_option")
@@ -160,6 +162,10 @@ class Graph:
         self.info = self._info()
         self.input_nodes = [v for v in range(n) if not any(e.tgt == v for e in self.edges)]
         self.output_node = self.info["output_node"]
+        self._in_shapes = [(batch, self.nodes[v].h, self.nodes[v].w, self.nodes[v].c) for v in self.input_nodes]
+        self._ptr_array = ctypes.c_void_p * len(self.input_nodes)
+        nd = self.nodes[self.output_node]
+        self._out_shape = (batch, nd.c) if nd.h == 1 and nd.w == 1 else (batch, nd.h, nd.w, nd.c)
 
     def __del__(self):
         try:
@@ -180,7 +186,7 @@ class Graph:
         return list(lv)
 
     def _stream(self):
-        return self._torch.cuda.current_stream().cuda_stream
+        return self._raw_stream(self._current_device())
 
     def set_weights(self, weights: Sequence[np.ndarray], biases: Optional[Sequence[np.ndarray]] = None):
         for ei, w in enumerate(weights):
@@ -192,27 +198,25 @@ class Graph:
                 _check(self._lib.sr_graph_set_node_bias(self._h, vi, b.ctypes.data), "sr_graph_set_node_bias")
 
     def _ptrs(self, tensors, frames: Optional[int] = None):
-        assert len(tensors) == len(self.input_nodes)
-        arr = (ctypes.c_void_p * len(tensors))()
-        for i, (t, v) in enumerate(zip(tensors, self.input_nodes)):
-            nd = self.nodes[v]
-            shape = (self.batch, nd.h, nd.w, nd.c) if frames is None else (frames, self.batch, nd.h, nd.w, nd.c)
-            assert t.is_cuda and t.is_contiguous() and t.dtype == self.tdtype and tuple(t.shape) == shape, (t.shape, shape)
-            arr[i] = t.data_ptr()
-        return arr
+        assert len(tensors) == len(self._in_shapes)
+        dtype, ptrs = self.tdtype, []
+        for t, shape in zip(tensors, self._in_shapes):
+            if frames is not None:
+                shape = (frames,) + shape
+            assert t.is_cuda and t.dtype is dtype and t.shape == shape and t.is_contiguous(), (t.shape, shape)
+            ptrs.append(t.data_ptr())
+        return self._ptr_array(*ptrs)
 
     def reset(self, in0):
         _check(self._lib.sr_graph_reset(self._h, self._ptrs(in0), self._stream()), "sr_graph_reset")
 
     def out_shape(self):
         """Shape of one frame of output: the output node's state, [B][C] for a dense node, else [B][H][W][C]."""
-        nd = self.nodes[self.output_node]
-        return (self.batch, nd.c) if nd.h == 1 and nd.w == 1 else (self.batch, nd.h, nd.w, nd.c)
+        return self._out_shape
 
     def step(self, in_next, out=None):
         if out is not None:
-            assert out.is_cuda and out.is_contiguous() and out.dtype == self._torch.float32
-            assert tuple(out.shape) == self.out_shape()
+            assert out.is_cuda and out.is_contiguous() and out.dtype is self._torch.float32 and out.shape == self._out_shape
         _check(self._lib.sr_rollout_step(self._h, self._ptrs(in_next), out.data_ptr() if out is not None else None,
                                          self._stream()), "sr_rollout_step")
 

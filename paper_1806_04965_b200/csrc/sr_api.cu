@@ -56,29 +56,6 @@ struct GraphCache {
     bool with_out = false;
 };
 
-// A second stream lets independent launches of one frame overlap: the CUDA-core kernel and the
-// tensor-core kernel of a launch group, and - when no input edge stays inside the frame - the copy
-// and staging of the next input frame, which nothing of the current update reads.
-struct SideStream {
-    cudaStream_t stream = nullptr;
-    cudaEvent_t fork = nullptr, join = nullptr;
-};
-
-SideStream* side_of(sr_graph* g)
-{
-    if (!g->side) {
-        SideStream* s = new SideStream();
-        if (cudaStreamCreateWithFlags(&s->stream, cudaStreamNonBlocking) != cudaSuccess ||
-            cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&s->join, cudaEventDisableTiming) != cudaSuccess) {
-            delete s;
-            return nullptr;
-        }
-        g->side = s;
-    }
-    return static_cast<SideStream*>(g->side);
-}
-
 float round_bf16_host(float f)
 {
     uint32_t u;
@@ -153,7 +130,7 @@ sr_status plan(sr_graph* g)
     g->group_item_offset.clear();
     g->group_item_count.clear();
     g->group_head_nodes.assign(g->groups.size(), {});
-    const int px = sr_direct_conv_pixels_per_block(), dco = sr_direct_dense_outputs_per_block(),
+    const int dco = sr_direct_dense_outputs_per_block(),
               dsb = sr_direct_dense_samples_per_block();
     for (size_t gi = 0; gi < g->groups.size(); ++gi) {
         g->group_item_offset.push_back((int)g->items.size());
@@ -168,11 +145,17 @@ sr_status plan(sr_graph* g)
                         for (int c0 = 0; c0 < n.d.c; c0 += dco) g->items.push_back(SrDirectItem{v, b0, c0, 0});
                 }
             } else {
-                const int HW = n.d.h * n.d.w;
-                for (int b = 0; b < g->batch; ++b)
-                    for (int p0 = 0; p0 < HW; p0 += px) g->items.push_back(SrDirectItem{v, b, p0, 0});
+                sr_direct_conv_items(g, v, g->items);
             }
         }
+        // the items with the longest reductions first: a launch ends when its last block ends
+        auto work = [&](const SrDirectItem& it) {
+            long long k = 0;
+            for (int e : g->nodes[it.node].in_edges) k += g->edges[e].K;
+            return k * (it.b0 < 0 ? 4 : 1);
+        };
+        std::stable_sort(g->items.begin() + g->group_item_offset.back(), g->items.end(),
+                         [&](const SrDirectItem& a, const SrDirectItem& b) { return work(a) > work(b); });
         g->group_item_count.push_back((int)g->items.size() - g->group_item_offset.back());
     }
     g->r_items = take(off, sizeof(SrDirectItem) * std::max<size_t>(1, g->items.size()));
@@ -215,41 +198,36 @@ sr_status ready(const sr_graph* g)
 int enqueue_frames(sr_graph* g, const SrFrameArgs& fr, int frames, cudaStream_t s, unsigned copies = ~0u, unsigned stems_R = 3u)
 {
     int launches = 0;
-    SideStream* side = g->opt_overlap ? side_of(g) : nullptr;
+    // events between two launches of a stream (the timing option) need plain launches around them
+    const bool chain = !g->opt_time_tc, overlap = g->opt_overlap != 0;
+    bool first = true;
+    auto follow = [&](bool beside, bool late) {
+        SrFollow how;
+        how.early = chain && !first;
+        how.beside = beside && chain;
+        how.late = late && chain;
+        first = false;
+        return how;
+    };
     g->frame = fr;
     for (int f = 0; f < frames; ++f, ++g->frame.off) {
-        bool forked = false;
-        auto fork = [&]() {
-            if (!forked) {
-                cudaEventRecord(side->fork, s);
-                cudaStreamWaitEvent(side->stream, side->fork, 0);
-                forked = true;
-            }
-        };
-        auto join = [&]() {
-            if (forked) {
-                cudaEventRecord(side->join, side->stream);
-                cudaStreamWaitEvent(s, side->join, 0);
-                forked = false;
-            }
-        };
-        // frame input: on the side stream if this frame's update does not read it, queued behind the first group's tensor-core
-        // kernel (whose CTAs each need most of an SM)
-        const bool input_beside = side && !g->input_feeds_same_frame;
-        if (input_beside) fork();
-        else launches += sr_launch_input(g, g->frame, copies, stems_R, false, s);
+        // The frame input: ahead of the first group if the update reads it (with its heads, where they can read the caller's
+        // frame themselves), else beside the first group.
+        const bool feeds = g->input_feeds_same_frame;
         for (int gi = 0; gi < (int)g->groups.size(); ++gi) {
-            // up to three independent launches: the heads go beside whatever else the group has, the other CUDA-core nodes
-            // beside the tensor-core kernel
+            // up to four independent launches: one of them leads, the others run beside it
             const bool has_heads = !g->group_heads[gi].empty(), has_items = g->group_item_count[gi] > 0, has_tc = sr_tc_group_has_work(g, gi);
-            if (side && ((has_heads && (has_items || has_tc)) || (has_items && has_tc))) fork();
-            launches += sr_tc_launch_group(g, gi, s);
-            if (gi == 0 && input_beside) launches += sr_launch_input(g, g->frame, copies, stems_R, true, side->stream);
-            if (has_heads) launches += sr_launch_heads(g, gi, side && (has_items || has_tc) ? side->stream : s);
-            if (has_items) launches += sr_launch_direct_group(g, gi, side && has_tc ? side->stream : s);
-            if (gi + 1 < (int)g->groups.size()) join();       // the next group reads what this one wrote
+            const bool heads_lead = !has_tc && !has_items;
+            const bool merged = gi == 0 && has_heads && (heads_lead || !feeds) && sr_heads_take_input(g, gi, g->frame, copies, stems_R);
+            if (gi == 0 && feeds && !merged) launches += sr_launch_input(g, g->frame, copies, stems_R, follow(false, false), s);
+            const bool input_beside = gi == 0 && !feeds && !merged;
+            const bool late = overlap && (input_beside || (has_tc + has_items + has_heads > 1));
+            if (has_tc) launches += sr_tc_launch_group(g, gi, follow(false, late), s);
+            if (has_items) launches += sr_launch_direct_group(g, gi, follow(overlap && has_tc, late && !has_tc), s);
+            if (input_beside && !heads_lead) launches += sr_launch_input(g, g->frame, copies, stems_R, follow(overlap, false), s);
+            if (has_heads) launches += sr_launch_heads(g, gi, merged, copies, stems_R, follow(overlap && !heads_lead, late && heads_lead), s);
+            if (input_beside && heads_lead) launches += sr_launch_input(g, g->frame, copies, stems_R, follow(overlap, false), s);
         }
-        join();
     }
     return launches;
 }
@@ -276,7 +254,7 @@ void stage_current(sr_graph* g, cudaStream_t s)
     SrFrameCtl c{};
     c.t = g->t - 1;                                              // "the input of frame t"
     for (size_t i = 0; i < g->input_nodes.size(); ++i) c.in_base[i] = g->ws + g->nodes[g->input_nodes[i]].state[g->t & 1].offset;
-    g->launches += sr_launch_input(g, by_value(c), 0u, 2u, false, s);
+    g->launches += sr_launch_input(g, by_value(c), 0u, 2u, SrFollow(), s);
 }
 
 // After a resident run they are brought up to date when the launch path is used next.
@@ -326,13 +304,6 @@ void sr_graph_destroy(sr_graph* g)
         if (c->exec) cudaGraphExecDestroy(c->exec);
         if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
         delete c;
-    }
-    if (g->side) {
-        SideStream* sd = static_cast<SideStream*>(g->side);
-        cudaEventDestroy(sd->fork);
-        cudaEventDestroy(sd->join);
-        cudaStreamDestroy(sd->stream);
-        delete sd;
     }
     sr_tc_destroy(g);
     sr_rs_destroy(g);
@@ -533,6 +504,7 @@ sr_status sr_graph_bind_workspace(sr_graph* g, void* workspace_dev, size_t bytes
                 x.src[1] = ws + s.state[1].offset;
                 x.w = reinterpret_cast<const float*>(ws + he.w_direct.offset);
                 x.HW = s.d.h * s.d.w; x.Cs = s.d.c; x.kind = he.d.kind; x.R = he.R; x.K = he.K;
+                x.slot = s.input_slot;
                 h.has_mean |= he.d.kind == SR_EDGE_MEAN_DENSE;
             }
             g->group_heads[gi].push_back(h);
@@ -671,7 +643,7 @@ sr_status sr_graph_reset(sr_graph* g, const void* const* in0_dev, void* stream)
     c.t = -1;                                                    // "the input of frame 0"
     for (size_t i = 0; i < g->input_nodes.size(); ++i) c.in_base[i] = in0_dev[i];
     const bool resident = sr_rs_available(g);                    // a resident run does not read staged edges
-    g->launches += sr_launch_input(g, by_value(c), ~0u, resident ? 0u : 2u, false, s);
+    g->launches += sr_launch_input(g, by_value(c), ~0u, resident ? 0u : 2u, SrFollow(), s);
     g->stage_dirty = resident;
     return cuda_ok(cudaGetLastError()) ? SR_OK : SR_ERR_CUDA;
 }
@@ -898,7 +870,7 @@ sr_status sr_rollout_window(sr_graph* g, const void* const* in_seq_dev, int W, f
     c.t = t_new - 1;
     for (size_t i = 0; i < g->input_nodes.size(); ++i)
         c.in_base[i] = static_cast<const char*>(in_seq_dev[i]) + node_elems(g, g->input_nodes[i]) * g->elem * (size_t)(W - 1);
-    w->launches += sr_launch_input(g, by_value(c), ~0u, 0u, false, s);
+    w->launches += sr_launch_input(g, by_value(c), ~0u, 0u, SrFollow(), s);
     for (size_t v = 0; v < g->nodes.size(); ++v) g->in_window[v] = !g->nodes[v].is_input;
     g->t = t_new;
     g->stage_dirty = true;

@@ -6,7 +6,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
-#include "sr_internal.h"
+#include "sr_input.cuh"
 #include "sr_kernels.h"
 
 namespace {
@@ -28,11 +28,18 @@ __device__ __forceinline__ void load4(const __nv_bfloat16* p, float (&v)[4])
     v[2] = __uint_as_float(q.y << 16); v[3] = __uint_as_float(q.y & 0xFFFF0000u);
 }
 
+__device__ __forceinline__ void store4(float* p, const float (&v)[4]) { *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]); }
+__device__ __forceinline__ void store4(__nv_bfloat16* p, const float (&v)[4])
+{
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
+    *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+}
+
 constexpr int kPix = 4;            // pixels per warp (conv nodes)
 constexpr int kWarps = 4;          // warps per block
 constexpr int kDenseB = 8;         // samples per warp (dense nodes)
 
-// Conv node: a block covers kWarps*kPix consecutive pixels of one sample; lanes run over output
+// Conv node whose channel count is not a multiple of four: a block covers kWarps*kPix consecutive pixels of one sample; lanes run over output
 // channels, so weight reads ([K][C_out] rows) and state writes (NHWC) are coalesced and the input
 // reads are warp-uniform broadcasts.
 template <typename T>
@@ -114,6 +121,110 @@ __device__ void conv_item(const SrDevNode& nd, const SrDevEdge* edges, const SrD
     }
 }
 
+// Conv node with a multiple of four channels.  A thread computes PX consecutive pixels of one sample x 4 channels; the threads of
+// a block are 2^qb_log2 channel quads x pixel groups, so weight rows ([K][C_out]) and states (NHWC) are read and written in
+// 16-byte vectors by neighbouring threads.  The reduction of an edge is one flat loop over a table in shared memory (offset
+// inside the window, filter row and column): no branch per tap, so the loads of several steps are in flight together.  What
+// bounds it is the latency of those loads for a small node and the load / store unit for a large one; PX = 4 loads a weight
+// vector once for four pixels and is taken when that still leaves threads enough (see sr_direct_conv_items).
+// Measured on B200 (was: a warp per four pixels, lanes over channels, a branch per tap), fp32, us per frame: MNIST net SR at 100
+// samples 49 -> 17.5, at one 34 -> 12.6; small CNN at 128 samples 260 -> 114, at one 80 -> 27.
+constexpr int kTab = 512;          // table entries at a time
+template <typename T, int PX>
+__device__ void conv_tile(const SrDevNode& nd, const SrDevEdge* edges, const SrDirectItem& it, int prev, int cur, float* out_f32, int2* tab)
+{
+    const int qlog = it.pad_ >> 24, c = (it.pad_ & 0xFFFFFF) + 4 * ((int)threadIdx.x & ((1 << qlog) - 1));
+    const int HW = nd.H * nd.W, C = nd.C, p_first = it.p0 + ((int)threadIdx.x >> qlog) * PX;
+    const bool cv = c < C;
+    int oy[PX], ox[PX];
+    float acc[PX][4];
+#pragma unroll
+    for (int j = 0; j < PX; ++j) {
+        const int p = p_first + j;
+        oy[j] = p < HW ? p / nd.W : 1 << 20;                                     // (a pixel that does not exist lies outside every image)
+        ox[j] = p % nd.W;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[j][q] = 0.f;
+    }
+    for (int ei = 0; ei < nd.n_edges; ++ei) {
+        const SrDevEdge& e = edges[nd.first_edge + ei];
+        const int Hs = e.Hs, Ws = e.Ws, Cs = e.Cs, k = e.k, vec = (Cs & 3) == 0 ? 4 : 1, n = e.K / vec, cg = Cs / vec;
+        const T* src = static_cast<const T*>(e.src[e.R ? prev : cur]) + (size_t)it.b0 * Hs * Ws * Cs;
+        const float* w = e.w + (cv ? c : 0);
+        int y0[PX], x0[PX], o0[PX];
+#pragma unroll
+        for (int j = 0; j < PX; ++j) {
+            y0[j] = oy[j] * e.stride - e.pad;
+            x0[j] = ox[j] * e.stride - e.pad;
+            o0[j] = oy[j] < (1 << 20) ? (y0[j] * Ws + x0[j]) * Cs : 0;
+            if (oy[j] >= (1 << 20)) y0[j] = -(1 << 20);
+        }
+        for (int e0 = 0; e0 < n; e0 += kTab) {
+            const int m = min(kTab, n - e0);
+            __syncthreads();
+            for (int i = threadIdx.x; i < m; i += kWarps * 32) {
+                const int tap = (e0 + i) / cg, ci = ((e0 + i) % cg) * vec, dy = tap / k, dx = tap % k;
+                tab[i] = make_int2((dy * Ws + dx) * Cs + ci, dy << 16 | dx);
+            }
+            __syncthreads();
+            if (vec == 4) {
+#pragma unroll 2
+                for (int i = 0; i < m; ++i) {
+                    const int2 t = tab[i];
+                    const int dy = t.y >> 16, dx = t.y & 0xFFFF;
+                    float4 wv[4];
+                    float x[PX][4];
+#pragma unroll
+                    for (int j = 0; j < PX; ++j) {
+                        x[j][0] = x[j][1] = x[j][2] = x[j][3] = 0.f;
+                        if ((unsigned)(y0[j] + dy) < (unsigned)Hs && (unsigned)(x0[j] + dx) < (unsigned)Ws) load4(src + o0[j] + t.x, x[j]);
+                    }
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) wv[q] = __ldg(reinterpret_cast<const float4*>(w + (size_t)((e0 + i) * 4 + q) * C));
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+#pragma unroll
+                        for (int j = 0; j < PX; ++j) {
+                            acc[j][0] = fmaf(wv[q].x, x[j][q], acc[j][0]); acc[j][1] = fmaf(wv[q].y, x[j][q], acc[j][1]);
+                            acc[j][2] = fmaf(wv[q].z, x[j][q], acc[j][2]); acc[j][3] = fmaf(wv[q].w, x[j][q], acc[j][3]);
+                        }
+                }
+            } else {
+#pragma unroll 8
+                for (int i = 0; i < m; ++i) {
+                    const int2 t = tab[i];
+                    const int dy = t.y >> 16, dx = t.y & 0xFFFF;
+                    const float4 wv = __ldg(reinterpret_cast<const float4*>(w + (size_t)(e0 + i) * C));
+#pragma unroll
+                    for (int j = 0; j < PX; ++j) {
+                        float x = 0.f;
+                        if ((unsigned)(y0[j] + dy) < (unsigned)Hs && (unsigned)(x0[j] + dx) < (unsigned)Ws) x = to_f(src[o0[j] + t.x]);
+                        acc[j][0] = fmaf(wv.x, x, acc[j][0]); acc[j][1] = fmaf(wv.y, x, acc[j][1]);
+                        acc[j][2] = fmaf(wv.z, x, acc[j][2]); acc[j][3] = fmaf(wv.w, x, acc[j][3]);
+                    }
+                }
+            }
+        }
+    }
+    if (!cv) return;
+    const float4 b = *reinterpret_cast<const float4*>(nd.bias + c);
+#pragma unroll
+    for (int j = 0; j < PX; ++j) {
+        const int p = p_first + j;
+        if (p >= HW) continue;
+        float z[4] = {acc[j][0] + b.x, acc[j][1] + b.y, acc[j][2] + b.z, acc[j][3] + b.w};
+        if (nd.act == 1)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) z[q] = fmaxf(z[q], 0.f);
+        const size_t o = ((size_t)it.b0 * HW + p) * C + c;
+        store4(static_cast<T*>(nd.state[cur]) + o, z);
+        if (out_f32) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) out_f32[o + q] = z[q];                  // (the caller's buffer: any alignment a float has)
+        }
+    }
+}
+
 // Dense node outside the limits of the head kernels: one warp per output channel and chunk of kDenseB samples; lanes stride over the
 // reduction index (coalesced weight and state reads), partial sums meet in a shuffle reduction.
 // A mean-dense edge is the dense edge whose weight index is k mod C_in, scaled by 1/(H*W).
@@ -177,26 +288,43 @@ constexpr int kHeadMaxC = 1024;    // channels of a node's mean-dense sources to
 
 struct HeadParams {
     SrFrameArgs fr;
-    int32_t n_nodes, B;
+    SrInputPart in;                // the frame input's blocks come first (n_blocks = 0: none)
+    int32_t n_nodes, B, follow, direct;      // direct: edges with R = 0 that leave an input node read the caller's frame (its
+                                             // copy in the state buffer is being made by this launch)
     int32_t first_block[SR_HEAD_NODES + 1];
     SrHeadNode nodes[SR_HEAD_NODES];
 };
 static_assert(sizeof(HeadParams) <= 4000, "kernel parameters");
 
+template <typename T>
+__device__ __forceinline__ const T* head_source(const HeadParams& P, const SrFrame& F, const SrHeadEdge& e)
+{
+    const int prev = (int)(F.t & 1);
+    if (P.direct && e.R == 0 && e.slot >= 0) return reinterpret_cast<const T*>(sr_frame_input(P.fr, F, e.slot));
+    return static_cast<const T*>(e.src[e.R ? prev : prev ^ 1]);
+}
+
 // Nodes with dense edges only: a block takes CO outputs of S samples; its threads stride over the reduction index in vectors
 // of four, every thread keeps S x CO partial sums (a weight vector serves S samples).  The sums of a warp meet by halving,
 // those of the warps in shared memory in a fixed order.
-template <typename T, int S, int CO>
+template <typename T, int S, int CO, bool WithInput>
 __global__ void __launch_bounds__(kHeadThreads) sr_head_kernel(const __grid_constant__ HeadParams P)
 {
     __shared__ float red[kHeadWarps][32];
+    __shared__ int2 tap[WithInput ? 128 : 1];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    sr_begin(P.follow);
     const SrFrame F = sr_frame(P.fr);
-    int ni = 0;
-    while (ni + 1 < P.n_nodes && (int)blockIdx.x >= P.first_block[ni + 1]) ++ni;
+    int bx = (int)blockIdx.x, ni = 0;
+    if (WithInput && (bx -= P.in.n_blocks) < 0) {
+        sr_input_block(P.in, P.fr, F, (int)blockIdx.x, tap);
+        sr_end(P.follow);
+        return;
+    }
+    while (ni + 1 < P.n_nodes && bx >= P.first_block[ni + 1]) ++ni;
     const SrHeadNode& nd = P.nodes[ni];
-    const int co_blocks = (nd.C + CO - 1) / CO, bi = (int)blockIdx.x - P.first_block[ni], b0 = (bi / co_blocks) * S, co0 = (bi % co_blocks) * CO;
-    const int nco = min(CO, nd.C - co0), prev = (int)(F.t & 1), cur = prev ^ 1;
+    const int co_blocks = (nd.C + CO - 1) / CO, bi = bx - P.first_block[ni], b0 = (bi / co_blocks) * S, co0 = (bi % co_blocks) * CO;
+    const int nco = min(CO, nd.C - co0), cur = (int)((F.t + 1) & 1);
     float* const out = nd.is_output ? sr_frame_output(P.fr, F) : nullptr;
     float acc[S][CO];
 #pragma unroll
@@ -206,10 +334,11 @@ __global__ void __launch_bounds__(kHeadThreads) sr_head_kernel(const __grid_cons
     for (int ei = 0; ei < nd.n_edges; ++ei) {
         const SrHeadEdge& e = nd.edges[ei];
         const int K = e.K;
+        const T* src = head_source<T>(P, F, e);
         const T* x[S];
         const float* w[CO];
 #pragma unroll
-        for (int s = 0; s < S; ++s) x[s] = static_cast<const T*>(e.src[e.R ? prev : cur]) + (size_t)min(b0 + s, P.B - 1) * K;   // samples and rows beyond
+        for (int s = 0; s < S; ++s) x[s] = src + (size_t)min(b0 + s, P.B - 1) * K;   // samples and rows beyond
 #pragma unroll
         for (int o = 0; o < CO; ++o) w[o] = e.w + (size_t)(co0 + min(o, nco - 1)) * K;                                          // the last repeat it
         if ((K & 3) == 0) {
@@ -274,6 +403,7 @@ __global__ void __launch_bounds__(kHeadThreads) sr_head_kernel(const __grid_cons
             if (out) out[(size_t)b * nd.C + co0 + o] = z;
         }
     }
+    sr_end(P.follow);
 }
 
 // Nodes with a mean-dense edge: a block takes one sample.  First the means of the sources (groups of Cs / 4 threads share the
@@ -282,13 +412,19 @@ template <typename T>
 __global__ void __launch_bounds__(kHeadThreads) sr_mean_head_kernel(const __grid_constant__ HeadParams P)
 {
     __shared__ __align__(16) float mean[kHeadMaxC];
-    __shared__ float part[4 * kHeadThreads];
+    __shared__ __align__(16) float part[4 * kHeadThreads];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    sr_begin(P.follow);
     const SrFrame F = sr_frame(P.fr);
-    int ni = 0;
-    while (ni + 1 < P.n_nodes && (int)blockIdx.x >= P.first_block[ni + 1]) ++ni;
+    int bx = (int)blockIdx.x, ni = 0;
+    if ((bx -= P.in.n_blocks) < 0) {
+        sr_input_block(P.in, P.fr, F, (int)blockIdx.x, reinterpret_cast<int2*>(part));
+        sr_end(P.follow);
+        return;
+    }
+    while (ni + 1 < P.n_nodes && bx >= P.first_block[ni + 1]) ++ni;
     const SrHeadNode& nd = P.nodes[ni];
-    const int b = (int)blockIdx.x - P.first_block[ni], prev = (int)(F.t & 1), cur = prev ^ 1;
+    const int b = bx - P.first_block[ni], cur = (int)((F.t + 1) & 1);
     float* const out = nd.is_output ? sr_frame_output(P.fr, F) : nullptr;
     int m_off = 0;
     for (int ei = 0; ei < nd.n_edges; ++ei) {
@@ -296,7 +432,7 @@ __global__ void __launch_bounds__(kHeadThreads) sr_mean_head_kernel(const __grid
         if (e.kind != SR_EDGE_MEAN_DENSE) continue;
         const int vc = e.Cs / 4, groups = kHeadThreads / vc, col = tid % vc, grp = tid / vc;
         if (grp < groups) {
-            const T* xs = static_cast<const T*>(e.src[e.R ? prev : cur]) + (size_t)b * e.HW * e.Cs + 4 * col;
+            const T* xs = head_source<T>(P, F, e) + (size_t)b * e.HW * e.Cs + 4 * col;
             float s4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 8
             for (int px = grp; px < e.HW; px += groups) {
@@ -332,7 +468,7 @@ __global__ void __launch_bounds__(kHeadThreads) sr_mean_head_kernel(const __grid
                 }
                 m_off += e.Cs;
             } else {
-                const T* x = static_cast<const T*>(e.src[e.R ? prev : cur]) + (size_t)b * e.K;
+                const T* x = head_source<T>(P, F, e) + (size_t)b * e.K;
 #pragma unroll 4
                 for (int k = lane; k < e.K; k += 32) a = fmaf(__ldg(w + k), to_f(x[k]), a);
             }
@@ -346,65 +482,125 @@ __global__ void __launch_bounds__(kHeadThreads) sr_mean_head_kernel(const __grid
             if (out) out[(size_t)b * nd.C + o] = z;
         }
     }
+    sr_end(P.follow);
 }
 
+struct DirectParams {
+    SrFrameArgs fr;
+    const SrDevNode* nodes;
+    const SrDevEdge* edges;
+    const SrDirectItem* items;
+    int32_t B, follow;
+};
+
 template <typename T>
-__global__ void __launch_bounds__(kWarps * 32)
-sr_direct_group_kernel(const SrDevNode* __restrict__ nodes, const SrDevEdge* __restrict__ edges,
-                       const SrDirectItem* __restrict__ items, const __grid_constant__ SrFrameArgs fr, int B)
+__global__ void __launch_bounds__(kWarps * 32) sr_direct_group_kernel(const __grid_constant__ DirectParams P)
 {
-    const SrDirectItem it = items[blockIdx.x];
-    const SrDevNode& nd = nodes[it.node];
-    const SrFrame F = sr_frame(fr);
+    __shared__ int2 tab[kTab];
+    sr_begin(P.follow);
+    const SrDirectItem it = P.items[blockIdx.x];
+    const SrDevNode& nd = P.nodes[it.node];
+    const SrFrame F = sr_frame(P.fr);
     const int prev = (int)(F.t & 1), cur = prev ^ 1;
-    float* out = nd.is_output ? sr_frame_output(fr, F) : nullptr;
-    if (nd.H == 1 && nd.W == 1 && edges[nd.first_edge].kind != SR_EDGE_CONV) dense_item<T>(nd, edges, it, prev, cur, B, out);
-    else conv_item<T>(nd, edges, it, prev, cur, out);
+    float* out = nd.is_output ? sr_frame_output(P.fr, F) : nullptr;
+    if (nd.H == 1 && nd.W == 1 && P.edges[nd.first_edge].kind != SR_EDGE_CONV) dense_item<T>(nd, P.edges, it, prev, cur, P.B, out);
+    else if (nd.C % 4 != 0) conv_item<T>(nd, P.edges, it, prev, cur, out);
+    else if (it.b0 >= 0) conv_tile<T, 1>(nd, P.edges, it, prev, cur, out, tab);
+    else {
+        SrDirectItem four = it;
+        four.b0 = ~it.b0;
+        conv_tile<T, 4>(nd, P.edges, four, prev, cur, out, tab);
+    }
+    sr_end(P.follow);
 }
 
 }  // namespace
 
-int sr_launch_direct_group(const sr_graph* g, int group, cudaStream_t s)
+int sr_launch_direct_group(const sr_graph* g, int group, SrFollow how, cudaStream_t s)
 {
     const int n = g->group_item_count[group];
     if (n == 0) return 0;
-    const SrDevNode* nodes = reinterpret_cast<const SrDevNode*>(g->ws + g->r_nodes.offset);
-    const SrDevEdge* edges = reinterpret_cast<const SrDevEdge*>(g->ws + g->r_edges.offset);
-    const SrDirectItem* items = reinterpret_cast<const SrDirectItem*>(g->ws + g->r_items.offset) + g->group_item_offset[group];
-    if (g->dtype == SR_DTYPE_BF16)
-        sr_direct_group_kernel<__nv_bfloat16><<<n, kWarps * 32, 0, s>>>(nodes, edges, items, g->frame, g->batch);
-    else
-        sr_direct_group_kernel<float><<<n, kWarps * 32, 0, s>>>(nodes, edges, items, g->frame, g->batch);
+    DirectParams P;
+    P.fr = g->frame;
+    P.nodes = reinterpret_cast<const SrDevNode*>(g->ws + g->r_nodes.offset);
+    P.edges = reinterpret_cast<const SrDevEdge*>(g->ws + g->r_edges.offset);
+    P.items = reinterpret_cast<const SrDirectItem*>(g->ws + g->r_items.offset) + g->group_item_offset[group];
+    P.B = g->batch;
+    P.follow = how.flags();
+    if (g->dtype == SR_DTYPE_BF16) sr_launch(sr_direct_group_kernel<__nv_bfloat16>, n, kWarps * 32, 0, s, how.early, P);
+    else sr_launch(sr_direct_group_kernel<float>, n, kWarps * 32, 0, s, how.early, P);
     return 1;
 }
 
-int sr_launch_heads(const sr_graph* g, int group, cudaStream_t s)
+// Dense nodes: with 16 samples or more a block takes 4 x 8 (samples x outputs), with fewer 1 x 2, which spreads a small batch over
+// more blocks and keeps four steps of the reduction in flight.
+static bool head_wide(const sr_graph* g) { return g->batch >= 16; }
+
+static int head_blocks(const sr_graph* g, const SrHeadNode& h)
+{
+    if (h.has_mean) return g->batch;
+    const int S = head_wide(g) ? 4 : 1, CO = head_wide(g) ? 8 : 2;
+    return (g->batch + S - 1) / S * ((h.C + CO - 1) / CO);
+}
+
+// The frame input goes with the heads of a group if there is one launch of them (not of the wide kind, whose registers leave
+// room for one block beside the tensor-core kernel), and input and heads together are one block per SM at most: a launch less
+// counts where a frame takes microseconds, while a large input is better off with small blocks of its own.
+bool sr_heads_take_input(const sr_graph* g, int group, const SrFrameArgs& fr, unsigned copies, unsigned stems_R)
+{
+    const std::vector<SrHeadNode>& heads = g->group_heads[group];
+    const std::vector<const SrStem*> stems = sr_stems(g, stems_R);
+    if (heads.empty() || heads.size() > SR_HEAD_NODES || stems.size() > kStemsPerLaunch) return false;
+    int blocks = 0, mean = 0;
+    for (const SrHeadNode& h : heads) {
+        blocks += head_blocks(g, h);
+        mean += h.has_mean;
+    }
+    if (mean != 0 && mean != (int)heads.size()) return false;
+    if (mean == 0 && head_wide(g)) return false;
+    if (g->input_feeds_same_frame) {
+        // then the heads read the caller's frame itself, in vectors of four elements
+        if (fr.ctl || !stems.empty()) return false;
+        for (size_t i = 0; i < g->input_nodes.size(); ++i)
+            if (reinterpret_cast<uintptr_t>(fr.v.in_base[i]) & 15 || fr.v.in_stride_bytes[i] & 15) return false;
+    }
+    size_t next = 0;
+    return blocks + sr_plan_input(g, copies, stems, next, true).n_blocks <= 148;
+}
+
+int sr_launch_heads(const sr_graph* g, int group, bool with_input, unsigned copies, unsigned stems_R, SrFollow how, cudaStream_t s)
 {
     int launches = 0;
     for (int cls = 0; cls < 2; ++cls) {                                      // 0: nodes with a mean-dense edge, 1: without
-        // Dense nodes: with 16 samples or more a block takes 4 x 8 (samples x outputs), with fewer 1 x 2, which spreads a small
-        // batch over more blocks and keeps four steps of the reduction in flight.
-        const bool wide = g->batch >= 16;
-        const int S = cls == 0 ? 1 : (wide ? 4 : 1), CO = cls == 0 ? 1 << 30 : (wide ? 8 : 2);
+        const bool wide = head_wide(g);
         HeadParams P;
-        P.B = g->batch;
         P.fr = g->frame;
+        P.B = g->batch;
+        P.direct = with_input && g->input_feeds_same_frame ? 1 : 0;
+        P.in.n_blocks = 0;
         P.n_nodes = 0;
         int blocks = 0;
         auto flush = [&]() {
             if (P.n_nodes == 0) return;
+            if (with_input) {
+                size_t next = 0;
+                P.in = sr_plan_input(g, copies, sr_stems(g, stems_R), next, true);
+            }
+            P.follow = how.flags();
             const bool bf = g->dtype == SR_DTYPE_BF16;
+            const int n = P.in.n_blocks + blocks;
             if (cls == 0) {
-                if (bf) sr_mean_head_kernel<__nv_bfloat16><<<blocks, kHeadThreads, 0, s>>>(P);
-                else sr_mean_head_kernel<float><<<blocks, kHeadThreads, 0, s>>>(P);
+                if (bf) sr_launch(sr_mean_head_kernel<__nv_bfloat16>, n, kHeadThreads, 0, s, how.early, P);
+                else sr_launch(sr_mean_head_kernel<float>, n, kHeadThreads, 0, s, how.early, P);
             } else if (wide) {
-                if (bf) sr_head_kernel<__nv_bfloat16, 4, 8><<<blocks, kHeadThreads, 0, s>>>(P);
-                else sr_head_kernel<float, 4, 8><<<blocks, kHeadThreads, 0, s>>>(P);
+                if (bf) sr_launch(sr_head_kernel<__nv_bfloat16, 4, 8, false>, n, kHeadThreads, 0, s, how.early, P);
+                else sr_launch(sr_head_kernel<float, 4, 8, false>, n, kHeadThreads, 0, s, how.early, P);
             } else {
-                if (bf) sr_head_kernel<__nv_bfloat16, 1, 2><<<blocks, kHeadThreads, 0, s>>>(P);
-                else sr_head_kernel<float, 1, 2><<<blocks, kHeadThreads, 0, s>>>(P);
+                if (bf) sr_launch(sr_head_kernel<__nv_bfloat16, 1, 2, true>, n, kHeadThreads, 0, s, how.early, P);
+                else sr_launch(sr_head_kernel<float, 1, 2, true>, n, kHeadThreads, 0, s, how.early, P);
             }
             ++launches;
+            how.early = true;
             P.n_nodes = 0;
             blocks = 0;
         };
@@ -412,7 +608,7 @@ int sr_launch_heads(const sr_graph* g, int group, cudaStream_t s)
             if ((h.has_mean ? 0 : 1) != cls) continue;
             P.nodes[P.n_nodes] = h;
             P.first_block[P.n_nodes++] = blocks;
-            blocks += (g->batch + S - 1) / S * (cls == 0 ? 1 : (h.C + CO - 1) / CO);
+            blocks += head_blocks(g, h);
             P.first_block[P.n_nodes] = blocks;
             if (P.n_nodes == SR_HEAD_NODES) flush();
         }
@@ -421,7 +617,27 @@ int sr_launch_heads(const sr_graph* g, int group, cudaStream_t s)
     return launches;
 }
 
-int sr_direct_conv_pixels_per_block() { return kWarps * kPix; }
+// The work items of a convolutional node on the CUDA cores.
+void sr_direct_conv_items(const sr_graph* g, int v, std::vector<SrDirectItem>& items)
+{
+    const sr_node_desc& d = g->nodes[v].d;
+    const int HW = d.h * d.w;
+    if (d.c % 4 != 0) {
+        for (int b = 0; b < g->batch; ++b)
+            for (int p0 = 0; p0 < HW; p0 += kWarps * kPix) items.push_back(SrDirectItem{v, b, p0, 0});
+        return;
+    }
+    int qlog = 0;
+    while (qlog < 5 && (4 << qlog) < d.c) ++qlog;
+    // Four pixels per thread once that still gives every SM 256 threads; marked by the complement of the sample.  Measured on
+    // B200, fp32, us per frame with one / four pixels everywhere: small CNN (28 x 28 x 32, 14 x 14 x 32, 7 x 7 x 64) at 128
+    // samples 161 / 133 (this rule: 114), at 32 samples (sequential) 90 / 144, at one 27 / 51; MNIST net at 256 samples 35 / 53.
+    const bool four = (size_t)g->batch * HW * (d.c / 4) / 4 >= (size_t)148 * 256;
+    const int px = (kWarps * 32 >> qlog) * (four ? 4 : 1);
+    for (int b = 0; b < g->batch; ++b)
+        for (int p0 = 0; p0 < HW; p0 += px)
+            for (int c0 = 0; c0 < d.c; c0 += 4 << qlog) items.push_back(SrDirectItem{v, four ? ~b : b, p0, c0 | qlog << 24});
+}
 int sr_direct_dense_outputs_per_block() { return kWarps; }
 int sr_direct_dense_samples_per_block() { return kDenseB; }
 
@@ -444,6 +660,6 @@ bool sr_head_takes(const sr_graph* g, int v)
 bool sr_direct_share_sm()
 {
     auto ask = [](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess; };
-    return ask(sr_head_kernel<__nv_bfloat16, 4, 8>) && ask(sr_head_kernel<__nv_bfloat16, 1, 2>) && ask(sr_mean_head_kernel<__nv_bfloat16>) &&
+    return ask(sr_head_kernel<__nv_bfloat16, 4, 8, false>) && ask(sr_head_kernel<__nv_bfloat16, 1, 2, true>) && ask(sr_mean_head_kernel<__nv_bfloat16>) &&
            ask(sr_direct_group_kernel<__nv_bfloat16>);
 }

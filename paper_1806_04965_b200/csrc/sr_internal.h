@@ -35,18 +35,18 @@ struct SrDevNode {
 // One block's work in a grouped direct launch.
 struct SrDirectItem {
     int32_t node;        // index into the SrDevNode table
-    int32_t b0;          // first sample (dense nodes: sample chunk)
+    int32_t b0;          // first sample (dense nodes: sample chunk); its complement: four pixels per thread (conv_tile)
     int32_t p0;          // first pixel (conv nodes) or first output channel (dense nodes)
-    int32_t pad_;
+    int32_t pad_;        // conv nodes with a multiple of four channels: first channel | log2(channel quads per block) << 24
 };
 
 // Dense / mean-dense nodes as the head kernels see them: passed as kernel parameters.
 #define SR_HEAD_EDGES 6
-#define SR_HEAD_NODES 8
+#define SR_HEAD_NODES 6
 struct SrHeadEdge {
     const void* src[2];
     const float* w;              // [C_out][K]
-    int32_t HW, Cs, kind, R, K, pad_;
+    int32_t HW, Cs, kind, R, K, slot;        // slot: the source's place among the input nodes, or -1
 };
 struct SrHeadNode {
     void* state[2];
@@ -73,7 +73,50 @@ struct SrFrameArgs {
     SrFrameCtl v;
 };
 
+// How the launches of a rollout follow one another in ONE stream (programmatic dependent launch): a kernel launched with
+// `early` may be scheduled as soon as every block of the kernel before it has let its successor start, and
+// sr_wait_for_predecessor returns when that kernel has completed and its writes are visible.
+//   main     waits before it touches anything an earlier kernel reads or writes;
+//   beside   does not depend on the main kernel of its group and runs beside it: the main kernel (`late`) lets its successor
+//            start only after its own wait, so everything before the group is complete when a beside kernel starts; it does its
+//            work at once and ONE of its blocks waits for its predecessor at the end, so that it completes after the main kernel
+//            and whoever waits for it has waited for both.
+// (Before, a second stream joined by events carried the beside kernels; measured on B200 the fork and join cost 1-3 us per frame
+// on the GPU and four calls on the host.)
+struct SrFollow {
+    bool early = false, beside = false, late = false;
+    int flags() const { return (beside ? 1 : 0) | (late ? 2 : 0); }
+};
 #ifdef __CUDACC__
+__device__ __forceinline__ void sr_wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void sr_let_successor_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void sr_begin(int follow_flags)
+{
+    if (!(follow_flags & 2)) sr_let_successor_start();
+    if (!(follow_flags & 1)) sr_wait_for_predecessor();
+    if (follow_flags & 2) sr_let_successor_start();
+}
+__device__ __forceinline__ void sr_end(int follow_flags)
+{
+    if ((follow_flags & 1) && blockIdx.x == 0) sr_wait_for_predecessor();
+}
+
+template <typename Params>
+inline cudaError_t sr_launch(void (*kernel)(const Params), int blocks, int threads, size_t smem, cudaStream_t stream, bool early, const Params& p)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, p);
+}
+
 struct SrFrame { long long t, run_t; };   // this launch computes frame t+1 from frame t
 __device__ __forceinline__ SrFrame sr_frame(const SrFrameArgs& a)
 {
@@ -165,7 +208,6 @@ struct sr_graph {
     void* dn = nullptr;                            // dense resident engine state (opaque here)
     std::vector<unsigned char> dn_headers;         // its per-rank table images, uploaded when a workspace is bound
     void* graphs = nullptr;                        // CUDA-graph cache (opaque here)
-    void* side = nullptr;                          // side stream and fork / join events (opaque here)
     bool input_feeds_same_frame = false;           // some edge that leaves an input node has R = 0
     // deep-window mode: a second graph of the same network whose batch holds the W frames of a window side by side
     sr_graph* window = nullptr;

@@ -60,7 +60,7 @@ constexpr int kMaxW = 12;                             // weight ring depth (one 
 constexpr int kItems = 8;                             // work items the keeper may be ahead of the epilogue
 constexpr int kTables = 3;                            // node tables in shared memory
 // Dynamic shared memory of a CTA.  With the 19 KiB of static shared memory this leaves about 12 KiB of the SM's 228 KiB
-// free: the other kernels of a frame (input staging, dense heads: up to 7.4 KiB per block) run on a second stream beside
+// free: the other kernels of a frame (input staging, dense heads: up to 7.4 KiB per block) run beside
 // the persistent CTAs, and measured on B200 they queue behind them, frame after frame, once less than about 10 KiB of
 // the SM's shared-memory partition is left (a 117 us frame then takes 170 us).
 constexpr int kSmemBudget = 196 * 1024;
@@ -142,7 +142,7 @@ struct TcParams {
     int* sched;                     // counters of the shared list, or null
     long long wait_limit;
     int n_tiles, n_own;             // items in all; those of the matrix
-    int B;
+    int B, follow;
     int table_bytes;                // shared memory of one node table
     int n_w, w_slot;                // weight ring: slots and their size
     int ring_kb;                    // activation ring in KiB
@@ -303,10 +303,12 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
     __shared__ __align__(16) uint16_t epi_buf[kEpiWarps][32 * 32];   // per epilogue warp: 32 pixels x 32 channels, bf16
     __shared__ int pix_off[2][kMaxCols];                   // element offset of every pixel of an item, -1 = not stored
 
+    if (!(P.follow & 2)) sr_let_successor_start();
     const long long wait_limit = P.wait_limit;
     // A wait limit of zero (a host-side test hook) means "every wait has already expired": report it and return
     // before any barrier, tensor memory, copy or MMA is touched.
     if (wait_limit <= 0) {
+        sr_wait_for_predecessor();
         if (threadIdx.x == 0) atomicExch(P.error, 1);
         return;
     }
@@ -355,6 +357,8 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
 
     if (warp == 2) {
         // ---------------------------------------------------------------- keeper
+        // (It does not wait for the predecessor to look at tables; the shared list's counter is the predecessor's too.)
+        bool waited = false;
         int slot_node = -1, slot_gen = -1;                 // lane s < kTables: the node whose table slot s holds, the last item that uses it
         int slot = -1, cached = -1;
         bool own = true, ok = true;
@@ -379,6 +383,8 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
             }
             if (!own && P.sched && P.n_own < P.n_tiles) {
                 int v = 0;
+                if (!waited) sr_wait_for_predecessor();
+                waited = true;
                 if (lane == 0) v = P.n_own + atomicAdd(P.sched, 1);
                 v = __shfl_sync(0xffffffffu, v, 0);
                 if (v < P.n_tiles) tl = P.tiles[v];
@@ -464,6 +470,9 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
         // ---------------------------------------------------------------- activation producer
         // Box j uses barrier pair j % kBoxes and the bytes [pos, pos + size) of the ring; it wraps as a whole.  `head` counts KiB
         // from the start of the launch, skipped ones included: head minus the start of the oldest box is what is in use.
+        // (The weights do not depend on the predecessor, so their producer does not wait for it; the activations do.)
+        sr_wait_for_predecessor();
+        if (P.follow & 2) sr_let_successor_start();
         if (elect_one()) {
             uint32_t n = 0, n_free = 0;                           // boxes started; boxes known to be released
             uint32_t pos = 0, head = 0;
@@ -669,6 +678,7 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
         // the warp as one 64-byte run.  The element offset of every pixel of the work item (or -1 for separator
         // rows and pixels outside the image) is tabulated once per item, in one of two tables, so that one barrier per
         // item is enough; that barrier also makes giving up a joint decision.
+        sr_wait_for_predecessor();
         const int ew = warp - 4, quarter = ew & 3, half = ew >> 2;      // TMEM lanes 32*quarter .. +31 belong to this warp
         const int et = threadIdx.x - 128;                               // 0..255 among the epilogue threads
         uint16_t* tbuf = &epi_buf[ew][0];
@@ -1557,7 +1567,7 @@ bool sr_tc_stages(const sr_graph* g, int edge)
     return g->nodes[g->edges[edge].d.tgt].use_tc && is_stem(g, g->edges[edge]);
 }
 
-int sr_tc_launch_group(sr_graph* g, int group, cudaStream_t s)
+int sr_tc_launch_group(sr_graph* g, int group, SrFollow how, cudaStream_t s)
 {
     TcEngine* E = eng(g);
     if (!E || E->group_tiles[group].empty()) return 0;
@@ -1593,7 +1603,8 @@ int sr_tc_launch_group(sr_graph* g, int group, cudaStream_t s)
     P.n_w = E->group_n_w[group];
     P.w_slot = E->group_w_slot[group];
     P.ring_kb = E->group_ring_kb[group];
-    sr_tc_group_kernel<<<E->group_grid[group], kThreads, smem, s>>>(P);
+    P.follow = how.flags();
+    sr_launch(sr_tc_group_kernel, E->group_grid[group], kThreads, smem, s, how.early && !timed, P);
     if (timed) {
         cudaEventRecord(E->ev[E->ev_used + 1], s);
         E->ev_used += 2;

@@ -282,3 +282,17 @@ def test_staged_input_edges(cin, k, stride, size):
     g.patterns = {"p": [i % 2 for i in range(n)] + [1] * (len(edges) - n)}
     parity.check_stepwise(g, "p", zero_bias=False)
     parity.check_run(g, "p", graph_frames=2, resident=False)
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("batch,size,cin,c", [(3, 5, 3, 4), (3, 7, 8, 12), (2, 9, 60, 132), (130, 16, 4, 128)])
+def test_cuda_core_convolutions_at_the_edges_of_their_tiles(batch, size, cin, c, dtype):
+    # channel quads per block 1 .. 32 with a remainder, pixels that do not fill a block, reductions longer than the table in
+    # shared memory (9 x 60 / 4 and 9 x 132 / 4 vectors, 25 x 3 scalars), one and (the last case) four pixels per thread
+    from workloads.graphs import CONV, GAP_DENSE, IDENTITY, Edge, GraphSpec, Node, check_shapes
+    nodes = [Node("in", size, size, cin, IDENTITY), Node("a", size, size, c), Node("b", (size + 1) // 2, (size + 1) // 2, c, IDENTITY), Node("o", 1, 1, 3, IDENTITY)]
+    edges = [Edge(0, 1, CONV, 5 if cin == 3 else 3, 1), Edge(1, 1, CONV, 3, 1), Edge(1, 2, CONV, 3, 2), Edge(0, 2, CONV, 1, 2), Edge(2, 3, GAP_DENSE)]
+    g = GraphSpec("tiles", nodes, edges, batch=batch, frames=2, dtype=dtype, seed=93)
+    check_shapes(g)
+    g.patterns = {"p": [1, 1, 1, 0, 1]}
+    parity.check_stepwise(g, "p", engine="direct", zero_bias=False, samples=[0, batch - 1])
