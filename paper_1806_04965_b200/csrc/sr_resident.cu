@@ -980,6 +980,44 @@ bool rs_layout(const sr_graph* g, RsEngine& E, int cs, int warps)
 
 RsEngine* rs_of(const sr_graph* g) { return static_cast<RsEngine*>(g->rs); }
 
+typedef void (*RsKernel)(const unsigned char*, int, const SrFrameCtl, int, int);
+
+RsKernel rs_kernel_of(const RsEngine& E) { return E.warps <= 16 ? sr_resident_kernel<512> : E.warps <= 24 ? sr_resident_kernel<768> : sr_resident_kernel<1024>; }
+
+cudaLaunchConfig_t rs_config(const RsEngine& E, int batch, cudaStream_t s, cudaLaunchAttribute* at)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(batch * E.cs));
+    cfg.blockDim = dim3((unsigned)(E.warps * 32));
+    cfg.dynamicSmemBytes = (size_t)E.smem_bytes;
+    cfg.stream = s;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)E.cs;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = E.cs > 1 ? 1 : 0;
+    return cfg;
+}
+
+// Clusters (sequences) the device holds at once.
+int rs_clusters_held(const RsEngine& E)
+{
+    int sms = 148, dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int n = std::max(1, sms / E.cs);
+    if (E.cs > 1) {
+        cudaLaunchAttribute at[1];
+        const cudaLaunchConfig_t cfg = rs_config(E, 1, nullptr, at);
+        int held = 0;
+        if (cudaFuncSetAttribute(rs_kernel_of(E), cudaFuncAttributeMaxDynamicSharedMemorySize, kRsSmemMax) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&held, rs_kernel_of(E), &cfg) == cudaSuccess && held > 0)
+            n = held;
+        cudaGetLastError();
+    }
+    return n;
+}
+
 }  // namespace
 
 void sr_rs_destroy(sr_graph* g)
@@ -1118,27 +1156,26 @@ sr_status sr_rs_plan(sr_graph* g, size_t& offset)
             L[kk] = (uint32_t)((tap / he.k_eff) * P + (tap % he.k_eff) * Cs + ci);
         }
     }
-    // cluster size: the largest that still gives every sequence its own cluster in one wave, else the
-    // smallest that fits
-    int sms = 148, dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    std::vector<int> order;
-    if (g->opt_rs_cluster > 0) {
-        order.push_back(g->opt_rs_cluster);
-    } else {
-        for (int c = kRsMaxCluster; c >= 1; c >>= 1)
-            if (g->batch * c <= sms) order.push_back(c);
-        for (int c = 1; c <= kRsMaxCluster; c <<= 1)
-            if (g->batch * c > sms) order.push_back(c);
-    }
     // 24 warps (80 registers each) hide the shared-memory latencies best on B200; with 32 the 64-register build spills
     const int warps = std::min(kRsMaxWarps, g->opt_rs_warps > 0 ? g->opt_rs_warps : 24);
+    // Cluster size: the one that ends first.  A run of more sequences than the device holds clusters takes several waves, and the
+    // device holds fewer clusters than its SMs suggest (a cluster does not span GPCs: of 148 SMs, 37 clusters of four do not fit
+    // at once: a pass of 37 sequences x 20 sequential frames of the small CNN takes 452 us in clusters of four and 284 in
+    // clusters of two; 33 sequences 236 against 283).  Time per frame of one wave, measured on that network: 4.2 us in clusters
+    // of four, 6.5 of two.
     bool placed = false;
-    for (int c : order)
-        if (rs_layout(g, *E, c, warps)) {
-            placed = true;
-            break;
-        }
+    double best = 0.0;
+    for (int c = kRsMaxCluster; c >= 1; c >>= 1) {
+        if (g->opt_rs_cluster > 0 && c != g->opt_rs_cluster) continue;
+        RsEngine F = *E;
+        if (!rs_layout(g, F, c, warps)) continue;
+        const int held = rs_clusters_held(F);
+        const double cost = (double)((g->batch + held - 1) / held) * (1.9 + 9.2 / c);
+        if (placed && cost >= best) continue;
+        placed = true;
+        best = cost;
+        *E = F;
+    }
     if (!placed) {
         delete E;
         return SR_OK;
@@ -1393,24 +1430,11 @@ sr_status sr_rs_launch(sr_graph* g, int T, const SrFrameCtl& init, cudaStream_t 
     RsEngine* E = rs_of(g);
     if (!E) return SR_ERR_STATE;
     if (!E->attr_set) {
-        if (cudaFuncSetAttribute(sr_resident_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, E->smem_bytes) != cudaSuccess ||
-            cudaFuncSetAttribute(sr_resident_kernel<768>, cudaFuncAttributeMaxDynamicSharedMemorySize, E->smem_bytes) != cudaSuccess ||
-            cudaFuncSetAttribute(sr_resident_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, E->smem_bytes) != cudaSuccess)
-            return SR_ERR_CUDA;
+        if (cudaFuncSetAttribute(rs_kernel_of(*E), cudaFuncAttributeMaxDynamicSharedMemorySize, kRsSmemMax) != cudaSuccess) return SR_ERR_CUDA;
         E->attr_set = true;
     }
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(g->batch * E->cs));
-    cfg.blockDim = dim3((unsigned)(E->warps * 32));
-    cfg.dynamicSmemBytes = (size_t)E->smem_bytes;
-    cfg.stream = s;
     cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)E->cs;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = E->cs > 1 ? 1 : 0;
+    const cudaLaunchConfig_t cfg = rs_config(*E, g->batch, s, at);
     const unsigned char* blobs = reinterpret_cast<const unsigned char*>(g->ws + E->r_blobs.offset);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     bool timed = g->opt_time_tc != 0 && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
@@ -1424,10 +1448,7 @@ sr_status sr_rs_launch(sr_graph* g, int T, const SrFrameCtl& init, cudaStream_t 
         if (E->ev_used + 2 > E->ev.size()) timed = false;
     }
     if (timed) cudaEventRecord(E->ev[E->ev_used], s);
-    cudaError_t le;
-    if (E->warps <= 16) le = cudaLaunchKernelEx(&cfg, sr_resident_kernel<512>, blobs, E->blob_bytes, init, T, E->cs);
-    else if (E->warps <= 24) le = cudaLaunchKernelEx(&cfg, sr_resident_kernel<768>, blobs, E->blob_bytes, init, T, E->cs);
-    else le = cudaLaunchKernelEx(&cfg, sr_resident_kernel<1024>, blobs, E->blob_bytes, init, T, E->cs);
+    const cudaError_t le = cudaLaunchKernelEx(&cfg, rs_kernel_of(*E), blobs, E->blob_bytes, init, T, E->cs);
     if (le != cudaSuccess) return SR_ERR_CUDA;
     if (timed) {
         cudaEventRecord(E->ev[E->ev_used + 1], s);

@@ -166,3 +166,10 @@ def test_resident_and_launch_path_agree_at_full_size():
         G.sync_status()
     assert np.abs(outs[1]).max() > 0
     assert parity.rel_err(outs[0], outs[1].astype(np.float64)) <= parity.TOL["bf16"]
+
+
+def test_more_sequences_than_clusters_of_four_fit():
+    # 37 sequences: 148 CTAs in clusters of four, which a device of 148 SMs does not hold at once
+    g = graphs.build("c2", batch=37, frames=3)
+    for p in g.patterns:
+        parity.check_run(g, p, samples=[0, 18, 36])
