@@ -200,7 +200,10 @@ int enqueue_frames(sr_graph* g, const SrFrameArgs& fr, int frames, cudaStream_t 
     int launches = 0;
     // events between two launches of a stream (the timing option) need plain launches around them
     const bool chain = !g->opt_time_tc, overlap = g->opt_overlap != 0;
-    bool first = true;
+    // The first launch may start early as well: what comes before it in the stream (an earlier call's kernel, the caller's own
+    // work) either lets it or, not knowing, holds it until it has completed.  Not while a capture records the stream.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    bool first = cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
     auto follow = [&](bool beside, bool late) {
         SrFollow how;
         how.early = chain && !first;
