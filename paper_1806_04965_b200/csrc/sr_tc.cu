@@ -59,11 +59,11 @@ constexpr int kBoxes = 8;                             // activation boxes in fli
 constexpr int kMaxW = 12;                             // weight ring depth (one weight group per slot)
 constexpr int kItems = 8;                             // work items the keeper may be ahead of the epilogue
 constexpr int kTables = 3;                            // node tables in shared memory
-// Dynamic shared memory of a CTA.  With the 19 KiB of static shared memory this leaves about 12 KiB of the SM's 228 KiB
+// Dynamic shared memory of a CTA.  With the 11 KiB of static shared memory this leaves about 12 KiB of the SM's 228 KiB
 // free: the other kernels of a frame (input staging, dense heads: up to 7.4 KiB per block) run beside
 // the persistent CTAs, and measured on B200 they queue behind them, frame after frame, once less than about 10 KiB of
 // the SM's shared-memory partition is left (a 117 us frame then takes 170 us).
-constexpr int kSmemBudget = 196 * 1024;
+constexpr int kSmemBudget = 204 * 1024;
 constexpr int kMaxNodeKb = 128;                       // K-blocks per node
 
 // A run of equally wide K-blocks of a node's reduction as the weight producer sees it: n_groups weight groups (one copy
@@ -266,17 +266,16 @@ __device__ __forceinline__ void tc_commit(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32])
+// 16 TMEM lanes x 16 columns: thread T gets columns 2 * (T % 4), + 1 (and those + 8: r[4..7]) of lanes T / 4 (r[0, 1]) and T / 4 + 8
+// (r[2, 3]), i.e. the fragments that stmatrix takes.
+__device__ __forceinline__ void tc_ld_16x16(uint32_t taddr, uint32_t (&r)[8])
 {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr) : "memory");
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void stmatrix_x4_trans(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
@@ -300,7 +299,7 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
     __shared__ TcTile items[kItems];                       // the item ring; node -1 = end of the list
     __shared__ uint32_t box_start[kBoxes];                 // the activation producer's own: `head` at the start of each box
     __shared__ volatile int epi_done;                      // items the epilogue has finished
-    __shared__ __align__(16) uint16_t epi_buf[kEpiWarps][32 * 32];   // per epilogue warp: 32 pixels x 32 channels, bf16
+    __shared__ __align__(16) uint16_t epi_buf[kEpiWarps][16 * 32];   // per epilogue warp: 16 pixels x 32 channels, bf16
     __shared__ int pix_off[2][kMaxCols];                   // element offset of every pixel of an item, -1 = not stored
 
     if (!(P.follow & 2)) sr_let_successor_start();
@@ -672,16 +671,21 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
     } else if (warp >= 4) {
         // ---------------------------------------------------------------- epilogue (warps 4..11)
         // TMEM lane = output channel, TMEM column = pixel.  Two warps share each quarter of the 128 lanes and take
-        // alternate 32-column chunks.  A warp turns 32 channels x 32 pixels into NHWC order through a 2 KiB
-        // shared-memory buffer: every thread writes its channel of 32 pixels (bias, ReLU, bf16), then reads back
-        // 8 consecutive channels of one pixel and stores them as one 16-byte word, so a pixel's 32 channels leave
-        // the warp as one 64-byte run.  The element offset of every pixel of the work item (or -1 for separator
+        // alternate 16-column chunks.  A warp turns 32 channels x 16 pixels into NHWC order through a 1 KiB shared-memory buffer:
+        // bias, ReLU and bf16 on fragments of 8 x 8 that stmatrix stores transposed, then every thread reads back 8 consecutive
+        // channels of one pixel and stores them as one 16-byte word, so a pixel's 32 channels leave the warp as one 64-byte
+        // run.  (With one 2-byte store per value the deepest CIFAR10 network took 74.6 us per frame, so 72.5.)  The element offset of every pixel of the work item (or -1 for separator
         // rows and pixels outside the image) is tabulated once per item, in one of two tables, so that one barrier per
         // item is enough; that barrier also makes giving up a joint decision.
         sr_wait_for_predecessor();
         const int ew = warp - 4, quarter = ew & 3, half = ew >> 2;      // TMEM lanes 32*quarter .. +31 belong to this warp
         const int et = threadIdx.x - 128;                               // 0..255 among the epilogue threads
         uint16_t* tbuf = &epi_buf[ew][0];
+        // the buffer holds 64 bytes per pixel; its four 16-byte chunks (8 channels each) are stored at chunk ^ (pixel / 2 % 4), which
+        // keeps both the matrix stores (rows = pixels) and the reads (8 pixels x 4 chunks) free of bank conflicts
+        const int st_px = lane & 7, ld_px = lane >> 2;
+        const uint32_t st_addr = smem_u32(tbuf) + st_px * 64 + (((lane >> 3) ^ ((st_px >> 1) & 3)) * 16);
+        const uint32_t ld_off = (uint32_t)(ld_px * 64 + (((lane & 3) ^ ((ld_px >> 1) & 3)) * 16));
         bool ok = true;
         for (int it = 0;; ++it) {
             ok = ok && mbar_wait(bar_item + 8 * (it & (kItems - 1)), (it / kItems) & 1, abortp, wait_limit);
@@ -711,8 +715,12 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
             const bool second = fused && quarter >= 2;              // this warp's TMEM lanes belong to the plan's second node
             __nv_bfloat16* out = static_cast<__nv_bfloat16*>(second ? nd->state2[cur] : nd->state[cur]);
             const int co_w = fused ? (quarter & 1) * 32 : tl.m0 + quarter * 32;   // first channel of this warp
-            const int co = co_w + lane;                             // TMEM lane = output channel
-            const float bias = co < C ? __ldg((second ? nd->bias2 : nd->bias) + co) : 0.f;
+            float bias[4];                                          // of channels co_w + lane / 4 + 0, 8, 16, 24
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int co = co_w + (lane >> 2) + 8 * q;
+                bias[q] = co < C ? __ldg((second ? nd->bias2 : nd->bias) + co) : 0.f;
+            }
             const int act = second ? nd->act2 : nd->act;
             const bool gvalid = co_w + (lane & 3) * 8 < C;          // this thread's group of 8 channels exists
             ok = mbar_wait(bar_tfull + 8 * acc, ((uint32_t)it >> 1) & 1u, abortp, wait_limit);
@@ -720,24 +728,36 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
             if (!ok) continue;                                      // to the joint decision at the next barrier
             tc_fence_after();
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * kMaxCols;
-            for (int c0 = half * 32; c0 < n_cols; c0 += 64) {
-                uint32_t v[32];
-                tc_ld32(taddr + c0, v);
+            uint32_t lo[8], hi[8];                                  // TMEM lanes 0..15 and 16..31 of the quarter
+            const int c_first = half * 16;
+            if (c_first < n_cols) {
+                tc_ld_16x16(taddr + c_first, lo);
+                tc_ld_16x16(taddr + (16u << 16) + c_first, hi);
+            }
+            for (int c0 = c_first; c0 < n_cols; c0 += 32) {
                 tc_wait_ld();
+                uint32_t h[2][4];                                   // [8 pixels][8 channels]: two pixels of one channel per word
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    float z = __uint_as_float(v[j]) + bias;
-                    if (act == 1) z = fmaxf(z, 0.f);
-                    const __nv_bfloat16 hz = __float2bfloat16_rn(z);
-                    tbuf[j * 32 + lane] = *reinterpret_cast<const uint16_t*>(&hz);
+                for (int pb = 0; pb < 2; ++pb)
+#pragma unroll
+                    for (int cb = 0; cb < 4; ++cb) {
+                        const uint32_t* r = (cb < 2 ? lo : hi) + pb * 4 + (cb & 1) * 2;
+                        __nv_bfloat162 z = __floats2bfloat162_rn(__uint_as_float(r[0]) + bias[cb], __uint_as_float(r[1]) + bias[cb]);
+                        if (act == 1) z = __hmax2(z, __floats2bfloat162_rn(0.f, 0.f));
+                        h[pb][cb] = *reinterpret_cast<const uint32_t*>(&z);
+                    }
+                if (c0 + 32 < n_cols) {                             // the next chunk, on its way during the stores
+                    tc_ld_16x16(taddr + c0 + 32, lo);
+                    tc_ld_16x16(taddr + (16u << 16) + c0 + 32, hi);
                 }
+                stmatrix_x4_trans(st_addr, h[0][0], h[0][1], h[0][2], h[0][3]);
+                stmatrix_x4_trans(st_addr + 512, h[1][0], h[1][1], h[1][2], h[1][3]);
                 __syncwarp();
 #pragma unroll
-                for (int pass = 0; pass < 4; ++pass) {
-                    const int p = pass * 8 + (lane >> 2);
-                    const int o = poff[c0 + p];
+                for (int pass = 0; pass < 2; ++pass) {
+                    const int o = poff[c0 + pass * 8 + (lane >> 2)];
                     if (o >= 0 && gvalid) {
-                        const uint4 w = *reinterpret_cast<const uint4*>(tbuf + p * 32 + (lane & 3) * 8);
+                        const uint4 w = *reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(tbuf) + pass * 512 + ld_off);
                         *reinterpret_cast<uint4*>(out + (size_t)o + co_w + (lane & 3) * 8) = w;
                     }
                 }
@@ -1048,6 +1068,18 @@ void build_groups(NodePlan& P)
     P.k_total = k_off;
 }
 
+// Two consecutive weight groups are one burst if their K-blocks are equally wide.
+bool one_burst(const NodePlan& P, size_t gi)
+{
+    return gi + 1 < P.wgroups.size() && P.kbs[P.wgroups[gi + 1].first_kb].bk == P.kbs[P.wgroups[gi].first_kb].bk;
+}
+int count_bursts(const NodePlan& P)
+{
+    int n = 0;
+    for (size_t gi = 0; gi < P.wgroups.size(); ++n) gi += one_burst(P, gi) ? 2 : 1;
+    return n;
+}
+
 std::vector<TcTile> node_tiles(const sr_graph* g, const NodePlan& P, int node_index)
 {
     const SrHostNode& n = g->nodes[P.node];
@@ -1256,8 +1288,12 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
             if (tl.size() > 8 * (size_t)E->sm_count) break;        // plenty of items: smaller tiles only cost copies
         }
         const std::vector<std::pair<long long, TcTile>> tl = plan_tiles(best_cols);
-        // Shared memory: six weight slots, the node tables, and the rest for activation boxes, of which two of the largest
-        // should fit.
+        // Shared memory: weight slots, the node tables, and the rest for activation boxes, of which two of the largest should
+        // fit.  A launch with several items per CTA is better off with room for a third box (a box read by one tap only lasts
+        // 512 cycles of MMAs, and the one after it has to be on its way before that), one with an item or two per CTA with a
+        // deeper weight ring.  Measured on B200, us per frame with six / five / four slots: six-node network at 256 samples
+        // 146.3 / 143.0 / 147.8, ten-node at 128 115.1 / 112.7 / 117.9, stress graph at 32 253.9 / 246.2 / 250.7, deep window
+        // 100.8 / 100.4 / 103.3; six-node hybrid at 37 samples (one item per CTA) 57.3 / 59.1 / 64.0.
         int w_slot = 1024, box_kb = 1, n_tab = 0;
         for (int ni : members) {
             const NodePlan& P = E->nodes[ni];
@@ -1268,16 +1304,16 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
                 bk_max = std::max(bk_max, kb.bk);
             }
             w_slot = std::max(w_slot, (int)sr_align_up((size_t)std::min(P.rows_total(g), 128) * std::max(64, bk_max) * 2, 1024));
-            n_tab = std::max(n_tab, 2 * (int)P.kbs.size() + n_act);
+            build_groups(E->nodes[ni]);
+            n_tab = std::max(n_tab, 2 * count_bursts(P) + n_act);
         }
         const int table_bytes = (int)sizeof(TcNode) + n_tab * 16;
         const int avail = kSmemBudget - 1024 - kTables * table_bytes;
-        int n_w = g->opt_b_units > 0 ? std::min(kMaxW, std::max(2, g->opt_b_units)) : 6;
+        int n_w = g->opt_b_units > 0 ? std::min(kMaxW, std::max(2, g->opt_b_units)) : (best_cols == kMaxCols && tl.size() > 2 * (size_t)E->sm_count ? 5 : 6);
         while (n_w > 3 && (avail - n_w * w_slot) / 1024 < 2 * box_kb) --n_w;
         while (n_w > 2 && (avail - n_w * w_slot) / 1024 < box_kb) --n_w;
         const int ring_kb = (avail - n_w * w_slot) / 1024;
         if (!members.empty() && (ring_kb < box_kb || box_kb > 255)) return SR_ERR_UNSUPPORTED;
-        for (int ni : members) build_groups(E->nodes[ni]);
         // Work lists: the items go, longest first, to the CTA with the least work so far; CTA c walks column c of a
         // matrix with one row per round (entries of node -1 pad the shorter columns).  Unless the lists are asked to be
         // static, the smallest items - a fifth of the work, if the launch has more than two items per CTA - stay out of
@@ -1460,7 +1496,7 @@ sr_status sr_tc_bind(sr_graph* g)
         std::vector<TcBurst> db;
         for (size_t gi = 0; gi < P.wgroups.size();) {
             const int i0 = P.wgroups[gi].first_kb, bk = P.kbs[i0].bk;
-            const bool two = gi + 1 < P.wgroups.size() && P.kbs[P.wgroups[gi + 1].first_kb].bk == bk;
+            const bool two = one_burst(P, gi);
             TcBurst b{};
             b.w_hi = dm[i0].w_hi;
             b.l1_off16 = (uint16_t)(8 * bk * 2 >> 4);                          // a lane's window lies 8 pixels after the one before
@@ -1544,11 +1580,16 @@ sr_status sr_tc_set_weights(sr_graph* g, int edge, const float* w_eff)
         for (size_t j = i; j < end; ++j) {
             const KbHost& kb = P.kbs[j];
             const int n_src = kb.stem ? std::max(0, std::min(kb.bk, he.K - kb.src_col)) : kb.bk;
-            for (int co = 0; co < t.d.c; ++co)
-                for (int k = 0; k < n_src; ++k) {
-                    const __nv_bfloat16 b = __float2bfloat16_rn(w_eff[(size_t)co * he.K + kb.src_col + k]);
-                    std::memcpy(&h[(size_t)co * width + col + k], &b, 2);
+            for (int co = 0; co < t.d.c; ++co) {
+                const float* src = w_eff + (size_t)co * he.K + kb.src_col;
+                uint16_t* dst = &h[(size_t)co * width + col];
+                for (int k = 0; k < n_src; ++k) {                 // to the nearest bfloat16, ties to even; NaN stays NaN
+                    uint32_t u;
+                    std::memcpy(&u, &src[k], 4);
+                    const uint32_t r = (u + 0x7FFFu + ((u >> 16) & 1u)) >> 16;
+                    dst[k] = (uint16_t)((u & 0x7FFFFFFFu) > 0x7F800000u ? 0x7FFFu : r);
                 }
+            }
             col += kb.bk;
         }
         const int row_off = P.kbs[i].edge == edge ? P.kbs[i].row_off : 64;
