@@ -3,25 +3,28 @@
 //
 // Such a network (the paper's H2 / O layers, a tiny MLP) moves a few hundred kilobytes of weights per frame and does a
 // million multiply-adds: launched frame by frame it is pure launch latency.  Here a cluster of eight or sixteen CTAs
-// keeps ALL weights in shared memory, split by output rows, and walks the frames of eight sequences by itself:
-//   - every CTA holds a full copy of every node state of its eight sequences (two buffers by frame parity; input
+// keeps ALL weights in shared memory, split by output rows, and walks the frames of two, four or eight sequences by itself:
+//   - every CTA holds a full copy of every node state of its sequences (two buffers by frame parity; input
 //     nodes three, because the next input frame is fetched with cp.async while the current update still reads the
 //     previous one);
 //   - a work unit is up to four output rows of one node; a warp takes a unit, its lanes stride over the reduction
-//     index with 16-byte loads (one weight vector per row, one state vector per sequence: 12 loads feed 128
-//     multiply-adds; what bounds a frame is the shared-memory bandwidth, and two-row units needed 10 loads per 64),
-//     shuffles sum the lanes (halving the number of values per step until a group of four lanes holds the four
-//     rows of one sequence), and the results (bias, ReLU) are written as one 16-byte word into the state copies of
-//     ALL CTAs of the cluster through distributed shared memory; warps never wait for each other inside a level.
-//     (Measured alternatives, both slower: eight-row jobs whose reduction index is split over warps with two
-//     block-wide barriers per level; four-row units cut along the reduction index into parts on up to fourteen warps
-//     that hand their partial sums to the unit's first part through shared memory and a named barrier, 3.1 against
-//     2.8 us per frame: the shared-memory traffic stays the same and every part pays the reduction over the lanes.)
+//     index with 16-byte loads (one weight vector per row, one state vector per sequence), multiply-adds are two to an
+//     instruction (fma.rn.f32x2 on neighbouring elements of the vectors), shuffles sum the
+//     lanes (halving the number of values per step until a group of lanes holds the four rows of one sequence), and the
+//     results (bias, ReLU) are written as one 16-byte word into the state copies of ALL CTAs of the cluster; warps never wait
+//     for each other inside a level.  (Measured alternative: four-row units cut along the reduction index into parts on up to
+//     fourteen warps that hand their partial sums on through shared memory, 3.1 against 2.8 us per frame at the time: the
+//     shared-memory traffic stays the same and every part pays the reduction over the lanes.)
 //   - units are given to the warps longest first (host side); the warps left without a unit in the first level fetch
 //     the next input frame;
-//   - a tableau level (Eq. 4) ends at a cluster barrier; a streaming frame has one.
-// The sums run in a fixed order, so results are reproducible bit for bit.  There is no spin-wait: the only
-// synchronisation is the hardware cluster barrier, reached by every thread the same number of times.
+//   - a tableau level (Eq. 4) ends when its new states have arrived: the stores into the other CTAs (st.async) count their
+//     bytes on a barrier there, one per level and frame parity, which every warp waits for (bounded: on expiry the kernel
+//     records an error and returns).  No cluster-wide barrier per frame.
+// What bounds it: latency.  On the 784-128-128-10 network, B = 8, 256 frames took 721 us (2.70 per further frame) with eight
+// sequences per cluster, sixteen warps, scalar multiply-adds and a cluster barrier per frame, 656 us (2.49) with the packed
+// multiply-adds and the counted stores, whose shared-memory loads per step stayed the same, and take 388 us (1.45) with two
+// sequences per cluster.
+// The sums run in a fixed order, so results are reproducible bit for bit.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -34,9 +37,10 @@
 namespace {
 
 constexpr int kDnMaxNodes = 16, kDnMaxEdges = 32, kDnMaxLevels = 16, kDnMaxUnits = 128;
+constexpr int kDnMaxSamples = 8;       // sequences per cluster, most
+constexpr int kDnMoreThanHalf = 120 * 1024;   // of an SM's shared memory, bytes
 constexpr int kDnMaxCluster = 16;      // CTAs per cluster: 8, or 16 (a non-portable size) for rollouts with one level per frame
-constexpr int kDnSamples = 8;          // sequences per cluster
-constexpr int kDnWarps = 16;
+constexpr int kDnWarps = 8;            // 256 threads: a work unit keeps 64 registers of packed accumulators and its operands
 constexpr int kDnRows = 4;             // output rows per work unit
 constexpr int kDnSmemMax = 220 * 1024;
 
@@ -68,9 +72,9 @@ static_assert(sizeof(DnUnit) == 48, "read as three 16-byte words");
 constexpr int kDnMaxTerms = 256;
 
 struct DnBlobHdr {                     // head of a rank's blob; the rank's weight slices follow
-    int32_t n_units, fetch_warp0, pad_[2];                   // fetch_warp0: first of the warps that fetch input frames
+    int32_t n_units, fetch_mask, idle, pad_;                 // fetch_mask: warps that fetch input frames; idle: the rank has no unit
     int32_t level_begin[kDnMaxLevels + 1];                   // units of level l: [level_begin[l-1], level_begin[l]); warp w
-    int32_t pad2_[3];                                        // takes entries w, w + 16, ... of a level
+    int32_t pad2_[3];                                        // takes entries w, w + kDnWarps, ... of a level
     DnUnit units[kDnMaxUnits];
     DnTerm terms[kDnMaxTerms];
 };
@@ -79,7 +83,10 @@ static_assert(offsetof(DnBlobHdr, units) % 16 == 0 && offsetof(DnBlobHdr, terms)
 
 struct DnParams {
     int32_t n_nodes, n_edges, n_levels, B;
-    int32_t blob_bytes, hdr_floats, total_floats, pad_;
+    int32_t blob_bytes, hdr_floats, total_floats, n_idle;    // n_idle: ranks without a unit
+    int32_t level_bytes[kDnMaxLevels];                       // bytes that a level's new states are, in one CTA's copy
+    int32_t* error;                                          // device-side error code
+    long long wait_limit;                                    // cycles after which a wait gives up
     const unsigned char* blobs;        // one blob of blob_bytes per rank of the cluster
     DnNode nodes[kDnMaxNodes];
     DnEdge edges[kDnMaxEdges];
@@ -94,19 +101,42 @@ __device__ __forceinline__ void dn_cluster_sync()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ __forceinline__ uint32_t dn_map_rank(const float* local, uint32_t rank)
+__device__ __forceinline__ uint32_t dn_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t dn_map_rank(uint32_t local, uint32_t rank)
 {
     uint32_t remote;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"((uint32_t)__cvta_generic_to_shared(local)), "r"(rank));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
     return remote;
 }
-__device__ __forceinline__ void dn_st_cluster(const float* local, uint32_t rank, float v)
+// Stores into another CTA's shared memory that count their bytes on a barrier there: whoever waits for the barrier sees them.
+__device__ __forceinline__ void dn_st_async(uint32_t cell, uint32_t bar, uint32_t rank, float v)
 {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(dn_map_rank(local, rank)), "f"(v) : "memory");
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];"
+                 ::"r"(dn_map_rank(cell, rank)), "f"(v), "r"(dn_map_rank(bar, rank)) : "memory");
 }
-__device__ __forceinline__ void dn_st_cluster4(const float* local, uint32_t rank, const float (&v)[4])
+__device__ __forceinline__ void dn_st_async4(uint32_t cell, uint32_t bar, uint32_t rank, const float (&v)[4])
 {
-    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dn_map_rank(local, rank)), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]) : "memory");
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(dn_map_rank(cell, rank)), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"(dn_map_rank(bar, rank)) : "memory");
+}
+// Bounded wait for a phase of a barrier that other CTAs' stores complete.
+__device__ __forceinline__ bool dn_wait(uint32_t bar, uint32_t parity, volatile int* gave_up, long long limit)
+{
+    long long t0 = 0;
+    for (int i = 0;; ++i) {
+        uint32_t ok;
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.b32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (ok) return true;
+        if ((i & 31) == 31) {
+            const long long t = clock64();
+            if (t0 == 0) t0 = t;
+            if (*gave_up || t - t0 > limit) {
+                *gave_up = 1;
+                return false;
+            }
+        }
+    }
 }
 
 // Fetch `n` floats (a multiple of 4, 16-byte aligned on both sides) with cp.async.
@@ -115,130 +145,151 @@ __device__ __forceinline__ void dn_fetch(float* dst, const float* src, int n, in
     for (int i = tid * 4; i < n; i += nthr * 4) dn_cp_async16(dst + i, src + i);
 }
 
-// acc[r][b0 + b] += a[r] . x[b] for four sequences, the four components of the vectors added in the order x, y, z, w.
-// Written component by component so that consecutive multiply-adds are independent of each other.
-template <int R>
-__device__ __forceinline__ void dn_fma4(float (&acc)[R][kDnSamples], const float4 (&a)[R], const float4 (&x)[4], int b0)
+// Two fp32 multiply-adds in one instruction: (acc.lo, acc.hi) += (a.lo * x.lo, a.hi * x.hi).
+__device__ __forceinline__ void dn_fma2(unsigned long long& acc, unsigned long long a, unsigned long long x)
+{
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(x));
+}
+// acc[r][b0 + b] += a[r] . x[b] for G sequences: the even and the odd elements of the vectors are summed side by side.  Written
+// component by component so that consecutive multiply-adds are independent of each other.
+template <int R, int S, int G>
+__device__ __forceinline__ void dn_fma(unsigned long long (&acc)[R][S], const ulonglong2 (&a)[R], const ulonglong2 (&x)[G], int b0)
 {
 #pragma unroll
-    for (int b = 0; b < 4; ++b)
+    for (int b = 0; b < G; ++b)
 #pragma unroll
-        for (int r = 0; r < R; ++r) acc[r][b0 + b] = fmaf(a[r].x, x[b].x, acc[r][b0 + b]);
+        for (int r = 0; r < R; ++r) dn_fma2(acc[r][b0 + b], a[r].x, x[b].x);
 #pragma unroll
-    for (int b = 0; b < 4; ++b)
+    for (int b = 0; b < G; ++b)
 #pragma unroll
-        for (int r = 0; r < R; ++r) acc[r][b0 + b] = fmaf(a[r].y, x[b].y, acc[r][b0 + b]);
-#pragma unroll
-    for (int b = 0; b < 4; ++b)
-#pragma unroll
-        for (int r = 0; r < R; ++r) acc[r][b0 + b] = fmaf(a[r].z, x[b].z, acc[r][b0 + b]);
-#pragma unroll
-    for (int b = 0; b < 4; ++b)
-#pragma unroll
-        for (int r = 0; r < R; ++r) acc[r][b0 + b] = fmaf(a[r].w, x[b].w, acc[r][b0 + b]);
+        for (int r = 0; r < R; ++r) dn_fma2(acc[r][b0 + b], a[r].y, x[b].y);
 }
 
-// One work unit: up to R rows of a node for the eight sequences of the cluster, relative frame f -> f + 1.
-// The loads of a reduction step are issued ahead of the multiply-adds that use them: the weights and the first four
-// sequences of step i + 1 while the last four sequences of step i are still being multiplied.
-template <int R, int CL>
-__device__ __forceinline__ void dn_unit(const DnBlobHdr* H, const DnUnit& un, float* dn_smem, const float* wsm,
-                                        const SrFrameCtl& init, int f, int lane, int b0, int nb, long long run0)
+// One halving step of the sum over the lanes: with distance D a lane keeps the half of its N values per row that matches its bit D
+// and adds the partner's.
+template <int R, int N, int D>
+__device__ __forceinline__ void dn_halve(float (&out)[R][N / 2], const float (&v)[R][N], int lane)
 {
-    float acc[R][kDnSamples];
+    const bool up = (lane & D) != 0;
 #pragma unroll
     for (int r = 0; r < R; ++r)
 #pragma unroll
-        for (int b = 0; b < kDnSamples; ++b) acc[r][b] = 0.f;
+        for (int j = 0; j < N / 2; ++j) {
+            const float keep = up ? v[r][j + N / 2] : v[r][j], send = up ? v[r][j] : v[r][j + N / 2];
+            out[r][j] = keep + __shfl_xor_sync(0xffffffffu, send, D);
+        }
+}
+
+// One work unit: up to R rows of a node for the S sequences of the cluster, relative frame f -> f + 1.
+// The loads of a reduction step are issued ahead of the multiply-adds that use them: the weights and the first four
+// sequences of step i + 1 while the last four sequences of step i are still being multiplied.
+template <int R, int CL, int S>
+__device__ __forceinline__ void dn_unit(const DnBlobHdr* H, const DnUnit& un, float* dn_mem, const float* wsm,
+                                        const SrFrameCtl& init, int f, int lane, int b0, int nb, long long run0, uint32_t bar)
+{
+    unsigned long long acc2[R][S];
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int b = 0; b < S; ++b) acc2[r][b] = 0ull;
     for (int ti = un.term0; ti < un.term0 + un.n_terms; ++ti) {
         const DnTerm tm = H->terms[ti];
         const int sf = f + 1 - tm.R;                                  // Eq. 2: the source frame
         const int bi = tm.n_buf == 3 ? sf % 3 : (sf & 1);
-        const float* xs = dn_smem + (bi == 0 ? tm.buf[0] : (bi == 1 ? tm.buf[1] : tm.buf[2])) + lane * 4;
+        const float* xs = dn_mem + (bi == 0 ? tm.buf[0] : (bi == 1 ? tm.buf[1] : tm.buf[2])) + lane * 4;
         const float* w0 = wsm + tm.w_off + lane * 4;
         int ro[R];                                                    // rows the unit does not have repeat row 0 (their sums are dropped)
 #pragma unroll
         for (int r = 0; r < R; ++r) ro[r] = r < un.nrows ? r * tm.Kpad : 0;
         const int xp = tm.xp, n_k = tm.Kpad - lane * 4;               // this lane's steps: k = 0, 128, ... < n_k
         if (n_k <= 0) continue;
-        float4 a[R], xa[4], xb[4];
+        constexpr int G = S < 4 ? S : 4;                              // sequences whose loads are issued together
+        ulonglong2 a[R], xa[G];
 #pragma unroll
-        for (int r = 0; r < R; ++r) a[r] = *reinterpret_cast<const float4*>(w0 + ro[r]);
+        for (int r = 0; r < R; ++r) a[r] = *reinterpret_cast<const ulonglong2*>(w0 + ro[r]);
 #pragma unroll
-        for (int b = 0; b < 4; ++b) xa[b] = *reinterpret_cast<const float4*>(xs + b * xp);
+        for (int b = 0; b < G; ++b) xa[b] = *reinterpret_cast<const ulonglong2*>(xs + b * xp);
         for (int k = 0; k < n_k; k += 128) {
-#pragma unroll
-            for (int b = 0; b < 4; ++b) xb[b] = *reinterpret_cast<const float4*>(xs + (b + 4) * xp + k);
-            dn_fma4<R>(acc, a, xa, 0);
-            float4 an[R];
+            ulonglong2 an[R], xb[G];
             const int kn = k + 128 < n_k ? k + 128 : k;               // the last step re-reads itself (no branch)
+            if (S > G) {
 #pragma unroll
-            for (int r = 0; r < R; ++r) an[r] = *reinterpret_cast<const float4*>(w0 + ro[r] + kn);
+                for (int b = 0; b < G; ++b) xb[b] = *reinterpret_cast<const ulonglong2*>(xs + (b + G) * xp + k);
+                dn_fma<R, S, G>(acc2, a, xa, 0);
 #pragma unroll
-            for (int b = 0; b < 4; ++b) xa[b] = *reinterpret_cast<const float4*>(xs + b * xp + kn);
-            dn_fma4<R>(acc, a, xb, 4);
+                for (int r = 0; r < R; ++r) an[r] = *reinterpret_cast<const ulonglong2*>(w0 + ro[r] + kn);
+#pragma unroll
+                for (int b = 0; b < G; ++b) xa[b] = *reinterpret_cast<const ulonglong2*>(xs + b * xp + kn);
+                dn_fma<R, S, G>(acc2, a, xb, S - G);
+            } else {
+#pragma unroll
+                for (int r = 0; r < R; ++r) an[r] = *reinterpret_cast<const ulonglong2*>(w0 + ro[r] + kn);
+#pragma unroll
+                for (int b = 0; b < G; ++b) xb[b] = *reinterpret_cast<const ulonglong2*>(xs + b * xp + kn);
+                dn_fma<R, S, G>(acc2, a, xa, 0);
+#pragma unroll
+                for (int b = 0; b < G; ++b) xa[b] = xb[b];
+            }
 #pragma unroll
             for (int r = 0; r < R; ++r) a[r] = an[r];
         }
     }
-    // Sum over the lanes by halving: in the step with distance d a lane keeps the half of its sequences that matches
-    // its bit d and adds the partner's; after distances 16, 8 and 4 lane L holds the R rows of sequence L >> 2, summed
-    // over the lanes that share L's two low bits; distances 2 and 1 complete the sums in all four lanes of a group.
-    float v16[R][4], v8[R][2], z[R];
-    {
-        const bool up = (lane & 16) != 0;
+    float acc[R][S];
 #pragma unroll
-        for (int r = 0; r < R; ++r)
+    for (int r = 0; r < R; ++r)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float keep = up ? acc[r][j + 4] : acc[r][j], send = up ? acc[r][j] : acc[r][j + 4];
-                v16[r][j] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-            }
-    }
-    {
-        const bool up = (lane & 8) != 0;
+        for (int b = 0; b < S; ++b) acc[r][b] = __uint_as_float((uint32_t)acc2[r][b]) + __uint_as_float((uint32_t)(acc2[r][b] >> 32));
+    // Sum over the lanes: halving steps until a lane holds the R rows of ONE sequence, lane / (32 / S), then plain butterflies
+    // among the 32 / S lanes that hold the same one.
+    float z[R];
+    if constexpr (S == 8) {
+        float v4[R][4], v2[R][2], v1[R][1];
+        dn_halve<R, 8, 16>(v4, acc, lane);
+        dn_halve<R, 4, 8>(v2, v4, lane);
+        dn_halve<R, 2, 4>(v1, v2, lane);
 #pragma unroll
-        for (int r = 0; r < R; ++r)
+        for (int r = 0; r < R; ++r) z[r] = v1[r][0];
+    } else if constexpr (S == 4) {
+        float v2[R][2], v1[R][1];
+        dn_halve<R, 4, 16>(v2, acc, lane);
+        dn_halve<R, 2, 8>(v1, v2, lane);
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
-                const float keep = up ? v16[r][j + 2] : v16[r][j], send = up ? v16[r][j] : v16[r][j + 2];
-                v8[r][j] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-            }
-    }
-    {
-        const bool up = (lane & 4) != 0;
+        for (int r = 0; r < R; ++r) z[r] = v1[r][0];
+    } else {
+        float v1[R][1];
+        dn_halve<R, 2, 16>(v1, acc, lane);
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const float keep = up ? v8[r][1] : v8[r][0], send = up ? v8[r][0] : v8[r][1];
-            z[r] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-        }
+        for (int r = 0; r < R; ++r) z[r] = v1[r][0];
     }
 #pragma unroll
-    for (int r = 0; r < R; ++r) z[r] += __shfl_xor_sync(0xffffffffu, z[r], 2);
+    for (int d = 16 / S; d > 0; d >>= 1)
 #pragma unroll
-    for (int r = 0; r < R; ++r) z[r] += __shfl_xor_sync(0xffffffffu, z[r], 1);
-    const int b = lane >> 2;
+        for (int r = 0; r < R; ++r) z[r] += __shfl_xor_sync(0xffffffffu, z[r], d);
+    constexpr int kLanes = 32 / S;                                    // lanes that hold the same sequence
+    const int b = lane / kLanes;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        z[r] += dn_smem[un.bias_off + un.row0 + (r < un.nrows ? r : 0)];
+        z[r] += dn_mem[un.bias_off + un.row0 + (r < un.nrows ? r : 0)];
         if (un.flags & 1) z[r] = fmaxf(z[r], 0.f);
     }
-    const float* cell = dn_smem + (((f + 1) & 1) ? un.buf[1] : un.buf[0]) + b * un.Cpad + un.row0;
-    constexpr uint32_t kPerLane = CL / 4;                             // the four lanes of a group serve a quarter of the ranks each
-    const uint32_t q = (uint32_t)(lane & 3) * kPerLane;
-    if (R == 4 && un.nrows == 4 && (un.row0 & 3) == 0) {
+    const uint32_t cell = dn_smem(dn_mem + (((f + 1) & 1) ? un.buf[1] : un.buf[0]) + b * un.Cpad + un.row0);
+    constexpr uint32_t kPerLane = CL > kLanes ? CL / kLanes : 1;      // ranks that each of them serves
+    const uint32_t q = (uint32_t)(lane % kLanes) * kPerLane;
+    if (q >= CL) {
+        // (more lanes than ranks: nothing to send)
+    } else if (R == 4 && un.nrows == 4 && (un.row0 & 3) == 0) {
         const float z4[4] = {z[0], z[1], z[2 % R], z[3 % R]};
 #pragma unroll
-        for (uint32_t i = 0; i < kPerLane; ++i) dn_st_cluster4(cell, q + i, z4);
+        for (uint32_t i = 0; i < kPerLane; ++i) dn_st_async4(cell, bar, q + i, z4);
     } else {
 #pragma unroll
         for (int r = 0; r < R; ++r)
             if (r < un.nrows) {
 #pragma unroll
-                for (uint32_t i = 0; i < kPerLane; ++i) dn_st_cluster(cell + r, q + i, z[r]);
+                for (uint32_t i = 0; i < kPerLane; ++i) dn_st_async(cell + 4 * r, bar, q + i, z[r]);
             }
     }
-    if ((un.flags & 2) && init.out_base && (lane & 3) == 0 && b < nb) {
+    if ((un.flags & 2) && init.out_base && lane % kLanes == 0 && b < nb) {
         float* o = init.out_base + (run0 + f) * init.out_stride + (long long)(b0 + b) * un.C + un.row0;
 #pragma unroll
         for (int r = 0; r < R; ++r)
@@ -246,32 +297,36 @@ __device__ __forceinline__ void dn_unit(const DnBlobHdr* H, const DnUnit& un, fl
     }
 }
 
-template <int CL>
+template <int CL, int S>
 __global__ void __launch_bounds__(kDnWarps * 32, 1)
 sr_dense_kernel(const DnParams P, const SrFrameCtl init, int T)
 {
-    extern __shared__ __align__(16) float dn_smem[];
+    extern __shared__ __align__(16) float dn_mem[];
     // the input nodes as the fetching warps need them: first float of this cluster's sequences in the caller's frame 0
     // of the run, floats from one frame to the next, floats per frame, the three shared-memory buffers
     __shared__ const float* in_src[SR_MAX_INPUTS];
     __shared__ long long in_step[SR_MAX_INPUTS];
     __shared__ int in_len[SR_MAX_INPUTS], in_buf[SR_MAX_INPUTS][3], n_in;
+    __shared__ uint64_t bars[kDnMaxLevels][2];               // per level and frame parity: the level's new states have arrived
+    __shared__ int gave_up;
     const int tid = threadIdx.x, nthr = blockDim.x, warp = tid >> 5, lane = tid & 31;
+    sr_let_successor_start();
     uint32_t rank;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-    const int b0 = (int)(blockIdx.x / CL) * kDnSamples;
-    const int nb = min(kDnSamples, P.B - b0);
-    const DnBlobHdr* H = reinterpret_cast<const DnBlobHdr*>(dn_smem);
-    const float* wsm = dn_smem + P.hdr_floats;
+    const int b0 = (int)(blockIdx.x / CL) * S;
+    const int nb = min(S, P.B - b0);
+    const DnBlobHdr* H = reinterpret_cast<const DnBlobHdr*>(dn_mem);
+    const float* wsm = dn_mem + P.hdr_floats;
 
     // this rank's tables and weight slices, and zeros in every state buffer (padding columns and unused sequences stay zero)
     {
         const float* blob = reinterpret_cast<const float*>(P.blobs + (size_t)rank * P.blob_bytes);
-        dn_fetch(dn_smem, blob, P.blob_bytes / 4, tid, nthr);
-        for (int i = P.blob_bytes / 4 + tid; i < P.total_floats; i += nthr) dn_smem[i] = 0.f;
+        dn_fetch(dn_mem, blob, P.blob_bytes / 4, tid, nthr);
+        for (int i = P.blob_bytes / 4 + tid; i < P.total_floats; i += nthr) dn_mem[i] = 0.f;
     }
     const long long t0 = init.t, run0 = init.run_t;
     if (tid == 0) {
+        gave_up = 0;
         int n = 0;
         for (int v = 0; v < P.n_nodes; ++v) {
             const DnNode& nd = P.nodes[v];
@@ -286,44 +341,67 @@ sr_dense_kernel(const DnParams P, const SrFrameCtl init, int T)
     }
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
     __syncthreads();
+    if (tid < 2 * P.n_levels) {
+        // one arrival announces the bytes; in the last level every fetching thread arrives when its copies have landed, and
+        // every rank that sends no states does once per frame
+        const int l = tid >> 1, n_arrive = 1 + (l == P.n_levels - 1 ? 32 * __popc(H->fetch_mask) + P.n_idle : 0);
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(dn_smem(&bars[l][tid & 1])), "r"(n_arrive) : "memory");
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    // (Weights and tables do not depend on the kernel before this one; states and input frames do.)
+    sr_wait_for_predecessor();
     // frame t of every node from the state buffers in global memory (relative frame 0)
     const int par0 = (int)(t0 & 1);
     for (int v = 0; v < P.n_nodes; ++v) {
         const DnNode& nd = P.nodes[v];
         const float* gsrc = nd.gstate[par0] + (size_t)b0 * nd.C;
-        float* dst = dn_smem + nd.buf[0];
+        float* dst = dn_mem + nd.buf[0];
         if (nd.Cpad == nd.C) dn_fetch(dst, gsrc, nb * nd.C, tid, nthr);                  // rows are contiguous: 16-byte copies
         else
             for (int i = tid; i < nb * nd.C; i += nthr) dst[(i / nd.C) * nd.Cpad + (i % nd.C)] = gsrc[i];
         if (!nd.is_input)
-            for (int i = tid; i < nd.C; i += nthr) dn_smem[nd.bias_off + i] = nd.bias[i];
+            for (int i = tid; i < nd.C; i += nthr) dn_mem[nd.bias_off + i] = nd.bias[i];
     }
-    // Input frame k of the run (relative frame k) -> buffer k % 3, by the warps from fetch_warp0 on.
-    const int f_tid = tid - H->fetch_warp0 * 32, f_nthr = nthr - H->fetch_warp0 * 32;
+    // Input frame k of the run (relative frame k) -> buffer k % 3, by the warps of fetch_mask.
+    const int f_nthr = 32 * __popc(H->fetch_mask);
+    const int f_tid = (H->fetch_mask >> warp) & 1 ? 32 * __popc(H->fetch_mask & ((1 << warp) - 1)) + lane : -1;
     auto fetch_inputs = [&](int k) {
         if (f_tid < 0) return;
-        for (int i = 0; i < n_in; ++i) dn_fetch(dn_smem + in_buf[i][k % 3], in_src[i] + (k - 1) * in_step[i], in_len[i], f_tid, f_nthr);
+        for (int i = 0; i < n_in; ++i) dn_fetch(dn_mem + in_buf[i][k % 3], in_src[i] + (k - 1) * in_step[i], in_len[i], f_tid, f_nthr);
     };
     fetch_inputs(1);
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
     dn_cluster_sync();                                       // every CTA of the cluster has its buffers in place before remote writes start
 
-    for (int f = 0; f < T; ++f) {                            // relative frame f -> f + 1
-        // the input frame after the next one is on its way during this update; it has landed, and is made visible
-        // to the whole CTA, at the cluster barrier that ends the update
+    for (int f = 0; f < T && !*(volatile int*)&gave_up; ++f) {                // relative frame f -> f + 1
+        // the input frame after the next one is on its way during this update; it has landed when the last level's barrier
+        // completes
+        const int par = (f + 1) & 1;
+        const uint32_t phase = (uint32_t)(f >> 1) & 1u;
         if (f + 1 < T) fetch_inputs(f + 2);
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (f_tid >= 0) asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(dn_smem(&bars[P.n_levels - 1][par])) : "memory");
         for (int l = 1; l <= P.n_levels; ++l) {
+            const uint32_t bar = dn_smem(&bars[l - 1][par]);
+            if (tid == 0)
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(P.level_bytes[l - 1]) : "memory");
+            // Nobody runs more than a frame ahead of a rank, because a level needs the states of every rank with a unit in it;
+            // a rank without any says so instead.
+            if (H->idle && l == P.n_levels && tid < CL)
+                asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(dn_map_rank(bar, (uint32_t)tid)) : "memory");
             for (int u = H->level_begin[l - 1] + warp; u < H->level_begin[l]; u += kDnWarps) {
                 const DnUnit un = H->units[u];
                 if (un.nrows == 0) continue;
-                if (un.nrows > 2) dn_unit<4, CL>(H, un, dn_smem, wsm, init, f, lane, b0, nb, run0);
-                else dn_unit<2, CL>(H, un, dn_smem, wsm, init, f, lane, b0, nb, run0);
+                if (un.nrows > 2) dn_unit<4, CL, S>(H, un, dn_mem, wsm, init, f, lane, b0, nb, run0, bar);
+                else dn_unit<2, CL, S>(H, un, dn_mem, wsm, init, f, lane, b0, nb, run0, bar);
             }
-            if (l == P.n_levels) asm volatile("cp.async.wait_group 0;" ::: "memory");
-            dn_cluster_sync();                               // the level is complete in every CTA's copy
+            if (!dn_wait(bar, phase, &gave_up, P.wait_limit)) break;    // the level is complete in this CTA's copy
         }
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (*(volatile int*)&gave_up) __nanosleep(100000);       // stores on their way to this CTA land before it leaves
+    __syncwarp();
+    dn_cluster_sync();                                       // no CTA leaves while another one may still store into it
+    if (tid == 0 && gave_up) atomicExch(P.error, 1);
 
     // relative frame T back to the state buffers in global memory (parity of t + T); every rank holds a full copy and
     // writes its share of it
@@ -332,7 +410,7 @@ sr_dense_kernel(const DnParams P, const SrFrameCtl init, int T)
         const int gtid = (int)rank * nthr + tid, gthr = CL * nthr;
         for (int v = 0; v < P.n_nodes; ++v) {
             const DnNode& nd = P.nodes[v];
-            const float* src = dn_smem + (nd.is_input ? nd.buf[T % 3] : nd.buf[T & 1]);
+            const float* src = dn_mem + (nd.is_input ? nd.buf[T % 3] : nd.buf[T & 1]);
             float* gdst = nd.gstate[parT] + (size_t)b0 * nd.C;
             if (nd.Cpad == nd.C)
                 for (int i = gtid * 4; i < nb * nd.C; i += gthr * 4) *reinterpret_cast<float4*>(gdst + i) = *reinterpret_cast<const float4*>(src + i);
@@ -347,6 +425,7 @@ struct DnEngine {
     DnParams P{};
     std::vector<int> edge_of_host;                 // host edge -> index in P.edges
     int cluster = 8;                               // CTAs per cluster
+    int samples = 8;                               // sequences per cluster
     std::vector<int> row_lo;                       // [node][rank] first row of the rank's slice, cluster + 1 entries per node
     std::vector<std::vector<int>> w_off;           // [rank][edge]
     std::vector<DnBlobHdr> hdrs;                   // per rank
@@ -368,15 +447,22 @@ bool dn_prepare(DnKernel kernel, int cluster, int smem_bytes)
     return true;
 }
 
-// Can at least one cluster of this size and shared-memory footprint be resident on the device?
-bool dn_cluster_fits(int cluster, int smem_bytes)
+DnKernel dn_kernel_of(int cluster, int samples)
 {
-    DnKernel kernel = cluster == 16 ? sr_dense_kernel<16> : sr_dense_kernel<8>;
-    if (!dn_prepare(kernel, cluster, smem_bytes)) { cudaGetLastError(); return false; }
+    if (cluster == 16) return samples == 8 ? sr_dense_kernel<16, 8> : samples == 4 ? sr_dense_kernel<16, 4> : sr_dense_kernel<16, 2>;
+    return samples == 8 ? sr_dense_kernel<8, 8> : samples == 4 ? sr_dense_kernel<8, 4> : sr_dense_kernel<8, 2>;
+}
+
+// Clusters of this size and shared-memory footprint that the device holds at once with one CTA per SM (0: none): two CTAs on an SM
+// share its shared-memory pipe, so a second one there gains little over a second wave.
+int dn_clusters_held(int cluster, int samples, int smem_bytes)
+{
+    DnKernel kernel = dn_kernel_of(cluster, samples);
+    if (!dn_prepare(kernel, cluster, std::max(smem_bytes, kDnMoreThanHalf))) { cudaGetLastError(); return 0; }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)cluster);
     cfg.blockDim = dim3((unsigned)(kDnWarps * 32));
-    cfg.dynamicSmemBytes = (size_t)smem_bytes;
+    cfg.dynamicSmemBytes = (size_t)std::max(smem_bytes, kDnMoreThanHalf);
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)cluster;
@@ -385,17 +471,18 @@ bool dn_cluster_fits(int cluster, int smem_bytes)
     cfg.attrs = at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); return false; }
-    return n >= 1;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+    return n;
 }
 
 // Plans the engine for a cluster of CL CTAs: rows of every node split evenly over the ranks.  Null if it does not fit.
-DnEngine* dn_build(const sr_graph* g, int CL)
+DnEngine* dn_build(const sr_graph* g, int CL, int S)
 {
     const int n_nodes = (int)g->nodes.size(), n_edges = (int)g->edges.size();
     DnEngine* E = new DnEngine();
     DnParams& P = E->P;
     E->cluster = CL;
+    E->samples = S;
     P.n_nodes = n_nodes;
     P.n_edges = n_edges;
     P.n_levels = (int)g->groups.size();
@@ -445,12 +532,16 @@ DnEngine* dn_build(const sr_graph* g, int CL)
         d.is_output = v == g->info.output_node ? 1 : 0;
         for (int i = 0; i < (n.is_input ? 3 : 2); ++i) {
             d.buf[i] = off;
-            off += kDnSamples * d.Cpad;
+            off += S * d.Cpad;
         }
         d.bias_off = off;
         if (!n.is_input) off += d.Cpad;
     }
     P.total_floats = off;
+    for (int l = 0; l < P.n_levels; ++l) {
+        P.level_bytes[l] = 0;
+        for (int v : g->groups[l]) P.level_bytes[l] += g->nodes[v].d.c * S * 4;
+    }
     E->smem_bytes = off * 4;
     if (E->smem_bytes > kDnSmemMax) {
         delete E;
@@ -458,7 +549,7 @@ DnEngine* dn_build(const sr_graph* g, int CL)
     }
     // Per rank: units (up to four rows of a node each) with their terms (one per incoming edge).  The units of a level
     // go longest first onto the warp with the least work so far; warp w's i-th unit of the level is entry
-    // level_begin + 16 i + w (gaps have nrows = 0).
+    // level_begin + kDnWarps * i + w (gaps have nrows = 0).
     std::vector<DnBlobHdr>& hdrs = E->hdrs;
     hdrs.assign(CL, DnBlobHdr{});
     for (int r = 0; r < CL; ++r) {
@@ -521,15 +612,20 @@ DnEngine* dn_build(const sr_graph* g, int CL)
                 for (int w = 0; w < kDnWarps; ++w) h.units[n_units++] = i < of_warp[w].size() ? of_warp[w][i] : DnUnit{};
             h.level_begin[l] = n_units;
             if (l == 1) {
-                // warps without a unit in the first level fetch the input frames, if there are at least four of them
-                int last = -1;
+                // warps without a unit in the first level fetch the input frames, if there are at least two of them
+                int idle_warps = 0;
                 for (int w = 0; w < kDnWarps; ++w)
-                    if (!of_warp[w].empty()) last = w;
-                h.fetch_warp0 = last + 1 <= kDnWarps - 4 ? last + 1 : 0;
+                    if (of_warp[w].empty()) h.fetch_mask |= 1 << w;
+                for (int w = 0; w < kDnWarps; ++w) idle_warps += (h.fetch_mask >> w) & 1;
+                if (idle_warps < 2) h.fetch_mask = (1 << kDnWarps) - 1;
             }
         }
         for (int l = P.n_levels + 1; l <= kDnMaxLevels; ++l) h.level_begin[l] = n_units;
         h.n_units = n_units;
+        h.idle = 1;
+        for (int u = 0; u < n_units; ++u)
+            if (h.units[u].nrows > 0) h.idle = 0;
+        P.n_idle += h.idle;
         if (!fits) {
             delete E;
             return nullptr;
@@ -572,19 +668,41 @@ sr_status sr_dn_plan(sr_graph* g, size_t& offset)
     }
     for (const SrHostEdge& e : g->edges)
         if (e.d.kind == SR_EDGE_CONV) return SR_OK;
-    // With one level per frame (the streaming rollout) a frame is one round of work units and one cluster barrier:
-    // sixteen CTAs (a non-portable cluster size) halve the units of each CTA (measured on the 784-128-128-10 network:
-    // 2.8 against 3.2 us per frame), while with several levels per frame the costlier barrier of the larger cluster
-    // outweighs that (6.2 against 5.7).  The larger cluster is used only if the device can hold one.
+    // With one level per frame (the streaming rollout) a frame is one round of work units and one exchange: sixteen CTAs (a
+    // non-portable cluster size) halve the units of each CTA, while with several levels per frame the costlier exchange of the
+    // larger cluster outweighs that.  Measured on the 784-128-128-10 network, four clusters of two sequences, per frame: streaming
+    // 1.45 us with sixteen, 2.19 with eight; sequential 3.4 and 3.3.  The device holds fewer than half as many of the larger
+    // clusters (7 against 15), and a second wave costs more than they win (64 sequences, 64 frames: 342 us against 254), so they
+    // are used only where all of a run go out at once.
     DnEngine* E = nullptr;
     if (g->groups.size() == 1) {
-        E = dn_build(g, kDnMaxCluster);
-        if (E && !dn_cluster_fits(kDnMaxCluster, E->smem_bytes)) {
+        E = dn_build(g, kDnMaxCluster, kDnMaxSamples);
+        if (E && (g->batch + kDnMaxSamples - 1) / kDnMaxSamples > dn_clusters_held(kDnMaxCluster, kDnMaxSamples, E->smem_bytes)) {
             delete E;
             E = nullptr;
         }
     }
-    if (!E) E = dn_build(g, 8);
+    if (!E) E = dn_build(g, 8, kDnMaxSamples);
+    // Fewer sequences per cluster shorten a frame, because the loads of the states shrink with them: per frame of one wave of that
+    // network 1.45, 1.87 and 2.50 us with two, four and eight sequences and sixteen CTAs, 2.19, 2.79 and 3.68 with eight CTAs
+    // (sequential 3.3, 4.2, 5.4).  The split whose waves end first by these ratios is taken.
+    if (E) {
+        const int cl = E->cluster;
+        double best = 0.0;
+        int best_s = 0;
+        for (int S = kDnMaxSamples; S >= 2; S /= 2) {
+            DnEngine* F = S == kDnMaxSamples ? E : dn_build(g, cl, S);
+            if (!F) continue;
+            const int clusters = (g->batch + S - 1) / S, held = std::max(dn_clusters_held(cl, S, F->smem_bytes), 1);
+            const double cost = (clusters + held - 1) / held * (S == 8 ? 1.0 : S == 4 ? 0.76 : 0.6);
+            if (F != E) delete F;
+            if (best_s == 0 || cost < best) { best = cost; best_s = S; }
+        }
+        if (best_s != E->samples) {
+            delete E;
+            E = dn_build(g, cl, best_s);
+        }
+    }
     if (!E) return SR_OK;
     const int CL = E->cluster;
     DnParams& P = E->P;
@@ -646,25 +764,31 @@ sr_status sr_dn_launch(sr_graph* g, int T, const SrFrameCtl& init, cudaStream_t 
     DnEngine* E = dn_of(g);
     if (!E) return SR_ERR_STATE;
     const int CL = E->cluster;
-    auto kernel = CL == 16 ? sr_dense_kernel<16> : sr_dense_kernel<8>;
+    const int S = E->samples;
+    auto kernel = dn_kernel_of(CL, S);
     if (!E->attr_set) {
         if (!dn_prepare(kernel, CL, E->smem_bytes)) return SR_ERR_CUDA;
         E->attr_set = true;
     }
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)((g->batch + kDnSamples - 1) / kDnSamples * CL));
+    cfg.gridDim = dim3((unsigned)((g->batch + S - 1) / S * CL));
     cfg.blockDim = dim3((unsigned)(kDnWarps * 32));
     cfg.dynamicSmemBytes = (size_t)E->smem_bytes;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)CL;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    bool timed = g->opt_time_tc != 0 && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    const bool plain = cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    bool timed = g->opt_time_tc != 0 && plain;
+    cfg.numAttrs = plain && !timed ? 2 : 1;                   // may start early (see SrFollow)
+    E->P.error = reinterpret_cast<int32_t*>(g->ws + g->r_flags.offset);
+    E->P.wait_limit = (long long)std::max(1, g->opt_wait_ms) * 2000000LL;
     if (timed && E->ev_used + 2 > E->ev.size()) {
         if (E->ev.size() >= 4096) timed = false;
         for (int i = 0; timed && i < 2; ++i) {

@@ -75,3 +75,12 @@ def test_results_are_reproducible_bit_for_bit():
         G = parity.make_graph(g, "streaming", "auto", 0, W, Bi)
         outs.append(G.rollout([parity.to_device(g, X[0])]).cpu().numpy())
     assert np.array_equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("batch", [1, 3, 15, 28, 130])
+def test_sequences_per_cluster_and_ranks_without_rows(batch):
+    # few rows: most CTAs of a cluster have no work unit in a level and only take part in the exchange; the batches make clusters
+    # of two, four and eight sequences (and, the last, more clusters of sixteen CTAs than a device holds), the last one ragged
+    g = mlp(batch, 6, sizes=(4, 3, 2, 5), seed=77)
+    for p in g.patterns:
+        parity.check_run(g, p, expect_resident=8 if batch == 130 else CLUSTER[p])
