@@ -426,6 +426,7 @@ struct DnEngine {
     std::vector<int> edge_of_host;                 // host edge -> index in P.edges
     int cluster = 8;                               // CTAs per cluster
     int samples = 8;                               // sequences per cluster
+    bool one_wave = false;                         // the device holds all clusters of the batch at once
     std::vector<int> row_lo;                       // [node][rank] first row of the rank's slice, cluster + 1 entries per node
     std::vector<std::vector<int>> w_off;           // [rank][edge]
     std::vector<DnBlobHdr> hdrs;                   // per rank
@@ -645,6 +646,7 @@ void sr_dn_destroy(sr_graph* g)
 }
 
 bool sr_dn_available(const sr_graph* g) { return g->dn != nullptr; }
+bool sr_dn_one_wave(const sr_graph* g) { return g->dn != nullptr && dn_of(g)->one_wave; }
 
 void sr_dn_describe(const sr_graph* g, int* cluster_size, int* smem_bytes)
 {
@@ -689,19 +691,21 @@ sr_status sr_dn_plan(sr_graph* g, size_t& offset)
     if (E) {
         const int cl = E->cluster;
         double best = 0.0;
-        int best_s = 0;
+        int best_s = 0, best_waves = 0;
         for (int S = kDnMaxSamples; S >= 2; S /= 2) {
             DnEngine* F = S == kDnMaxSamples ? E : dn_build(g, cl, S);
             if (!F) continue;
             const int clusters = (g->batch + S - 1) / S, held = std::max(dn_clusters_held(cl, S, F->smem_bytes), 1);
-            const double cost = (clusters + held - 1) / held * (S == 8 ? 1.0 : S == 4 ? 0.76 : 0.6);
+            const int waves = (clusters + held - 1) / held;
+            const double cost = waves * (S == 8 ? 1.0 : S == 4 ? 0.76 : 0.6);
             if (F != E) delete F;
-            if (best_s == 0 || cost < best) { best = cost; best_s = S; }
+            if (best_s == 0 || cost < best) { best = cost; best_s = S; best_waves = waves; }
         }
         if (best_s != E->samples) {
             delete E;
             E = dn_build(g, cl, best_s);
         }
+        if (E) E->one_wave = best_waves == 1;
     }
     if (!E) return SR_OK;
     const int CL = E->cluster;

@@ -9,6 +9,7 @@ sr_status sr_dn_plan(sr_graph* g, size_t& offset);            // decides eligibi
 sr_status sr_dn_bind(sr_graph* g);
 sr_status sr_dn_set_weights(sr_graph* g, int edge, const float* w /* host, [C_out][K] */);
 bool sr_dn_available(const sr_graph* g);
+bool sr_dn_one_wave(const sr_graph* g);
 // Queues ONE kernel that performs the T frame updates described by `init` and leaves the state buffers
 // in global memory as T single-frame updates would.
 sr_status sr_dn_launch(sr_graph* g, int T, const SrFrameCtl& init, cudaStream_t s);

@@ -84,3 +84,27 @@ def test_sequences_per_cluster_and_ranks_without_rows(batch):
     g = mlp(batch, 6, sizes=(4, 3, 2, 5), seed=77)
     for p in g.patterns:
         parity.check_run(g, p, expect_resident=8 if batch == 130 else CLUSTER[p])
+
+
+@pytest.mark.parametrize("batch", [1, 9, 260])
+def test_single_steps(batch):
+    # frame by frame: on the engine, but for a frame that starts off a 16-byte boundary and for a batch of several waves (260)
+    import torch
+    from oracle import frame_update as fu
+    g = mlp(batch, 5)
+    X, W, Bi = data.make_inputs(g), data.make_weights(g), data.make_biases(g, zero=False)
+    for p in ("streaming", "sequential"):
+        want = fu.rollout_spec(g, p, X, W, Bi)
+        G = parity.make_graph(g, p, "auto", 0, W, Bi)
+        x = parity.to_device(g, X[0])
+        odd = torch.empty(x[3].numel() + 1, dtype=x.dtype, device=x.device)[1:].view(x[3].shape).copy_(x[3])
+        assert odd.data_ptr() % 16 != 0
+        G.reset([x[0]])
+        out = torch.empty((5,) + G.out_shape(), dtype=torch.float32, device="cuda:0")
+        for t in range(1, 6):
+            G.step([odd if t == 3 else x[t]], out[t - 1])
+        G.sync_status()
+        o = G.output_node
+        assert parity.rel_err(out.cpu().numpy().reshape(want[o][1:6].shape), want[o][1:6]) <= 1e-4
+        for v in range(len(g.nodes)):
+            assert parity.rel_err(G.get_state(v).cpu().numpy(), want[v][5]) <= 1e-4, g.nodes[v].name
