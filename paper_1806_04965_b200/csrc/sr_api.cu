@@ -222,14 +222,14 @@ int enqueue_frames(sr_graph* g, const SrFrameArgs& fr, int frames, cudaStream_t 
             const bool has_heads = !g->group_heads[gi].empty(), has_items = g->group_item_count[gi] > 0, has_tc = sr_tc_group_has_work(g, gi);
             const bool heads_lead = !has_tc && !has_items;
             const bool merged = gi == 0 && has_heads && (heads_lead || !feeds) && sr_heads_take_input(g, gi, g->frame, copies, stems_R);
-            if (gi == 0 && feeds && !merged) launches += sr_launch_input(g, g->frame, copies, stems_R, follow(false, false), s);
+            if (gi == 0 && feeds && !merged) launches += sr_launch_input(g, g->frame, copies, stems_R, follow(false, false), nullptr, s);
             const bool input_beside = gi == 0 && !feeds && !merged;
             const bool late = overlap && (input_beside || (has_tc + has_items + has_heads > 1));
             if (has_tc) launches += sr_tc_launch_group(g, gi, follow(false, late), s);
             if (has_items) launches += sr_launch_direct_group(g, gi, follow(overlap && has_tc, late && !has_tc), s);
-            if (input_beside && !heads_lead) launches += sr_launch_input(g, g->frame, copies, stems_R, follow(overlap, false), s);
+            if (input_beside && !heads_lead) launches += sr_launch_input(g, g->frame, copies, stems_R, follow(overlap, false), nullptr, s);
             if (has_heads) launches += sr_launch_heads(g, gi, merged, copies, stems_R, follow(overlap && !heads_lead, late && heads_lead), s);
-            if (input_beside && heads_lead) launches += sr_launch_input(g, g->frame, copies, stems_R, follow(overlap, false), s);
+            if (input_beside && heads_lead) launches += sr_launch_input(g, g->frame, copies, stems_R, follow(overlap, false), nullptr, s);
         }
     }
     return launches;
@@ -257,7 +257,7 @@ void stage_current(sr_graph* g, cudaStream_t s)
     SrFrameCtl c{};
     c.t = g->t - 1;                                              // "the input of frame t"
     for (size_t i = 0; i < g->input_nodes.size(); ++i) c.in_base[i] = g->ws + g->nodes[g->input_nodes[i]].state[g->t & 1].offset;
-    g->launches += sr_launch_input(g, by_value(c), 0u, 2u, SrFollow(), s);
+    g->launches += sr_launch_input(g, by_value(c), 0u, 2u, SrFollow(), nullptr, s);
 }
 
 // After a resident run they are brought up to date when the launch path is used next.
@@ -643,10 +643,9 @@ sr_status sr_graph_reset(sr_graph* g, const void* const* in0_dev, void* stream)
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     for (size_t i = 0; i < g->input_nodes.size(); ++i)
         if (!in0_dev[i]) return SR_ERR_INVALID_ARG;
-    // One memset: the non-input states of frame 0 (those of the other parity are written before they are read), a reported
-    // device-side error (an expired wait: the rollout starts over) and the shared work list's counters (every launch leaves
-    // them at zero; this covers a launch cut short).
-    if (!cuda_ok(cudaMemsetAsync(g->ws + g->r_clear.offset, 0, g->r_clear.bytes, s))) return SR_ERR_CUDA;
+    // Zeroed with the input: the non-input states of frame 0 (those of the other parity are written before they are read), a
+    // reported device-side error (an expired wait: the rollout starts over) and the shared work list's counters (every launch
+    // leaves them at zero; this covers a launch cut short).
     if (g->window && g->window->ws && !cuda_ok(cudaMemsetAsync(g->window->ws + g->window->r_flags.offset, 0, g->window->r_flags.bytes, s)))
         return SR_ERR_CUDA;
     g->t = 0;
@@ -655,7 +654,7 @@ sr_status sr_graph_reset(sr_graph* g, const void* const* in0_dev, void* stream)
     c.t = -1;                                                    // "the input of frame 0"
     for (size_t i = 0; i < g->input_nodes.size(); ++i) c.in_base[i] = in0_dev[i];
     const bool resident = sr_rs_available(g);                    // a resident run does not read staged edges
-    g->launches += sr_launch_input(g, by_value(c), ~0u, resident ? 0u : 2u, SrFollow(), s);
+    g->launches += sr_launch_input(g, by_value(c), ~0u, resident ? 0u : 2u, SrFollow(), &g->r_clear, s);
     g->stage_dirty = resident;
     return cuda_ok(cudaGetLastError()) ? SR_OK : SR_ERR_CUDA;
 }
@@ -888,7 +887,7 @@ sr_status sr_rollout_window(sr_graph* g, const void* const* in_seq_dev, int W, f
     c.t = t_new - 1;
     for (size_t i = 0; i < g->input_nodes.size(); ++i)
         c.in_base[i] = static_cast<const char*>(in_seq_dev[i]) + node_elems(g, g->input_nodes[i]) * g->elem * (size_t)(W - 1);
-    w->launches += sr_launch_input(g, by_value(c), ~0u, 0u, SrFollow(), s);
+    w->launches += sr_launch_input(g, by_value(c), ~0u, 0u, SrFollow(), nullptr, s);
     for (size_t v = 0; v < g->nodes.size(); ++v) g->in_window[v] = !g->nodes[v].is_input;
     g->t = t_new;
     g->stage_dirty = true;

@@ -9,16 +9,24 @@ namespace {
 struct InputParams {
     SrFrameArgs fr;
     SrInputPart in;
-    int32_t follow;
+    int32_t follow, clear_blocks;                  // blocks behind those of `in` that zero `clear`
+    uint4* clear;
+    size_t n_clear;                                // 16-byte words
 };
 static_assert(sizeof(InputParams) <= 4000, "kernel parameters");
 
 // (Registers for six blocks per SM: three of them fit beside a CTA of the tensor-core kernel.)
-__global__ void __launch_bounds__(kInputThreads, 6) sr_input_kernel(const __grid_constant__ InputParams P)
+template <bool CLEAR>
+__global__ void __launch_bounds__(kInputThreads, CLEAR ? 1 : 6) sr_input_kernel(const __grid_constant__ InputParams P)
 {
     __shared__ int2 tap[128];
     sr_begin(P.follow);
-    sr_input_block(P.in, P.fr, sr_frame(P.fr), (int)blockIdx.x, tap);
+    if (!CLEAR || (int)blockIdx.x < P.in.n_blocks) {
+        sr_input_block(P.in, P.fr, sr_frame(P.fr), (int)blockIdx.x, tap);
+    } else {
+        const size_t nth = (size_t)P.clear_blocks * kInputThreads;
+        for (size_t i = (size_t)((int)blockIdx.x - P.in.n_blocks) * kInputThreads + threadIdx.x; i < P.n_clear; i += nth) P.clear[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
     sr_end(P.follow);
 }
 
@@ -33,16 +41,22 @@ __global__ void sr_advance_kernel(SrFrameCtl* ctl, int n)
 }  // namespace
 
 // Queues the input of the frame that `fr` describes.  copies: bit i = input node i's state takes it; stems_R: see sr_stems.
-// Returns launches.
-int sr_launch_input(const sr_graph* g, const SrFrameArgs& fr, unsigned copies, unsigned stems_R, SrFollow how, cudaStream_t s)
+// `clear` (or null): a region, in whole 16-byte words, that the same launch zeroes (a reset: as a memset of its own it took
+// 2 us of a small network's pass on the GPU, and a launch on the host).  Returns launches.
+int sr_launch_input(const sr_graph* g, const SrFrameArgs& fr, unsigned copies, unsigned stems_R, SrFollow how, const SrRegion* clear, cudaStream_t s)
 {
     int launches = 0;
     const std::vector<const SrStem*> stems = sr_stems(g, stems_R);
     size_t next = 0;
     do {
-        InputParams P{fr, sr_plan_input(g, launches == 0 ? copies : 0u, stems, next, how.beside), how.flags()};
-        if (P.in.n_blocks == 0) break;
-        sr_launch(sr_input_kernel, P.in.n_blocks, kInputThreads, 0, s, how.early, P);
+        InputParams P{fr, sr_plan_input(g, launches == 0 ? copies : 0u, stems, next, how.beside), how.flags(), 0, nullptr, 0};
+        if (clear && launches == 0) {
+            P.clear = reinterpret_cast<uint4*>(g->ws + clear->offset);
+            P.n_clear = clear->bytes / 16;
+            P.clear_blocks = (int)std::min<size_t>(148 * 6, (P.n_clear + 4 * kInputThreads - 1) / (4 * kInputThreads));
+        }
+        if (P.in.n_blocks + P.clear_blocks == 0) break;
+        sr_launch(P.clear_blocks ? sr_input_kernel<true> : sr_input_kernel<false>, P.in.n_blocks + P.clear_blocks, kInputThreads, 0, s, how.early, P);
         ++launches;
         how.early = true;
     } while (next < stems.size());
@@ -63,5 +77,5 @@ void sr_launch_advance(const sr_graph* g, int n, cudaStream_t s)
 // SM changes its partition only when it is empty, so with another one the tensor-core kernel waits for them to drain.
 bool sr_input_share_sm()
 {
-    return cudaFuncSetAttribute(sr_input_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
+    return cudaFuncSetAttribute(sr_input_kernel<false>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
 }

@@ -5,7 +5,7 @@
 #include "sr_internal.h"
 
 int sr_launch_direct_group(const sr_graph* g, int group, SrFollow how, cudaStream_t s);
-int sr_launch_input(const sr_graph* g, const SrFrameArgs& fr, unsigned copies, unsigned stems_R, SrFollow how, cudaStream_t s);
+int sr_launch_input(const sr_graph* g, const SrFrameArgs& fr, unsigned copies, unsigned stems_R, SrFollow how, const SrRegion* clear, cudaStream_t s);
 void sr_launch_set_ctl(const sr_graph* g, const SrFrameCtl& v, cudaStream_t s);
 void sr_launch_advance(const sr_graph* g, int n, cudaStream_t s);
 void sr_direct_conv_items(const sr_graph* g, int v, std::vector<SrDirectItem>& items);

@@ -509,6 +509,7 @@ __device__ __forceinline__ void rs_kernel_body(const unsigned char* __restrict__
     const int tid = threadIdx.x, nthr = blockDim.x;
     const uint32_t rank = cs > 1 ? rs_cluster_rank() : 0u;
     const int b = blockIdx.x / cs;                                    // the sequence this cluster rolls out
+    sr_let_successor_start();
     {
         const uint4* src = reinterpret_cast<const uint4*>(blobs + (size_t)rank * blob_stride);
         const int n16 = reinterpret_cast<const RsHeader*>(src)->blob_bytes >> 4;
@@ -552,6 +553,9 @@ __device__ __forceinline__ void rs_kernel_body(const unsigned char* __restrict__
             }
         }
     }
+    // (Tables and weights do not depend on the kernel before this one; states and input frames do.  With this and the reset in one
+    // launch a pass of the small CNN, 64 sequences x 32 frames, went from 240.4 to 234.4 us.)
+    sr_wait_for_predecessor();
     // frame t of every node (relative frame 0), and the first input frame of the run (relative frame 1)
     // `init` describes this run (frame counter, the caller's input sequences and output)
     const SrFrameCtl* const ctl = &init;
@@ -984,7 +988,8 @@ typedef void (*RsKernel)(const unsigned char*, int, const SrFrameCtl, int, int);
 
 RsKernel rs_kernel_of(const RsEngine& E) { return E.warps <= 16 ? sr_resident_kernel<512> : E.warps <= 24 ? sr_resident_kernel<768> : sr_resident_kernel<1024>; }
 
-cudaLaunchConfig_t rs_config(const RsEngine& E, int batch, cudaStream_t s, cudaLaunchAttribute* at)
+// at: room for two attributes; early: the launch may start before its predecessor in the stream has completed (see SrFollow)
+cudaLaunchConfig_t rs_config(const RsEngine& E, int batch, bool early, cudaStream_t s, cudaLaunchAttribute* at)
 {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(batch * E.cs));
@@ -995,8 +1000,10 @@ cudaLaunchConfig_t rs_config(const RsEngine& E, int batch, cudaStream_t s, cudaL
     at[0].val.clusterDim.x = (unsigned)E.cs;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = E.cs > 1 ? 1 : 0;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = E.cs > 1 ? at : at + 1;
+    cfg.numAttrs = (E.cs > 1 ? 1 : 0) + (early ? 1 : 0);
     return cfg;
 }
 
@@ -1007,8 +1014,8 @@ int rs_clusters_held(const RsEngine& E)
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     int n = std::max(1, sms / E.cs);
     if (E.cs > 1) {
-        cudaLaunchAttribute at[1];
-        const cudaLaunchConfig_t cfg = rs_config(E, 1, nullptr, at);
+        cudaLaunchAttribute at[2];
+        const cudaLaunchConfig_t cfg = rs_config(E, 1, false, nullptr, at);
         int held = 0;
         if (cudaFuncSetAttribute(rs_kernel_of(E), cudaFuncAttributeMaxDynamicSharedMemorySize, kRsSmemMax) == cudaSuccess &&
             cudaOccupancyMaxActiveClusters(&held, rs_kernel_of(E), &cfg) == cudaSuccess && held > 0)
@@ -1433,11 +1440,12 @@ sr_status sr_rs_launch(sr_graph* g, int T, const SrFrameCtl& init, cudaStream_t 
         if (cudaFuncSetAttribute(rs_kernel_of(*E), cudaFuncAttributeMaxDynamicSharedMemorySize, kRsSmemMax) != cudaSuccess) return SR_ERR_CUDA;
         E->attr_set = true;
     }
-    cudaLaunchAttribute at[1];
-    const cudaLaunchConfig_t cfg = rs_config(*E, g->batch, s, at);
     const unsigned char* blobs = reinterpret_cast<const unsigned char*>(g->ws + E->r_blobs.offset);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    bool timed = g->opt_time_tc != 0 && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    const bool plain = cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    bool timed = g->opt_time_tc != 0 && plain;
+    cudaLaunchAttribute at[2];
+    const cudaLaunchConfig_t cfg = rs_config(*E, g->batch, plain && !timed, s, at);
     if (timed && E->ev_used + 2 > E->ev.size()) {
         if (E->ev.size() >= 4096) timed = false;
         for (int i = 0; timed && i < 2; ++i) {
