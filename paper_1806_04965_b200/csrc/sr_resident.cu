@@ -22,9 +22,15 @@
 //     costs >= 110 cycles however few columns it has), which is why this engine uses the warp-level
 //     tensor path and the batch-tiled tcgen05 kernel serves the large networks.
 //   * Few-channel edges (C_in * k * k <= 64, the first layer of an image network) build their A
-//     fragments from scalar shared-memory loads through a small per-edge lookup table.
-//   * Dense and mean-dense heads run on CUDA cores: every warp reduces a slice of the flattened
-//     source into a slot, slots of all CTAs are summed in a fixed order after the barrier.
+//     fragments from scalar shared-memory loads through a small per-edge lookup table; a node fed by one such edge only takes
+//     up to four tiles to a unit (rs_few_unit).
+//   * Dense and mean-dense heads: every warp reduces a slice of the flattened source into a slot (on the tensor pipe, see
+//     rs_dense_unit), slots of all CTAs are summed in a fixed order after the barrier.
+//   * What bounds it: instructions and shared-memory latency around the multiplies.  Measured on B200 (small CNN 28 x 28 x 1, us per
+//     pass, before / after heads on the tensor pipe, several first-layer tiles to a unit, and the slot sums as records of two
+//     loads that are charged to the level they run beside): 64 sequences x 128 streaming frames 861.6 / 843.7, 37 sequences
+//     x 80 sequential frames 1053.8 / 949.9.  Dealing a tile's edges to several warps, which add their sums through shared
+//     memory, was slower (948 and 1162 against 865 and 1053 at the time): the shared-memory pipe is shared by all of them.
 // State layout in shared memory: [row][col][C] bf16 in 16-byte chunks, chunk q stored at
 // (q & ~7) | ((q ^ (q >> 3)) & 7) so that the eight row addresses of an ldmatrix phase fall into
 // different bank groups for unit-stride and stride-2 taps.
@@ -44,14 +50,15 @@ namespace {
 constexpr int kRsMaxCluster = 4;
 constexpr int kRsSmemMax = 232448 - 128;      // 227 KiB per CTA minus the kernel's static shared memory
 constexpr int kRsMaxWarps = 32;
-constexpr int kRsDenseUnitChunks = 64;        // 16-byte chunks of the source per dense unit
+constexpr long kRsFewCost = 600;              // estimated cycles of one of its tiles
+constexpr int kRsFewTiles = 4;                // 16-pixel tiles per unit of a few-channel node, most
 constexpr int kRsMaxDenseC = 64;
 constexpr int kRsFinalizeWarp = 0;            // sums the dense slots after a level's barrier
 constexpr int kRsFetchWarp = 1;               // fetches the next input frame
 
 enum { RS_INPUT = 0, RS_CONV = 1, RS_DENSE = 2 };
 enum { RS_E_MMA = 0, RS_E_GATHER = 1, RS_E_DENSE = 2, RS_E_MEAN = 3 };
-enum { RS_U_CONV = 0, RS_U_DENSE = 1 };
+enum { RS_U_CONV = 0, RS_U_DENSE = 1, RS_U_FEW = 2 };
 
 // The first five 16-byte groups of RsNode and the first three of RsEdge are what a work unit needs; the unit
 // fetches them with 128-bit loads (a quarter of the shared-memory instructions of field-by-field reads, which
@@ -91,11 +98,15 @@ static_assert(offsetof(RsEdge, src) == 0 && offsetof(RsEdge, pad) == 16 && offse
 struct RsUnit { int32_t kind, node, a, b, c, d; };
 struct RsCopy { const char* src; int32_t dst, bytes; };
 
+// What the sum of a dense node's slots needs (32 bytes: two loads).  act: bit 0 ReLU, bit 1 the output node.
+struct alignas(16) RsSum { int32_t level, slot_off, n_slots, C, bias_off, buf[2], act; };
+
 struct RsHeader {
     int32_t n_nodes, n_edges, n_levels, n_warps;
     int32_t off_nodes, off_edges, off_units, off_ubegin;
     int32_t off_copies, n_copies, zero_off, smem_bytes;
-    int32_t dense_level_mask, sync_after_finalize, blob_bytes, pad_;
+    int32_t dense_level_mask, sync_after_finalize, blob_bytes, off_sums;
+    int32_t n_sums, pad_[3];
 };
 
 // ------------------------------------------------------------------------------------------------ device helpers
@@ -273,6 +284,61 @@ __device__ __forceinline__ void rs_mma_edge_generic(float (&acc)[2 * NB][4], int
     }
 }
 
+// Where a node's outputs of relative frame f + 1 go, for the lane's eight channels from n0 on.
+struct RsTileOut {
+    int W, nslo, d_up, d_dn;
+    uint32_t nchd, ch, dbuf, buf_bytes;
+    bool relu;
+    __device__ __forceinline__ RsTileOut(const RsNode& nd, int f, int n0, int lane)
+    {
+        const uint4* np = reinterpret_cast<const uint4*>(&nd);
+        const uint4 nq0 = np[0], nq1 = np[1], nq2 = np[2], nq4 = np[4];
+        W = (int)nq0.y;
+        nslo = (int)nq0.w;
+        nchd = nq0.z >> 3;
+        ch = (uint32_t)((n0 >> 3) + (lane & 3));
+        dbuf = ((f + 1) & 1) ? nq1.z : nq1.y;
+        buf_bytes = nq2.w;
+        relu = nq2.z == 1;
+        d_up = (nslo - (int)nq4.z) * W;
+        d_dn = (nslo - (int)nq4.w) * W;
+    }
+};
+
+// Activation, bf16, one 16-byte (8-byte for a 16-channel tile) store per pixel, and one into the neighbour's halo where the pixel
+// table says so.  t: the table's entries of accumulator rows g and g + 8; sub: byte offset of a 16-channel tile in its chunk.
+template <int NB>
+__device__ __forceinline__ void rs_store_tile(const RsCtx& cx, const RsTileOut& o, const float (&acc)[2 * NB][4], const uint32_t (&t)[2], uint32_t sub)
+{
+    auto put = [&](uint32_t off, const uint32_t (&pk)[4], int peer) {
+        if (off >= o.buf_bytes) return;
+        if (peer < 0) {
+            if (NB == 2) *reinterpret_cast<uint4*>(cx.smem + o.dbuf + off) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+            else *reinterpret_cast<uint2*>(cx.smem + o.dbuf + off + sub) = make_uint2(pk[0], pk[1]);
+        } else {
+            const uint32_t ra = rs_mapa(cx.sbase + o.dbuf + off + sub, (uint32_t)peer);
+            if (NB == 2) rs_st_cluster_v4(ra, pk);
+            else rs_st_cluster_v2(ra, pk[0], pk[1]);
+        }
+    };
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        if (t[r] == 0xFFFFFFFFu) continue;
+        const int y = (int)((t[r] >> 15) & 0x7FFFu), x = (int)(t[r] & 0x7FFFu);
+        uint32_t pk[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+        for (int nt = 0; nt < 2 * NB; ++nt) {
+            __nv_bfloat162 v = __floats2bfloat162_rn(acc[nt][2 * r], acc[nt][2 * r + 1]);
+            if (o.relu) v = __hmax2(v, __floats2bfloat162_rn(0.f, 0.f));
+            pk[nt] = *reinterpret_cast<const uint32_t*>(&v);
+        }
+        const int lin = (y - o.nslo) * o.W + x;
+        put(rs_swz((uint32_t)lin * o.nchd + o.ch) * 16u, pk, -1);
+        if (t[r] & 0x80000000u) put(rs_swz((uint32_t)(lin + o.d_up) * o.nchd + o.ch) * 16u, pk, (int)cx.rank - 1);   // halo of the previous CTA
+        if (t[r] & 0x40000000u) put(rs_swz((uint32_t)(lin + o.d_dn) * o.nchd + o.ch) * 16u, pk, (int)cx.rank + 1);   // of the next one
+    }
+}
+
 // One (16 pixels x NB * 16 channels) tile of a convolutional node: all k-steps of all incoming edges into one
 // accumulator, then bias, activation, bf16 cast and the stores into the next frame's buffer (own copy and,
 // for halo rows, the neighbour's).  `f` is the frame index relative to the start of the run: the update
@@ -284,8 +350,8 @@ __device__ __forceinline__ void rs_conv_unit(const RsCtx& cx, const RsNode& nd, 
 {
     const int lane = cx.lane;
     const uint4* np = reinterpret_cast<const uint4*>(&nd);
-    const uint4 nq0 = np[0], nq3 = np[3], nq4 = np[4];
-    const int W = (int)nq0.y, C = (int)nq0.z, nslo = (int)nq0.w, n_edges = (int)nq3.x, first_edge = (int)nq3.y;
+    const uint4 nq3 = np[3], nq4 = np[4];
+    const int n_edges = (int)nq3.x, first_edge = (int)nq3.y;
     const uint32_t zaddr = cx.sbase + cx.H->zero_off;
     // Column c of n-tile nt of a block holds output channel n0 + (c >> 1) * 8 + nt * 2 + (c & 1) (the host packs the
     // weights that way), so a lane's accumulator columns are consecutive channels: n0 + tq * 8 .. + 7 for a
@@ -393,108 +459,130 @@ __device__ __forceinline__ void rs_conv_unit(const RsCtx& cx, const RsNode& nd, 
             }
         }
     }
-    // epilogue: activation, bf16, one 16-byte (8-byte for a 16-channel tile) store per pixel, and one into the
-    // neighbour's halo where the pixel table says so
-    const uint32_t nchd = (uint32_t)(C >> 3), ch = (uint32_t)((n0 >> 3) + tq), sub = NB == 1 ? (uint32_t)half * 8u : 0u;
-    const uint4 nq1 = np[1], nq2 = np[2], nq4e = np[4];      // fetched here, not kept in registers across the main loop
-    const uint32_t dbuf = ((f + 1) & 1) ? nq1.z : nq1.y, buf_bytes = nq2.w;
-    const bool relu = nq2.z == 1;
-    const int d_up = (nslo - (int)nq4e.z) * W, d_dn = (nslo - (int)nq4e.w) * W;
-    auto put = [&](uint32_t off, const uint32_t (&pk)[4], int peer) {
-        if (off >= buf_bytes) return;
-        if (peer < 0) {
-            if (NB == 2) *reinterpret_cast<uint4*>(cx.smem + dbuf + off) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-            else *reinterpret_cast<uint2*>(cx.smem + dbuf + off + sub) = make_uint2(pk[0], pk[1]);
-        } else {
-            const uint32_t ra = rs_mapa(cx.sbase + dbuf + off + sub, (uint32_t)peer);
-            if (NB == 2) rs_st_cluster_v4(ra, pk);
-            else rs_st_cluster_v2(ra, pk[0], pk[1]);
-        }
-    };
+    // epilogue
+    const RsTileOut o(nd, f, n0, lane);
+    uint32_t t[2];
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const uint32_t t = pix[j0 + g + 8 * r];
-        if (t == 0xFFFFFFFFu) continue;
-        const int y = (int)((t >> 15) & 0x7FFFu), x = (int)(t & 0x7FFFu);
-        uint32_t pk[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-        for (int nt = 0; nt < 2 * NB; ++nt) {
-            __nv_bfloat162 v = __floats2bfloat162_rn(acc[nt][2 * r], acc[nt][2 * r + 1]);
-            if (relu) v = __hmax2(v, __floats2bfloat162_rn(0.f, 0.f));
-            pk[nt] = *reinterpret_cast<const uint32_t*>(&v);
-        }
-        const int lin = (y - nslo) * W + x;
-        put(rs_swz((uint32_t)lin * nchd + ch) * 16u, pk, -1);
-        if (t & 0x80000000u) put(rs_swz((uint32_t)(lin + d_up) * nchd + ch) * 16u, pk, (int)cx.rank - 1);   // halo of the previous CTA
-        if (t & 0x40000000u) put(rs_swz((uint32_t)(lin + d_dn) * nchd + ch) * 16u, pk, (int)cx.rank + 1);   // of the next one
-    }
+    for (int r = 0; r < 2; ++r) t[r] = pix[j0 + g + 8 * r];
+    rs_store_tile<NB>(cx, o, acc, t, NB == 1 ? (uint32_t)half * 8u : 0u);
 }
 
-__device__ __forceinline__ void rs_unpack8(const uint4& q, float (&v)[8])
+// A row of up to kRsFewTiles such tiles of a node whose only edge is a few-channel one of KS k-steps: the lookup table,
+// the bias and (one k-step) the weights stay in registers for all of them, and the loads of a tile are then issued before the
+// stores of the one before it.
+template <int KS>
+__device__ __forceinline__ void rs_few_unit(const RsCtx& cx, const RsNode& nd, int j0, int n0, int n_tiles, int f)
 {
-    v[0] = __uint_as_float(q.x << 16); v[1] = __uint_as_float(q.x & 0xFFFF0000u);
-    v[2] = __uint_as_float(q.y << 16); v[3] = __uint_as_float(q.y & 0xFFFF0000u);
-    v[4] = __uint_as_float(q.z << 16); v[5] = __uint_as_float(q.z & 0xFFFF0000u);
-    v[6] = __uint_as_float(q.w << 16); v[7] = __uint_as_float(q.w & 0xFFFF0000u);
+    const int lane = cx.lane, g = lane >> 2, tq = lane & 3;
+    const uint4* np = reinterpret_cast<const uint4*>(&nd);
+    const uint4 nq3 = np[3], nq4 = np[4];
+    const RsEdge& e = cx.edges[(int)nq3.y];
+    const uint4* ep = reinterpret_cast<const uint4*>(&e);
+    const uint4 eq0 = ep[0], eq1 = ep[1], eq2 = ep[2];
+    const RsNode& sn = cx.nodes[eq0.x];
+    const uint4 sq1 = reinterpret_cast<const uint4*>(&sn)[1];
+    const int fb = f + 1 - (int)eq1.y, bi = fb % sn.in_nb, tail = sn.in_tail;
+    const uint16_t* src = reinterpret_cast<const uint16_t*>(cx.smem + (bi == 0 ? sq1.y : bi == 1 ? sq1.z : sq1.w));
+    const uint32_t* lut = reinterpret_cast<const uint32_t*>(cx.smem + eq1.w);
+    const int g_const = (int)eq2.x, g_ys = (int)eq2.y, g_xs = (int)eq2.z;
+    const uint32_t* pix = reinterpret_cast<const uint32_t*>(cx.smem + nq3.z) + j0 + g;
+    uint2 L[KS][2];
+    uint32_t w[2][4];
+    const uint32_t waddr = cx.sbase + nq4.x + (uint32_t)(n0 >> 5) * nq4.y * 1024u + lane * 16;
+#pragma unroll
+    for (int ks = 0; ks < KS; ++ks) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) L[ks][h] = *reinterpret_cast<const uint2*>(lut + ks * 16 + h * 8 + 2 * tq);
+        if (KS == 1) {
+            rs_ldsm4(w[0], waddr);
+            rs_ldsm4(w[1], waddr + 512);
+        }
+    }
+    const float* bias = reinterpret_cast<const float*>(cx.smem + nq3.w) + n0 + tq * 8;
+    const float4 bl = *reinterpret_cast<const float4*>(bias), bh = *reinterpret_cast<const float4*>(bias + 4);
+    const RsTileOut o(nd, f, n0, lane);
+    uint32_t t[2], a[KS][4];
+    auto gather = [&](int i) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            t[r] = pix[i * 16 + 8 * r];
+            const uint16_t* x = src + (t[r] != 0xFFFFFFFFu ? g_const + (int)((t[r] >> 15) & 0x7FFFu) * g_ys + (int)(t[r] & 0x7FFFu) * g_xs : tail);
+#pragma unroll
+            for (int ks = 0; ks < KS; ++ks)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) a[ks][h * 2 + r] = (uint32_t)x[(int)L[ks][h].x] | ((uint32_t)x[(int)L[ks][h].y] << 16);
+        }
+    };
+    gather(0);
+    for (int i = 0; i < n_tiles; ++i) {
+        float acc[4][4];
+        acc[0][0] = acc[0][2] = bl.x; acc[0][1] = acc[0][3] = bl.y;
+        acc[1][0] = acc[1][2] = bl.z; acc[1][1] = acc[1][3] = bl.w;
+        acc[2][0] = acc[2][2] = bh.x; acc[2][1] = acc[2][3] = bh.y;
+        acc[3][0] = acc[3][2] = bh.z; acc[3][1] = acc[3][3] = bh.w;
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) {
+            if (KS > 1) {
+                rs_ldsm4(w[0], waddr + ks * 1024);
+                rs_ldsm4(w[1], waddr + ks * 1024 + 512);
+            }
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt) rs_mma(acc[nt], a[ks], w[nt >> 1][(nt & 1) * 2], w[nt >> 1][(nt & 1) * 2 + 1]);
+        }
+        const uint32_t tc[2] = {t[0], t[1]};
+        if (KS == 1 && i + 1 < n_tiles) gather(i + 1);
+        rs_store_tile<2>(cx, o, acc, tc, 0u);
+        if (KS > 1 && i + 1 < n_tiles) gather(i + 1);           // (no registers left to have two in flight)
+    }
 }
 
 // A slice of a dense / mean-dense edge: this warp's partial dot products of the 16-byte chunks
 // [c_begin, c_end) of the CTA's part of the source with the matching weight columns, for every output,
 // written to slot `slot` of the target node in every CTA of the cluster.
+// Sixteen outputs are the rows of an m16n8k16 whose eight columns all hold the source: four chunks a step, lane tq's chunk
+// supplying its words 0, 1 to the first and 2, 3 to the second multiply (the order of k is free as long as both operands agree).
+template <bool WS>
 __device__ __forceinline__ void rs_dense_unit(const RsCtx& cx, const RsNode& nd, const RsEdge& e, int c_begin, int c_end,
                                               int slot, int f)
 {
-    const int lane = cx.lane;
+    const int lane = cx.lane, g = lane >> 2, tq = lane & 3;
     const RsNode& sn = cx.nodes[e.src];
     const int fb = f + 1 - e.R;
     const unsigned char* xb = cx.smem + sn.buf[fb & 1];
     const bool swz = sn.kind == RS_CONV;
-    const char* wb = e.wd_off >= 0 ? reinterpret_cast<const char*>(cx.smem + e.wd_off) : e.wd_global;
-    const long long ld = e.wd_off >= 0 ? (long long)e.wd_ld : (long long)e.wd_gld;
     const uint32_t slot_base = (uint32_t)nd.slot_off + (uint32_t)((((f + 1) & 1) * nd.n_slots + slot) * nd.C) * 4u;
     const int C = nd.C, wmod = e.wchunk_mod, x0 = e.x_chunk0;
     const float scale = e.scale;
+    const long long ld = WS ? (long long)e.wd_ld : (long long)e.wd_gld;
     for (int ob = 0; ob < C; ob += 16) {
-        float acc[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) acc[j] = 0.f;
-        for (int cl = c_begin + lane; cl < c_end; cl += 32) {
+        const bool r0 = ob + g < C, r1 = ob + g + 8 < C;
+        const unsigned char* ws = cx.smem + e.wd_off + (ob + g) * (int)ld * 2;
+        const char* wg = e.wd_global + (long long)(ob + g) * ld * 2;
+        const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+        float d0[4] = {0.f, 0.f, 0.f, 0.f}, d1[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+        for (int c = c_begin; c < c_end; c += 4) {
+            const int cl = c + tq;
+            const bool in = cl < c_end;
             const uint32_t q = (uint32_t)(x0 + cl);
-            const uint4 xq = *reinterpret_cast<const uint4*>(xb + (swz ? rs_swz(q) : q) * 16u);
-            float x[8];
-            rs_unpack8(xq, x);
-            const int wc = wmod ? cl % wmod : cl;
-            const char* wp = wb + ((long long)ob * ld + (long long)wc * 8) * 2;
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                if (ob + j < C) {
-                    const uint4 wq = *reinterpret_cast<const uint4*>(wp + (long long)j * ld * 2);
-                    float w[8];
-                    rs_unpack8(wq, w);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) acc[j] = fmaf(w[i], x[i], acc[j]);
-                }
-            }
+            const int wo = (wmod ? cl % wmod : cl) * 16;
+            uint4 x = zero, a = zero, b = zero;
+            if (in) x = *reinterpret_cast<const uint4*>(xb + (swz ? rs_swz(q) : q) * 16u);
+            if (in && r0) a = WS ? *reinterpret_cast<const uint4*>(ws + wo) : __ldg(reinterpret_cast<const uint4*>(wg + wo));
+            if (in && r1) b = WS ? *reinterpret_cast<const uint4*>(ws + (int)ld * 16 + wo) : __ldg(reinterpret_cast<const uint4*>(wg + ld * 16 + wo));
+            const uint32_t a0[4] = {a.x, b.x, a.y, b.y}, a1[4] = {a.z, b.z, a.w, b.w};
+            rs_mma(d0, a0, x.x, x.y);
+            rs_mma(d1, a1, x.z, x.w);
         }
-        // reduce-scatter over the warp: every step halves the values a lane keeps and adds the partner's copy of
-        // them (16 shuffles for 16 outputs instead of 80); lane l ends with the total of output ob + (l & 15)
-        float v8[8], v4[4], v2[2];
-        const bool h3 = lane & 8, h2 = lane & 4, h1 = lane & 2, h0 = lane & 1;
+        // all columns are equal: lane tq of a row's four writes it to rank tq
+        if (tq < cx.cs) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) v8[i] = (h3 ? acc[i + 8] : acc[i]) + __shfl_xor_sync(0xffffffffu, h3 ? acc[i] : acc[i + 8], 8);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) v4[i] = (h2 ? v8[i + 4] : v8[i]) + __shfl_xor_sync(0xffffffffu, h2 ? v8[i] : v8[i + 4], 4);
-#pragma unroll
-        for (int i = 0; i < 2; ++i) v2[i] = (h1 ? v4[i + 2] : v4[i]) + __shfl_xor_sync(0xffffffffu, h1 ? v4[i] : v4[i + 2], 2);
-        float v = (h0 ? v2[1] : v2[0]) + __shfl_xor_sync(0xffffffffu, h0 ? v2[0] : v2[1], 1);
-        v += __shfl_xor_sync(0xffffffffu, v, 16);
-        if (lane < 16 && ob + lane < C) {
-            v *= scale;
-            const uint32_t a = cx.sbase + slot_base + (uint32_t)(ob + lane) * 4u;
-            if (cx.cs > 1) {
-                for (int r = 0; r < cx.cs; ++r) rs_st_cluster_u32(rs_mapa(a, (uint32_t)r), __float_as_uint(v));
-            } else {
-                *reinterpret_cast<float*>(cx.smem + slot_base + (uint32_t)(ob + lane) * 4u) = v;
+            for (int h = 0; h < 2; ++h) {
+                if (h ? !r1 : !r0) continue;
+                const float v = (d0[2 * h] + d1[2 * h]) * scale;
+                const uint32_t at = slot_base + (uint32_t)(ob + g + 8 * h) * 4u;
+                if (cx.cs > 1) rs_st_cluster_u32(rs_mapa(cx.sbase + at, (uint32_t)tq), __float_as_uint(v));
+                else *reinterpret_cast<float*>(cx.smem + at) = v;
             }
         }
     }
@@ -610,26 +698,40 @@ __device__ __forceinline__ void rs_kernel_body(const unsigned char* __restrict__
                     if (un.c == 2) rs_conv_unit<2>(cx, nd, un.a, un.b, 0, f);
                     else rs_conv_unit<1>(cx, nd, un.a, un.b, un.c, f);
                 }
-                else rs_dense_unit(cx, nd, cx.edges[un.a], un.b, un.c, un.d, f);
+                else if (un.kind == RS_U_FEW) {
+                    if (un.d == 1) rs_few_unit<1>(cx, nd, un.a, un.b, un.c, f);
+                    else rs_few_unit<2>(cx, nd, un.a, un.b, un.c, f);
+                }
+                else if (cx.edges[un.a].wd_off >= 0) rs_dense_unit<true>(cx, nd, cx.edges[un.a], un.b, un.c, un.d, f);
+                else rs_dense_unit<false>(cx, nd, cx.edges[un.a], un.b, un.c, un.d, f);
             }
             if (l == H.n_levels - 1) rs_cp_async_wait_all();
             rs_level_barrier(cs);
             if ((H.dense_level_mask >> l) & 1) {
                 // dense nodes of this level: fixed-order sum of the slots (the bias is slot-independent), activation
                 if (warp == kRsFinalizeWarp) {
-                    for (int v = 0; v < H.n_nodes; ++v) {
-                        const RsNode& nd = cx.nodes[v];
-                        if (nd.kind != RS_DENSE || nd.level != l) continue;
-                        const int C = nd.C, n_slots = nd.n_slots;
-                        const float* slots = reinterpret_cast<const float*>(smem + nd.slot_off) + ((f + 1) & 1) * n_slots * C;
-                        const float* bias = reinterpret_cast<const float*>(smem + nd.bias_off);
-                        for (int o = cx.lane; o < C; o += 32) {
-                            float z = 0.f;
-                            for (int s = 0; s < n_slots; ++s) z += slots[s * C + o];
-                            z += bias[o];
-                            if (nd.act == 1) z = fmaxf(z, 0.f);
-                            reinterpret_cast<__nv_bfloat16*>(smem + nd.buf[(f + 1) & 1])[o] = __float2bfloat16_rn(z);
-                            if (nd.is_output && rank == 0 && out_base) out_base[(run0 + f) * out_stride + (long long)b * C + o] = z;
+                    const RsSum* sums = reinterpret_cast<const RsSum*>(smem + H.off_sums);
+                    for (int k = 0; k < H.n_sums; ++k) {
+                        const int4 q0 = reinterpret_cast<const int4*>(sums + k)[0], q1 = reinterpret_cast<const int4*>(sums + k)[1];
+                        if (q0.x != l) continue;
+                        const int n_slots = q0.z, C = q0.w;
+                        const float* slots = reinterpret_cast<const float*>(smem + q0.y) + ((f + 1) & 1) * n_slots * C;
+                        __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(smem + (((f + 1) & 1) ? q1.z : q1.y));
+                        // the halves of the warp take a half of the slots each
+                        const int s_half = (n_slots + 1) >> 1, s0 = cx.lane < 16 ? 0 : s_half, s1 = cx.lane < 16 ? s_half : n_slots;
+                        for (int o0 = 0; o0 < C; o0 += 16) {
+                            const int o = o0 + (cx.lane & 15);
+                            float z = cx.lane < 16 && o < C ? reinterpret_cast<const float*>(smem + q1.x)[o] : 0.f;
+                            if (o < C) {
+#pragma unroll 4
+                                for (int s = s0; s < s1; ++s) z += slots[s * C + o];
+                            }
+                            z += __shfl_down_sync(0xffffffffu, z, 16);
+                            if (cx.lane < 16 && o < C) {
+                                if (q1.w & 1) z = fmaxf(z, 0.f);
+                                dst[o] = __float2bfloat16_rn(z);
+                                if ((q1.w & 2) && rank == 0 && out_base) out_base[(run0 + f) * out_stride + (long long)b * C + o] = z;
+                            }
                         }
                     }
                 }
@@ -692,7 +794,7 @@ struct RsPlanEdge {
     int wd_off[kRsMaxCluster] = {-1, -1, -1, -1};
 };
 
-struct RsOffsets { int nodes = 0, edges = 0, units = 0, ubegin = 0, copies = 0; };   // table offsets inside a rank's blob
+struct RsOffsets { int nodes = 0, edges = 0, units = 0, ubegin = 0, copies = 0, sums = 0; };   // table offsets inside a rank's blob
 
 struct RsEngine {
     int cs = 1, warps = 16, smem_bytes = 0, blob_bytes = 0, n_levels = 1;
@@ -716,7 +818,8 @@ int rs_up16(int x) { return (x + 15) / 16 * 16; }
 int rs_up128(int x) { return (x + 127) / 128 * 128; }
 
 // Lays the engine out for a cluster of `cs` CTAs; false if the network does not fit.
-bool rs_layout(const sr_graph* g, RsEngine& E, int cs, int warps)
+// dense_chunks: 16-byte chunks of the source per unit of a dense edge.
+bool rs_layout(const sr_graph* g, RsEngine& E, int cs, int warps, int dense_chunks)
 {
     const int n_nodes = (int)g->nodes.size();
     E.cs = cs;
@@ -774,28 +877,34 @@ bool rs_layout(const sr_graph* g, RsEngine& E, int cs, int warps)
     // which nodes are cut into 16-channel tiles: those whose 32-channel tile alone would take more than half of a
     // warp's fair share of its level
     std::vector<char> split(n_nodes, 0);
-    if (g->opt_rs_split != 0) {
-        std::vector<long> level_cost(E.n_levels, 0), unit_cost(n_nodes, 0);
+    std::vector<long> level_cost(E.n_levels, 0), unit_cost(n_nodes, 0);
+    auto few = [&](int v) {                            // the node's only edge is a few-channel one of at most two k-steps
+        return E.pn[v].kind == RS_CONV && g->nodes[v].in_edges.size() == 1 && E.pe[E.pn[v].first_edge].type == RS_E_GATHER && E.pe[E.pn[v].first_edge].ksteps <= 2;
+    };
+    {
         for (int v = 0; v < n_nodes; ++v) {
             const RsPlanNode& p = E.pn[v];
             const SrHostNode& hn = g->nodes[v];
             if (p.kind == RS_INPUT) continue;
             long c = 1700, units = 0;
-            if (p.kind == RS_CONV) {
+            if (few(v)) {
+                c = kRsFewCost;
+                units = (long)(((p.lo[1] - p.lo[0]) * hn.d.w + 15) / 16) * (hn.d.c / 32);
+            } else if (p.kind == RS_CONV) {
                 for (int ei = 0; ei < (int)hn.in_edges.size(); ++ei) {
                     const RsPlanEdge& pe = E.pe[p.first_edge + ei];
                     c += (long)pe.ksteps * (pe.type == RS_E_MMA ? 160 : 400);
                 }
                 units = (long)(((p.lo[1] - p.lo[0]) * hn.d.w + 15) / 16) * (hn.d.c / 32);
             } else {
-                c = 5000;
-                units = 4;
+                c = 1500;
+                units = 8;
             }
             unit_cost[v] = c;
             level_cost[hn.level - 1] += c * units;
         }
-        for (int v = 0; v < n_nodes; ++v)
-            if (E.pn[v].kind == RS_CONV && (g->opt_rs_split == 1 || unit_cost[v] * 2 * warps > level_cost[g->nodes[v].level - 1]))
+        for (int v = 0; v < n_nodes && g->opt_rs_split != 0; ++v)
+            if (E.pn[v].kind == RS_CONV && !few(v) && (g->opt_rs_split == 1 || unit_cost[v] * 2 * warps > level_cost[g->nodes[v].level - 1]))
                 split[v] = 1;
     }
     for (int v = 0; v < n_nodes; ++v) {
@@ -814,9 +923,16 @@ bool rs_layout(const sr_graph* g, RsEngine& E, int cs, int warps)
             // a unit is a 16-pixel x 32-channel tile (c = 2), or, for nodes with many k-steps when the CTA has more
             // warps than such tiles, its two 16-channel halves (c = 0, 1): they load the A operand twice but halve the
             // longest dependent chain of a frame
+            // Few-channel nodes: as many tiles to a unit as keep it below half of a warp's fair share of its level.
+            const int few_tiles = few(v) ? (int)std::max(1L, std::min((long)kRsFewTiles, level_cost[level] / (2 * warps * kRsFewCost))) : 0;
             for (int r = 0; r < cs; ++r) {
                 const int npix = (p.lo[r + 1] - p.lo[r]) * hn.d.w;
-                for (int j0 = 0; j0 < npix; j0 += 16)
+                for (int j0 = 0; few_tiles && j0 < npix; j0 += 16 * few_tiles)
+                    for (int n0 = 0; n0 < hn.d.c; n0 += 32) {
+                        const int nt = std::min(few_tiles, (npix - j0 + 15) / 16);
+                        cand[r].push_back(Cand{RsUnit{RS_U_FEW, v, j0, n0, nt, E.pe[p.first_edge].ksteps}, level, 600 + nt * kRsFewCost});
+                    }
+                for (int j0 = 0; !few_tiles && j0 < npix; j0 += 16)
                     for (int n0 = 0; n0 < hn.d.c; n0 += 32) {
                         if (split[v]) {
                             cand[r].push_back(Cand{RsUnit{RS_U_CONV, v, j0, n0, 0, 0}, level, 1400 + (cost - 1700) * 6 / 10});
@@ -836,11 +952,11 @@ bool rs_layout(const sr_graph* g, RsEngine& E, int cs, int warps)
                     if (sp.kind == RS_CONV) n = (sp.lo[r + 1] - sp.lo[r]) * sd.w * (sd.c / 8);
                     else if (r == 0) n = sd.c / 8;
                     if (n == 0) continue;
-                    const int parts = (n + kRsDenseUnitChunks - 1) / kRsDenseUnitChunks;
+                    const int parts = (n + dense_chunks - 1) / dense_chunks;
                     const int per = (n + parts - 1) / parts;
                     for (int c0 = 0; c0 < n; c0 += per) {
                         const int c1 = std::min(n, c0 + per);
-                        const long cost = 2200 + (long)((c1 - c0 + 31) / 32) * 250 * hn.d.c;
+                        const long cost = 800 + (long)((c1 - c0 + 3) / 4) * 100 * ((hn.d.c + 15) / 16);
                         cand[r].push_back(Cand{RsUnit{RS_U_DENSE, v, p.first_edge + ei, c0, c1, slot_count[v]++}, level, cost});
                     }
                 }
@@ -858,13 +974,14 @@ bool rs_layout(const sr_graph* g, RsEngine& E, int cs, int warps)
                 if (c.level == l) cs_l.push_back(c);
             std::stable_sort(cs_l.begin(), cs_l.end(), [](const Cand& a, const Cand& b) { return a.cost > b.cost; });
             std::vector<long> wl(warps, 0), pl(4, 0);
-            // fixed duties: the slot sums of the dense nodes of this level, the input fetch (last level's barrier waits for it)
-            bool dense_here = false;
+            // fixed duties: the slot sums of the dense nodes of the level before (they follow its barrier), the input fetch (the last
+            // level's barrier waits for it)
+            bool dense_before = false;
             for (int v = 0; v < n_nodes; ++v)
-                if (E.pn[v].kind == RS_DENSE && g->nodes[v].level - 1 == l) dense_here = true;
-            if (dense_here && kRsFinalizeWarp < warps) {
-                wl[kRsFinalizeWarp] += 3500;
-                pl[kRsFinalizeWarp % 4] += 3500;
+                if (E.pn[v].kind == RS_DENSE && (g->nodes[v].level - 1 + 1) % E.n_levels == l) dense_before = true;
+            if (dense_before && kRsFinalizeWarp < warps) {
+                wl[kRsFinalizeWarp] += 2000;
+                pl[kRsFinalizeWarp % 4] += 2000;
             }
             if (l == 0 && kRsFetchWarp < warps) {
                 wl[kRsFetchWarp] += 2500;
@@ -912,6 +1029,9 @@ bool rs_layout(const sr_graph* g, RsEngine& E, int cs, int warps)
         if (he.d.kind != SR_EDGE_CONV) dense_rows += g->nodes[he.d.tgt].d.c;
     }
     const int off_copies = take((int)sizeof(RsCopy) * (n_copies + dense_rows), 16);
+    int n_sums = 0;
+    for (int v = 0; v < n_nodes; ++v) n_sums += E.pn[v].kind == RS_DENSE;
+    const int off_sums = take((int)sizeof(RsSum) * n_sums, 16);
     for (size_t i = 0; i < E.pe.size(); ++i)
         if (E.pe[i].type == RS_E_GATHER) E.pe[i].lut_off = take((int)E.luts[i].size() * 4, 16);
     for (int v = 0; v < n_nodes; ++v) {
@@ -979,6 +1099,7 @@ bool rs_layout(const sr_graph* g, RsEngine& E, int cs, int warps)
     E.offs.units = off_units;
     E.offs.ubegin = off_ubegin;
     E.offs.copies = off_copies;
+    E.offs.sums = off_sums;
     return true;
 }
 
@@ -1175,7 +1296,12 @@ sr_status sr_rs_plan(sr_graph* g, size_t& offset)
     for (int c = kRsMaxCluster; c >= 1; c >>= 1) {
         if (g->opt_rs_cluster > 0 && c != g->opt_rs_cluster) continue;
         RsEngine F = *E;
-        if (!rs_layout(g, F, c, warps)) continue;
+        // (Smaller dense units finish sooner but need more slots; the dense weights' place in shared memory is worth more.)
+        if (!rs_layout(g, F, c, warps, 32)) continue;
+        if (!F.dense_in_smem) {
+            RsEngine F2 = *E;
+            if (rs_layout(g, F2, c, warps, 64)) F = F2;
+        }
         const int held = rs_clusters_held(F);
         const double cost = (double)((g->batch + held - 1) / held) * (1.9 + 9.2 / c);
         if (placed && cost >= best) continue;
@@ -1230,6 +1356,8 @@ sr_status sr_rs_bind(sr_graph* g)
         RsUnit* units = reinterpret_cast<RsUnit*>(blob.data() + O.units);
         int32_t* ubegin = reinterpret_cast<int32_t*>(blob.data() + O.ubegin);
         RsCopy* copies = reinterpret_cast<RsCopy*>(blob.data() + O.copies);
+        RsSum* sums = reinterpret_cast<RsSum*>(blob.data() + O.sums);
+        int n_sums = 0;
         int n_copies = 0, dense_mask = 0, sync_after = 0;
         for (int v = 0; v < n_nodes; ++v) {
             const SrHostNode& hn = g->nodes[v];
@@ -1288,6 +1416,7 @@ sr_status sr_rs_bind(sr_graph* g)
             d.gstate[1] = g->ws + hn.state[1].offset;
             if (p.kind == RS_DENSE) {
                 dense_mask |= 1 << d.level;
+                sums[n_sums++] = RsSum{d.level, p.slot_off, p.n_slots, d.C, p.bias_off, {p.buf[0], p.buf[1]}, (d.act == 1 ? 1 : 0) | (d.is_output ? 2 : 0)};
                 if (p.has_consumers) sync_after = 1;
             }
             if (p.kind != RS_INPUT) copies[n_copies++] = RsCopy{g->ws + hn.bias.offset, p.bias_off, rs_up16(hn.d.c * 4)};
@@ -1370,6 +1499,8 @@ sr_status sr_rs_bind(sr_graph* g)
         H->dense_level_mask = dense_mask;
         H->sync_after_finalize = sync_after;
         H->blob_bytes = E.blob_bytes;
+        H->off_sums = O.sums;
+        H->n_sums = n_sums;
         if (cudaMemcpy(g->ws + E.r_blobs.offset + (size_t)r * E.blob_bytes, blob.data(), blob.size(), cudaMemcpyHostToDevice) !=
             cudaSuccess)
             return SR_ERR_CUDA;

@@ -173,3 +173,19 @@ def test_more_sequences_than_clusters_of_four_fit():
     g = graphs.build("c2", batch=37, frames=3)
     for p in g.patterns:
         parity.check_run(g, p, samples=[0, 18, 36])
+
+
+@pytest.mark.parametrize("cin,k,stride,size,c,classes", [(1, 3, 1, 12, 32, 10), (3, 3, 1, 10, 64, 17), (1, 5, 2, 28, 32, 5), (2, 1, 1, 6, 32, 33), (4, 3, 1, 8, 32, 12)])
+def test_few_channel_nodes_and_dense_heads_at_edges(cin, k, stride, size, c, classes):
+    """First layers of one, two and more k-steps (several tiles to a unit, a ragged last one), dense nodes of more and of fewer
+    outputs than an instruction has rows, of chunk counts that are no multiple of its four, fed by another dense node."""
+    from workloads.graphs import CONV, DENSE, GAP_DENSE, IDENTITY, Edge, GraphSpec, Node, check_shapes
+    out = size // stride
+    nodes = [Node("in", size, size, cin, IDENTITY), Node("a", out, out, c), Node("h", 1, 1, 40), Node("o", 1, 1, classes, IDENTITY)]
+    edges = [Edge(0, 1, CONV, k, stride), Edge(1, 2, DENSE), Edge(2, 3, DENSE), Edge(1, 3, GAP_DENSE)]
+    for cluster in (1, 2):
+        for R in ([1, 1, 1, 1], [0, 0, 0, 0], [0, 1, 0, 1]):
+            g = GraphSpec("few", nodes, edges, batch=2, frames=3, dtype="bf16", seed=7)
+            g.patterns = {"p": R}
+            check_shapes(g)
+            parity.check_run(g, "p", expect_resident=cluster, resident_cluster=cluster)
