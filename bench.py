@@ -43,11 +43,11 @@ PAPER_NETS = {"dsr0": dict(batch=128, frames=16), "dsr6": dict(batch=128, frames
 # the kernel source it was taken from; the number is reported only while that source is unchanged, else null.
 TRAFFIC = {
     # workload: (bytes per launch, kernel source file, sha256[:12] of that file at capture time, summary under profiles/)
-    "c5": (615.7e6, "sr_tc.cu", "6985e1c55246", "profiles/sr_tc_group_kernel_counters.md"),
-    "c3": (245.2e6, "sr_tc.cu", "6985e1c55246", "profiles/sr_tc_group_kernel_counters.md"),
-    "c4": (165.1e6, "sr_tc.cu", "6985e1c55246", "profiles/sr_tc_group_kernel_counters.md"),
-    "c2": (8.0e6, "sr_resident.cu", "89436108f1ff", "profiles/sr_resident_kernel_c2.md"),     # one launch = all 32 frames
-    "c1": (1.30e6, "sr_dense.cu", "9f15eb3bde12", "profiles/sr_dense_kernel_c1.md"),           # one launch = all 16 frames
+    "c5": (604.6e6, "sr_tc.cu", "e7c1b36fa98f", "profiles/sr_tc_group_kernel_counters.md"),
+    "c3": (247.8e6, "sr_tc.cu", "e7c1b36fa98f", "profiles/sr_tc_group_kernel_counters.md"),
+    "c4": (162.4e6, "sr_tc.cu", "e7c1b36fa98f", "profiles/sr_tc_group_kernel_counters.md"),
+    "c2": (8.0e6, "sr_resident.cu", "91cb355416fc", "profiles/sr_resident_kernel_c2.md"),     # one launch = all 32 frames
+    "c1": (1.30e6, "sr_dense.cu", "056cb3783d12", "profiles/sr_dense_kernel_c1.md"),           # one launch = all 16 frames
 }
 
 
