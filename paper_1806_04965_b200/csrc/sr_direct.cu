@@ -39,7 +39,7 @@ constexpr int kPix = 4;            // pixels per warp (conv nodes)
 constexpr int kWarps = 4;          // warps per block
 constexpr int kDenseB = 8;         // samples per warp (dense nodes)
 
-// Conv node whose channel count is not a multiple of four: a block covers kWarps*kPix consecutive pixels of one sample; lanes run over output
+// Conv node that conv_tile does not take (see sr_direct_conv_items): a block covers kWarps*kPix consecutive pixels of one sample; lanes run over output
 // channels, so weight reads ([K][C_out] rows) and state writes (NHWC) are coalesced and the input
 // reads are warp-uniform broadcasts.
 template <typename T>
@@ -141,7 +141,7 @@ __device__ void conv_tile(const SrDevNode& nd, const SrDevEdge* edges, const SrD
 #pragma unroll
     for (int j = 0; j < PX; ++j) {
         const int p = p_first + j;
-        oy[j] = p < HW ? p / nd.W : 1 << 20;                                     // (a pixel that does not exist lies outside every image)
+        oy[j] = p < HW ? p / nd.W : -1;                                          // (-1: the pixel does not exist)
         ox[j] = p % nd.W;
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[j][q] = 0.f;
@@ -154,10 +154,9 @@ __device__ void conv_tile(const SrDevNode& nd, const SrDevEdge* edges, const SrD
         int y0[PX], x0[PX], o0[PX];
 #pragma unroll
         for (int j = 0; j < PX; ++j) {
-            y0[j] = oy[j] * e.stride - e.pad;
+            y0[j] = oy[j] >= 0 ? oy[j] * e.stride - e.pad : -(1 << 30);          // (then outside every image)
             x0[j] = ox[j] * e.stride - e.pad;
-            o0[j] = oy[j] < (1 << 20) ? (y0[j] * Ws + x0[j]) * Cs : 0;
-            if (oy[j] >= (1 << 20)) y0[j] = -(1 << 20);
+            o0[j] = oy[j] >= 0 ? (y0[j] * Ws + x0[j]) * Cs : 0;
         }
         for (int e0 = 0; e0 < n; e0 += kTab) {
             const int m = min(kTab, n - e0);
@@ -504,7 +503,7 @@ __global__ void __launch_bounds__(kWarps * 32) sr_direct_group_kernel(const __gr
     const int prev = (int)(F.t & 1), cur = prev ^ 1;
     float* out = nd.is_output ? sr_frame_output(P.fr, F) : nullptr;
     if (nd.H == 1 && nd.W == 1 && P.edges[nd.first_edge].kind != SR_EDGE_CONV) dense_item<T>(nd, P.edges, it, prev, cur, P.B, out);
-    else if (nd.C % 4 != 0) conv_item<T>(nd, P.edges, it, prev, cur, out);
+    else if (it.pad_ < 0) conv_item<T>(nd, P.edges, it, prev, cur, out);
     else if (it.b0 >= 0) conv_tile<T, 1>(nd, P.edges, it, prev, cur, out, tab);
     else {
         SrDirectItem four = it;
@@ -622,9 +621,17 @@ void sr_direct_conv_items(const sr_graph* g, int v, std::vector<SrDirectItem>& i
 {
     const sr_node_desc& d = g->nodes[v].d;
     const int HW = d.h * d.w;
-    if (d.c % 4 != 0) {
+    // conv_tile takes channels in vectors of four and counts the elements of a source sample in 32 bits (from the corner of a window
+    // that leaves the image, hence the margin).
+    bool tile = d.c % 4 == 0 && d.c < 1 << 24;
+    for (int e : g->nodes[v].in_edges) {
+        const SrHostEdge& he = g->edges[e];
+        const sr_node_desc& s = g->nodes[he.d.src].d;
+        tile = tile && (double)(s.h + 2 * he.k_eff) * (s.w + 2 * he.k_eff) * s.c < 2147483648.0;
+    }
+    if (!tile) {
         for (int b = 0; b < g->batch; ++b)
-            for (int p0 = 0; p0 < HW; p0 += kWarps * kPix) items.push_back(SrDirectItem{v, b, p0, 0});
+            for (int p0 = 0; p0 < HW; p0 += kWarps * kPix) items.push_back(SrDirectItem{v, b, p0, -1});
         return;
     }
     int qlog = 0;

@@ -37,7 +37,7 @@ struct SrDirectItem {
     int32_t node;        // index into the SrDevNode table
     int32_t b0;          // first sample (dense nodes: sample chunk); its complement: four pixels per thread (conv_tile)
     int32_t p0;          // first pixel (conv nodes) or first output channel (dense nodes)
-    int32_t pad_;        // conv nodes with a multiple of four channels: first channel | log2(channel quads per block) << 24
+    int32_t pad_;        // conv nodes: first channel | log2(channel quads per block) << 24, or -1 (conv_item)
 };
 
 // Dense / mean-dense nodes as the head kernels see them: passed as kernel parameters.

@@ -296,3 +296,39 @@ def test_cuda_core_convolutions_at_the_edges_of_their_tiles(batch, size, cin, c,
     check_shapes(g)
     g.patterns = {"p": [1, 1, 1, 0, 1]}
     parity.check_stepwise(g, "p", engine="direct", zero_bias=False, samples=[0, batch - 1])
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+def test_cuda_core_convolutions_of_images_with_a_million_rows(dtype):
+    # one-dimensional signals of more than 2^20 samples, the last pixels of which do not fill a block; one and four pixels per thread
+    from workloads.graphs import CONV, GAP_DENSE, IDENTITY, Edge, GraphSpec, Node, check_shapes
+    h = (1 << 20) + 37
+    for stride, c in ((1, 4), (32, 8)):
+        out = (h + stride - 1) // stride
+        nodes = [Node("in", h, 1, 1, IDENTITY), Node("a", out, 1, c), Node("o", 1, 1, 2, IDENTITY)]
+        g = GraphSpec("signal", nodes, [Edge(0, 1, CONV, 3, stride), Edge(1, 2, GAP_DENSE)], batch=1, frames=2, dtype=dtype, seed=95)
+        check_shapes(g)
+        g.patterns = {"p": [1, 1]}
+        parity.check_stepwise(g, "p", engine="direct", zero_bias=False)
+
+
+def test_cuda_core_convolution_of_a_sample_beyond_32_bit_offsets():
+    # a source sample of 2^31 elements: the last rows and columns, which lie behind the middle of it, against a product made on the
+    # GPU by torch in fp32 (the sums have four terms: 1e-2 is the rounding of the state to bf16, 2^-9, with room)
+    import torch
+    from paper_1806_04965_b200 import Graph
+    from workloads.graphs import CONV, GAP_DENSE, IDENTITY, Edge, Node
+    H, W, s = 1 << 15, 1 << 14, 64
+    nodes = [Node("in", H, W, 4, IDENTITY), Node("a", H // s, W // s, 8, IDENTITY), Node("o", 1, 1, 2, IDENTITY)]
+    G = Graph(nodes, [Edge(0, 1, CONV, 1, s), Edge(1, 2, GAP_DENSE)], [1, 1], batch=1, dtype="bf16", engine="direct")
+    w = np.random.default_rng(4).standard_normal((8, 1, 1, 4)).astype(np.float32)
+    G.set_weights([w, np.ones((2, 8), np.float32)], [np.zeros(n.c, np.float32) for n in nodes])
+    x = torch.zeros((1, H, W, 4), dtype=torch.bfloat16, device="cuda:0")
+    sub = torch.randn((H // s, W // s, 4), device="cuda:0", generator=torch.Generator(device="cuda:0").manual_seed(5)).to(torch.bfloat16)
+    x[0, ::s, ::s] = sub
+    G.reset([x])
+    G.step([x])
+    G.sync_status()
+    want = torch.einsum("hwc,oc->hwo", sub.float(), torch.from_numpy(w.reshape(8, 4)).to("cuda:0").to(torch.bfloat16).float())
+    got = G.get_state(1)[0].float()
+    assert float((got - want).abs().max()) <= 1e-2 * float(want.abs().max())
