@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
     __shared__ uint32_t box_start[kBoxes];                 // the activation producer's own: `head` at the start of each box
     __shared__ volatile int epi_done;                      // items the epilogue has finished
     __shared__ __align__(16) uint16_t epi_buf[kEpiWarps][16 * 32];   // per epilogue warp: 16 pixels x 32 channels, bf16
-    __shared__ int pix_off[2][kMaxCols];                   // element offset of every pixel of an item, -1 = not stored
+    __shared__ int pix_off[2][kMaxCols];                   // number of every pixel of an item in its node's state, -1 = not stored
 
     if (!(P.follow & 2)) sr_let_successor_start();
     const long long wait_limit = P.wait_limit;
@@ -674,9 +674,10 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
         // alternate 16-column chunks.  A warp turns 32 channels x 16 pixels into NHWC order through a 1 KiB shared-memory buffer:
         // bias, ReLU and bf16 on fragments of 8 x 8 that stmatrix stores transposed, then every thread reads back 8 consecutive
         // channels of one pixel and stores them as one 16-byte word, so a pixel's 32 channels leave the warp as one 64-byte
-        // run.  (With one 2-byte store per value the deepest CIFAR10 network took 74.6 us per frame, so 72.5.)  The element offset of every pixel of the work item (or -1 for separator
-        // rows and pixels outside the image) is tabulated once per item, in one of two tables, so that one barrier per
-        // item is enough; that barrier also makes giving up a joint decision.
+        // run.  (With one 2-byte store per value the deepest CIFAR10 network took 74.6 us per frame, so 72.5.)  The number of
+        // every pixel of the work item in the state (or -1 for separator rows and pixels outside the image) is tabulated
+        // once per item, in one of two tables, so that one barrier per item is enough; that barrier also makes giving up a
+        // joint decision.
         sr_wait_for_predecessor();
         const int ew = warp - 4, quarter = ew & 3, half = ew >> 2;      // TMEM lanes 32*quarter .. +31 belong to this warp
         const int et = threadIdx.x - 128;                               // 0..255 among the epilogue threads
@@ -700,7 +701,7 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                 const int l = et / lane_cols, nn = et - l * lane_cols, x = nn % tw, q = nn / tw, r = q % rows, bi = q / rows;
                 const int b = tl.b0 + bi, y = tl.h0 + r, xx = tl.w0 + l * tw + x;
                 const bool in = l < nl && r < th && bi < nd->tb && b < P.B && y < nd->H && xx < nd->W;
-                poff[et] = in ? (int)((((size_t)b * nd->H + y) * nd->W + xx) * nd->C) : -1;
+                poff[et] = in ? (b * nd->H + y) * nd->W + xx : -1;
             }
             uint32_t stop;
             asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, 1, 256, p;\n\tselp.b32 %0, 1, 0, q;\n\t}"
@@ -758,7 +759,7 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                     const int o = poff[c0 + pass * 8 + (lane >> 2)];
                     if (o >= 0 && gvalid) {
                         const uint4 w = *reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(tbuf) + pass * 512 + ld_off);
-                        *reinterpret_cast<uint4*>(out + (size_t)o + co_w + (lane & 3) * 8) = w;
+                        *reinterpret_cast<uint4*>(out + (size_t)o * C + co_w + (lane & 3) * 8) = w;
                     }
                 }
                 __syncwarp();
@@ -1123,7 +1124,8 @@ long long spread_items(const std::vector<std::pair<long long, TcTile>>& tl, size
 }  // namespace
 
 // A node goes to the tensor cores if it sums convolutions only, has at least 16 output channels in
-// multiples of 8, and every incoming edge either has C_in % 16 == 0 or is a few-channel input edge.
+// multiples of 8, and every incoming edge either has C_in % 16 == 0 or is a few-channel input edge.  Its pixels (and the
+// 16-byte chunks of a staged edge, see sr_input.cuh) are counted in 32 bits.
 void sr_tc_select_nodes(sr_graph* g)
 {
     for (size_t v = 0; v < g->nodes.size(); ++v) {
@@ -1131,12 +1133,14 @@ void sr_tc_select_nodes(sr_graph* g)
         n.use_tc = false;
         if (n.is_input || n.dense_target || (int)v == g->info.output_node) continue;
         if (n.d.c % 8 != 0 || n.d.c < 16 || n.d.c > 1024) continue;
-        bool ok = true;
+        const long long pixels = (long long)g->batch * n.d.h * n.d.w;
+        bool ok = pixels < 1LL << 31;
         int n_blocks = 0;
         for (int e : n.in_edges) {
             const SrHostEdge& he = g->edges[e];
             const SrHostNode& s = g->nodes[he.d.src];
             if (he.d.kind != SR_EDGE_CONV) ok = false;
+            else if (is_stem(g, he) && pixels * ((he.K + 7) / 8) >= (1LL << 32) - (1LL << 24)) ok = false;
             else if (s.d.c % 16 != 0 && !is_stem(g, he)) ok = false;
             else if (he.k_eff > 8) ok = false;
             else n_blocks += is_stem(g, he) ? 2 : he.k_eff * he.k_eff * (s.d.c / block_k(s.d.c));

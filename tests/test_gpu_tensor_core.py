@@ -141,3 +141,24 @@ def test_gtsrb_network_variant():
     from workloads import graphs
     g = graphs.dsr(4, batch=2, frames=3, classes=43, h1_recurrence=False)
     parity.check_stepwise(g, "streaming", zero_bias=False)
+
+
+def test_a_state_of_more_than_2_31_elements():
+    # 514 samples of 128 x 128 x 256: the last samples lie beyond 32-bit element offsets; first and last ones against the oracle
+    import numpy as np
+    from oracle import frame_update as fu
+    from workloads import data
+    g = tiny("large", [Node("in", 128, 128, 1, IDENTITY), Node("a", 128, 128, 256), Node("o", 1, 1, 4, IDENTITY)],
+             [Edge(0, 1, CONV, 3, 1), Edge(1, 2, GAP_DENSE)], batch=514, frames=2)
+    assert g.batch * 128 * 128 * 256 > 1 << 31
+    X, W, Bi = data.make_inputs(g), data.make_weights(g), data.make_biases(g, zero=False)
+    samples = [0, 511, 512, 513]
+    want = fu.rollout_spec(g, "p", X, W, Bi, samples=samples)
+    G = parity.make_graph(g, "p", "auto", 0, W, Bi)
+    assert G.info["n_tensor_core_nodes"] == 1
+    out = G.rollout([parity.to_device(g, X[0])])
+    G.sync_status()
+    assert parity.rel_err(out.cpu().numpy()[:, samples].reshape(want[2][1:].shape), want[2][1:]) <= parity.TOL["bf16"]
+    state = G.get_state(1)
+    for i, b in enumerate(samples):
+        assert parity.rel_err(state[b].float().cpu().numpy(), want[1][2][i]) <= parity.TOL["bf16"], b
