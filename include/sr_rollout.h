@@ -187,7 +187,8 @@ sr_status sr_graph_set_node_bias(sr_graph* g, int node, const float* bias_host);
  *                  shared-memory barrier, on a descriptor queue) gives up; the kernel then records an error, waits
  *                  for its own copies in flight, frees its tensor memory and returns, and sr_graph_sync_status
  *                  reports SR_ERR_TIMEOUT.  0 is a test hook: every tensor-core launch reports the error at once and
- *                  returns before it touches a barrier, a copy or an MMA.  May be set at any time.
+ *                  returns before it touches a barrier, a copy or an MMA.  May be set at any time; holds for a bound
+ *                  window as well.
  *           key 11 "tile pairs" (0, 1, 2) and key 12 "staged boxes in the weight ring" (0, 1, 2): accepted for the callers
  *                  that set them, without effect any more: the library chooses the columns of a tile that share their
  *                  weights, and the activation ring takes boxes of any size.
@@ -265,7 +266,7 @@ sr_status sr_graph_launch_count(const sr_graph* g, int64_t* n);
 /* Sum of the event-timed durations (milliseconds) and the number of tensor-core group launches and resident
  * launches since the previous call (option key 5); waits for those launches to finish. */
 sr_status sr_graph_kernel_time(sr_graph* g, double* ms, int64_t* launches);
-/* Synchronises `stream` and reports SR_ERR_CUDA / SR_ERR_TIMEOUT if queued work failed.  A recorded time-out stays
+/* Synchronises `stream` and reports SR_ERR_CUDA / SR_ERR_TIMEOUT if queued work failed, a bound window's included.  A recorded time-out stays
  * recorded, and is reported by every later call, until sr_graph_reset starts the rollout over. */
 sr_status sr_graph_sync_status(sr_graph* g, void* stream);
 

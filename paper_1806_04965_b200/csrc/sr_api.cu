@@ -430,6 +430,7 @@ sr_status sr_graph_set_option(sr_graph* g, int key, int value)
             if (c->exec) cudaGraphExecDestroy(c->exec);
             c->exec = nullptr;
         }
+        if (g->window) g->window->opt_wait_ms = value;
         return SR_OK;
     }
     return SR_ERR_INVALID_ARG;
@@ -955,9 +956,12 @@ sr_status sr_graph_sync_status(sr_graph* g, void* stream)
     if (!g) return SR_ERR_INVALID_ARG;
     if (g->batch <= 0 || !g->ws) return SR_ERR_STATE;
     if (!cuda_ok(cudaStreamSynchronize(static_cast<cudaStream_t>(stream)))) return SR_ERR_CUDA;
-    int error = 0;
-    if (!cuda_ok(cudaMemcpy(&error, g->ws + g->r_flags.offset, sizeof(error), cudaMemcpyDeviceToHost))) return SR_ERR_CUDA;
-    if (error != 0) return SR_ERR_TIMEOUT;
+    for (const sr_graph* q : {static_cast<const sr_graph*>(g), static_cast<const sr_graph*>(g->window)}) {   // a window's launches report to its own word
+        int error = 0;
+        if (!q || !q->ws) continue;
+        if (!cuda_ok(cudaMemcpy(&error, q->ws + q->r_flags.offset, sizeof(error), cudaMemcpyDeviceToHost))) return SR_ERR_CUDA;
+        if (error != 0) return SR_ERR_TIMEOUT;
+    }
     return SR_OK;
 }
 

@@ -267,6 +267,34 @@ def test_states_after_a_deep_window():
     assert float(G.get_state(2).abs().max()) == 0.0
 
 
+def test_expired_wait_in_a_deep_window_is_reported():
+    # the host-side hook of a zero wait limit, set once the window is bound: nothing on the GPU actually waits
+    import torch
+    from oracle import frame_update as fu
+    from paper_1806_04965_b200 import SrError
+    g = graphs.dsr(2, batch=2, frames=4, h1_recurrence=False)
+    X, Wt, Bi = data.make_inputs(g), data.make_weights(g), data.make_biases(g, zero=False)
+    want = fu.rollout_spec(g, "sequential", X, Wt, Bi)
+    G = parity.make_graph(g, "sequential", "auto", 0, Wt, Bi)
+    G.bind_window(2)
+    x, o = parity.to_device(g, X[0]), G.output_node
+    G.set_option(10, 0)
+    G.reset([x[0]])
+    G.rollout_window([x[1:3]])
+    with pytest.raises(SrError) as e:
+        G.sync_status()
+    assert e.value.status == "SR_ERR_TIMEOUT"
+    G.set_option(10, 1000)
+    with pytest.raises(SrError):                        # recorded until the rollout starts over
+        G.sync_status()
+    G.reset([x[0]])
+    out = torch.empty((4,) + G.out_shape(), dtype=torch.float32, device="cuda:0")
+    for t in (0, 2):
+        G.rollout_window([x[t + 1:t + 3]], out[t:t + 2])
+    G.sync_status()
+    assert parity.rel_err(out.cpu().numpy().reshape(want[o][1:].shape), want[o][1:]) <= parity.TOL["bf16"]
+
+
 @pytest.mark.parametrize("cin,k,stride,size", [(1, 1, 1, 9), (5, 5, 1, 11), (3, 3, 2, 10), (3, 3, 4, 32), (2, 7, 1, 8), (14, 3, 3, 13)])
 def test_staged_input_edges(cin, k, stride, size):
     # receptive fields of 1 .. 126 values (filters are odd) (partial and full 16-byte chunks), windows that leave the image on every side,
