@@ -441,9 +441,10 @@ DnEngine* dn_of(const sr_graph* g) { return static_cast<DnEngine*>(g->dn); }
 
 typedef void (*DnKernel)(const DnParams, const SrFrameCtl, int);
 
-bool dn_prepare(DnKernel kernel, int cluster, int smem_bytes)
+// (The limit belongs to the kernel, not to a graph: always the same value, or a small network would lower a larger one's.)
+bool dn_prepare(DnKernel kernel, int cluster)
 {
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes) != cudaSuccess) return false;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDnSmemMax) != cudaSuccess) return false;
     if (cluster > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return false;
     return true;
 }
@@ -459,7 +460,7 @@ DnKernel dn_kernel_of(int cluster, int samples)
 int dn_clusters_held(int cluster, int samples, int smem_bytes)
 {
     DnKernel kernel = dn_kernel_of(cluster, samples);
-    if (!dn_prepare(kernel, cluster, std::max(smem_bytes, kDnMoreThanHalf))) { cudaGetLastError(); return 0; }
+    if (!dn_prepare(kernel, cluster)) { cudaGetLastError(); return 0; }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)cluster);
     cfg.blockDim = dim3((unsigned)(kDnWarps * 32));
@@ -771,7 +772,7 @@ sr_status sr_dn_launch(sr_graph* g, int T, const SrFrameCtl& init, cudaStream_t 
     const int S = E->samples;
     auto kernel = dn_kernel_of(CL, S);
     if (!E->attr_set) {
-        if (!dn_prepare(kernel, CL, E->smem_bytes)) return SR_ERR_CUDA;
+        if (!dn_prepare(kernel, CL)) return SR_ERR_CUDA;
         E->attr_set = true;
     }
     cudaLaunchConfig_t cfg{};

@@ -108,3 +108,28 @@ def test_single_steps(batch):
         assert parity.rel_err(out.cpu().numpy().reshape(want[o][1:6].shape), want[o][1:6]) <= 1e-4
         for v in range(len(g.nodes)):
             assert parity.rel_err(G.get_state(v).cpu().numpy(), want[v][5]) <= 1e-4, g.nodes[v].name
+
+
+@pytest.mark.parametrize("pattern", ["streaming", "sequential"])
+@pytest.mark.parametrize("batch", [8, 64, 128])
+def test_a_smaller_network_leaves_a_larger_one_runnable(pattern, batch):
+    # both run on the same kernels (cluster size and sequences per cluster follow from batch and pattern), whose shared-memory limit
+    # they share; the larger network runs before and after the smaller one was planned and run
+    import torch
+    from oracle import frame_update as fu
+    g, small = graphs.build("c1", batch=batch, frames=4), mlp(batch, 4)
+    X, W, Bi = data.make_inputs(g), data.make_weights(g), data.make_biases(g, zero=False)
+    samples = [0, batch - 1]
+    want = fu.rollout_spec(g, pattern, X, W, Bi, samples=samples)
+    G = parity.make_graph(g, pattern, "auto", 0, W, Bi)
+    x, o = parity.to_device(g, X[0]), G.output_node
+    for _ in range(2):
+        out = torch.empty((4,) + G.out_shape(), dtype=torch.float32, device="cuda:0")
+        G.reset([x[0]])
+        G.run([x[1:3]], out[:2])
+        for t in (3, 4):
+            G.step([x[t]], out[t - 1])
+        G.sync_status()
+        assert parity.rel_err(out.cpu().numpy()[:, samples].reshape(want[o][1:].shape), want[o][1:]) <= 1e-4
+        parity.check_run(small, pattern, samples=samples)
+        parity.check_stepwise(small, pattern, samples=samples)
