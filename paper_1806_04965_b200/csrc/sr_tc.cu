@@ -194,7 +194,9 @@ __device__ __forceinline__ bool elect_one()
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.b32 %0, 1, 0, p;\n\t}" : "=r"(p)::"memory");
     return p != 0;
 }
-// Bounded wait.  Returns false if the limit expired or another role already gave up.
+// Bounded wait.  Returns false if the limit expired or another role already gave up.  A launch may start early, while a run of many
+// frames before it is still on; the limit must not count that time, so every role waits for the predecessor ahead of its first
+// bounded wait that depends, through whatever other role, on the predecessor.
 __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long limit)
 {
     const long long t0 = clock64();
@@ -372,6 +374,8 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
             // room in the item ring (and, for an item of the shared list, not too far ahead)
             const int ahead = own ? kItems : kAhead;
             if (it - epi_done >= ahead) {
+                if (!waited) sr_wait_for_predecessor();    // (the epilogue does; see mbar_wait_slow)
+                waited = true;
                 const long long t0 = clock64();
                 while (ok && it - epi_done >= ahead) {
                     if (*abortp || clock64() - t0 > wait_limit) ok = false;
@@ -400,6 +404,10 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                     for (int q = 1; q < kTables; ++q) {
                         const int gq = __shfl_sync(0xffffffffu, slot_gen, q);
                         if (gq < oldest) { oldest = gq; slot = q; }
+                    }
+                    if (epi_done <= oldest && !waited) {
+                        sr_wait_for_predecessor();
+                        waited = true;
                     }
                     const long long t0 = clock64();
                     while (ok && epi_done <= oldest) {
@@ -434,8 +442,13 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
         if (elect_one()) {
             uint32_t n = 0, s = 0, ph = 1;                        // copies started; next slot, parity of its release
             const uint32_t n_w = (uint32_t)P.n_w, w_slot = (uint32_t)P.w_slot;
-            bool ok = true;
+            bool ok = true, waited = false;
             for (int it = 0; ok; ++it) {
+                // (the first item and the first n_w slots come without the predecessor, the rest is up to the issuer and the epilogue)
+                if (it > 0 && !waited && !mbar_test_wait(bar_item + 8 * (it & (kItems - 1)), (it / kItems) & 1)) {
+                    sr_wait_for_predecessor();
+                    waited = true;
+                }
                 ok = mbar_wait(bar_item + 8 * (it & (kItems - 1)), (it / kItems) & 1, abortp, wait_limit);
                 if (!ok) break;
                 const TcTile& tl = items[it & (kItems - 1)];
@@ -452,6 +465,10 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                     int blk = 0;
                     for (; gi < end; ++gi) {
                         const uint32_t two = R.map1 == R.map2 ? 0u : (nd->pairs[gi >> 5] >> (gi & 31)) & 1u;
+                        if (n == n_w && !waited) {
+                            sr_wait_for_predecessor();
+                            waited = true;
+                        }
                         ok = mbar_wait(bar_wempty + 8 * s, ph, abortp, wait_limit);
                         if (!ok) break;
                         mbar_expect_tx(bar_wfull + 8 * s, bytes << two);
@@ -587,6 +604,7 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                 const uint32_t acc = (uint32_t)it & 1u, d0 = tmem_base + acc * kMaxCols, d1 = d0 + lane_cols;
                 Burst c;
                 decode(tab[0], tab[1], c);
+                if (it == 0) sr_wait_for_predecessor();
                 ok = mbar_wait(bar_tempty + 8 * acc, (((uint32_t)it >> 1) & 1u) ^ 1u, abortp, wait_limit);
                 if (!ok) break;
                 tc_fence_after();                                     // the accumulator was just handed back

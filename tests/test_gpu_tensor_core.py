@@ -162,3 +162,30 @@ def test_a_state_of_more_than_2_31_elements():
     state = G.get_state(1)
     for i, b in enumerate(samples):
         assert parity.rel_err(state[b].float().cpu().numpy(), want[1][2][i]) <= parity.TOL["bf16"], b
+
+
+@pytest.mark.parametrize("name,kw", [("c3", dict(batch=40, frames=2, size=16)), ("c4", dict(batch=3, frames=2, size=16))])
+def test_the_wait_limit_does_not_count_the_run_before(name, kw):
+    # a launch that starts early, beside a run of another graph that takes far longer (4000 frames of the resident kernel, some 15 ms)
+    # than the limit of its own waits (1 ms); c4 has more nodes than a CTA keeps tables, c3 several work items per CTA
+    import torch
+    from oracle import frame_update as fu
+    from workloads import data
+    long = build("c2", batch=8, frames=1)
+    L = parity.make_graph(long, "streaming", "auto", 0, data.make_weights(long), data.make_biases(long))
+    assert L.info["resident_cluster"] > 0
+    xl = torch.zeros((4001, 8, 28, 28, 1), dtype=torch.bfloat16, device="cuda:0")
+    g = build(name, **kw)
+    X, W, Bi = data.make_inputs(g), data.make_weights(g), data.make_biases(g, zero=False)
+    samples = [0, g.batch - 1]
+    want = fu.rollout_spec(g, "streaming", X, W, Bi, samples=samples)
+    G = parity.make_graph(g, "streaming", "auto", 0, W, Bi, wait_limit_ms=1)
+    x, o = parity.to_device(g, X[0]), G.output_node
+    out = torch.empty((2,) + G.out_shape(), dtype=torch.float32, device="cuda:0")
+    L.reset([xl[0]])
+    G.reset([x[0]])
+    for t in (1, 2):
+        L.run([xl[1:]])
+        G.step([x[t]], out[t - 1])
+        G.sync_status()
+    assert parity.rel_err(out.cpu().numpy()[:, samples].reshape(want[o][1:].shape), want[o][1:]) <= parity.TOL["bf16"]
