@@ -81,6 +81,12 @@ struct SrFrameArgs {
 //            start only after its own wait, so everything before the group is complete when a beside kernel starts; it does its
 //            work at once and ONE of its blocks waits for its predecessor at the end, so that it completes after the main kernel
 //            and whoever waits for it has waited for both.
+// What the blocks of a beside kernel that never wait rely on: the programming model promises visibility to whoever executes
+// griddepcontrol.wait, and none of them does.  They read what kernels ahead of the main one wrote.  Those had completed, with
+// their writes performed for the whole device, when the main kernel's wait returned; every block of the main kernel signals
+// after that wait, and a beside kernel starts only once all of them have.  So the values stand in L2 when it starts, and what is
+// left is a line that its SM's L1 may hold from an earlier frame: the fence at its start (an acquire at device scope) drops
+// those.  Nothing of it is read through the non-coherent path but weights, which only the host writes.
 // (Before, a second stream joined by events carried the beside kernels; measured on B200 the fork and join cost 1-3 us per frame
 // on the GPU and four calls on the host.)
 struct SrFollow {
@@ -94,6 +100,7 @@ __device__ __forceinline__ void sr_begin(int follow_flags)
 {
     if (!(follow_flags & 2)) sr_let_successor_start();
     if (!(follow_flags & 1)) sr_wait_for_predecessor();
+    else __threadfence();
     if (follow_flags & 2) sr_let_successor_start();
 }
 __device__ __forceinline__ void sr_end(int follow_flags)
