@@ -477,7 +477,7 @@ sr_status sr_graph_bind_workspace(sr_graph* g, void* workspace_dev, size_t bytes
         d.first_edge = pos;
         d.n_edges = (int)n.in_edges.size();
         d.is_output = v == g->info.output_node;
-        d.input_slot = n.input_slot;
+        d.untiled = sr_direct_untiled(g, v);
         for (int e : n.in_edges) {
             const SrHostEdge& he = g->edges[e];
             const SrHostNode& s = g->nodes[he.d.src];

@@ -29,7 +29,7 @@ struct SrDevNode {
     int32_t H, W, C, act;
     int32_t first_edge, n_edges;     // range in the SrDevEdge table
     int32_t is_output;
-    int32_t input_slot;              // >= 0 for input nodes: index into SrFrameCtl::in_base
+    int32_t untiled;                 // conv nodes: 1 if conv_item takes them
 };
 
 // One block's work in a grouped direct launch.
@@ -37,7 +37,7 @@ struct SrDirectItem {
     int32_t node;        // index into the SrDevNode table
     int32_t b0;          // first sample (dense nodes: sample chunk); its complement: four pixels per thread (conv_tile)
     int32_t p0;          // first pixel (conv nodes) or first output channel (dense nodes)
-    int32_t pad_;        // conv nodes: first channel | log2(channel quads per block) << 24, or -1 (conv_item)
+    int32_t pad_;        // conv nodes on conv_tile: first channel | log2(channel quads per block) << 24
 };
 
 // Dense / mean-dense nodes as the head kernels see them: passed as kernel parameters.

@@ -8,6 +8,7 @@ int sr_launch_direct_group(const sr_graph* g, int group, SrFollow how, cudaStrea
 int sr_launch_input(const sr_graph* g, const SrFrameArgs& fr, unsigned copies, unsigned stems_R, SrFollow how, const SrRegion* clear, cudaStream_t s);
 void sr_launch_set_ctl(const sr_graph* g, const SrFrameCtl& v, cudaStream_t s);
 void sr_launch_advance(const sr_graph* g, int n, cudaStream_t s);
+bool sr_direct_untiled(const sr_graph* g, int v);
 void sr_direct_conv_items(const sr_graph* g, int v, std::vector<SrDirectItem>& items);
 int sr_direct_dense_outputs_per_block();
 int sr_direct_dense_samples_per_block();
