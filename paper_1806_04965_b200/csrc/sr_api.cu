@@ -138,7 +138,7 @@ sr_status plan(sr_graph* g)
             const SrHostNode& n = g->nodes[v];
             if (n.use_tc) continue;
             if (n.dense_target) {
-                if (sr_head_takes(g, v)) {
+                if (sr_head_class(g, v) != 0) {
                     g->group_head_nodes[gi].push_back(v);
                 } else {
                     for (int b0 = 0; b0 < g->batch; b0 += dsb)
@@ -219,7 +219,7 @@ int enqueue_frames(sr_graph* g, const SrFrameArgs& fr, int frames, cudaStream_t 
         const bool feeds = g->input_feeds_same_frame;
         for (int gi = 0; gi < (int)g->groups.size(); ++gi) {
             // up to four independent launches: one of them leads, the others run beside it
-            const bool has_heads = !g->group_heads[gi].empty(), has_items = g->group_item_count[gi] > 0, has_tc = sr_tc_group_has_work(g, gi);
+            const bool has_heads = !g->group_head_nodes[gi].empty(), has_items = g->group_item_count[gi] > 0, has_tc = sr_tc_group_has_work(g, gi);
             const bool heads_lead = !has_tc && !has_items;
             const bool merged = gi == 0 && has_heads && (heads_lead || !feeds) && sr_heads_take_input(g, gi, g->frame, copies, stems_R);
             if (gi == 0 && feeds && !merged) launches += sr_launch_input(g, g->frame, copies, stems_R, follow(false, false), nullptr, s);
@@ -500,30 +500,11 @@ sr_status sr_graph_bind_workspace(sr_graph* g, void* workspace_dev, size_t bytes
                             cudaMemcpyHostToDevice)))
         return SR_ERR_CUDA;
     g->group_heads.assign(g->groups.size(), {});
-    for (size_t gi = 0; gi < g->groups.size(); ++gi)
-        for (int v : g->group_head_nodes[gi]) {
-            const SrHostNode& n = g->nodes[v];
-            SrHeadNode h{};
-            h.state[0] = ws + n.state[0].offset;
-            h.state[1] = ws + n.state[1].offset;
-            h.bias = reinterpret_cast<const float*>(ws + n.bias.offset);
-            h.C = n.d.c; h.act = n.d.act;
-            h.is_output = v == g->info.output_node;
-            for (int e : n.in_edges) {
-                const SrHostEdge& he = g->edges[e];
-                const SrHostNode& s = g->nodes[he.d.src];
-                SrHeadEdge& x = h.edges[h.n_edges++];
-                x.src[0] = ws + s.state[0].offset;
-                x.src[1] = ws + s.state[1].offset;
-                x.w = reinterpret_cast<const float*>(ws + he.w_direct.offset);
-                x.HW = s.d.h * s.d.w; x.Cs = s.d.c; x.kind = he.d.kind; x.R = he.R; x.K = he.K;
-                x.slot = s.input_slot;
-                h.has_mean |= he.d.kind == SR_EDGE_MEAN_DENSE;
-            }
-            g->group_heads[gi].push_back(h);
-        }
+    g->group_wide.assign(g->groups.size(), {});
+    g->group_wide_edges.assign(g->groups.size(), {});
     g->stems.clear();
     g->ws = ws;
+    for (size_t gi = 0; gi < g->groups.size(); ++gi) sr_describe_heads(g, (int)gi);
     st = sr_tc_bind(g);
     if (st == SR_OK && g->info.n_tensor_core_nodes > 0 && (!sr_input_share_sm() || !sr_direct_share_sm())) st = SR_ERR_CUDA;
     if (st == SR_OK) st = sr_rs_bind(g);

@@ -6,6 +6,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "sr_input.cuh"
 #include "sr_kernels.h"
 
@@ -406,8 +408,10 @@ __global__ void __launch_bounds__(kHeadThreads) sr_head_kernel(const __grid_cons
     sr_end(P.follow);
 }
 
-// Nodes with a mean-dense edge: a block takes one sample.  First the means of the sources (groups of Cs / 4 threads share the
-// pixels, the groups' sums are added in group order), then every warp takes outputs by itself.
+// Nodes with a mean-dense edge: a block takes one sample and mean_q outputs per warp (see sr_head_mean_outputs).  First the means of
+// the sources (groups of Cs / 4 threads share the pixels, the groups' sums are added in group order), then every warp takes
+// outputs by itself.  (With all outputs of a sample in one block, and dense edges read value by value, 64 channels of 8 x 8 by their
+// mean and by all 4096 values to 100 outputs took 4472 us for 16 frames of one sample, fp32, so 174.)
 template <typename T>
 __global__ void __launch_bounds__(kHeadThreads) sr_mean_head_kernel(const __grid_constant__ HeadParams P)
 {
@@ -424,7 +428,8 @@ __global__ void __launch_bounds__(kHeadThreads) sr_mean_head_kernel(const __grid
     }
     while (ni + 1 < P.n_nodes && bx >= P.first_block[ni + 1]) ++ni;
     const SrHeadNode& nd = P.nodes[ni];
-    const int b = bx - P.first_block[ni], cur = (int)((F.t + 1) & 1);
+    const int per_block = kHeadWarps * nd.mean_q, co_blocks = (nd.C + per_block - 1) / per_block, bi = bx - P.first_block[ni];
+    const int b = bi / co_blocks, o_first = (bi % co_blocks) * per_block, o_end = min(nd.C, o_first + per_block), cur = (int)((F.t + 1) & 1);
     float* const out = nd.is_output ? sr_frame_output(P.fr, F) : nullptr;
     int m_off = 0;
     for (int ei = 0; ei < nd.n_edges; ++ei) {
@@ -454,7 +459,7 @@ __global__ void __launch_bounds__(kHeadThreads) sr_mean_head_kernel(const __grid
         __syncthreads();
         m_off += e.Cs;
     }
-    for (int o = warp; o < nd.C; o += kHeadWarps) {
+    for (int o = o_first + warp; o < o_end; o += kHeadWarps) {
         float a = 0.f;
         m_off = 0;
         for (int ei = 0; ei < nd.n_edges; ++ei) {
@@ -469,13 +474,151 @@ __global__ void __launch_bounds__(kHeadThreads) sr_mean_head_kernel(const __grid
                 m_off += e.Cs;
             } else {
                 const T* x = head_source<T>(P, F, e) + (size_t)b * e.K;
+                if ((e.K & 3) == 0) {
 #pragma unroll 4
-                for (int k = lane; k < e.K; k += 32) a = fmaf(__ldg(w + k), to_f(x[k]), a);
+                    for (int k = 4 * lane; k < e.K; k += 128) {
+                        float v[4];
+                        load4(x + k, v);
+                        const float4 q = __ldg(reinterpret_cast<const float4*>(w + k));
+                        a = fmaf(q.x, v[0], a); a = fmaf(q.y, v[1], a); a = fmaf(q.z, v[2], a); a = fmaf(q.w, v[3], a);
+                    }
+                } else {
+#pragma unroll 4
+                    for (int k = lane; k < e.K; k += 32) a = fmaf(__ldg(w + k), to_f(x[k]), a);
+                }
             }
         }
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) a += __shfl_xor_sync(0xffffffffu, a, d);
         if (lane == 0) {
+            float z = a + nd.bias[o];
+            if (nd.act == 1) z = fmaxf(z, 0.f);
+            from_f(static_cast<T*>(nd.state[cur]) + (size_t)b * nd.C + o, z);
+            if (out) out[(size_t)b * nd.C + o] = z;
+        }
+    }
+    sr_end(P.follow);
+}
+
+// Dense nodes that the two kernels above do not take: a mean-dense edge whose channels are no multiple of four or lie beyond kHeadMaxC
+// with those of the node's other ones, or more than SR_HEAD_EDGES edges.  A block takes one sample and one or up to Q = kWideQ outputs
+// per warp, whose weight rows are loaded side by side; edge by edge, a mean-dense one in pieces of kHeadMaxC channels: first the means
+// of the piece (groups of threads share the pixels, the groups' sums are added in group order), then their products.
+// Measured on B200, us per 16 frames, on dense_item (a warp per output and eight samples) -> here: means of 2 x 768 channels of 4 x 4
+// to 100 outputs at 8 samples 7820 -> 249; mean of 10 channels of 32 x 32 to 10 outputs at 32 samples 3709 -> 133; eight
+// means of 64 channels of 8 x 8 to 10 outputs at 8 samples 4433 -> 233.
+constexpr int kWideQ = 8;
+
+struct WideParams {
+    SrFrameArgs fr;
+    int32_t n_nodes, B, follow;
+    int32_t first_block[SR_WIDE_NODES + 1];
+    SrWideNode nodes[SR_WIDE_NODES];
+    SrHeadEdge edges[SR_WIDE_EDGES];
+};
+static_assert(sizeof(WideParams) <= 4000, "kernel parameters");
+
+// Adds w[row q * kHeadWarps] . x over n values, spread over the lanes, to acc[q] of the warp's n_q outputs.
+template <int Q, typename X>
+__device__ __forceinline__ void wide_dot(float (&acc)[Q], const float* w, size_t row, const X* x, int n, int n_q, bool vec, int lane)
+{
+    if (vec) {
+#pragma unroll(Q == 1 ? 8 : 2)
+        for (int k = 4 * lane; k < n; k += 128) {
+            float xv[4];
+            load4(x + k, xv);
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                if (q >= n_q) break;
+                const float4 wv = __ldg(reinterpret_cast<const float4*>(w + q * kHeadWarps * row + k));
+                acc[q] = fmaf(wv.x, xv[0], acc[q]); acc[q] = fmaf(wv.y, xv[1], acc[q]);
+                acc[q] = fmaf(wv.z, xv[2], acc[q]); acc[q] = fmaf(wv.w, xv[3], acc[q]);
+            }
+        }
+    } else {
+#pragma unroll 4
+        for (int k = lane; k < n; k += 32) {
+            const float xv = to_f(x[k]);
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                if (q >= n_q) break;
+                acc[q] = fmaf(__ldg(w + q * kHeadWarps * row + k), xv, acc[q]);
+            }
+        }
+    }
+}
+
+template <typename T, int Q>
+__global__ void __launch_bounds__(kHeadThreads) sr_wide_head_kernel(const __grid_constant__ WideParams P)
+{
+    __shared__ __align__(16) float mean[kHeadMaxC];
+    __shared__ __align__(16) float part[4 * kHeadThreads];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    sr_begin(P.follow);
+    const SrFrame F = sr_frame(P.fr);
+    int ni = 0;
+    while (ni + 1 < P.n_nodes && (int)blockIdx.x >= P.first_block[ni + 1]) ++ni;
+    const SrWideNode& nd = P.nodes[ni];
+    const int per_block = kHeadWarps * nd.q, co_blocks = (nd.C + per_block - 1) / per_block, bi = (int)blockIdx.x - P.first_block[ni];
+    const int b = bi / co_blocks, o0 = (bi % co_blocks) * per_block + warp, o_end = min(nd.C, (bi % co_blocks + 1) * per_block);
+    const int n_q = o0 < o_end ? (o_end - o0 + kHeadWarps - 1) / kHeadWarps : 0;       // outputs o0 + kHeadWarps * q
+    const int prev = (int)(F.t & 1), cur = prev ^ 1;
+    float* const out = nd.is_output ? sr_frame_output(P.fr, F) : nullptr;
+    float acc[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) acc[q] = 0.f;
+    for (int ei = 0; ei < nd.n_edges; ++ei) {
+        const SrHeadEdge& e = P.edges[nd.first_edge + ei];
+        const T* src = static_cast<const T*>(e.src[e.R ? prev : cur]) + (size_t)b * e.HW * e.Cs;
+        const float* w = e.w + (size_t)o0 * e.K;
+        const bool vec = (e.K & 3) == 0;
+        if (e.kind != SR_EDGE_MEAN_DENSE) {
+            wide_dot(acc, w, e.K, src, e.K, n_q, vec, lane);
+            continue;
+        }
+        const float inv = 1.f / (float)e.HW;
+        for (int c0 = 0; c0 < e.Cs; c0 += kHeadMaxC) {
+            const int n = min(kHeadMaxC, e.Cs - c0), cols = vec ? n / 4 : n, groups = max(1, kHeadThreads / cols);
+            if (tid < groups * cols) {
+                const int grp = tid / cols;
+                for (int col = tid % cols; col < cols; col += kHeadThreads) {      // (more than one round: more columns than threads)
+                    if (vec) {
+                        float s4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+                        for (int px = grp; px < e.HW; px += groups) {
+                            float x[4];
+                            load4(src + c0 + 4 * col + (size_t)px * e.Cs, x);
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) s4[q] += x[q];
+                        }
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) part[grp * n + 4 * col + q] = s4[q];
+                    } else {
+                        float s1 = 0.f;
+#pragma unroll 8
+                        for (int px = grp; px < e.HW; px += groups) s1 += to_f(src[c0 + col + (size_t)px * e.Cs]);
+                        part[grp * n + col] = s1;
+                    }
+                }
+            }
+            __syncthreads();
+            for (int c = tid; c < n; c += kHeadThreads) {
+                float m = 0.f;
+                for (int gq = 0; gq < groups; ++gq) m += part[gq * n + c];
+                mean[c] = m * inv;
+            }
+            __syncthreads();
+            wide_dot(acc, w + c0, e.K, mean, n, n_q, vec, lane);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        if (q >= n_q) break;
+        float a = acc[q];
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) a += __shfl_xor_sync(0xffffffffu, a, d);
+        if (lane == 0) {
+            const int o = o0 + q * kHeadWarps;
             float z = a + nd.bias[o];
             if (nd.act == 1) z = fmaxf(z, 0.f);
             from_f(static_cast<T*>(nd.state[cur]) + (size_t)b * nd.C + o, z);
@@ -538,9 +681,23 @@ int sr_launch_direct_group(const sr_graph* g, int group, SrFollow how, cudaStrea
 // more blocks and keeps four steps of the reduction in flight.
 static bool head_wide(const sr_graph* g) { return g->batch >= 16; }
 
+// Outputs per warp of a node with a mean-dense edge (at most `most`): few, because a warp takes them one after the other, as long as
+// the blocks number 500 at most, from where on they queue and every one computes the sample's means again; a batch that has a
+// block for every SM anyway does not part two outputs.  Measured on B200, us per 16 frames with 1 / 2 / 3 / 8 / 16 outputs per
+// warp and with all: 256 channels of 8 x 8 to 1000 outputs at one sample 92 / 104 / 115 / 179 / 280 / 1617, at 32 samples 466 /
+// 311 / 258 / 230 / 324 / 1710 (this rule: 9); 32 channels of 16 x 16 to 43 outputs at 8 samples 75 / 85 / 96 / 125 with six, at
+// 128 samples 131 / 111 / 113 / 140; 256 channels of 8 x 8 to 10 outputs at 256 samples, fp32, 311 / 300.
+static int head_mean_outputs(const sr_graph* g, int channels, int most)
+{
+    const int all = (channels + kHeadWarps - 1) / kHeadWarps;
+    int q = g->batch >= 148 ? std::min(2, all) : 1;
+    while (q < all && q < most && (long long)g->batch * ((channels + kHeadWarps * q - 1) / (kHeadWarps * q)) > 500) ++q;
+    return q;
+}
+
 static int head_blocks(const sr_graph* g, const SrHeadNode& h)
 {
-    if (h.has_mean) return g->batch;
+    if (h.has_mean) return g->batch * ((h.C + kHeadWarps * h.mean_q - 1) / (kHeadWarps * h.mean_q));
     const int S = head_wide(g) ? 4 : 1, CO = head_wide(g) ? 8 : 2;
     return (g->batch + S - 1) / S * ((h.C + CO - 1) / CO);
 }
@@ -552,7 +709,7 @@ bool sr_heads_take_input(const sr_graph* g, int group, const SrFrameArgs& fr, un
 {
     const std::vector<SrHeadNode>& heads = g->group_heads[group];
     const std::vector<const SrStem*> stems = sr_stems(g, stems_R);
-    if (heads.empty() || heads.size() > SR_HEAD_NODES || stems.size() > kStemsPerLaunch) return false;
+    if (heads.empty() || heads.size() > SR_HEAD_NODES || !g->group_wide[group].empty() || stems.size() > kStemsPerLaunch) return false;
     int blocks = 0, mean = 0;
     for (const SrHeadNode& h : heads) {
         blocks += head_blocks(g, h);
@@ -616,6 +773,34 @@ int sr_launch_heads(const sr_graph* g, int group, bool with_input, unsigned copi
         }
         flush();
     }
+    for (int few = 0; few < 2; ++few) {                                      // 1: nodes of one output per warp
+        WideParams P;
+        P.fr = g->frame;
+        P.B = g->batch;
+        P.n_nodes = 0;
+        int blocks = 0, n_edges = 0;
+        auto flush = [&]() {
+            if (P.n_nodes == 0) return;
+            P.follow = how.flags();
+            auto kernel = [&](auto q) { return g->dtype == SR_DTYPE_BF16 ? sr_wide_head_kernel<__nv_bfloat16, q> : sr_wide_head_kernel<float, q>; };
+            sr_launch(few ? kernel(std::integral_constant<int, 1>()) : kernel(std::integral_constant<int, kWideQ>()), blocks, kHeadThreads, 0, s, how.early, P);
+            ++launches;
+            how.early = true;
+            P.n_nodes = blocks = n_edges = 0;
+        };
+        for (const SrWideNode& h : g->group_wide[group]) {
+            if ((h.q == 1) != (few == 1)) continue;
+            if (P.n_nodes == SR_WIDE_NODES || n_edges + h.n_edges > SR_WIDE_EDGES) flush();
+            std::copy_n(g->group_wide_edges[group].begin() + h.first_edge, h.n_edges, P.edges + n_edges);
+            P.nodes[P.n_nodes] = h;
+            P.nodes[P.n_nodes].first_edge = n_edges;
+            P.first_block[P.n_nodes++] = blocks;
+            n_edges += h.n_edges;
+            blocks += g->batch * ((h.C + kHeadWarps * h.q - 1) / (kHeadWarps * h.q));
+            P.first_block[P.n_nodes] = blocks;
+        }
+        flush();
+    }
     return launches;
 }
 
@@ -656,25 +841,71 @@ void sr_direct_conv_items(const sr_graph* g, int v, std::vector<SrDirectItem>& i
 int sr_direct_dense_outputs_per_block() { return kWarps; }
 int sr_direct_dense_samples_per_block() { return kDenseB; }
 
-// Can the head kernels take the node?
-bool sr_head_takes(const sr_graph* g, int v)
+// Which head kernel takes the node: 1: sr_head_kernel or sr_mean_head_kernel, 2: sr_wide_head_kernel, 0: none.
+int sr_head_class(const sr_graph* g, int v)
 {
     const SrHostNode& n = g->nodes[v];
-    if (n.in_edges.size() > SR_HEAD_EDGES) return false;
+    if (n.in_edges.size() > SR_WIDE_EDGES) return 0;
     int channels = 0;
     for (int e : n.in_edges) {
         const SrHostEdge& he = g->edges[e];
         if (he.d.kind != SR_EDGE_MEAN_DENSE) continue;
         const int cs = g->nodes[he.d.src].d.c;
-        if (cs % 4 != 0) return false;
+        if (cs % 4 != 0 || cs > kHeadMaxC) return 2;
         channels += cs;
     }
-    return channels <= kHeadMaxC;
+    return n.in_edges.size() > SR_HEAD_EDGES || channels > kHeadMaxC ? 2 : 1;
+}
+
+// Fills g's lists of the group's head nodes for the workspace that is being bound.
+void sr_describe_heads(sr_graph* g, int group)
+{
+    char* const ws = g->ws;
+    for (int v : g->group_head_nodes[group]) {
+        const SrHostNode& n = g->nodes[v];
+        std::vector<SrHeadEdge> edges;
+        bool has_mean = false;
+        for (int e : n.in_edges) {
+            const SrHostEdge& he = g->edges[e];
+            const SrHostNode& s = g->nodes[he.d.src];
+            SrHeadEdge x{};
+            x.src[0] = ws + s.state[0].offset;
+            x.src[1] = ws + s.state[1].offset;
+            x.w = reinterpret_cast<const float*>(ws + he.w_direct.offset);
+            x.HW = s.d.h * s.d.w; x.Cs = s.d.c; x.kind = he.d.kind; x.R = he.R; x.K = he.K;
+            x.slot = s.input_slot;
+            has_mean |= he.d.kind == SR_EDGE_MEAN_DENSE;
+            edges.push_back(x);
+        }
+        auto describe = [&](auto& h) {
+            h.state[0] = ws + n.state[0].offset;
+            h.state[1] = ws + n.state[1].offset;
+            h.bias = reinterpret_cast<const float*>(ws + n.bias.offset);
+            h.C = n.d.c; h.act = n.d.act;
+            h.is_output = v == g->info.output_node;
+            h.n_edges = (int)edges.size();
+        };
+        if (sr_head_class(g, v) == 1) {
+            SrHeadNode h{};
+            describe(h);
+            h.has_mean = has_mean;
+            if (has_mean) h.mean_q = head_mean_outputs(g, h.C, h.C);
+            std::copy(edges.begin(), edges.end(), h.edges);
+            g->group_heads[group].push_back(h);
+        } else {
+            SrWideNode h{};
+            describe(h);
+            h.q = head_mean_outputs(g, h.C, kWideQ);
+            h.first_edge = (int)g->group_wide_edges[group].size();
+            g->group_wide_edges[group].insert(g->group_wide_edges[group].end(), edges.begin(), edges.end());
+            g->group_wide[group].push_back(h);
+        }
+    }
 }
 
 bool sr_direct_share_sm()
 {
     auto ask = [](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess; };
-    return ask(sr_head_kernel<__nv_bfloat16, 4, 8, false>) && ask(sr_head_kernel<__nv_bfloat16, 1, 2, true>) && ask(sr_mean_head_kernel<__nv_bfloat16>) &&
+    return ask(sr_head_kernel<__nv_bfloat16, 4, 8, false>) && ask(sr_head_kernel<__nv_bfloat16, 1, 2, true>) && ask(sr_mean_head_kernel<__nv_bfloat16>) && ask(sr_wide_head_kernel<__nv_bfloat16, 1>) && ask(sr_wide_head_kernel<__nv_bfloat16, kWideQ>) &&
            ask(sr_direct_group_kernel<__nv_bfloat16>);
 }

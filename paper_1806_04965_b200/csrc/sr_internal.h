@@ -52,8 +52,18 @@ struct SrHeadNode {
     void* state[2];
     const float* bias;
     int32_t C, act, is_output, n_edges;
-    int32_t has_mean, pad_[3];
+    int32_t has_mean, mean_q, pad_[2];       // mean_q: outputs per warp (nodes with a mean-dense edge)
     SrHeadEdge edges[SR_HEAD_EDGES];
+};
+
+// The nodes of sr_wide_head_kernel: their edges lie in one list.
+#define SR_WIDE_EDGES 48
+#define SR_WIDE_NODES 8
+struct SrWideNode {
+    void* state[2];
+    const float* bias;
+    int32_t C, act, is_output, n_edges;
+    int32_t first_edge, q;                   // q: outputs per warp
 };
 
 // What a launch needs to know about its frame.  Plain launches carry it by value; launches recorded in a CUDA graph read it
@@ -206,6 +216,8 @@ struct sr_graph {
     std::vector<int> group_item_offset;
     std::vector<std::vector<int>> group_head_nodes;       // per group: nodes of the head kernels
     std::vector<std::vector<SrHeadNode>> group_heads;     // and what they need to know about them (filled when a workspace is bound)
+    std::vector<std::vector<SrWideNode>> group_wide;
+    std::vector<std::vector<SrHeadEdge>> group_wide_edges;
     // dynamic state
     SrFrameArgs frame{};                           // of the launches being queued
     int64_t t = 0;

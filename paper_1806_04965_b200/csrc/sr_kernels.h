@@ -12,7 +12,8 @@ bool sr_direct_untiled(const sr_graph* g, int v);
 void sr_direct_conv_items(const sr_graph* g, int v, std::vector<SrDirectItem>& items);
 int sr_direct_dense_outputs_per_block();
 int sr_direct_dense_samples_per_block();
-bool sr_head_takes(const sr_graph* g, int v);
+int sr_head_class(const sr_graph* g, int v);
+void sr_describe_heads(sr_graph* g, int group);
 // The heads of a group; with_input: the frame input goes with them (copies, stems_R as for sr_launch_input).
 bool sr_heads_take_input(const sr_graph* g, int group, const SrFrameArgs& fr, unsigned copies, unsigned stems_R);
 int sr_launch_heads(const sr_graph* g, int group, bool with_input, unsigned copies, unsigned stems_R, SrFollow how, cudaStream_t s);      // returns launches queued

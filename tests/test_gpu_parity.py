@@ -237,6 +237,28 @@ def test_heads_at_the_edges_of_their_blocks(batch, c_mid, c_out, dtype):
         parity.check_stepwise(g, p, zero_bias=False, resident=False)
 
 
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("batch,classes", [(1, 1), (1, 300), (3, 65), (37, 17), (150, 9), (150, 41)])
+def test_mean_heads_in_several_blocks(batch, classes, dtype):
+    # blocks of 8, 16, ... outputs with a ragged last one.  m: two means and a dense edge of K % 4 == 0; s: a dense edge of odd K;
+    # w1: channels that are no multiple of four, fewer and more than threads; w2: more channels than a block's means, alone and
+    # beside others; w3: more than six edges, dense and mean.  R = 0 edges read the frame's own input.
+    from workloads.graphs import CONV, DENSE, GAP_DENSE, IDENTITY, Edge, GraphSpec, Node, check_shapes
+    nodes = [Node("in", 4, 4, 12, IDENTITY), Node("odd", 3, 3, 9, IDENTITY), Node("wide", 2, 2, 1028, IDENTITY), Node("m", 1, 1, classes),
+             Node("s", 1, 1, 5), Node("w1", 1, 1, classes), Node("w2", 1, 1, classes, IDENTITY), Node("w3", 1, 1, classes), Node("big", 1, 1, 301),
+             Node("w4", 1, 1, 6, IDENTITY), Node("o", 1, 1, 3, IDENTITY)]
+    edges = [Edge(0, 3, GAP_DENSE), Edge(0, 3, DENSE), Edge(0, 3, GAP_DENSE), Edge(0, 4, GAP_DENSE), Edge(1, 4, DENSE), Edge(1, 5, GAP_DENSE),
+             Edge(0, 5, GAP_DENSE), Edge(2, 6, GAP_DENSE), Edge(1, 6, GAP_DENSE)]
+    edges += [Edge(i % 2, 7, GAP_DENSE if i % 3 else DENSE) for i in range(9)]
+    edges += [Edge(0, 8, DENSE), Edge(8, 9, GAP_DENSE), Edge(2, 9, DENSE)] + [Edge(v, 10, DENSE) for v in (3, 4, 5, 6, 7, 9)]
+    g = GraphSpec("heads", nodes, edges, batch=batch, frames=3, dtype=dtype, seed=89)
+    check_shapes(g)
+    g.patterns = {"p": [1] * len(edges), "q": [i % 2 for i in range(len(edges))]}
+    for p in g.patterns:
+        parity.check_stepwise(g, p, zero_bias=False, resident=False, samples=[0, batch - 1])
+        parity.check_run(g, p, graph_frames=2, resident=False, samples=[0, batch - 1])
+
+
 def test_states_after_a_deep_window():
     # the states a window leaves behind can be read, replaced one by one, and are superseded by the next update
     import torch
