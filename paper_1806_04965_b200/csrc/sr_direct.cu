@@ -30,6 +30,30 @@ __device__ __forceinline__ void load4(const __nv_bfloat16* p, float (&v)[4])
     v[2] = __uint_as_float(q.y << 16); v[3] = __uint_as_float(q.y & 0xFFFF0000u);
 }
 
+// One value, or four, of a state; BESIDE: past L1 (see SrFollow).
+template <bool BESIDE>
+__device__ __forceinline__ float head_load1(const float* p) { return BESIDE ? sr_load_past_l1(p) : *p; }
+template <bool BESIDE>
+__device__ __forceinline__ float head_load1(const __nv_bfloat16* p)
+{
+    return BESIDE ? __uint_as_float((uint32_t)sr_load_past_l1(reinterpret_cast<const unsigned short*>(p)) << 16) : to_f(*p);
+}
+template <bool BESIDE>
+__device__ __forceinline__ void head_load4(const float* p, float (&v)[4])
+{
+    if (!BESIDE) return load4(p, v);
+    const float4 q = sr_load_past_l1(reinterpret_cast<const float4*>(p));
+    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+}
+template <bool BESIDE>
+__device__ __forceinline__ void head_load4(const __nv_bfloat16* p, float (&v)[4])
+{
+    if (!BESIDE) return load4(p, v);
+    const uint2 q = sr_load_past_l1(reinterpret_cast<const uint2*>(p));
+    v[0] = __uint_as_float(q.x << 16); v[1] = __uint_as_float(q.x & 0xFFFF0000u);
+    v[2] = __uint_as_float(q.y << 16); v[3] = __uint_as_float(q.y & 0xFFFF0000u);
+}
+
 __device__ __forceinline__ void store4(float* p, const float (&v)[4]) { *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]); }
 __device__ __forceinline__ void store4(__nv_bfloat16* p, const float (&v)[4])
 {
@@ -309,7 +333,7 @@ __device__ __forceinline__ const T* head_source(const HeadParams& P, const SrFra
 // Nodes with dense edges only: a block takes CO outputs of S samples; its threads stride over the reduction index in vectors
 // of four, every thread keeps S x CO partial sums (a weight vector serves S samples).  The sums of a warp meet by halving,
 // those of the warps in shared memory in a fixed order.
-template <typename T, int S, int CO, bool WithInput>
+template <typename T, int S, int CO, bool WithInput, bool BESIDE>
 __global__ void __launch_bounds__(kHeadThreads) sr_head_kernel(const __grid_constant__ HeadParams P)
 {
     __shared__ float red[kHeadWarps][32];
@@ -319,7 +343,7 @@ __global__ void __launch_bounds__(kHeadThreads) sr_head_kernel(const __grid_cons
     const SrFrame F = sr_frame(P.fr);
     int bx = (int)blockIdx.x, ni = 0;
     if (WithInput && (bx -= P.in.n_blocks) < 0) {
-        sr_input_block(P.in, P.fr, F, (int)blockIdx.x, tap);
+        sr_input_block<BESIDE>(P.in, P.fr, F, (int)blockIdx.x, tap);
         sr_end(P.follow);
         return;
     }
@@ -349,7 +373,7 @@ __global__ void __launch_bounds__(kHeadThreads) sr_head_kernel(const __grid_cons
                 float4 wv[CO];
                 float xv[S][4];
 #pragma unroll
-                for (int s = 0; s < S; ++s) load4(x[s] + k, xv[s]);
+                for (int s = 0; s < S; ++s) head_load4<BESIDE>(x[s] + k, xv[s]);
 #pragma unroll
                 for (int o = 0; o < CO; ++o) wv[o] = __ldg(reinterpret_cast<const float4*>(w[o] + k));
 #pragma unroll
@@ -366,7 +390,7 @@ __global__ void __launch_bounds__(kHeadThreads) sr_head_kernel(const __grid_cons
                 for (int o = 0; o < CO; ++o) {
                     const float wk = __ldg(w[o] + k);
 #pragma unroll
-                    for (int s = 0; s < S; ++s) acc[s][o] = fmaf(wk, to_f(x[s][k]), acc[s][o]);
+                    for (int s = 0; s < S; ++s) acc[s][o] = fmaf(wk, head_load1<BESIDE>(x[s] + k), acc[s][o]);
                 }
         }
     }
@@ -408,11 +432,11 @@ __global__ void __launch_bounds__(kHeadThreads) sr_head_kernel(const __grid_cons
     sr_end(P.follow);
 }
 
-// Nodes with a mean-dense edge: a block takes one sample and mean_q outputs per warp (see sr_head_mean_outputs).  First the means of
+// Nodes with a mean-dense edge: a block takes one sample and mean_q outputs per warp (see head_mean_outputs).  First the means of
 // the sources (groups of Cs / 4 threads share the pixels, the groups' sums are added in group order), then every warp takes
 // outputs by itself.  (With all outputs of a sample in one block, and dense edges read value by value, 64 channels of 8 x 8 by their
 // mean and by all 4096 values to 100 outputs took 4472 us for 16 frames of one sample, fp32, so 174.)
-template <typename T>
+template <typename T, bool BESIDE>
 __global__ void __launch_bounds__(kHeadThreads) sr_mean_head_kernel(const __grid_constant__ HeadParams P)
 {
     __shared__ __align__(16) float mean[kHeadMaxC];
@@ -422,7 +446,7 @@ __global__ void __launch_bounds__(kHeadThreads) sr_mean_head_kernel(const __grid
     const SrFrame F = sr_frame(P.fr);
     int bx = (int)blockIdx.x, ni = 0;
     if ((bx -= P.in.n_blocks) < 0) {
-        sr_input_block(P.in, P.fr, F, (int)blockIdx.x, reinterpret_cast<int2*>(part));
+        sr_input_block<BESIDE>(P.in, P.fr, F, (int)blockIdx.x, reinterpret_cast<int2*>(part));
         sr_end(P.follow);
         return;
     }
@@ -442,7 +466,7 @@ __global__ void __launch_bounds__(kHeadThreads) sr_mean_head_kernel(const __grid
 #pragma unroll 8
             for (int px = grp; px < e.HW; px += groups) {
                 float x[4];
-                load4(xs + (size_t)px * e.Cs, x);
+                head_load4<BESIDE>(xs + (size_t)px * e.Cs, x);
 #pragma unroll
                 for (int q = 0; q < 4; ++q) s4[q] += x[q];
             }
@@ -478,13 +502,13 @@ __global__ void __launch_bounds__(kHeadThreads) sr_mean_head_kernel(const __grid
 #pragma unroll 4
                     for (int k = 4 * lane; k < e.K; k += 128) {
                         float v[4];
-                        load4(x + k, v);
+                        head_load4<BESIDE>(x + k, v);
                         const float4 q = __ldg(reinterpret_cast<const float4*>(w + k));
                         a = fmaf(q.x, v[0], a); a = fmaf(q.y, v[1], a); a = fmaf(q.z, v[2], a); a = fmaf(q.w, v[3], a);
                     }
                 } else {
 #pragma unroll 4
-                    for (int k = lane; k < e.K; k += 32) a = fmaf(__ldg(w + k), to_f(x[k]), a);
+                    for (int k = lane; k < e.K; k += 32) a = fmaf(__ldg(w + k), head_load1<BESIDE>(x + k), a);
                 }
             }
         }
@@ -555,6 +579,7 @@ __global__ void __launch_bounds__(kHeadThreads) sr_wide_head_kernel(const __grid
     __shared__ __align__(16) float part[4 * kHeadThreads];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     sr_begin(P.follow);
+    sr_drop_old_lines(P.follow);
     const SrFrame F = sr_frame(P.fr);
     int ni = 0;
     while (ni + 1 < P.n_nodes && (int)blockIdx.x >= P.first_block[ni + 1]) ++ni;
@@ -641,6 +666,7 @@ __global__ void __launch_bounds__(kWarps * 32) sr_direct_group_kernel(const __gr
 {
     __shared__ int2 tab[kTab];
     sr_begin(P.follow);
+    sr_drop_old_lines(P.follow);
     const SrDirectItem it = P.items[blockIdx.x];
     const SrDevNode& nd = P.nodes[it.node];
     const SrFrame F = sr_frame(P.fr);
@@ -746,18 +772,13 @@ int sr_launch_heads(const sr_graph* g, int group, bool with_input, unsigned copi
                 P.in = sr_plan_input(g, copies, sr_stems(g, stems_R), next, true);
             }
             P.follow = how.flags();
-            const bool bf = g->dtype == SR_DTYPE_BF16;
-            const int n = P.in.n_blocks + blocks;
-            if (cls == 0) {
-                if (bf) sr_launch(sr_mean_head_kernel<__nv_bfloat16>, n, kHeadThreads, 0, s, how.early, P);
-                else sr_launch(sr_mean_head_kernel<float>, n, kHeadThreads, 0, s, how.early, P);
-            } else if (wide) {
-                if (bf) sr_launch(sr_head_kernel<__nv_bfloat16, 4, 8, false>, n, kHeadThreads, 0, s, how.early, P);
-                else sr_launch(sr_head_kernel<float, 4, 8, false>, n, kHeadThreads, 0, s, how.early, P);
-            } else {
-                if (bf) sr_launch(sr_head_kernel<__nv_bfloat16, 1, 2, true>, n, kHeadThreads, 0, s, how.early, P);
-                else sr_launch(sr_head_kernel<float, 1, 2, true>, n, kHeadThreads, 0, s, how.early, P);
-            }
+            auto kernel = [&](auto beside) {
+                const bool bf = g->dtype == SR_DTYPE_BF16;
+                if (cls == 0) return bf ? sr_mean_head_kernel<__nv_bfloat16, beside> : sr_mean_head_kernel<float, beside>;
+                if (wide) return bf ? sr_head_kernel<__nv_bfloat16, 4, 8, false, beside> : sr_head_kernel<float, 4, 8, false, beside>;
+                return bf ? sr_head_kernel<__nv_bfloat16, 1, 2, true, beside> : sr_head_kernel<float, 1, 2, true, beside>;
+            };
+            sr_launch(how.beside ? kernel(std::true_type()) : kernel(std::false_type()), P.in.n_blocks + blocks, kHeadThreads, 0, s, how.early, P);
             ++launches;
             how.early = true;
             P.n_nodes = 0;
@@ -906,6 +927,10 @@ void sr_describe_heads(sr_graph* g, int group)
 bool sr_direct_share_sm()
 {
     auto ask = [](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess; };
-    return ask(sr_head_kernel<__nv_bfloat16, 4, 8, false>) && ask(sr_head_kernel<__nv_bfloat16, 1, 2, true>) && ask(sr_mean_head_kernel<__nv_bfloat16>) && ask(sr_wide_head_kernel<__nv_bfloat16, 1>) && ask(sr_wide_head_kernel<__nv_bfloat16, kWideQ>) &&
-           ask(sr_direct_group_kernel<__nv_bfloat16>);
+    auto heads = [&](auto beside) {
+        return ask(sr_head_kernel<__nv_bfloat16, 4, 8, false, beside>) && ask(sr_head_kernel<__nv_bfloat16, 1, 2, true, beside>) &&
+               ask(sr_mean_head_kernel<__nv_bfloat16, beside>);
+    };
+    return heads(std::false_type()) && heads(std::true_type()) && ask(sr_wide_head_kernel<__nv_bfloat16, 1>) &&
+           ask(sr_wide_head_kernel<__nv_bfloat16, kWideQ>) && ask(sr_direct_group_kernel<__nv_bfloat16>);
 }

@@ -16,13 +16,13 @@ struct InputParams {
 static_assert(sizeof(InputParams) <= 4000, "kernel parameters");
 
 // (Registers for six blocks per SM: three of them fit beside a CTA of the tensor-core kernel.)
-template <bool CLEAR>
+template <bool CLEAR, bool BESIDE>
 __global__ void __launch_bounds__(kInputThreads, CLEAR ? 1 : 6) sr_input_kernel(const __grid_constant__ InputParams P)
 {
     __shared__ int2 tap[128];
     sr_begin(P.follow);
     if (!CLEAR || (int)blockIdx.x < P.in.n_blocks) {
-        sr_input_block(P.in, P.fr, sr_frame(P.fr), (int)blockIdx.x, tap);
+        sr_input_block<BESIDE>(P.in, P.fr, sr_frame(P.fr), (int)blockIdx.x, tap);
     } else {
         const size_t nth = (size_t)P.clear_blocks * kInputThreads;
         for (size_t i = (size_t)((int)blockIdx.x - P.in.n_blocks) * kInputThreads + threadIdx.x; i < P.n_clear; i += nth) P.clear[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -56,7 +56,7 @@ int sr_launch_input(const sr_graph* g, const SrFrameArgs& fr, unsigned copies, u
             P.clear_blocks = (int)std::min<size_t>(148 * 6, (P.n_clear + 4 * kInputThreads - 1) / (4 * kInputThreads));
         }
         if (P.in.n_blocks + P.clear_blocks == 0) break;
-        sr_launch(P.clear_blocks ? sr_input_kernel<true> : sr_input_kernel<false>, P.in.n_blocks + P.clear_blocks, kInputThreads, 0, s, how.early, P);
+        sr_launch(P.clear_blocks ? sr_input_kernel<true, false> : how.beside ? sr_input_kernel<false, true> : sr_input_kernel<false, false>, P.in.n_blocks + P.clear_blocks, kInputThreads, 0, s, how.early, P);
         ++launches;
         how.early = true;
     } while (next < stems.size());
@@ -77,5 +77,6 @@ void sr_launch_advance(const sr_graph* g, int n, cudaStream_t s)
 // SM changes its partition only when it is empty, so with another one the tensor-core kernel waits for them to drain.
 bool sr_input_share_sm()
 {
-    return cudaFuncSetAttribute(sr_input_kernel<false>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess;
+    auto ask = [](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) == cudaSuccess; };
+    return ask(sr_input_kernel<false, false>) && ask(sr_input_kernel<false, true>);
 }

@@ -32,7 +32,8 @@ struct SrInputPart {
 };
 
 // Block bx of the input's n_blocks.  tap: 128 words of shared memory; per element of a window: offset from the (unpadded) window
-// origin; dy << 16 | dx.
+// origin; dy << 16 | dx.  BESIDE: for a launch that does not wait for the one before it (see SrFollow).
+template <bool BESIDE>
 __device__ __forceinline__ void sr_input_block(const SrInputPart& P, const SrFrameArgs& fr, const SrFrame& F, int bx, int2* tap)
 {
     const int cur = (int)((F.t + 1) & 1);
@@ -47,13 +48,17 @@ __device__ __forceinline__ void sr_input_block(const SrInputPart& P, const SrFra
         const size_t tid = (size_t)(bx - c.first_block) * kInputThreads + threadIdx.x, nth = (size_t)blocks * kInputThreads;
         if (((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0) {
             const size_t nv = c.bytes / 16;
-            for (size_t j = tid; j < nv; j += nth) reinterpret_cast<uint4*>(dst)[j] = reinterpret_cast<const uint4*>(src)[j];
+            const uint4* v = reinterpret_cast<const uint4*>(src);
+            for (size_t j = tid; j < nv; j += nth) reinterpret_cast<uint4*>(dst)[j] = BESIDE ? sr_load_past_l1(v + j) : v[j];
+            if (BESIDE && nv * 16 < c.bytes) __threadfence();
             for (size_t j = nv * 16 + tid; j < c.bytes; j += nth) dst[j] = src[j];
         } else {
+            if (BESIDE) __threadfence();
             for (size_t j = tid; j < c.bytes; j += nth) dst[j] = src[j];
         }
         return;
     }
+    if (BESIDE) __threadfence();
     int i = 0;
     while (i + 1 < P.n_stem && bx >= P.stem[i + 1].first_block) ++i;
     const SrStemPart& st = P.stem[i];

@@ -95,8 +95,10 @@ struct SrFrameArgs {
 // griddepcontrol.wait, and none of them does.  They read what kernels ahead of the main one wrote.  Those had completed, with
 // their writes performed for the whole device, when the main kernel's wait returned; every block of the main kernel signals
 // after that wait, and a beside kernel starts only once all of them have.  So the values stand in L2 when it starts, and what is
-// left is a line that its SM's L1 may hold from an earlier frame: the fence at its start (an acquire at device scope) drops
-// those.  Nothing of it is read through the non-coherent path but weights, which only the host writes.
+// left is a line that its SM's L1 may hold from an earlier frame.  What a beside kernel reads once it reads past L1
+// (sr_load_past_l1); one that reads a value many times (staging, convolutions) begins with a fence, an acquire at device scope,
+// which drops those lines (and takes 0.5 us, or 1 us beside a running main kernel).  Nothing is read through the non-coherent path
+// but weights, which only the host writes.
 // (Before, a second stream joined by events carried the beside kernels; measured on B200 the fork and join cost 1-3 us per frame
 // on the GPU and four calls on the host.)
 struct SrFollow {
@@ -110,8 +112,42 @@ __device__ __forceinline__ void sr_begin(int follow_flags)
 {
     if (!(follow_flags & 2)) sr_let_successor_start();
     if (!(follow_flags & 1)) sr_wait_for_predecessor();
-    else __threadfence();
     if (follow_flags & 2) sr_let_successor_start();
+}
+__device__ __forceinline__ void sr_drop_old_lines(int follow_flags)
+{
+    if (follow_flags & 1) __threadfence();
+}
+// (Not volatile: a beside kernel may load as early as it likes.)
+__device__ __forceinline__ float4 sr_load_past_l1(const float4* p)
+{
+    float4 v;
+    asm("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint4 sr_load_past_l1(const uint4* p)
+{
+    uint4 v;
+    asm("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint2 sr_load_past_l1(const uint2* p)
+{
+    uint2 v;
+    asm("ld.global.cg.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float sr_load_past_l1(const float* p)
+{
+    float v;
+    asm("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ unsigned short sr_load_past_l1(const unsigned short* p)
+{
+    unsigned short v;
+    asm("ld.global.cg.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return v;
 }
 __device__ __forceinline__ void sr_end(int follow_flags)
 {
