@@ -798,6 +798,7 @@ struct RsOffsets { int nodes = 0, edges = 0, units = 0, ubegin = 0, copies = 0, 
 
 struct RsEngine {
     int cs = 1, warps = 16, smem_bytes = 0, blob_bytes = 0, n_levels = 1;
+    double frame_us = 0.0;                         // estimated time of a frame of one wave (see sr_rs_plan)
     RsOffsets offs;                             // written by rs_layout, read when the blobs are filled
     std::vector<RsPlanNode> pn;
     std::vector<RsPlanEdge> pe;                 // ordered by target node, then by the node's in-edge order
@@ -964,7 +965,9 @@ bool rs_layout(const sr_graph* g, RsEngine& E, int cs, int warps, int dense_chun
         }
     }
     for (int v = 0; v < n_nodes; ++v) E.pn[v].n_slots = slot_count[v];
+    E.frame_us = 0.0;
     for (int r = 0; r < cs; ++r) {
+        double rank_us = 0.0;
         // longest-processing-time-first: level by level, to the least loaded scheduler partition
         // (warp id mod 4), then to its least loaded warp
         std::vector<std::vector<std::vector<RsUnit>>> lists(E.n_levels, std::vector<std::vector<RsUnit>>(warps));
@@ -998,7 +1001,9 @@ bool rs_layout(const sr_graph* g, RsEngine& E, int cs, int warps, int dense_chun
                 pl[bp] += c.cost;
                 lists[l][bw].push_back(c.u);
             }
+            rank_us += 0.3e-3 * *std::max_element(wl.begin(), wl.end()) + 0.2e-3 * *std::max_element(pl.begin(), pl.end()) + 0.5;
         }
+        E.frame_us = std::max(E.frame_us, rank_us);
         for (int l = 0; l < E.n_levels; ++l)
             for (int w = 0; w < warps; ++w) {
                 E.ubegin[r].push_back((int)E.units[r].size());
@@ -1289,8 +1294,11 @@ sr_status sr_rs_plan(sr_graph* g, size_t& offset)
     // Cluster size: the one that ends first.  A run of more sequences than the device holds clusters takes several waves, and the
     // device holds fewer clusters than its SMs suggest (a cluster does not span GPCs: of 148 SMs, 37 clusters of four do not fit
     // at once: a pass of 37 sequences x 20 sequential frames of the small CNN takes 452 us in clusters of four and 284 in
-    // clusters of two; 33 sequences 236 against 283).  Time per frame of one wave, measured on that network: 4.2 us in clusters
-    // of four, 6.5 of two.
+    // clusters of two; 33 sequences 236 against 283).  A frame of one wave is estimated from the work lists: level by level 0.3 ns
+    // per cycle of the longest warp, 0.2 per cycle of the fullest scheduler and 0.5 us.  Fitted to six networks (small CNNs, 1 to
+    // 5 levels, 1 to 600 sequences): the chosen size takes 0.2 % more than the best one on average and 7 % at most.  (Before, the
+    // small CNN's times stood for every network, 11.1, 6.5 and 4.2 us for one, two and four CTAs: a network of half its
+    // channels at 300 sequences took 2619 instead of 1625 us for 32 sequential frames, in five waves instead of three.)
     bool placed = false;
     double best = 0.0;
     for (int c = kRsMaxCluster; c >= 1; c >>= 1) {
@@ -1303,7 +1311,7 @@ sr_status sr_rs_plan(sr_graph* g, size_t& offset)
             if (rs_layout(g, F2, c, warps, 64)) F = F2;
         }
         const int held = rs_clusters_held(F);
-        const double cost = (double)((g->batch + held - 1) / held) * (1.9 + 9.2 / c);
+        const double cost = (double)((g->batch + held - 1) / held) * F.frame_us;
         if (placed && cost >= best) continue;
         placed = true;
         best = cost;

@@ -169,10 +169,19 @@ def test_resident_and_launch_path_agree_at_full_size():
 
 
 def test_more_sequences_than_clusters_of_four_fit():
-    # 37 sequences: 148 CTAs in clusters of four, which a device of 148 SMs does not hold at once
-    g = graphs.build("c2", batch=37, frames=3)
+    # 37 sequences: 148 CTAs in clusters of four, which a device of 148 SMs does not hold at once; 20 sequences fit
+    for batch, cluster in ((37, 2), (20, 4)):
+        g = graphs.build("c2", batch=batch, frames=3)
+        for p in g.patterns:
+            parity.check_run(g, p, samples=[0, 18, batch - 1], expect_resident=cluster)
+
+
+@pytest.mark.parametrize("batch,cluster", [(20, 4), (34, 2), (100, 1), (150, 1), (300, 1)])
+def test_cluster_size_of_a_network_of_little_work(batch, cluster):
+    # a frame of a small network takes nearly as long in a cluster as on one CTA: with more than one wave a CTA per sequence ends first
+    g = graphs.build("mini", batch=batch, frames=3)
     for p in g.patterns:
-        parity.check_run(g, p, samples=[0, 18, 36])
+        parity.check_run(g, p, samples=[0, batch - 1], expect_resident=cluster)
 
 
 @pytest.mark.parametrize("cin,k,stride,size,c,classes", [(1, 3, 1, 12, 32, 10), (3, 3, 1, 10, 64, 17), (1, 5, 2, 28, 32, 5), (2, 1, 1, 6, 32, 33), (4, 3, 1, 8, 32, 12)])
