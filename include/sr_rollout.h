@@ -128,7 +128,7 @@ sr_status sr_graph_bind_workspace(sr_graph* g, void* workspace_dev, size_t bytes
  * whose memory pool is owned and sized by another component, a late start-up phase after the device
  * has been handed over fully committed.  Such a caller cannot produce the buffer that
  * sr_graph_bind_workspace wants.  This call needs none: the workspace is a fixed array of
- * SR_STATIC_WORKSPACE_BYTES that lives in the library's device image, so every GPU that loads the
+ * SR_STATIC_WORKSPACE_BYTES (and 1/256 of that) that lives in the library's device image, so every GPU that loads the
  * library holds that much memory until the process exits, whether or not this call is ever made.
  *
  * Behaviour
@@ -139,7 +139,8 @@ sr_status sr_graph_bind_workspace(sr_graph* g, void* workspace_dev, size_t bytes
  *   - the first call on a device looks the array's address up for that device (the device must be
  *     current) and remembers it; make that first call before any stream capture begins;
  *   - a graph whose sr_graph_workspace_bytes exceeds SR_STATIC_WORKSPACE_BYTES is refused with
- *     SR_ERR_TOO_LARGE and stays unbound;
+ *     SR_ERR_TOO_LARGE and stays unbound (work lists of the CUDA-core kernels do not count: the array has
+ *     1/256 of its size of room for them);
  *   - all graphs bound this way share the one array.  It still holds what the previous user left, so
  *     binding clears the part the new graph uses (states start at zero) and parameters must be set
  *     again.  Only one such graph may be in use at a time: work of two graphs bound to the built-in

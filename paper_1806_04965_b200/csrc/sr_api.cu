@@ -17,8 +17,10 @@
 
 // Built-in workspace for callers that may not allocate device memory.  In host code the array's name
 // is only a handle: its device address is looked up once per device and that pointer is what the
-// kernels get (through the ordinary bind path).
-static __device__ __align__(256) unsigned char sr_static_workspace[SR_STATIC_WORKSPACE_BYTES];
+// kernels get (through the ordinary bind path).  The work lists of the CUDA-core kernels (16 bytes per 16 pixels and 128 channels, so
+// at most one part in 512 of the states) have room beyond the size that callers know.
+constexpr size_t kStaticBytes = SR_STATIC_WORKSPACE_BYTES + SR_STATIC_WORKSPACE_BYTES / 256;
+static __device__ __align__(256) unsigned char sr_static_workspace[kStaticBytes];
 
 namespace {
 
@@ -525,7 +527,7 @@ sr_status sr_graph_bind_static_workspace(sr_graph* g)
     size_t need = 0;
     sr_status st = sr_graph_workspace_bytes(g, &need);
     if (st != SR_OK) return st;
-    if (need > (size_t)SR_STATIC_WORKSPACE_BYTES) return SR_ERR_TOO_LARGE;
+    if (need - g->r_items.bytes > (size_t)SR_STATIC_WORKSPACE_BYTES || need > kStaticBytes) return SR_ERR_TOO_LARGE;
     int dev = -1;
     if (!cuda_ok(cudaGetDevice(&dev)) || dev < 0 || dev >= 64) return SR_ERR_CUDA;
     std::lock_guard<std::mutex> lock(static_mutex);
@@ -537,7 +539,7 @@ sr_status sr_graph_bind_static_workspace(sr_graph* g)
     }
     if (slot.owner && slot.owner != g) unbind(slot.owner);
     slot.owner = nullptr;
-    st = sr_graph_bind_workspace(g, slot.address, (size_t)SR_STATIC_WORKSPACE_BYTES);
+    st = sr_graph_bind_workspace(g, slot.address, kStaticBytes);
     if (st != SR_OK) return st;
     slot.owner = g;
     g->static_device = dev;

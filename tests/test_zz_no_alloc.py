@@ -79,3 +79,24 @@ def test_graph_larger_than_the_built_in_workspace_is_refused():
         Graph(spec.nodes, spec.edges, spec.patterns["streaming"], batch=spec.batch, dtype=spec.dtype,
               static_workspace=True)
     assert e.value.status == "SR_ERR_TOO_LARGE"
+
+
+def test_work_lists_do_not_count_against_the_built_in_workspace():
+    # states and weights of 31.99 MiB, and work lists of a node of 512 channels that take the total beyond 32 MiB
+    from workloads.graphs import CONV, GAP_DENSE, IDENTITY, Edge, GraphSpec, Node, check_shapes
+    g = GraphSpec("limit", [Node("in", 56, 29, 4, IDENTITY), Node("a", 56, 29, 512), Node("o", 1, 1, 4, IDENTITY)],
+                  [Edge(0, 1, CONV, 1, 1), Edge(1, 2, GAP_DENSE)], batch=5, frames=2, dtype="fp32", seed=96)
+    check_shapes(g)
+    g.patterns = {"streaming": [1, 1]}
+    from paper_1806_04965_b200 import Graph
+    import torch
+    X, W, Bi = data.make_inputs(g), data.make_weights(g), data.make_biases(g, zero=False)
+    outs = []
+    for static in (False, True):
+        G = Graph(g.nodes, g.edges, [1, 1], batch=g.batch, dtype="fp32", engine="direct", static_workspace=static)
+        assert 32 << 20 < G.workspace_bytes < (32 << 20) + (128 << 10) or not static
+        G.set_weights(W, Bi)
+        outs.append(G.rollout([parity.to_device(g, X[0])]))
+        G.sync_status()
+        torch.cuda.synchronize()
+    assert torch.equal(outs[0], outs[1])
