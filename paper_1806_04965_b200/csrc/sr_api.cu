@@ -508,6 +508,11 @@ sr_status sr_graph_bind_workspace(sr_graph* g, void* workspace_dev, size_t bytes
     g->ws = ws;
     for (size_t gi = 0; gi < g->groups.size(); ++gi) sr_describe_heads(g, (int)gi);
     st = sr_tc_bind(g);
+    for (unsigned mask = 0; mask < 4; ++mask) {
+        g->stems_of[mask].clear();
+        for (const SrStem& stem : g->stems)
+            if ((mask >> stem.R) & 1u) g->stems_of[mask].push_back(&stem);
+    }
     if (st == SR_OK && g->info.n_tensor_core_nodes > 0 && (!sr_input_share_sm() || !sr_direct_share_sm())) st = SR_ERR_CUDA;
     if (st == SR_OK) st = sr_rs_bind(g);
     if (st == SR_OK) st = sr_dn_bind(g);

@@ -734,7 +734,7 @@ static int head_blocks(const sr_graph* g, const SrHeadNode& h)
 bool sr_heads_take_input(const sr_graph* g, int group, const SrFrameArgs& fr, unsigned copies, unsigned stems_R)
 {
     const std::vector<SrHeadNode>& heads = g->group_heads[group];
-    const std::vector<const SrStem*> stems = sr_stems(g, stems_R);
+    const std::vector<const SrStem*>& stems = sr_stems(g, stems_R);
     if (heads.empty() || heads.size() > SR_HEAD_NODES || !g->group_wide[group].empty() || stems.size() > kStemsPerLaunch) return false;
     int blocks = 0, mean = 0;
     for (const SrHeadNode& h : heads) {

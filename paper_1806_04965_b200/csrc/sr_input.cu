@@ -46,7 +46,7 @@ __global__ void sr_advance_kernel(SrFrameCtl* ctl, int n)
 int sr_launch_input(const sr_graph* g, const SrFrameArgs& fr, unsigned copies, unsigned stems_R, SrFollow how, const SrRegion* clear, cudaStream_t s)
 {
     int launches = 0;
-    const std::vector<const SrStem*> stems = sr_stems(g, stems_R);
+    const std::vector<const SrStem*>& stems = sr_stems(g, stems_R);
     size_t next = 0;
     do {
         InputParams P{fr, sr_plan_input(g, launches == 0 ? copies : 0u, stems, next, how.beside), how.flags(), 0, nullptr, 0};

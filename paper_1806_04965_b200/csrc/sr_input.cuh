@@ -143,10 +143,4 @@ inline SrInputPart sr_plan_input(const sr_graph* g, unsigned copies, const std::
 }
 
 // The staged edges that stems_R names (bit 0: those that read the frame's input within the frame, R = 0; bit 1: a frame later).
-inline std::vector<const SrStem*> sr_stems(const sr_graph* g, unsigned stems_R)
-{
-    std::vector<const SrStem*> stems;
-    for (const SrStem& st : g->stems)
-        if ((stems_R >> st.R) & 1u) stems.push_back(&st);
-    return stems;
-}
+inline const std::vector<const SrStem*>& sr_stems(const sr_graph* g, unsigned stems_R) { return g->stems_of[stems_R & 3u]; }
