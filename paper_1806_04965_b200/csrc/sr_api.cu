@@ -90,6 +90,8 @@ sr_status plan(sr_graph* g)
     if (g->batch <= 0) return SR_ERR_STATE;
     if (g->planned) return SR_OK;                                // asking for the size and binding share one plan
     const int n_nodes = (int)g->nodes.size(), n_edges = (int)g->edges.size();
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0) g->sm_count = sms;
     for (int v = 0; v < n_nodes; ++v) {
         SrHostNode& n = g->nodes[v];
         n.dense_target = false;

@@ -716,7 +716,7 @@ static bool head_wide(const sr_graph* g) { return g->batch >= 16; }
 static int head_mean_outputs(const sr_graph* g, int channels, int most)
 {
     const int all = (channels + kHeadWarps - 1) / kHeadWarps;
-    int q = g->batch >= 148 ? std::min(2, all) : 1;
+    int q = g->batch >= g->sm_count ? std::min(2, all) : 1;
     while (q < all && q < most && (long long)g->batch * ((channels + kHeadWarps * q - 1) / (kHeadWarps * q)) > 500) ++q;
     return q;
 }
@@ -750,7 +750,7 @@ bool sr_heads_take_input(const sr_graph* g, int group, const SrFrameArgs& fr, un
             if (reinterpret_cast<uintptr_t>(fr.v.in_base[i]) & 15 || fr.v.in_stride_bytes[i] & 15) return false;
     }
     size_t next = 0;
-    return blocks + sr_plan_input(g, copies, stems, next, true).n_blocks <= 148;
+    return blocks + sr_plan_input(g, copies, stems, next, true).n_blocks <= g->sm_count;
 }
 
 int sr_launch_heads(const sr_graph* g, int group, bool with_input, unsigned copies, unsigned stems_R, SrFollow how, cudaStream_t s)
@@ -853,7 +853,7 @@ void sr_direct_conv_items(const sr_graph* g, int v, std::vector<SrDirectItem>& i
     // Four pixels per thread once that still gives every SM 256 threads; marked by the complement of the sample.  Measured on
     // B200, fp32, us per frame with one / four pixels everywhere: small CNN (28 x 28 x 32, 14 x 14 x 32, 7 x 7 x 64) at 128
     // samples 161 / 133 (this rule: 114), at 32 samples (sequential) 90 / 144, at one 27 / 51; MNIST net at 256 samples 35 / 53.
-    const bool four = (size_t)g->batch * HW * (d.c / 4) / 4 >= (size_t)148 * 256;
+    const bool four = (size_t)g->batch * HW * (d.c / 4) / 4 >= (size_t)g->sm_count * 256;
     const int px = (kWarps * 32 >> qlog) * (four ? 4 : 1);
     for (int b = 0; b < g->batch; ++b)
         for (int p0 = 0; p0 < HW; p0 += px)

@@ -53,7 +53,7 @@ int sr_launch_input(const sr_graph* g, const SrFrameArgs& fr, unsigned copies, u
         if (clear && launches == 0) {
             P.clear = reinterpret_cast<uint4*>(g->ws + clear->offset);
             P.n_clear = clear->bytes / 16;
-            P.clear_blocks = (int)std::min<size_t>(148 * 6, (P.n_clear + 4 * kInputThreads - 1) / (4 * kInputThreads));
+            P.clear_blocks = (int)std::min<size_t>((size_t)g->sm_count * 6, (P.n_clear + 4 * kInputThreads - 1) / (4 * kInputThreads));
         }
         if (P.in.n_blocks + P.clear_blocks == 0) break;
         sr_launch(P.clear_blocks ? sr_input_kernel<true, false> : how.beside ? sr_input_kernel<false, true> : sr_input_kernel<false, false>, P.in.n_blocks + P.clear_blocks, kInputThreads, 0, s, how.early, P);

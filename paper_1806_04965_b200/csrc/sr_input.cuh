@@ -111,7 +111,7 @@ inline SrInputPart sr_plan_input(const sr_graph* g, unsigned copies, const std::
 {
     // Beside a tensor-core kernel: few blocks (every SM has threads and registers left for all of them), else as many as there
     // is work for.
-    const size_t per_part = beside ? 148 * 2 : 148 * 16;
+    const size_t sms = (size_t)g->sm_count, per_part = beside ? sms * 2 : sms * 16;
     SrInputPart P;
     P.B = g->batch;
     P.n_copy = P.n_stem = 0;
@@ -125,7 +125,7 @@ inline SrInputPart sr_plan_input(const sr_graph* g, unsigned copies, const std::
         c.bytes = (size_t)g->batch * n.d.h * n.d.w * n.d.c * g->elem;
         c.slot = (int)i;
         c.first_block = blocks;
-        blocks += (int)std::min<size_t>(beside ? 148 : 296, (c.bytes / 16 + kInputThreads - 1) / kInputThreads + 1);
+        blocks += (int)std::min<size_t>(beside ? sms : sms * 2, (c.bytes / 16 + kInputThreads - 1) / kInputThreads + 1);
     }
     for (; next < stems.size() && P.n_stem < kStemsPerLaunch; ++next) {
         const SrStem& st = *stems[next];

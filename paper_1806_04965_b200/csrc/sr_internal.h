@@ -244,6 +244,7 @@ struct sr_graph {
     SrRegion r_nodes, r_edges, r_ctl, r_items;
     SrRegion r_clear;                              // what a reset zeroes: the flags, then the non-input nodes' parity-0 states
     SrRegion r_flags;                              // int 0: device-side error code (0 = none); ints 16, 17: the shared work list's counters
+    int sm_count = 148;                            // of the device that is current when the graph is planned
     std::vector<SrStem> stems;                     // filled when a workspace is bound
     std::vector<const SrStem*> stems_of[4];        // those that a mask of R names (see sr_stems): nothing is allocated on a launch
     unsigned input_read = 0;                       // bit i: some edge reads input node i's state itself (not a staged copy)

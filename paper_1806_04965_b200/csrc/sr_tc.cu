@@ -862,7 +862,6 @@ struct TcEngine {
     std::vector<int> group_tile_offset, group_grid, group_n_own, group_n_w, group_w_slot, group_ring_kb, group_table_bytes;
     SrRegion r_maps, r_nodes, r_tables, r_tiles;
     int n_maps = 0, n_kbs = 0, n_tiles = 0;
-    int sm_count = 148;
     // optional timing of the group launches with CUDA events on the launching stream
     std::vector<cudaEvent_t> ev;             // pairs: start, stop
     size_t ev_used = 0;
@@ -1175,9 +1174,6 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
     if (!any) return SR_OK;
     TcEngine* E = new TcEngine();
     g->tc = E;
-    int dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&E->sm_count, cudaDevAttrMultiProcessorCount, dev);
-    if (E->sm_count <= 0) E->sm_count = 148;
     E->node_of.assign(g->nodes.size(), -1);
     E->stem_of_edge.assign(g->edges.size(), -1);
     auto take = [&](size_t bytes) {
@@ -1302,12 +1298,12 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
         long long best_span = -1;
         for (int max_cols = kMaxCols; max_cols >= 64 && !members.empty(); max_cols /= 2) {
             const auto tl = plan_tiles(max_cols);
-            const long long span = spread_items(tl, tl.size(), (int)std::min<size_t>(tl.size(), (size_t)E->sm_count), nullptr);
+            const long long span = spread_items(tl, tl.size(), (int)std::min<size_t>(tl.size(), (size_t)g->sm_count), nullptr);
             if (best_span < 0 || span < best_span) {
                 best_span = span;
                 best_cols = max_cols;
             }
-            if (tl.size() > 8 * (size_t)E->sm_count) break;        // plenty of items: smaller tiles only cost copies
+            if (tl.size() > 8 * (size_t)g->sm_count) break;        // plenty of items: smaller tiles only cost copies
         }
         const std::vector<std::pair<long long, TcTile>> tl = plan_tiles(best_cols);
         // Shared memory: weight slots, the node tables, and the rest for activation boxes, of which two of the largest should
@@ -1331,7 +1327,7 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
         }
         const int table_bytes = (int)sizeof(TcNode) + n_tab * 16;
         const int avail = kSmemBudget - 1024 - kTables * table_bytes;
-        int n_w = g->opt_b_units > 0 ? std::min(kMaxW, std::max(2, g->opt_b_units)) : (best_cols == kMaxCols && tl.size() > 2 * (size_t)E->sm_count ? 5 : 6);
+        int n_w = g->opt_b_units > 0 ? std::min(kMaxW, std::max(2, g->opt_b_units)) : (best_cols == kMaxCols && tl.size() > 2 * (size_t)g->sm_count ? 5 : 6);
         while (n_w > 3 && (avail - n_w * w_slot) / 1024 < 2 * box_kb) --n_w;
         while (n_w > 2 && (avail - n_w * w_slot) / 1024 < box_kb) --n_w;
         const int ring_kb = (avail - n_w * w_slot) / 1024;
@@ -1340,7 +1336,7 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
         // matrix with one row per round (entries of node -1 pad the shorter columns).  Unless the lists are asked to be
         // static, the smallest items - a fifth of the work, if the launch has more than two items per CTA - stay out of
         // the matrix and follow it as one shared list (see the kernel).
-        const int grid = (int)std::min<size_t>(tl.size(), (size_t)E->sm_count);
+        const int grid = (int)std::min<size_t>(tl.size(), (size_t)g->sm_count);
         std::vector<std::vector<TcTile>> lists(std::max(grid, 1));
         size_t n_matrix = tl.size();
         if (g->opt_tc_lists == 0 && tl.size() > 2 * (size_t)grid) {
