@@ -55,7 +55,6 @@ struct GraphCache {
     cudaGraphExec_t exec = nullptr;
     int frames = 0;
     int kernels = 0;
-    bool with_out = false;
 };
 
 float round_bf16_host(float f)
@@ -402,11 +401,9 @@ sr_status sr_graph_set_option(sr_graph* g, int key, int value)
         g->opt_rs_warps = value;
         return SR_OK;
     }
-    if (key == 11) {
+    if (key == 11 || key == 12) {                        // accepted, without effect
         if (g->ws) return SR_ERR_STATE;
-        if (value < 0 || value > 2) return SR_ERR_INVALID_ARG;
-        g->opt_tc_pair = value;
-        return SR_OK;
+        return value < 0 || value > 2 ? SR_ERR_INVALID_ARG : SR_OK;
     }
     if (key == 14) {
         if (g->ws) return SR_ERR_STATE;
@@ -418,12 +415,6 @@ sr_status sr_graph_set_option(sr_graph* g, int key, int value)
         if (g->ws) return SR_ERR_STATE;
         if (value < 0 || value > 1) return SR_ERR_INVALID_ARG;
         g->opt_tc_lists = value;
-        return SR_OK;
-    }
-    if (key == 12) {
-        if (g->ws) return SR_ERR_STATE;
-        if (value < 0 || value > 2) return SR_ERR_INVALID_ARG;
-        g->opt_stem_ring = value;
         return SR_OK;
     }
     if (key == 10) {
@@ -807,8 +798,6 @@ sr_status sr_graph_window_workspace_bytes(sr_graph* g, int W, size_t* bytes)
         w->opt_b_units = g->opt_b_units;
         w->opt_tile_w = g->opt_tile_w;
         w->opt_overlap = g->opt_overlap;
-        w->opt_tc_pair = g->opt_tc_pair;
-        w->opt_stem_ring = g->opt_stem_ring;
         w->opt_tc_lists = g->opt_tc_lists;
         w->opt_tc_fuse = g->opt_tc_fuse;
         w->opt_wait_ms = g->opt_wait_ms;
