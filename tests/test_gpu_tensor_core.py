@@ -17,14 +17,14 @@ def tiny(name, nodes, edges, batch=3, frames=3, R=None):
 
 
 def run(g):
-    # single tiles (work items from the shared list, then from per-CTA lists), then pairs of tiles that share every
-    # weight box
+    # as the library chooses; a work list per CTA instead of the shared list, on tiles of one lane of eight columns; tiles of four
+    # lanes (or as many as the image is wide) with the shallowest weight ring
     from paper_1806_04965_b200 import Graph
     G = Graph(g.nodes, g.edges, g.patterns["p"], batch=g.batch, dtype="bf16")
     assert G.info["n_tensor_core_nodes"] >= 1, G.info
-    parity.check_stepwise(g, "p", zero_bias=False, tc_pair=1)
-    parity.check_stepwise(g, "p", zero_bias=False, tc_lists=1)      # a work list per CTA instead of the shared list
-    return parity.check_stepwise(g, "p", zero_bias=False, tc_pair=2)
+    parity.check_stepwise(g, "p", zero_bias=False, tc_lists=1, tile_width=8)
+    parity.check_stepwise(g, "p", zero_bias=False, tile_width=32, weight_ring_units=2)
+    return parity.check_stepwise(g, "p", zero_bias=False)
 
 
 @pytest.mark.parametrize("cin,cout,k,stride,size", [
@@ -47,17 +47,16 @@ def test_few_channel_input_edges_are_staged():
                  [Edge(0, 1, CONV, k, 1), Edge(1, 2, CONV, 3, 1), Edge(0, 2, CONV, k, 1), Edge(1, 1, CONV, 3, 1),
                   Edge(2, 3, GAP_DENSE)], frames=4, R=[1, 1, 0, 1, 0])
         run(g)
-        # the staged edge's activation box in an activation slot (0) / in the weight ring behind its weights (2)
-        for stem_ring in (0, 2):
-            parity.check_stepwise(g, "p", zero_bias=False, stem_ring=stem_ring)
+        for ring in (3, 8):
+            parity.check_stepwise(g, "p", zero_bias=False, weight_ring_units=ring)
 
 
 def test_a_node_fed_by_a_staged_edge_only():
-    # every K-block of node a travels in the weight ring: the activation ring stays empty for its tiles
+    # no tap of node a shares an activation box: flat tiles (0), or tiles of lanes where a width is asked for
     g = tiny("stem_only", [Node("in", 32, 32, 3, IDENTITY), Node("a", 32, 32, 64), Node("b", 32, 32, 128), Node("o", 1, 1, 4, IDENTITY)],
              [Edge(0, 1, CONV, 3, 1), Edge(1, 2, CONV, 3, 1), Edge(2, 3, GAP_DENSE)], batch=5, frames=4)
-    for stem_ring in (0, 1, 2):
-        parity.check_stepwise(g, "p", zero_bias=False, stem_ring=stem_ring)
+    for tile_width in (0, 8, 32):
+        parity.check_stepwise(g, "p", zero_bias=False, tile_width=tile_width)
 
 
 @pytest.mark.parametrize("c,act_b", [(64, RELU), (32, IDENTITY)])
@@ -70,7 +69,7 @@ def test_two_narrow_nodes_that_share_a_source_run_as_one_plan(c, act_b):
               Edge(1, 3, CONV, 3, 2), Edge(2, 3, CONV, 1, 2), Edge(3, 4, GAP_DENSE)], batch=5, frames=4)
     for fuse in (1, 0):
         parity.check_stepwise(g, "p", zero_bias=False, tc_fuse=fuse)
-    parity.check_stepwise(g, "p", zero_bias=False, tc_fuse=1, tc_lists=1, stem_ring=2)
+    parity.check_stepwise(g, "p", zero_bias=False, tc_fuse=1, tc_lists=1, weight_ring_units=2)
     # with a -> b inside the frame (R = 0) the two nodes are in different launch groups: nothing to fuse, same results
     g.patterns["q"] = [1, 1, 0, 1, 1, 1, 1, 1]
     parity.check_stepwise(g, "q", zero_bias=False)
@@ -102,14 +101,14 @@ def test_configs_reduced_tensor_cores(name, kw):
     g = build(name, **kw)
     for p in g.patterns:
         parity.check_stepwise(g, p, engine="auto", zero_bias=False)
-        parity.check_stepwise(g, p, engine="auto", zero_bias=False, tc_pair=2)
+        parity.check_stepwise(g, p, engine="auto", zero_bias=False, tile_width=32)
         parity.check_run(g, p, engine="auto", graph_frames=2)
-        parity.check_run(g, p, engine="auto", graph_frames=2, tc_pair=2, resident=False)
+        parity.check_run(g, p, engine="auto", graph_frames=2, tile_width=16, resident=False)
 
 
 @pytest.mark.parametrize("batch", [1, 2, 7])
-def test_pairs_with_ragged_batches_and_widths(batch):
-    # lane 1 of the last pair falls outside the batch (sample pairs) or outside the image (column pairs)
+def test_lanes_with_ragged_batches_and_widths(batch):
+    # the last lanes of a tile lie partly or wholly outside the image (20, 10 and 5 columns in lanes of eight)
     g = tiny("ragged", [Node("in", 20, 20, 64, IDENTITY), Node("a", 20, 20, 128), Node("b", 10, 10, 128), Node("c", 5, 5, 256),
                         Node("o", 1, 1, 4, IDENTITY)],
              [Edge(0, 1, CONV, 3, 1), Edge(1, 1, CONV, 3, 1), Edge(1, 2, CONV, 3, 2), Edge(2, 2, CONV, 3, 1), Edge(2, 3, CONV, 3, 2),
@@ -131,8 +130,8 @@ def test_paper_cifar10_networks_on_tensor_cores(k):
     S = Graph(g.nodes, g.edges, g.patterns["sequential"], batch=0)
     assert S.info["first_response_step"] == 4 + k and S.info["inference_factor"] == 4 + k
     for p in g.patterns:
-        parity.check_stepwise(g, p, zero_bias=False, tc_pair=1)
-        parity.check_stepwise(g, p, zero_bias=False, tc_pair=2)
+        parity.check_stepwise(g, p, zero_bias=False)
+        parity.check_stepwise(g, p, zero_bias=False, tile_width=16)
         parity.check_run(g, p, graph_frames=2)
 
 
@@ -141,6 +140,50 @@ def test_gtsrb_network_variant():
     from workloads import graphs
     g = graphs.dsr(4, batch=2, frames=3, classes=43, h1_recurrence=False)
     parity.check_stepwise(g, "streaming", zero_bias=False)
+
+
+@pytest.mark.parametrize("tile_width,ring", [(0, 0), (8, 0), (16, 4), (32, 3), (32, 8)])
+@pytest.mark.parametrize("size", [(9, 5), (7, 17), (5, 33), (3, 70)])
+def test_tile_widths_and_ring_depths(size, tile_width, ring):
+    # a width of 8, 16 or 32 makes tiles of one, two or four lanes of eight columns, as far as the image is wide, the last of them
+    # beyond it; blocks of 64, 32 and 16 channels and a staged edge in one reduction, which make bursts of two weight groups and of one
+    h, w = size
+    g = tiny("lanes", [Node("in", h, w, 3, IDENTITY), Node("a", h, w, 64), Node("b", h, w, 48), Node("c", h, w, 96), Node("d", (h + 1) // 2, (w + 1) // 2, 136),
+                       Node("o", 1, 1, 4, IDENTITY)],
+             [Edge(0, 1, CONV, 3, 1), Edge(1, 1, CONV, 3, 1), Edge(1, 2, CONV, 3, 1), Edge(0, 2, CONV, 1, 1), Edge(2, 3, CONV, 3, 1), Edge(1, 3, CONV, 1, 1),
+              Edge(3, 3, CONV, 3, 1), Edge(3, 4, CONV, 3, 2), Edge(2, 4, CONV, 1, 2), Edge(4, 5, GAP_DENSE)], batch=3, frames=3)
+    parity.check_stepwise(g, "p", zero_bias=False, tile_width=tile_width, weight_ring_units=ring)
+
+
+@pytest.mark.parametrize("h,w", [(1, 250), (2, 131), (1, 20001), (4, 20001)])
+def test_images_of_few_rows(h, w):
+    # tiles of as many lanes as an accumulator holds: four of 16 columns, two, eight of 16 and eight of 32 (a lane has at least 16
+    # columns, of which one row of eight pixels fills half)
+    g = tiny("rows", [Node("in", h, w, 64, IDENTITY), Node("a", h, w, 64), Node("b", h, w, 32), Node("o", 1, 1, 4, IDENTITY)],
+             [Edge(0, 1, CONV, 3, 1), Edge(1, 1, CONV, 3, 1), Edge(1, 2, CONV, 3, 1), Edge(2, 3, GAP_DENSE)], batch=1, frames=2)
+    parity.check_stepwise(g, "p", zero_bias=False)
+
+
+@pytest.mark.parametrize("name,kw", [("c3", dict(batch=3, frames=4, size=16)), ("c4", dict(batch=2, frames=4, size=16)), ("dsr2", dict(batch=2, frames=3)),
+                                     ("c2", dict(batch=2, frames=4, dtype="fp32")), ("mini", dict(batch=2, frames=4, dtype="fp32"))])
+def test_launches_one_after_the_other_give_the_same(name, kw):
+    # overlap off (option 4): every launch waits for the one before it; the same kernels on the same data, bit for bit, also recorded
+    # in CUDA graphs
+    import torch
+    from workloads import data, graphs
+    g = graphs.dsr(2, **kw) if name == "dsr2" else build(name, **kw)
+    X, W, Bi = data.make_inputs(g), data.make_weights(g), data.make_biases(g, zero=False)
+    for p in g.patterns:
+        seen = []
+        for overlap, graph_frames in ((1, 0), (0, 0), (0, 2), (1, 2)):
+            G = parity.make_graph(g, p, "auto", graph_frames, W, Bi, resident=False)
+            G.set_option(4, overlap)
+            out = G.rollout([parity.to_device(g, X[v]) for v in G.input_nodes])
+            G.sync_status()
+            seen.append([out] + [G.get_state(v) for v in range(len(g.nodes))])
+        for other in seen[1:]:
+            assert all(torch.equal(a, b) for a, b in zip(seen[0], other)), p
+        parity.check_run(g, p, resident=False)
 
 
 def test_a_state_of_more_than_2_31_elements():
