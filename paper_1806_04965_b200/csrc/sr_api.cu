@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstddef>
 #include <cstring>
 #include <mutex>
@@ -56,6 +57,14 @@ struct GraphCache {
     int frames = 0;
     int kernels = 0;
 };
+
+// Launches recorded in a CUDA graph are recorded anew by the next run.
+void forget_recorded(sr_graph* g)
+{
+    GraphCache* c = static_cast<GraphCache*>(g->graphs);
+    if (c && c->exec) cudaGraphExecDestroy(c->exec);
+    if (c) c->exec = nullptr;
+}
 
 float round_bf16_host(float f)
 {
@@ -420,11 +429,7 @@ sr_status sr_graph_set_option(sr_graph* g, int key, int value)
     if (key == 10) {
         if (value < 0 || value > 60000) return SR_ERR_INVALID_ARG;
         g->opt_wait_ms = value;
-        if (g->graphs) {                                 // recorded launches carry the old limit
-            GraphCache* c = static_cast<GraphCache*>(g->graphs);
-            if (c->exec) cudaGraphExecDestroy(c->exec);
-            c->exec = nullptr;
-        }
+        forget_recorded(g);                              // recorded launches carry the old limit
         if (g->window) g->window->opt_wait_ms = value;
         return SR_OK;
     }
@@ -449,11 +454,7 @@ sr_status sr_graph_bind_workspace(sr_graph* g, void* workspace_dev, size_t bytes
     if (!g || !workspace_dev) return SR_ERR_INVALID_ARG;
     if (g->ws) return SR_ERR_STATE;
     if (reinterpret_cast<uintptr_t>(workspace_dev) & 255) return SR_ERR_INVALID_ARG;
-    if (g->graphs) {                                     // launches recorded for an earlier binding point at its tables
-        GraphCache* c = static_cast<GraphCache*>(g->graphs);
-        if (c->exec) cudaGraphExecDestroy(c->exec);
-        c->exec = nullptr;
-    }
+    forget_recorded(g);                                  // launches recorded for an earlier binding point at its tables
     sr_status st = plan(g);
     if (st != SR_OK) return st;
     if (bytes < g->ws_bytes) return SR_ERR_INVALID_ARG;
@@ -485,6 +486,8 @@ sr_status sr_graph_bind_workspace(sr_graph* g, void* workspace_dev, size_t bytes
             x.R = he.R; x.K = he.K; x.src_is_input = s.is_input;
         }
     }
+    for (SrHostEdge& e : g->edges) e.w_finite = true;
+    for (SrHostNode& n : g->nodes) n.w_finite = true;
     if (!cuda_ok(cudaMemset(ws, 0, g->ws_bytes))) return SR_ERR_CUDA;
     if (!cuda_ok(cudaMemcpy(ws + g->r_nodes.offset, dn.data(), sizeof(SrDevNode) * n_nodes, cudaMemcpyHostToDevice)))
         return SR_ERR_CUDA;
@@ -592,6 +595,17 @@ sr_status sr_graph_set_edge_weights(sr_graph* g, int edge, const float* w, int i
         if (!cuda_ok(cudaMemcpy(g->ws + he.w_direct.offset, src, (size_t)he.K * Cout * sizeof(float),
                                 cudaMemcpyHostToDevice)))
             return SR_ERR_CUDA;
+        // a convolutional node with a weight that is not finite leaves conv_tile, and returns to it with its last one
+        he.w_finite = std::all_of(src, src + (size_t)he.K * Cout, [](float v) { return std::isfinite(v); });
+        const bool finite = std::all_of(t.in_edges.begin(), t.in_edges.end(), [&](int e) { return g->edges[e].w_finite; });
+        if (finite != t.w_finite) {
+            const int32_t untiled = sr_direct_untiled(g, he.d.tgt) ? 1 : finite ? 0 : 2;
+            if (!cuda_ok(cudaMemcpy(g->ws + g->r_nodes.offset + sizeof(SrDevNode) * he.d.tgt + offsetof(SrDevNode, untiled), &untiled, sizeof(untiled),
+                                    cudaMemcpyHostToDevice)))
+                return SR_ERR_CUDA;
+            g->nodes[he.d.tgt].w_finite = finite;
+            forget_recorded(g);
+        }
     } else {
         const sr_status st = sr_tc_set_weights(g, edge, eff.data());
         if (st != SR_OK) return st;

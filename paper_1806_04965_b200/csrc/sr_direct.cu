@@ -65,83 +65,93 @@ constexpr int kPix = 4;            // pixels per warp (conv nodes)
 constexpr int kWarps = 4;          // warps per block
 constexpr int kDenseB = 8;         // samples per warp (dense nodes)
 
-// Conv node that conv_tile does not take (see sr_direct_conv_items): a block covers kWarps*kPix consecutive pixels of one sample; lanes run over output
-// channels, so weight reads ([K][C_out] rows) and state writes (NHWC) are coalesced and the input
+// Conv node that conv_tile does not take (see sr_direct_untiled), or that has a weight which is not finite: a tap outside the image is
+// left out here, while conv_tile multiplies it by zero.  A block covers kWarps*kPix consecutive pixels of one sample at a time; lanes
+// run over output channels, so weight reads ([K][C_out] rows) and state writes (NHWC) are coalesced and the input
 // reads are warp-uniform broadcasts.
-template <typename T>
+template <typename T, bool ANY_ITEM>
 __device__ void conv_item(const SrDevNode& nd, const SrDevEdge* edges, const SrDirectItem& it, int prev, int cur,
                           float* out_f32)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int HW = nd.H * nd.W;
-    const int pbase = it.p0 + warp * kPix;
-    int oy[kPix], ox[kPix];
-    bool pv[kPix];
-#pragma unroll
-    for (int j = 0; j < kPix; ++j) {
-        const int p = pbase + j;
-        pv[j] = p < HW;
-        oy[j] = pv[j] ? p / nd.W : 0;
-        ox[j] = pv[j] ? p % nd.W : 0;
+    int b = it.b0, n_pix = kWarps * kPix, c_first = 0, c_end = nd.C;
+    if (ANY_ITEM && nd.untiled == 2) {                                                       // conv_tile's items: pixels and channels of their own
+        const int qlog = it.pad_ >> 24;
+        b = it.b0 < 0 ? ~it.b0 : it.b0;
+        n_pix = (kWarps * 32 >> qlog) * (it.b0 < 0 ? 4 : 1);
+        c_first = it.pad_ & 0xFFFFFF;
+        c_end = min(nd.C, c_first + (4 << qlog));
     }
-    T* dst = static_cast<T*>(nd.state[cur]) + (size_t)it.b0 * HW * nd.C;
-    for (int co0 = 0; co0 < nd.C; co0 += 32) {
-        const int co = co0 + lane;
-        const bool cv = co < nd.C;
-        float acc[kPix];
+    T* dst = static_cast<T*>(nd.state[cur]) + (size_t)b * HW * nd.C;
+    for (int pbase = it.p0 + warp * kPix; pbase < min(HW, it.p0 + n_pix); pbase += kWarps * kPix) {
+        int oy[kPix], ox[kPix];
+        bool pv[kPix];
 #pragma unroll
-        for (int j = 0; j < kPix; ++j) acc[j] = 0.f;
-        for (int ei = 0; ei < nd.n_edges; ++ei) {
-            const SrDevEdge& e = edges[nd.first_edge + ei];
-            const T* src = static_cast<const T*>(e.src[e.R ? prev : cur]) + (size_t)it.b0 * e.Hs * e.Ws * e.Cs;
-            const bool vec = (e.Cs & 3) == 0;
-            for (int ky = 0; ky < e.k; ++ky)
-                for (int kx = 0; kx < e.k; ++kx) {
-                    const T* xp[kPix];
-                    bool ok[kPix];
-                    bool any = false;
+        for (int j = 0; j < kPix; ++j) {
+            const int p = pbase + j;
+            pv[j] = p < HW;
+            oy[j] = pv[j] ? p / nd.W : 0;
+            ox[j] = pv[j] ? p % nd.W : 0;
+        }
+        for (int co0 = c_first; co0 < c_end; co0 += 32) {
+            const int co = co0 + lane;
+            const bool cv = co < c_end;
+            float acc[kPix];
 #pragma unroll
-                    for (int j = 0; j < kPix; ++j) {
-                        const int iy = oy[j] * e.stride + ky - e.pad, ix = ox[j] * e.stride + kx - e.pad;
-                        ok[j] = pv[j] && iy >= 0 && iy < e.Hs && ix >= 0 && ix < e.Ws;
-                        xp[j] = src + ((size_t)(ok[j] ? iy : 0) * e.Ws + (ok[j] ? ix : 0)) * e.Cs;
-                        any |= ok[j];
-                    }
-                    if (!any) continue;
-                    const float* wp = e.w + (size_t)(ky * e.k + kx) * e.Cs * nd.C + co;
-                    if (vec) {
-                        for (int ci = 0; ci < e.Cs; ci += 4) {
-                            float w[4];
+            for (int j = 0; j < kPix; ++j) acc[j] = 0.f;
+            for (int ei = 0; ei < nd.n_edges; ++ei) {
+                const SrDevEdge& e = edges[nd.first_edge + ei];
+                const T* src = static_cast<const T*>(e.src[e.R ? prev : cur]) + (size_t)b * e.Hs * e.Ws * e.Cs;
+                const bool vec = (e.Cs & 3) == 0;
+                for (int ky = 0; ky < e.k; ++ky)
+                    for (int kx = 0; kx < e.k; ++kx) {
+                        const T* xp[kPix];
+                        bool ok[kPix];
+                        bool any = false;
 #pragma unroll
-                            for (int q = 0; q < 4; ++q) w[q] = cv ? wp[(size_t)(ci + q) * nd.C] : 0.f;
+                        for (int j = 0; j < kPix; ++j) {
+                            const int iy = oy[j] * e.stride + ky - e.pad, ix = ox[j] * e.stride + kx - e.pad;
+                            ok[j] = pv[j] && iy >= 0 && iy < e.Hs && ix >= 0 && ix < e.Ws;
+                            xp[j] = src + ((size_t)(ok[j] ? iy : 0) * e.Ws + (ok[j] ? ix : 0)) * e.Cs;
+                            any |= ok[j];
+                        }
+                        if (!any) continue;
+                        const float* wp = e.w + (size_t)(ky * e.k + kx) * e.Cs * nd.C + co;
+                        if (vec) {
+                            for (int ci = 0; ci < e.Cs; ci += 4) {
+                                float w[4];
 #pragma unroll
-                            for (int j = 0; j < kPix; ++j) {
-                                if (!ok[j]) continue;
-                                float x[4];
-                                load4(xp[j] + ci, x);
+                                for (int q = 0; q < 4; ++q) w[q] = cv ? wp[(size_t)(ci + q) * nd.C] : 0.f;
 #pragma unroll
-                                for (int q = 0; q < 4; ++q) acc[j] = fmaf(w[q], x[q], acc[j]);
+                                for (int j = 0; j < kPix; ++j) {
+                                    if (!ok[j]) continue;
+                                    float x[4];
+                                    load4(xp[j] + ci, x);
+#pragma unroll
+                                    for (int q = 0; q < 4; ++q) acc[j] = fmaf(w[q], x[q], acc[j]);
+                                }
+                            }
+                        } else {
+                            for (int ci = 0; ci < e.Cs; ++ci) {
+                                const float w = cv ? wp[(size_t)ci * nd.C] : 0.f;
+#pragma unroll
+                                for (int j = 0; j < kPix; ++j)
+                                    if (ok[j]) acc[j] = fmaf(w, to_f(xp[j][ci]), acc[j]);
                             }
                         }
-                    } else {
-                        for (int ci = 0; ci < e.Cs; ++ci) {
-                            const float w = cv ? wp[(size_t)ci * nd.C] : 0.f;
-#pragma unroll
-                            for (int j = 0; j < kPix; ++j)
-                                if (ok[j]) acc[j] = fmaf(w, to_f(xp[j][ci]), acc[j]);
-                        }
                     }
-                }
-        }
-        if (cv) {
-            const float b = nd.bias[co];
+            }
+            if (cv) {
+                const float bias = nd.bias[co];
 #pragma unroll
-            for (int j = 0; j < kPix; ++j) {
-                if (!pv[j]) continue;
-                float z = acc[j] + b;
-                if (nd.act == 1) z = fmaxf(z, 0.f);
-                from_f(dst + (size_t)(pbase + j) * nd.C + co, z);
-                if (out_f32) out_f32[((size_t)it.b0 * HW + pbase + j) * nd.C + co] = z;
+                for (int j = 0; j < kPix; ++j) {
+                    if (!pv[j]) continue;
+                    float z = acc[j] + bias;
+                    if (nd.act == 1) z = fmaxf(z, 0.f);
+                    from_f(dst + (size_t)(pbase + j) * nd.C + co, z);
+                    if (out_f32) out_f32[((size_t)b * HW + pbase + j) * nd.C + co] = z;
+                }
             }
         }
     }
@@ -661,7 +671,10 @@ struct DirectParams {
     int32_t B, follow;
 };
 
-template <typename T>
+// NON_FINITE: nodes may have a weight that is not finite.  In fp32 a kernel of its own, because the compiler's choices for the tiled
+// convolutions change with everything beside them (32 -> 32 channels of 32 x 32, 64 samples: 570 us for eight frames, 626 in the
+// kernel that takes both); bf16 is as fast either way.
+template <typename T, bool NON_FINITE>
 __global__ void __launch_bounds__(kWarps * 32) sr_direct_group_kernel(const __grid_constant__ DirectParams P)
 {
     __shared__ int2 tab[kTab];
@@ -675,7 +688,7 @@ __global__ void __launch_bounds__(kWarps * 32) sr_direct_group_kernel(const __gr
     if (nd.H == 1 && nd.W == 1 && P.edges[nd.first_edge].kind != SR_EDGE_CONV) dense_item<T>(nd, P.edges, it, prev, cur, P.B, out);
     // (As two tests joined by ||, or a mark in the item, this took the compiler from 96 registers to 128, and 3 -> 32 channels of
     // 32 x 32 at 64 samples, fp32, from 171 us for eight frames to 202.)
-    else if ((nd.C | nd.untiled) % 4 != 0) conv_item<T>(nd, P.edges, it, prev, cur, out);
+    else if ((nd.C | nd.untiled) % 4 != 0) conv_item<T, NON_FINITE>(nd, P.edges, it, prev, cur, out);
     else if (it.b0 >= 0) conv_tile<T, 1>(nd, P.edges, it, prev, cur, out, tab);
     else {
         SrDirectItem four = it;
@@ -698,8 +711,11 @@ int sr_launch_direct_group(const sr_graph* g, int group, SrFollow how, cudaStrea
     P.items = reinterpret_cast<const SrDirectItem*>(g->ws + g->r_items.offset) + g->group_item_offset[group];
     P.B = g->batch;
     P.follow = how.flags();
-    if (g->dtype == SR_DTYPE_BF16) sr_launch(sr_direct_group_kernel<__nv_bfloat16>, n, kWarps * 32, 0, s, how.early, P);
-    else sr_launch(sr_direct_group_kernel<float>, n, kWarps * 32, 0, s, how.early, P);
+    bool finite = true;
+    for (int v : g->groups[group]) finite = finite && g->nodes[v].w_finite;
+    sr_launch(g->dtype == SR_DTYPE_BF16 ? sr_direct_group_kernel<__nv_bfloat16, true>
+                                        : finite ? sr_direct_group_kernel<float, false> : sr_direct_group_kernel<float, true>,
+              n, kWarps * 32, 0, s, how.early, P);
     return 1;
 }
 
@@ -932,5 +948,5 @@ bool sr_direct_share_sm()
                ask(sr_mean_head_kernel<__nv_bfloat16, beside>);
     };
     return heads(std::false_type()) && heads(std::true_type()) && ask(sr_wide_head_kernel<__nv_bfloat16, 1>) &&
-           ask(sr_wide_head_kernel<__nv_bfloat16, kWideQ>) && ask(sr_direct_group_kernel<__nv_bfloat16>);
+           ask(sr_wide_head_kernel<__nv_bfloat16, kWideQ>) && ask(sr_direct_group_kernel<__nv_bfloat16, true>);
 }

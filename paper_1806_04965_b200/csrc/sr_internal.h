@@ -29,7 +29,7 @@ struct SrDevNode {
     int32_t H, W, C, act;
     int32_t first_edge, n_edges;     // range in the SrDevEdge table
     int32_t is_output;
-    int32_t untiled;                 // conv nodes: 1 if conv_item takes them
+    int32_t untiled;                 // conv nodes: 0: conv_tile takes them; 1: conv_item; 2: conv_item on conv_tile's items
 };
 
 // One block's work in a grouped direct launch.
@@ -202,6 +202,7 @@ struct SrHostNode {
     std::vector<int> in_edges;
     bool dense_target = false;     // all incoming edges are dense / mean-dense
     bool use_tc = false;
+    bool w_finite = true;          // every weight of the incoming edges is finite (nodes of the CUDA-core kernels)
     SrRegion state[2], bias;
     bool bias_set = false;
 };
@@ -212,7 +213,7 @@ struct SrHostEdge {
     // the convolution actually executed (pooled edges are rewritten)
     int k_eff = 0, stride_eff = 0, pad_eff = 0, K = 0;
     SrRegion w_direct;
-    bool w_set = false;
+    bool w_set = false, w_finite = true;
 };
 
 // A few-channel input edge staged as im2col rows (see sr_input.cu).

@@ -382,3 +382,35 @@ def test_cuda_core_convolution_of_a_sample_beyond_32_bit_offsets():
     want = torch.einsum("hwc,oc->hwo", sub.float(), torch.from_numpy(w.reshape(8, 4)).to("cuda:0").to(torch.bfloat16).float())
     got = G.get_state(1)[0].float()
     assert float((got - want).abs().max()) <= 1e-2 * float(want.abs().max())
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("batch,size,cin,c", [(2, 5, 3, 4), (2, 7, 8, 132), (130, 16, 4, 64)])
+def test_infinite_weights_leave_pixels_alone_whose_window_they_miss(batch, size, cin, c, dtype):
+    # the weight of a corner tap is infinite: the first row and column, for which that tap lies outside the image, stay finite, with one
+    # and (the last case) four pixels per thread; finite weights afterwards bring the usual results back
+    import torch
+    from oracle import frame_update as fu
+    from workloads.graphs import CONV, GAP_DENSE, IDENTITY, Edge, GraphSpec, Node, check_shapes
+    nodes = [Node("in", size, size, cin, IDENTITY), Node("a", size, size, c, IDENTITY), Node("o", 1, 1, 3, IDENTITY)]
+    g = GraphSpec("inf", nodes, [Edge(0, 1, CONV, 3, 1), Edge(0, 1, CONV, 1, 1), Edge(1, 2, GAP_DENSE)], batch=batch, frames=1, dtype=dtype, seed=97)
+    check_shapes(g)
+    g.patterns = {"p": [1, 1, 1]}
+    X, W, Bi = data.make_inputs(g), data.make_weights(g), data.make_biases(g, zero=False)
+    bad = [w.copy() for w in W]
+    bad[0][c - 1, 0, 0, cin - 1] = np.inf
+    G = parity.make_graph(g, "p", "direct", 1, W, Bi)
+    x = parity.to_device(g, X[0])
+    samples = [0, batch - 1]
+    for weights in (W, bad, W):
+        with np.errstate(invalid="ignore"):
+            want = fu.rollout_spec(g, "p", X, weights, Bi, samples=samples)[1][1]
+        G.set_weights(weights)
+        G.reset([x[0]])
+        G.run([x[1:2]])                                 # (recorded in a CUDA graph)
+        G.sync_status()
+        got = G.get_state(1).float().cpu().numpy()[samples].reshape(want.shape)
+        finite = np.isfinite(want)
+        assert finite.all() == (weights is W) and np.array_equal(np.isfinite(got), finite)
+        assert np.array_equal(got[~finite], want[~finite].astype(np.float32), equal_nan=True)
+        assert parity.rel_err(got[finite], want[finite]) <= parity.TOL[dtype]
