@@ -174,13 +174,15 @@ sr_status sr_graph_set_node_bias(sr_graph* g, int node, const float* bias_host);
  *           key 5 "kernel timing": 1 brackets every tensor-core group launch and every resident launch with CUDA
  *                  events on the launching stream (plain launches only, not inside CUDA graphs); read with
  *                  sr_graph_kernel_time.
- *           key 6 "resident": 1 (default) lets sr_rollout_run use the resident kernel when the network qualifies
- *                  (bfloat16; per-sequence states and convolution weights fit in the shared memory of a
- *                  thread-block cluster): one cluster per sequence walks all T frames in one launch with
- *                  the states on chip; 0 = always the per-frame launch path.  sr_rollout_step always uses
- *                  the launch path.
- *           key 7 "resident cluster size": CTAs per sequence, 1, 2 or 4; 0 (default) = chosen by the library.
- *           key 8 "resident warps": warps per CTA of the resident kernel, 4..32; 0 = default.
+ *           key 6 "resident": 1 (default) lets sr_rollout_run use a resident kernel when the network qualifies: all T
+ *                  frames in one launch with weights and states in the shared memory of thread-block clusters.
+ *                  bfloat16 networks of convolutions with dense heads: one cluster per sequence.  float networks of
+ *                  dense edges only: one cluster per two, four or eight sequences, if every input frame starts on a 16-byte
+ *                  boundary; sr_rollout_step uses that one too while the device holds all clusters of the batch at
+ *                  once.  0 = always the per-frame launch path.
+ *           key 7 "resident cluster size": CTAs per sequence of the bfloat16 kernel, 1, 2 or 4; 0 (default) = chosen by the
+ *                  library.
+ *           key 8 "resident warps": warps per CTA of the bfloat16 kernel, 4..32; 0 = default.
  *           key 9 "resident tile width": 0 (default) = 16-pixel x 32-channel work units only, 1 = 16-channel units for
  *                  every convolutional node, 2 = 16-channel units for the nodes whose 32-channel unit would be the
  *                  longest dependent chain of a frame (more, shorter units; they load the activations twice).

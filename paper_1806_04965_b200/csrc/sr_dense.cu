@@ -688,7 +688,8 @@ sr_status sr_dn_plan(sr_graph* g, size_t& offset)
     if (!E) E = dn_build(g, 8, kDnMaxSamples);
     // Fewer sequences per cluster shorten a frame, because the loads of the states shrink with them: per frame of one wave of that
     // network 1.45, 1.87 and 2.50 us with two, four and eight sequences and sixteen CTAs, 2.19, 2.79 and 3.68 with eight CTAs
-    // (sequential 3.3, 4.2, 5.4).  The split whose waves end first by these ratios is taken.
+    // (sequential 3.3, 4.2, 5.4).  The split whose waves end first by these ratios is taken.  (They are that network's.  Networks of
+    // 64- and 256-wide layers at 1 to 512 sequences were faster by this rule than with eight sequences per cluster throughout.)
     if (E) {
         const int cl = E->cluster;
         double best = 0.0;

@@ -17,10 +17,10 @@
 //     gathered by ldmatrix straight from the NHWC state (one row address per lane = one pixel of one
 //     filter tap; out-of-image taps point at a zero line), the B fragments come from weights packed
 //     per k-step in ldmatrix order.  The sum over incoming edges is one accumulator walked over the
-//     k-steps of all edges (the concatenated-convolution view of Sec. A).  Tiles of 16 pixels of ONE
-//     sample are far below the size the tcgen05 pipe needs to pay off (an instruction with M = 128
-//     costs >= 110 cycles however few columns it has), which is why this engine uses the warp-level
-//     tensor path and the batch-tiled tcgen05 kernel serves the large networks.
+//     k-steps of all edges (the concatenated-convolution view of Sec. A).  The multiplies alone would be cheaper on tcgen05
+//     (an instruction with M = 128 costs 48 cycles at 64 columns: about 4 k cycles per CTA and frame of the small CNN, of 12 k
+//     that the frame takes); its operands would not: every state in the swizzled K-major layout, once per stride's residue
+//     class, with halo rows, written by an epilogue from tensor memory.
 //   * Few-channel edges (C_in * k * k <= 64, the first layer of an image network) build their A
 //     fragments from scalar shared-memory loads through a small per-edge lookup table; a node fed by one such edge only takes
 //     up to four tiles to a unit (rs_few_unit).

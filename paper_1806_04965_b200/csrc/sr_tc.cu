@@ -17,7 +17,7 @@
 // a dense box.  The node's weight matrix [C_out][K] (K-major) keeps its columns in the order the K loop
 // walks them, so that consecutive K-blocks of equal width are one 3-D tensor and a weight group (one slot of
 // the weight ring) is ONE TMA copy.  Few-channel input edges (C_in = 1 or 3) are staged per frame into an im2col
-// tensor with K padded to 16/32/64 so that they are ordinary K-blocks.
+// tensor with K padded to 16/32/64/128 so that they are ordinary K-blocks.
 //
 // Pixel tile.  A tile is tb samples x th rows x (8 * nl) columns; its nl "lanes" of 8 columns lie side by side in one
 // activation box and in one accumulator of up to 256 TMEM columns, and share every weight block (nl MMAs per K = 16
@@ -36,7 +36,7 @@
 // memory ahead of time); warp 0 = weight producer (a ring of equal slots); warp 3 = activation producer (a ring of bytes:
 // boxes differ in size); warp 1 = MMA issuer (owns TMEM; one host-made record per eight or so MMAs); warps 4..11 = epilogue
 // (TMEM lane = output channel; bias, ReLU, bf16, NHWC stores in which a warp writes 32 consecutive channels of one pixel).
-// Every wait is bounded; on expiry the kernel records an error in the frame control block, waits for its own copies, frees
+// Every wait is bounded; on expiry the kernel sets the graph's error word, waits for its own copies, frees
 // TMEM and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
