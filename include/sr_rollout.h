@@ -49,7 +49,8 @@ typedef struct sr_graph sr_graph;          /* opaque; owned by the library */
 
 typedef enum {
     SR_OK = 0,
-    SR_ERR_INVALID_ARG = 1,        /* null pointer, index out of range, bad size                      */
+    SR_ERR_INVALID_ARG = 1,        /* null pointer, index out of range, bad size (also one that the host's
+                                      memory does not hold)                                           */
     SR_ERR_NOT_A_NETWORK = 2,      /* |E| = 0 or not input-connected (Sec. 3, Definition "network")   */
     SR_ERR_INVALID_ROLLOUT = 3,    /* the rollout window of R has a cycle (Sec. 3, validity)          */
     SR_ERR_SHAPE_MISMATCH = 4,     /* an edge does not map its source shape to its target shape       */

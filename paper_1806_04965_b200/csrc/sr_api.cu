@@ -294,6 +294,9 @@ bool dense_resident_takes(const sr_graph* g, const void* const* in_dev)
 
 }  // namespace
 
+// No exception leaves a C entry: what can throw here is the host's memory, for a size that it does not hold.
+#define SR_NOTHROW catch (...) { return SR_ERR_INVALID_ARG; }
+
 extern "C" {
 
 sr_status sr_graph_create(const sr_node_desc* nodes, int n_nodes, const sr_edge_desc* edges, int n_edges,
@@ -302,7 +305,11 @@ sr_status sr_graph_create(const sr_node_desc* nodes, int n_nodes, const sr_edge_
     if (!out || batch < 0 || (dtype != SR_DTYPE_F32 && dtype != SR_DTYPE_BF16)) return SR_ERR_INVALID_ARG;
     sr_graph* g = new (std::nothrow) sr_graph();
     if (!g) return SR_ERR_INVALID_ARG;
-    const sr_status st = sr_compile(g, nodes, n_nodes, edges, n_edges, R);
+    sr_status st = SR_ERR_INVALID_ARG;
+    try {
+        st = sr_compile(g, nodes, n_nodes, edges, n_edges, R);
+    } catch (...) {
+    }
     if (st != SR_OK) {
         delete g;
         return st;
@@ -437,7 +444,7 @@ sr_status sr_graph_set_option(sr_graph* g, int key, int value)
 }
 
 sr_status sr_graph_workspace_bytes(const sr_graph* g, size_t* bytes)
-{
+try {
     if (!g || !bytes) return SR_ERR_INVALID_ARG;
     if (g->ws) {
         *bytes = g->ws_bytes;
@@ -447,10 +454,10 @@ sr_status sr_graph_workspace_bytes(const sr_graph* g, size_t* bytes)
     if (st != SR_OK) return st;
     *bytes = g->ws_bytes;
     return SR_OK;
-}
+} SR_NOTHROW
 
 sr_status sr_graph_bind_workspace(sr_graph* g, void* workspace_dev, size_t bytes)
-{
+try {
     if (!g || !workspace_dev) return SR_ERR_INVALID_ARG;
     if (g->ws) return SR_ERR_STATE;
     if (reinterpret_cast<uintptr_t>(workspace_dev) & 255) return SR_ERR_INVALID_ARG;
@@ -519,6 +526,9 @@ sr_status sr_graph_bind_workspace(sr_graph* g, void* workspace_dev, size_t bytes
     g->t = 0;
     g->in_window.assign(g->nodes.size(), 0);
     return SR_OK;
+} catch (...) {
+    g->ws = nullptr;                                     // (a bound graph is refused before anything can throw)
+    return SR_ERR_INVALID_ARG;
 }
 
 sr_status sr_graph_bind_static_workspace(sr_graph* g)
@@ -548,7 +558,7 @@ sr_status sr_graph_bind_static_workspace(sr_graph* g)
 }
 
 sr_status sr_graph_set_edge_weights(sr_graph* g, int edge, const float* w, int is_device)
-{
+try {
     if (!g || !w || edge < 0 || edge >= (int)g->edges.size()) return SR_ERR_INVALID_ARG;
     if (!g->ws) return SR_ERR_STATE;
     SrHostEdge& he = g->edges[edge];
@@ -617,10 +627,10 @@ sr_status sr_graph_set_edge_weights(sr_graph* g, int edge, const float* w, int i
     }
     he.w_set = true;
     return SR_OK;
-}
+} SR_NOTHROW
 
 sr_status sr_graph_set_node_bias(sr_graph* g, int node, const float* bias_host)
-{
+try {
     if (!g || !bias_host || node < 0 || node >= (int)g->nodes.size()) return SR_ERR_INVALID_ARG;
     if (!g->ws) return SR_ERR_STATE;
     SrHostNode& n = g->nodes[node];
@@ -630,7 +640,7 @@ sr_status sr_graph_set_node_bias(sr_graph* g, int node, const float* bias_host)
     if (g->kept_bias.size() != g->nodes.size()) g->kept_bias.assign(g->nodes.size(), std::vector<float>());
     g->kept_bias[node].assign(bias_host, bias_host + n.d.c);
     return SR_OK;
-}
+} SR_NOTHROW
 
 sr_status sr_graph_reset(sr_graph* g, const void* const* in0_dev, void* stream)
 {
@@ -656,7 +666,7 @@ sr_status sr_graph_reset(sr_graph* g, const void* const* in0_dev, void* stream)
 }
 
 sr_status sr_rollout_step(sr_graph* g, const void* const* in_next_dev, float* out_dev, void* stream)
-{
+try {
     sr_status st = ready(g);
     if (st != SR_OK) return st;
     if (!in_next_dev) return SR_ERR_INVALID_ARG;
@@ -679,10 +689,10 @@ sr_status sr_rollout_step(sr_graph* g, const void* const* in_next_dev, float* ou
     g->t += 1;
     leave_window(g);
     return cuda_ok(cudaGetLastError()) ? SR_OK : SR_ERR_CUDA;
-}
+} SR_NOTHROW
 
 sr_status sr_rollout_run(sr_graph* g, const void* const* in_seq_dev, int T, float* out_seq_dev, void* stream)
-{
+try {
     sr_status st = ready(g);
     if (st != SR_OK) return st;
     if (!in_seq_dev || T < 0) return SR_ERR_INVALID_ARG;
@@ -769,15 +779,15 @@ sr_status sr_rollout_run(sr_graph* g, const void* const* in_seq_dev, int T, floa
     }
     g->t += T;
     return cuda_ok(cudaGetLastError()) ? SR_OK : SR_ERR_CUDA;
-}
+} SR_NOTHROW
 
 // ------------------------------------------------------------------ deep windows (W > 1)
 sr_status sr_graph_window_tableau(const sr_graph* g, int W, int32_t* T_host)
-{
+try {
     if (!g || !T_host || W < 1 || W > 4096) return SR_ERR_INVALID_ARG;
     sr_window_tableau(g, W, T_host);
     return SR_OK;
-}
+} SR_NOTHROW
 
 static bool frames_independent(const sr_graph* g)
 {
@@ -787,7 +797,7 @@ static bool frames_independent(const sr_graph* g)
 }
 
 sr_status sr_graph_window_workspace_bytes(sr_graph* g, int W, size_t* bytes)
-{
+try {
     if (!g || !bytes || W < 1 || W > 4096) return SR_ERR_INVALID_ARG;
     if (g->batch <= 0) return SR_ERR_STATE;
     if (!frames_independent(g)) return SR_ERR_UNSUPPORTED;
@@ -820,10 +830,10 @@ sr_status sr_graph_window_workspace_bytes(sr_graph* g, int W, size_t* bytes)
         g->window_frames = W;
     }
     return sr_graph_workspace_bytes(g->window, bytes);
-}
+} SR_NOTHROW
 
 sr_status sr_graph_bind_window(sr_graph* g, int W, void* workspace_dev, size_t bytes)
-{
+try {
     if (!g || !workspace_dev) return SR_ERR_INVALID_ARG;
     sr_status st = ready(g);
     if (st != SR_OK) return st;
@@ -844,10 +854,10 @@ sr_status sr_graph_bind_window(sr_graph* g, int W, void* workspace_dev, size_t b
             if (st != SR_OK) return st;
         }
     return SR_OK;
-}
+} SR_NOTHROW
 
 sr_status sr_rollout_window(sr_graph* g, const void* const* in_seq_dev, int W, float* out_seq_dev, void* stream)
-{
+try {
     sr_status st = ready(g);
     if (st != SR_OK) return st;
     sr_graph* w = g->window;
@@ -888,7 +898,7 @@ sr_status sr_rollout_window(sr_graph* g, const void* const* in_seq_dev, int W, f
     g->launches += w->launches;
     w->launches = 0;
     return cuda_ok(cudaGetLastError()) ? SR_OK : SR_ERR_CUDA;
-}
+} SR_NOTHROW
 
 sr_status sr_graph_get_state(const sr_graph* g, int node, void* dst_dev, void* stream)
 {

@@ -154,3 +154,27 @@ def test_window_tableau_matches_the_oracle_for_every_window_size():
     assert all(T[i] == T[1] for i in range(1, 9)) and max(T[8]) == G.info["inference_factor"] == 8
     S = Graph(g.nodes, g.edges, g.patterns["streaming"], batch=0)
     assert max(S.window_tableau(8)[8]) == 8 and S.window_tableau(8)[3][len(g.nodes) - 1] == 3
+
+
+def test_a_size_beyond_the_hosts_memory_is_an_error_not_an_abort():
+    # a child process with 4 GiB of address space: the work lists of 2^30 samples do not fit; the graph stays usable as an object
+    import subprocess
+    import sys
+    code = """
+import ctypes, resource, sys
+sys.path.insert(0, %r)
+from paper_1806_04965_b200 import load_library
+from paper_1806_04965_b200.binding import _EdgeDesc, _NodeDesc
+lib = load_library()
+resource.setrlimit(resource.RLIMIT_AS, (4 << 30, 4 << 30))
+n = (_NodeDesc * 3)(_NodeDesc(4, 4, 4, 0), _NodeDesc(4, 4, 5, 1), _NodeDesc(1, 1, 2, 0))
+e = (_EdgeDesc * 2)(_EdgeDesc(0, 1, 0, 1, 1, 0), _EdgeDesc(1, 2, 2, 1, 1, 0))
+h, size = ctypes.c_void_p(), ctypes.c_size_t()
+assert lib.sr_graph_create(n, 3, e, 2, (ctypes.c_uint8 * 2)(1, 1), 1 << 30, 0, ctypes.byref(h)) == 0
+for _ in range(2):
+    assert lib.sr_graph_workspace_bytes(h, ctypes.byref(size)) == 1
+lib.sr_graph_destroy(h)
+print("ok")
+""" % ROOT
+    out = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0 and out.stdout.strip() == "ok", (out.returncode, out.stderr[-500:])
