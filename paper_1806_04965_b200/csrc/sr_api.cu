@@ -609,7 +609,7 @@ try {
         he.w_finite = std::all_of(src, src + (size_t)he.K * Cout, [](float v) { return std::isfinite(v); });
         const bool finite = std::all_of(t.in_edges.begin(), t.in_edges.end(), [&](int e) { return g->edges[e].w_finite; });
         if (finite != t.w_finite) {
-            const int32_t untiled = sr_direct_untiled(g, he.d.tgt) ? 1 : finite ? 0 : 2;
+            const int32_t untiled = sr_direct_untiled(g, he.d.tgt) ? 1 : finite ? 0 : g->dtype == SR_DTYPE_BF16 ? 2 : 4;
             if (!cuda_ok(cudaMemcpy(g->ws + g->r_nodes.offset + sizeof(SrDevNode) * he.d.tgt + offsetof(SrDevNode, untiled), &untiled, sizeof(untiled),
                                     cudaMemcpyHostToDevice)))
                 return SR_ERR_CUDA;

@@ -76,7 +76,7 @@ __device__ void conv_item(const SrDevNode& nd, const SrDevEdge* edges, const SrD
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int HW = nd.H * nd.W;
     int b = it.b0, n_pix = kWarps * kPix, c_first = 0, c_end = nd.C;
-    if (ANY_ITEM && nd.untiled == 2) {                                                       // conv_tile's items: pixels and channels of their own
+    if (ANY_ITEM && nd.untiled == (sizeof(T) == 2 ? 2 : 4)) {                                                       // conv_tile's items: pixels and channels of their own
         const int qlog = it.pad_ >> 24;
         b = it.b0 < 0 ? ~it.b0 : it.b0;
         n_pix = (kWarps * 32 >> qlog) * (it.b0 < 0 ? 4 : 1);
@@ -673,7 +673,8 @@ struct DirectParams {
 
 // NON_FINITE: nodes may have a weight that is not finite.  In fp32 a kernel of its own, because the compiler's choices for the tiled
 // convolutions change with everything beside them (32 -> 32 channels of 32 x 32, 64 samples: 570 us for eight frames, 626 in the
-// kernel that takes both); bf16 is as fast either way.
+// kernel that takes both); bf16 is as fast either way.  A launch that a caller recorded before the weight came keeps its kernel, and
+// its tiles.
 template <typename T, bool NON_FINITE>
 __global__ void __launch_bounds__(kWarps * 32) sr_direct_group_kernel(const __grid_constant__ DirectParams P)
 {
@@ -688,7 +689,7 @@ __global__ void __launch_bounds__(kWarps * 32) sr_direct_group_kernel(const __gr
     if (nd.H == 1 && nd.W == 1 && P.edges[nd.first_edge].kind != SR_EDGE_CONV) dense_item<T>(nd, P.edges, it, prev, cur, P.B, out);
     // (As two tests joined by ||, or a mark in the item, this took the compiler from 96 registers to 128, and 3 -> 32 channels of
     // 32 x 32 at 64 samples, fp32, from 171 us for eight frames to 202.)
-    else if ((nd.C | nd.untiled) % 4 != 0) conv_item<T, NON_FINITE>(nd, P.edges, it, prev, cur, out);
+    else if ((nd.C | nd.untiled | (NON_FINITE && sizeof(T) == 4 ? nd.untiled >> 2 : 0)) % 4 != 0) conv_item<T, NON_FINITE>(nd, P.edges, it, prev, cur, out);
     else if (it.b0 >= 0) conv_tile<T, 1>(nd, P.edges, it, prev, cur, out, tab);
     else {
         SrDirectItem four = it;

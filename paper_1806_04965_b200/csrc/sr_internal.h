@@ -29,7 +29,8 @@ struct SrDevNode {
     int32_t H, W, C, act;
     int32_t first_edge, n_edges;     // range in the SrDevEdge table
     int32_t is_output;
-    int32_t untiled;                 // conv nodes: 0: conv_tile takes them; 1: conv_item; 2: conv_item on conv_tile's items
+    int32_t untiled;                 // conv nodes: 0: conv_tile takes them; 1: conv_item; 2 (bf16), 4 (fp32): conv_item on
+                                     // conv_tile's items, in the kernel for weights that are not finite
 };
 
 // One block's work in a grouped direct launch.

@@ -414,3 +414,21 @@ def test_infinite_weights_leave_pixels_alone_whose_window_they_miss(batch, size,
         assert finite.all() == (weights is W) and np.array_equal(np.isfinite(got), finite)
         assert np.array_equal(got[~finite], want[~finite].astype(np.float32), equal_nan=True)
         assert parity.rel_err(got[finite], want[finite]) <= parity.TOL[dtype]
+    # a pass that the caller recorded with finite weights keeps its kernel: pixels inside the image come out as they should
+    out = torch.empty((1,) + G.out_shape(), dtype=torch.float32, device="cuda:0")
+    G.set_option(1, 0)
+    stream, recorded = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(recorded, stream=stream):
+        G.reset([x[0]])
+        G.run([x[1:2]], out)
+    G.set_weights(bad)
+    recorded.replay()
+    torch.cuda.synchronize()
+    with np.errstate(invalid="ignore"):
+        want = fu.rollout_spec(g, "p", X, bad, Bi, samples=samples)[1][1]
+    got = G.get_state(1).float().cpu().numpy()[samples].reshape(want.shape)
+    inside = np.isfinite(want)
+    inside[:, 0] = inside[:, :, 0] = False
+    assert parity.rel_err(got[inside], want[inside]) <= parity.TOL[dtype]
+    del recorded
