@@ -124,17 +124,19 @@ struct alignas(16) TcNode {
     int32_t tw, th, tb, sep;        // geometry of the tile (see the file comment): tw = columns of a lane
     int32_t nl, lane_cols;          // lanes, TMEM columns of each (N of the MMA)
     int32_t n_runs, n_act, n_bu;    // lengths of the node's tables
-    int32_t table_off;              // 16-byte words from the start of the table area: bursts, then activation boxes
+    int32_t pad_;
     uint32_t pairs[4];              // bit i: weight group i of the node has two blocks
     TcRun runs[kMaxRuns];
 };
 static_assert(sizeof(TcNode) % 16 == 0, "copied as 16-byte words");
 
-struct alignas(16) TcTile { int32_t node, b0, h0, w0, m0, slot, pad_[2]; };   // m0: first output channel; slot: node table (set by the keeper)
+// node: where its table begins, in 16-byte words from the start of the table area (on the host, until a workspace is bound: its plan):
+// a TcNode, bursts, activation boxes; words: how many it has.  m0: first output channel; slot: of the table in shared memory (set by
+// the keeper)
+struct alignas(16) TcTile { int32_t node, b0, h0, w0, m0, slot, words, pad_; };
 
 struct TcParams {
     const CUtensorMap* maps;
-    const TcNode* nodes;
     const uint4* tables;
     const TcTile* tiles;
     SrFrameArgs fr;
@@ -346,6 +348,10 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&tmem_slot)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    // (the keeper's first item is on its way meanwhile)
+    TcTile first;
+    first.node = -1;
+    if (warp == 2 && (int)blockIdx.x < P.n_own) first = P.tiles[blockIdx.x];
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -368,7 +374,8 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
             tl.node = -1;
             if (own) {
                 const long long idx = (long long)blockIdx.x + (long long)it * gridDim.x;
-                if (idx < P.n_own) tl = P.tiles[idx];
+                if (it == 0) tl = first;
+                else if (idx < P.n_own) tl = P.tiles[idx];
                 own = tl.node >= 0;                        // the rest of this CTA's column is padding
             }
             // room in the item ring (and, for an item of the shared list, not too far ahead)
@@ -417,11 +424,8 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) { *abortp = 1; break; }
                     uint4* dst = reinterpret_cast<uint4*>(smem_raw + tab_off + slot * P.table_bytes);
-                    const uint4* nd = reinterpret_cast<const uint4*>(P.nodes + tl.node);
-                    const uint4* tb = P.tables + P.nodes[tl.node].table_off;
-                    const int n_tab = 2 * P.nodes[tl.node].n_bu + P.nodes[tl.node].n_act;
-                    for (int i = lane; i < (int)(sizeof(TcNode) / 16); i += 32) dst[i] = nd[i];
-                    for (int i = lane; i < n_tab; i += 32) dst[sizeof(TcNode) / 16 + i] = tb[i];
+                    const uint4* src = P.tables + tl.node;
+                    for (int i = lane; i < tl.words; i += 32) dst[i] = src[i];
                     if (lane == slot) slot_node = tl.node;
                 }
                 cached = tl.node;
@@ -487,9 +491,10 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
         // Box j uses barrier pair j % kBoxes and the bytes [pos, pos + size) of the ring; it wraps as a whole.  `head` counts KiB
         // from the start of the launch, skipped ones included: head minus the start of the oldest box is what is in use.
         // (The weights do not depend on the predecessor, so their producer does not wait for it; the activations do.)
-        sr_wait_for_predecessor();
-        if (P.follow & 2) sr_let_successor_start();
+        // Everything up to the first request is done ahead of that wait: tables read, tensor map and instructions fetched (from the
+        // end of the wait to the request 0.4-0.6 us without that, 0.05-0.2 so).
         if (elect_one()) {
+            bool waited = false;
             uint32_t n = 0, n_free = 0;                           // boxes started; boxes known to be released
             uint32_t pos = 0, head = 0;
             const uint32_t ring = (uint32_t)P.ring_kb;
@@ -516,8 +521,15 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                     }
                     if (!ok) break;
                     const int par = (k.flags & 1) ? prev : cur;
+                    const CUtensorMap* map = &P.maps[par ? k.x_map1 : k.x_map0];
+                    if (!waited) {
+                        asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
+                        sr_wait_for_predecessor();
+                        if (P.follow & 2) sr_let_successor_start();
+                        waited = true;
+                    }
                     mbar_expect_tx(bar_afull + 8 * s, (uint32_t)k.x_bytes16 << 4);
-                    tma_load_4d(a_ring + pos * 1024u, &P.maps[par ? k.x_map1 : k.x_map0], bar_afull + 8 * s, (int)k.c0_16 << 4, w0 + k.qx, h0 + k.qy, b0);
+                    tma_load_4d(a_ring + pos * 1024u, map, bar_afull + 8 * s, (int)k.c0_16 << 4, w0 + k.qx, h0 + k.qy, b0);
                     box_start[s] = head;
                     head += size;
                     pos += size;
@@ -538,6 +550,10 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                         tma_prefetch_4d(&P.maps[pp ? p.x_map1 : p.x_map0], (int)p.c0_16 << 4, pw + p.qx, ph + p.qy, pb);
                     }
                 }
+            }
+            if (!waited) {
+                sr_wait_for_predecessor();
+                if (P.follow & 2) sr_let_successor_start();
             }
             for (uint32_t v = 0; v < kBoxes && v < n; ++v) mbar_wait_drain(bar_afull + 8 * v, ((n - 1 - v) / kBoxes) & 1, wait_limit);
         }
@@ -844,6 +860,7 @@ struct NodePlan {
     std::vector<KbHost> kbs;
     std::vector<WRun> runs;
     std::vector<WGroup> wgroups;
+    int table_off, table_words;     // see TcTile
     SrRegion wcat;
 };
 
@@ -860,7 +877,7 @@ struct TcEngine {
     std::vector<int> stem_of_edge;
     std::vector<std::vector<TcTile>> group_tiles;
     std::vector<int> group_tile_offset, group_grid, group_n_own, group_n_w, group_w_slot, group_ring_kb, group_table_bytes;
-    SrRegion r_maps, r_nodes, r_tables, r_tiles;
+    SrRegion r_maps, r_tables, r_tiles;
     int n_maps = 0, n_kbs = 0, n_tiles = 0;
     // optional timing of the group launches with CUDA events on the launching stream
     std::vector<cudaEvent_t> ev;             // pairs: start, stop
@@ -1105,7 +1122,7 @@ std::vector<TcTile> node_tiles(const sr_graph* g, const NodePlan& P, int node_in
     for (int b0 = 0; b0 < g->batch; b0 += P.tb)
         for (int h0 = 0; h0 < n.d.h; h0 += P.th)
             for (int w0 = 0; w0 < n.d.w; w0 += P.tw * P.nl)
-                for (int m0 = 0; m0 < P.rows_total(g); m0 += 128) out.push_back(TcTile{node_index, b0, h0, w0, m0, 0, {0, 0}});
+                for (int m0 = 0; m0 < P.rows_total(g); m0 += 128) out.push_back(TcTile{node_index, b0, h0, w0, m0, 0, 0, 0});
     return out;
 }
 
@@ -1350,7 +1367,7 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
             for (auto& l : lists) n_rows = std::max(n_rows, l.size());
             for (size_t r = 0; r < n_rows; ++r)
                 for (int c = 0; c < grid; ++c)
-                    E->group_tiles[gi].push_back(r < lists[c].size() ? lists[c][r] : TcTile{-1, 0, 0, 0, 0, 0, {0, 0}});
+                    E->group_tiles[gi].push_back(r < lists[c].size() ? lists[c][r] : TcTile{-1, 0, 0, 0, 0, 0, 0, 0});
         }
         E->group_n_own.push_back((int)E->group_tiles[gi].size());
         for (size_t i = n_matrix; i < tl.size(); ++i) E->group_tiles[gi].push_back(tl[i].second);
@@ -1371,8 +1388,7 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
     E->n_kbs = n_kbs;
     // upper bound on distinct tensor maps: two parities per K-block plus one weight map per (node, bk)
     E->r_maps = take(sizeof(CUtensorMap) * (size_t)(4 * n_kbs + 1));
-    E->r_nodes = take(sizeof(TcNode) * E->nodes.size());
-    E->r_tables = take(48 * (size_t)std::max(1, n_kbs));
+    E->r_tables = take(48 * (size_t)n_kbs + sizeof(TcNode) * E->nodes.size());
     E->r_tiles = take(sizeof(TcTile) * (size_t)std::max(1, n_tiles));
     return SR_OK;
 }
@@ -1411,9 +1427,8 @@ sr_status sr_tc_bind(sr_graph* g)
         cache[key] = (int)maps.size() - 1;
         return (int)maps.size() - 1;
     };
-    std::vector<TcNode> dn;
-    std::vector<uint4> dt;                             // per node: bursts (two words each), then activation boxes
-    for (const NodePlan& P : E->nodes) {
+    std::vector<uint4> dt;                             // per node: TcNode, bursts (two words each), activation boxes
+    for (NodePlan& P : E->nodes) {
         const SrHostNode& n = g->nodes[P.node];
         TcNode d{};
         d.state[0] = ws + n.state[0].offset;
@@ -1539,17 +1554,24 @@ sr_status sr_tc_bind(sr_graph* g)
         }
         d.n_bu = (int)db.size();
         d.n_act = (int)da.size();
-        d.table_off = (int)dt.size();
-        const size_t at = dt.size();
-        dt.resize(at + 2 * db.size() + da.size());
-        std::memcpy(dt.data() + at, db.data(), db.size() * sizeof(TcBurst));
-        std::memcpy(dt.data() + at + 2 * db.size(), da.data(), da.size() * sizeof(TcAct));
-        dn.push_back(d);
+        const size_t at = dt.size(), words = sizeof(TcNode) / 16;
+        P.table_off = (int)at;
+        P.table_words = (int)(words + 2 * db.size() + da.size());
+        dt.resize(at + P.table_words);
+        std::memcpy(dt.data() + at, &d, sizeof(d));
+        std::memcpy(dt.data() + at + words, db.data(), db.size() * sizeof(TcBurst));
+        std::memcpy(dt.data() + at + words + 2 * db.size(), da.data(), da.size() * sizeof(TcAct));
     }
     if (maps.size() * sizeof(CUtensorMap) > E->r_maps.bytes || dt.size() * sizeof(uint4) > E->r_tables.bytes) return SR_ERR_UNSUPPORTED;
     E->n_maps = (int)maps.size();
     std::vector<TcTile> tiles;
     for (auto& v : E->group_tiles) tiles.insert(tiles.end(), v.begin(), v.end());
+    for (TcTile& t : tiles)
+        if (t.node >= 0) {
+            const NodePlan& P = E->nodes[t.node];
+            t.node = P.table_off;
+            t.words = P.table_words;
+        }
     g->stems.clear();
     for (const StemPlan& S : E->stems) {
         const SrHostEdge& he = g->edges[S.edge];
@@ -1567,7 +1589,7 @@ sr_status sr_tc_bind(sr_graph* g)
     auto up = [&](const SrRegion& r, const void* p, size_t bytes) {
         return bytes == 0 || cudaMemcpy(ws + r.offset, p, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
     };
-    if (!up(E->r_maps, maps.data(), maps.size() * sizeof(CUtensorMap)) || !up(E->r_nodes, dn.data(), dn.size() * sizeof(TcNode)) ||
+    if (!up(E->r_maps, maps.data(), maps.size() * sizeof(CUtensorMap)) ||
         !up(E->r_tables, dt.data(), dt.size() * sizeof(uint4)) ||
         !up(E->r_tiles, tiles.data(), tiles.size() * sizeof(TcTile)))
         return SR_ERR_CUDA;
@@ -1648,7 +1670,6 @@ int sr_tc_launch_group(sr_graph* g, int group, SrFollow how, cudaStream_t s)
     }
     TcParams P{};
     P.maps = reinterpret_cast<const CUtensorMap*>(g->ws + E->r_maps.offset);
-    P.nodes = reinterpret_cast<const TcNode*>(g->ws + E->r_nodes.offset);
     P.tables = reinterpret_cast<const uint4*>(g->ws + E->r_tables.offset);
     P.tiles = reinterpret_cast<const TcTile*>(g->ws + E->r_tiles.offset) + E->group_tile_offset[group];
     P.fr = g->frame;
