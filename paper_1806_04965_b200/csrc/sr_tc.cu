@@ -65,6 +65,7 @@ constexpr int kTables = 3;                            // node tables in shared m
 // the SM's shared-memory partition is left (a 117 us frame then takes 170 us).
 constexpr int kSmemBudget = 204 * 1024;
 constexpr int kMaxNodeKb = 128;                       // K-blocks per node
+constexpr int kMaxParts = 8;                          // parts of an item's reduction
 
 // A run of equally wide K-blocks of a node's reduction as the weight producer sees it: n_groups weight groups (one copy
 // and one ring slot each) of one or two blocks (see TcNode::pairs).
@@ -72,6 +73,7 @@ struct TcRun {
     uint16_t map1, map2;                // tensor maps: dims (channels of a block, output channels, blocks), box of one / two blocks
     uint16_t bytes16;                   // bytes of a block's weights / 16
     uint16_t n_groups;
+    uint16_t blk0, pad_;                // the first of them
 };
 constexpr int kMaxRuns = 3;                           // block widths 64, 32, 16
 
@@ -127,13 +129,14 @@ struct alignas(16) TcNode {
     int32_t pad_;
     uint32_t pairs[4];              // bit i: weight group i of the node has two blocks
     TcRun runs[kMaxRuns];
+    int32_t part, n_parts, part_chunks;     // of a split item (see the kernel); part_chunks: 16-column chunks per part
 };
 static_assert(sizeof(TcNode) % 16 == 0, "copied as 16-byte words");
 
 // node: where its table begins, in 16-byte words from the start of the table area (on the host, until a workspace is bound: its plan):
-// a TcNode, bursts, activation boxes; words: how many it has.  m0: first output channel; slot: of the table in shared memory (set by
-// the keeper)
-struct alignas(16) TcTile { int32_t node, b0, h0, w0, m0, slot, words, pad_; };
+// a TcNode, bursts, activation boxes; words: how many it has (until then: the part of a split item).  m0: first output channel; slot:
+// of the table in shared memory (set by the keeper); rank0: the cluster rank that has part 0 of a split item
+struct alignas(16) TcTile { int32_t node, b0, h0, w0, m0, slot, words, rank0; };
 
 struct TcParams {
     const CUtensorMap* maps;
@@ -148,6 +151,7 @@ struct TcParams {
     int table_bytes;                // shared memory of one node table
     int n_w, w_slot;                // weight ring: slots and their size
     int ring_kb;                    // activation ring in KiB
+    int exch_off;                   // (SPLIT) where what other parts send lies: bytes from the start of the weight ring
 };
 
 // ------------------------------------------------------------------------------------------ PTX helpers
@@ -283,6 +287,23 @@ __device__ __forceinline__ void stmatrix_x4_trans(uint32_t addr, uint32_t a, uin
 }
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t map_rank(uint32_t local, uint32_t rank)
+{
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(rank));
+    return remote;
+}
+// A store into another CTA's shared memory that counts its bytes on a barrier there.
+__device__ __forceinline__ void st_async_v4(uint32_t remote, uint32_t remote_bar, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(remote), "r"(a), "r"(b), "r"(c), "r"(d), "r"(remote_bar) : "memory");
+}
+
 // ------------------------------------------------------------------------------------------ the kernel
 // Work items.  CTA c walks column c of a matrix of items made on the host (longest first onto the least loaded CTA).  The
 // kernel ends when its slowest CTA ends, and the cost of an item is only an estimate: measured on B200 such lists left
@@ -294,10 +315,27 @@ __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sy
 // An item of the shared list is asked for at most kAhead items ahead of the epilogue, so that a slow CTA does not hoard them.
 constexpr int kAhead = 3;
 
+// Split reductions (SPLIT: a launch in clusters).  Where a launch has fewer items than SMs, its time is that of the longest
+// reduction.  Such an item is cut along K into 2, 4 or 8 parts, one per CTA of a cluster: each part walks its K-blocks like an item
+// of its own (a TcNode of its own), with the weights and boxes of these blocks only.  The accumulators are summed through
+// distributed shared memory, every part for its share of the columns: a part sends the fp32 fragments of the others' columns to
+// them (st.async, 16 bytes per thread) and finishes its own: bias, activation, store.  The order of the sums is fixed.  A CTA has one
+// split item at most, the last of its list, so the room for what others send is used once, and one barrier, on which those bytes
+// count, is all there is between the CTAs.  Where that room would cost the weight ring its depth, it lies in the rings, which are
+// idle by then, and the parts tell each other first that they are (half a microsecond more).  Everything that others write into a
+// CTA it has waited for when it leaves.  Measured on B200, us per frame before / now: six-node network at one sample 14.3 / 8.8
+// (sequential 52.0 / 38.5), ten-node at 1 / 4 / 16 samples 22.5 / 9.8, 23.4 / 12.7, 32.5 / 26.4 (sequential at 16 110 / 94), stress graph
+// at 1 / 4 samples 34.1 / 18.9, 46.9 / 43.3 (sequential at 4 241 / 156), deepest CIFAR10 network at 1 / 16 19.8 / 7.9, 29.2 / 18.8.
+// Alternatives that lost: a cluster barrier at the end and the sums always in the rings (8.8 -> 10.5 with both); two threads that
+// start weight copies in turn (deepest CIFAR10 network at 16 samples 18.8 -> 22.5, at 128 73.8 -> 77.6); two issuing threads with an
+// accumulator each for tiles of up to 128 columns (8.8 -> 9.6); launches of half an SM's shared memory, so that the next one
+// sets up beside them (14.9 -> 22 before the split: the ring is too shallow).
+template <bool SPLIT>
 __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_constant__ TcParams P)
 {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t bars[2 * kBoxes + 2 * kMaxW + 4 + kItems];
+    __shared__ uint64_t bars[2 * kBoxes + 2 * kMaxW + 4 + kItems + 2];
+    __shared__ uint4 clear_words[SPLIT ? kMaxParts : 1];   // what the other parts of a split item say `clear` with
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     __shared__ TcTile items[kItems];                       // the item ring; node -1 = end of the list
@@ -324,6 +362,7 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
     const uint32_t bar_afull = smem_u32(&bars[0]), bar_aempty = smem_u32(&bars[kBoxes]);
     const uint32_t bar_wfull = smem_u32(&bars[2 * kBoxes]), bar_wempty = smem_u32(&bars[2 * kBoxes + kMaxW]);
     const uint32_t bar_tfull = smem_u32(&bars[2 * kBoxes + 2 * kMaxW]), bar_tempty = bar_tfull + 16, bar_item = bar_tempty + 16;
+    const uint32_t bar_sums = bar_item + 8 * kItems, bar_clear = bar_sums + 8;      // (SPLIT) what the other parts send has arrived; they may
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
@@ -341,6 +380,10 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
             mbar_init(bar_tempty + 8 * a, kEpiWarps);
         }
         for (int s = 0; s < kItems; ++s) mbar_init(bar_item + 8 * s, 1);
+        if (SPLIT) {
+            mbar_init(bar_sums, 1);
+            mbar_init(bar_clear, 1);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -353,7 +396,8 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
     first.node = -1;
     if (warp == 2 && (int)blockIdx.x < P.n_own) first = P.tiles[blockIdx.x];
     tc_fence_before();
-    __syncthreads();
+    if (SPLIT) cluster_sync();                             // (the other CTAs' barriers stand, too)
+    else __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = tmem_slot;
     volatile int* abortp = &abort_flag;
@@ -466,7 +510,7 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                     const CUtensorMap* map2 = &P.maps[R.map2];
                     const uint32_t bytes = (uint32_t)R.bytes16 << 4;
                     const int end = gi + R.n_groups;
-                    int blk = 0;
+                    int blk = R.blk0;
                     for (; gi < end; ++gi) {
                         const uint32_t two = R.map1 == R.map2 ? 0u : (nd->pairs[gi >> 5] >> (gi & 31)) & 1u;
                         if (n == n_w && !waited) {
@@ -721,7 +765,7 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
         const int st_px = lane & 7, ld_px = lane >> 2;
         const uint32_t st_addr = smem_u32(tbuf) + st_px * 64 + (((lane >> 3) ^ ((st_px >> 1) & 3)) * 16);
         const uint32_t ld_off = (uint32_t)(ld_px * 64 + (((lane & 3) ^ ((ld_px >> 1) & 3)) * 16));
-        bool ok = true;
+        bool ok = true, owed_sums = false;                              // the other parts of a split item may still send
         for (int it = 0;; ++it) {
             ok = ok && mbar_wait(bar_item + 8 * (it & (kItems - 1)), (it / kItems) & 1, abortp, wait_limit);
             const TcTile tl = items[it & (kItems - 1)];
@@ -743,6 +787,7 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
             if (et == 0) epi_done = it;                              // every warp has finished the items before this one
             if (stop) {
                 if (!ok) *abortp = 1;
+                if (SPLIT && owed_sums) mbar_wait_drain(bar_sums, 0, wait_limit);
                 break;
             }
             const uint32_t acc = (uint32_t)it & 1u;
@@ -765,12 +810,12 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * kMaxCols;
             uint32_t lo[8], hi[8];                                  // TMEM lanes 0..15 and 16..31 of the quarter
             const int c_first = half * 16;
-            if (c_first < n_cols) {
-                tc_ld_16x16(taddr + c_first, lo);
-                tc_ld_16x16(taddr + (16u << 16) + c_first, hi);
-            }
-            for (int c0 = c_first; c0 < n_cols; c0 += 32) {
-                tc_wait_ld();
+            auto fetch = [&](int c0) {
+                tc_ld_16x16(taddr + c0, lo);
+                tc_ld_16x16(taddr + (16u << 16) + c0, hi);
+            };
+            // the 32 channels x 16 pixels in lo, hi; `fetch_next` is called when their registers are free
+            auto finish = [&](int c0, auto fetch_next) {
                 uint32_t h[2][4];                                   // [8 pixels][8 channels]: two pixels of one channel per word
 #pragma unroll
                 for (int pb = 0; pb < 2; ++pb)
@@ -781,10 +826,7 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                         if (act == 1) z = __hmax2(z, __floats2bfloat162_rn(0.f, 0.f));
                         h[pb][cb] = *reinterpret_cast<const uint32_t*>(&z);
                     }
-                if (c0 + 32 < n_cols) {                             // the next chunk, on its way during the stores
-                    tc_ld_16x16(taddr + c0 + 32, lo);
-                    tc_ld_16x16(taddr + (16u << 16) + c0 + 32, hi);
-                }
+                fetch_next();
                 stmatrix_x4_trans(st_addr, h[0][0], h[0][1], h[0][2], h[0][3]);
                 stmatrix_x4_trans(st_addr + 512, h[1][0], h[1][1], h[1][2], h[1][3]);
                 __syncwarp();
@@ -797,6 +839,67 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                     }
                 }
                 __syncwarp();
+            };
+            if (SPLIT && nd->n_parts > 1) {
+                const int n_parts = nd->n_parts, me = nd->part, per = nd->part_chunks, n_chunks = n_cols / 16;
+                const int own0 = min(me * per, n_chunks), own1 = min(own0 + per, n_chunks);
+                // fragments of chunk c from part p: 8 KiB at ((p less one beyond me) * per + c - own0) * 8 KiB, of which this warp
+                // writes and reads the same 2 KiB, a thread the same 64 bytes
+                const uint32_t mine = w_ring + (uint32_t)(P.exch_off + quarter * 2048 + lane * 16);
+                owed_sums = true;
+                if (et == 0) mbar_expect_tx(bar_sums, (uint32_t)((n_parts - 1) * (own1 - own0)) * 8192u);
+                if (P.exch_off == 0) {
+                    // (into the rings, which are idle when all parts have come this far)
+                    if (et == 0) {
+                        mbar_expect_tx(bar_clear, 16u * (uint32_t)(n_parts - 1));
+                        for (int p = 0; p < n_parts; ++p)
+                            if (p != me) st_async_v4(map_rank(smem_u32(&clear_words[me]), tl.rank0 + p), map_rank(bar_clear, tl.rank0 + p), 1u, 1u, 1u, 1u);
+                    }
+                    ok = mbar_wait(bar_clear, 0, abortp, wait_limit);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) continue;
+                }
+                for (int c = half; c < n_chunks; c += 2) {
+                    const int to = c / per;
+                    if (to == me) continue;
+                    fetch(c * 16);
+                    const uint32_t dst = map_rank(mine + (uint32_t)((me < to ? me : me - 1) * per + c - to * per) * 8192u, tl.rank0 + to);
+                    const uint32_t bar = map_rank(bar_sums, tl.rank0 + to);
+                    tc_wait_ld();
+                    st_async_v4(dst, bar, lo[0], lo[1], lo[2], lo[3]);
+                    st_async_v4(dst + 512, bar, lo[4], lo[5], lo[6], lo[7]);
+                    st_async_v4(dst + 1024, bar, hi[0], hi[1], hi[2], hi[3]);
+                    st_async_v4(dst + 1536, bar, hi[4], hi[5], hi[6], hi[7]);
+                }
+                ok = mbar_wait(bar_sums, 0, abortp, wait_limit);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) continue;
+                owed_sums = false;
+                for (int c = own0 + ((own0 ^ half) & 1); c < own1; c += 2) {
+                    fetch(c * 16);
+                    tc_wait_ld();
+                    for (int p = 0; p + 1 < n_parts; ++p) {
+                        const uint4* x = reinterpret_cast<const uint4*>(smem_raw + (mine - smem_u32(smem_raw)) + (size_t)(p * per + c - own0) * 8192u);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const uint4 v = x[q * 32];
+                            uint32_t* r = (q < 2 ? lo : hi) + (q & 1) * 4;
+                            r[0] = __float_as_uint(__uint_as_float(r[0]) + __uint_as_float(v.x));
+                            r[1] = __float_as_uint(__uint_as_float(r[1]) + __uint_as_float(v.y));
+                            r[2] = __float_as_uint(__uint_as_float(r[2]) + __uint_as_float(v.z));
+                            r[3] = __float_as_uint(__uint_as_float(r[3]) + __uint_as_float(v.w));
+                        }
+                    }
+                    finish(c * 16, [] {});
+                }
+            } else {
+                if (c_first < n_cols) fetch(c_first);
+                for (int c0 = c_first; c0 < n_cols; c0 += 32) {
+                    tc_wait_ld();
+                    finish(c0, [&] {
+                        if (c0 + 32 < n_cols) fetch(c0 + 32);       // the next chunk, on its way during the stores
+                    });
+                }
             }
             tc_fence_before();
             __syncwarp();
@@ -806,6 +909,7 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
     __syncwarp();
     tc_fence_before();
     __syncthreads();
+    if (SPLIT && abort_flag) cluster_sync();               // (given up: those that have not left may still write to this CTA)
     if (threadIdx.x == 0 && abort_flag) atomicExch(P.error, 1);
     if (threadIdx.x == 0 && P.sched && P.n_own < P.n_tiles) {
         // the CTA that leaves last (none takes an item any more) puts the counters back for the next launch
@@ -839,7 +943,7 @@ struct KbHost {
     int run = 0;       // run of equally wide K-blocks this block belongs to, and its index inside the run
     int blk = 0;
     int w_off = 0;     // byte offset of this block's weights inside the group's slot
-    int ring_kb = 0;   // (loading block) KiB the box takes in the activation ring
+    int ring_kb = 0;   // KiB the box takes in the activation ring
     int row_off = 0;         // first row of `edge`'s weights in the plan's weight matrix (64: the second node of a fused plan)
     int edge2 = -1;          // fused plan: the second node's edge that shares this block (its weights take rows 64..127)
 };
@@ -859,8 +963,9 @@ struct NodePlan {
     int k_total;                    // columns of the concatenated weight matrix
     std::vector<KbHost> kbs;
     std::vector<WRun> runs;
-    std::vector<WGroup> wgroups;
-    int table_off, table_words;     // see TcTile
+    int n_parts = 1;                // parts of an item's reduction
+    struct Part { std::vector<KbHost> kbs; std::vector<WGroup> wgroups; int table_off, table_words; };   // (its table: see TcTile)
+    std::vector<Part> parts;
     SrRegion wcat;
 };
 
@@ -876,7 +981,16 @@ struct TcEngine {
     std::vector<StemPlan> stems;
     std::vector<int> stem_of_edge;
     std::vector<std::vector<TcTile>> group_tiles;
-    std::vector<int> group_tile_offset, group_grid, group_n_own, group_n_w, group_w_slot, group_ring_kb, group_table_bytes;
+    // per launch group: its items' place in the list of all, those of the matrix; grid and cluster (0: none); shared memory
+    struct Launch {
+        int first_tile = 0, n_own = 0, grid = 0, cluster = 0;
+        int n_w = 2, w_slot = 1024, ring_kb = 0, table_bytes = 0, exch = 0;      // exch: bytes for what the other parts of an item send
+        bool fits = false;
+        int rings() const { return n_w * w_slot + ring_kb * 1024 + kTables * table_bytes; }
+        int exch_off() const { return exch ? rings() : 0; }                      // 0: in the rings
+        size_t smem() const { return (size_t)rings() + exch + 1024; }
+    };
+    std::vector<Launch> launches;
     SrRegion r_maps, r_tables, r_tiles;
     int n_maps = 0, n_kbs = 0, n_tiles = 0;
     // optional timing of the group launches with CUDA events on the launching stream
@@ -924,6 +1038,10 @@ uint32_t desc_hi_of(int bk)
     const uint32_t layout = bk == 64 ? 2u : (bk == 32 ? 4u : 6u);        // 128B / 64B / 32B swizzle
     return sbo | (1u << 14) | (layout << 29);
 }
+
+// A launch on more than half of the SMs cannot set up its CTAs while the one before it runs: about as many cycles later.  One in
+// clusters starts up later than one without.
+constexpr long long kLateStart = 4000, kClusterStart = 1000;
 
 // Cycles of one MMA (M = 128, K = 16) of n columns, measured on B200 (see the file comment).
 double mma_cycles(int n) { return std::max(n / 2.0, (128 + n) / 4.0); }
@@ -1075,20 +1193,37 @@ void build_kblocks(const sr_graph* g, const TcEngine* E, NodePlan& P)
                         kb.box_rx = cl.first.second;
                         P.kbs.push_back(kb);
                     }
-                    P.kbs[first].ring_kb = ring_kb(P.kbs[first], max_shift);
+                    const int kb = ring_kb(P.kbs[first], max_shift);
+                    for (size_t i = first; i < P.kbs.size(); ++i) P.kbs[i].ring_kb = kb;
                 }
         }
     }
 }
 
+// Cycles of a K-block: those of its MMAs or of its copies (at 60 bytes per cycle), whichever are more; in a launch of few items
+// (ring_cycles > 0, see below) also at least its share of the time in which a slot of the weight ring comes round, and of the
+// issuing thread's work (720 cycles for two weight slots).
+double kb_cycles(const sr_graph* g, const NodePlan& P, const KbHost& kb, double ring_cycles)
+{
+    const double w_bytes = std::min(P.rows_total(g), 128) * 2.0;
+    const double c = std::max((kb.bk / 16) * P.nl * mma_cycles(P.lane_cols), (w_bytes * kb.bk + (kb.x_load ? kb.ring_kb * 1024.0 : 0.0)) / 60.0);
+    return ring_cycles > 0 ? std::max(c, (kb.bk == 64 ? 1.0 : 0.5) * std::max(330.0, ring_cycles)) : c;
+}
+// From the release of a slot to the arrival of the next weights, over the slots: 1 us, or 1.5 us where all SMs have several items.
+double ring_cycles(int n_w, bool crowded) { return (crowded ? 3000.0 : 2000.0) / n_w; }
+
 // Weight groups (one copy and one slot of the weight ring each): one K-block of 64 channels, or two narrower ones.
 // (Groups of twice the size make a ring of three slots out of one of six: with one of them in use two thirds are in
-// flight instead of five sixths.)  A group reads one activation box.
-void build_groups(NodePlan& P)
+// flight instead of five sixths.)  A group reads one activation box.  The plan's n_parts parts take about the same time each; a
+// box whose taps fall into two parts is loaded by both.
+void build_groups(const sr_graph* g, NodePlan& P)
 {
     P.runs.clear();
-    P.wgroups.clear();
+    P.parts.assign(P.n_parts, NodePlan::Part());
     int k_off = 0;
+    double total = 0, done = 0;
+    for (const KbHost& kb : P.kbs) total += kb_cycles(g, P, kb, ring_cycles(kMaxW, false));
+    size_t part = 0;
     for (size_t i = 0; i < P.kbs.size(); ++i) {
         KbHost& kb = P.kbs[i];
         kb.k_off = k_off;
@@ -1096,19 +1231,31 @@ void build_groups(NodePlan& P)
         if (P.runs.empty() || P.runs.back().bk != kb.bk) P.runs.push_back(WRun{kb.bk, kb.k_off, 0});
         kb.run = (int)P.runs.size() - 1;
         kb.blk = P.runs.back().n_blocks++;
-        if (kb.x_load || P.wgroups.back().run != kb.run || P.wgroups.back().n >= (kb.bk == 64 ? 1 : 2))
-            P.wgroups.push_back(WGroup{kb.run, kb.blk, 0, (int)i});
-        P.wgroups.back().n += 1;
+        // the next part begins here if this block's middle lies beyond this part's share, or if as many blocks are left as parts
+        const double cost = kb_cycles(g, P, kb, ring_cycles(kMaxW, false));
+        if (!P.parts[part].kbs.empty() && part + 1 < P.parts.size() &&
+            ((done + 0.5 * cost) * P.n_parts > total * (part + 1) || P.kbs.size() - i < P.parts.size() - part))
+            ++part;
+        done += cost;
+        NodePlan::Part& q = P.parts[part];
+        q.kbs.push_back(kb);
+        if (q.kbs.size() == 1 && !kb.x_load) {
+            q.kbs[0].x_load = true;
+            P.parts[part - 1].kbs.back().x_release = true;
+        }
+        if (q.kbs.back().x_load || q.wgroups.back().run != kb.run || q.wgroups.back().n >= (kb.bk == 64 ? 1 : 2))
+            q.wgroups.push_back(WGroup{kb.run, kb.blk, 0, (int)q.kbs.size() - 1});
+        q.wgroups.back().n += 1;
     }
     P.k_total = k_off;
 }
 
 // Two consecutive weight groups are one burst if their K-blocks are equally wide.
-bool one_burst(const NodePlan& P, size_t gi)
+bool one_burst(const NodePlan::Part& P, size_t gi)
 {
     return gi + 1 < P.wgroups.size() && P.kbs[P.wgroups[gi + 1].first_kb].bk == P.kbs[P.wgroups[gi].first_kb].bk;
 }
-int count_bursts(const NodePlan& P)
+int count_bursts(const NodePlan::Part& P)
 {
     int n = 0;
     for (size_t gi = 0; gi < P.wgroups.size(); ++n) gi += one_burst(P, gi) ? 2 : 1;
@@ -1126,33 +1273,117 @@ std::vector<TcTile> node_tiles(const sr_graph* g, const NodePlan& P, int node_in
     return out;
 }
 
-// Estimated cycles of one item of the plan: every K-block takes the time of its MMAs or of its weight copy (at 60 bytes per
-// cycle), plus start-up and the share of the epilogue that is not hidden.
-long long item_cycles(const sr_graph* g, const NodePlan& P)
+// Estimated cycles of one item of the plan: its K-blocks, start-up and the share of the epilogue that is not hidden.
+long long item_cycles(const sr_graph* g, const NodePlan& P, double ring_cycles)
 {
     double c = 1500.0;
-    const double w_bytes = std::min(P.rows_total(g), 128) * 2.0;
-    for (const KbHost& kb : P.kbs) c += std::max((kb.bk / 16) * P.nl * mma_cycles(P.lane_cols), (w_bytes * kb.bk + (kb.x_load ? kb.ring_kb * 1024.0 : 0.0)) / 60.0);
+    for (const KbHost& kb : P.kbs) c += kb_cycles(g, P, kb, ring_cycles);
     return (long long)c;
 }
 
+// An item as the work lists see it: cycles of one of its parts (estimated), parts, what the kernel reads.
+struct TcWork { long long cycles; int parts; TcTile tile; };
+
 // Longest processing time first: items (sorted, longest first) onto the least loaded of `grid` lists.  Returns the longest list's load.
-long long spread_items(const std::vector<std::pair<long long, TcTile>>& tl, size_t n, int grid, std::vector<std::vector<TcTile>>* lists)
+long long spread_items(const std::vector<TcWork>& work, size_t n, int grid, std::vector<std::vector<TcTile>>* lists)
 {
     std::vector<std::pair<long long, int>> heap;             // (-load, cta): the standard heap keeps the largest on top
     for (int c = 0; c < grid; ++c) heap.push_back({0, -c});
     std::make_heap(heap.begin(), heap.end());
+    if (lists) lists->assign(grid, {});
     long long longest = 0;
     for (size_t i = 0; i < n; ++i) {
         std::pop_heap(heap.begin(), heap.end());
         std::pair<long long, int> top = heap.back();
-        if (lists) (*lists)[-top.second].push_back(tl[i].second);
-        top.first -= tl[i].first;
+        if (lists) (*lists)[-top.second].push_back(work[i].tile);
+        top.first -= work[i].cycles;
         longest = std::max(longest, -top.first);
         heap.back() = top;
         std::push_heap(heap.begin(), heap.end());
     }
     return longest;
+}
+
+// 16-column chunks of the accumulator that one of an item's parts sums.
+int part_chunks(const NodePlan& P, int parts) { return (P.nl * P.lane_cols / 16 + parts - 1) / parts; }
+
+// Estimated cycles of one of the parts of an item of `cycles`: K-blocks and start, and what it sends to the others (8 KiB a chunk).
+long long part_cycles(const NodePlan& P, long long cycles, int parts, bool in_rings)
+{
+    if (parts <= 1) return cycles;
+    return 1500 + (cycles - 1500) / parts + 1200 + (in_rings ? 1200 : 0) + 320 * (P.nl * P.lane_cols / 16 - part_chunks(P, parts));
+}
+
+// Items (sorted, longest first) onto `grid` CTAs in clusters: an item of p > 1 parts goes to p neighbouring CTAs of one cluster that
+// have no part yet, behind what else they have; whole items to the least loaded CTAs.  Returns the longest list's load, or -1 if
+// the parts do not find room.
+long long spread_split(const std::vector<TcWork>& work, int grid, int cluster, std::vector<std::vector<TcTile>>* lists)
+{
+    std::vector<long long> load(grid, 0);
+    std::vector<char> taken(grid, 0);
+    std::vector<TcTile> part(grid);
+    if (lists) lists->assign(grid, {});
+    for (const TcWork& w : work) {
+        const int n = w.parts;
+        int at = -1;
+        long long least = 0;
+        for (int c = 0; c + n <= grid; c += n) {
+            long long l = 0;
+            bool room = true;
+            for (int q = 0; q < n; ++q) {
+                l = std::max(l, load[c + q]);
+                room = room && (n == 1 || !taken[c + q]);
+            }
+            if (room && (at < 0 || l < least)) { at = c; least = l; }
+        }
+        if (at < 0) return -1;
+        for (int q = 0; q < n; ++q) {
+            load[at + q] += w.cycles;
+            TcTile t = w.tile;
+            t.words = q;
+            t.rank0 = at % cluster;
+            if (n > 1) {
+                part[at + q] = t;
+                taken[at + q] = 1;
+            } else if (lists) {
+                (*lists)[at].push_back(t);
+            }
+        }
+    }
+    if (lists)
+        for (int c = 0; c < grid; ++c)
+            if (taken[c]) (*lists)[c].push_back(part[c]);
+    return *std::max_element(load.begin(), load.end());
+}
+
+cudaLaunchConfig_t cluster_config(int grid, int cluster, size_t smem, cudaStream_t stream, bool early, cudaLaunchAttribute (&at)[2])
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cluster;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = early ? 2 : 1;
+    return cfg;
+}
+
+// Clusters of a launch that the device holds at once, one CTA to an SM.
+int clusters_held(const sr_graph* g, int cluster)
+{
+    cudaLaunchAttribute at[2];
+    const cudaLaunchConfig_t cfg = cluster_config(cluster, cluster, kSmemBudget, nullptr, false, at);
+    int held = 0;
+    if (cudaFuncSetAttribute(sr_tc_group_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&held, sr_tc_group_kernel<true>, &cfg) == cudaSuccess && held > 0)
+        return std::min(held, g->sm_count / cluster);
+    cudaGetLastError();
+    return std::max(1, g->sm_count / cluster);
 }
 
 }  // namespace
@@ -1279,6 +1510,9 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
     }
     for (size_t v = 0; v < g->nodes.size(); ++v)
         if (leader[v] >= 0) E->node_of[v] = E->node_of[leader[v]];
+    std::map<int, int> held;
+    held[1] = g->sm_count;
+    for (int cluster = 2; cluster <= kMaxParts; cluster *= 2) held[cluster] = clusters_held(g, cluster);
     // per launch group: tile sizes, K-blocks, ring geometry, work lists
     E->group_tiles.assign(g->groups.size(), {});
     int n_tiles = 0;
@@ -1286,98 +1520,213 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
         std::vector<int> members;
         for (int v : g->groups[gi])
             if (E->node_of[v] >= 0 && leader[v] < 0) members.push_back(E->node_of[v]);
-        // Tile size: a launch with many items per SM takes the widest tiles (fewest copies per MMA); one with few takes the
-        // size that ends first by the estimate, because an MMA of 128 columns costs half of one of 256.
-        auto plan_tiles = [&](int max_cols) {
-            std::vector<std::pair<long long, TcTile>> tl;
-            for (int ni : members) {
-                NodePlan& P = E->nodes[ni];
-                const SrHostNode& n = g->nodes[P.node];
-                double blocks = 0, boxes = 0;
-                std::vector<int> in_edges(n.in_edges.begin(), n.in_edges.end());
-                if (P.node2 >= 0) in_edges.insert(in_edges.end(), g->nodes[P.node2].in_edges.begin(), g->nodes[P.node2].in_edges.end());
-                for (int e : in_edges) {
-                    const SrHostEdge& he = g->edges[e];
-                    const double cb = is_stem(g, he) ? 1.0 : (double)(g->nodes[he.d.src].d.c / block_k(g->nodes[he.d.src].d.c));
-                    const int kk = is_stem(g, he) ? 1 : he.k_eff, sd = is_stem(g, he) ? 1 : std::min(he.k_eff, he.stride_eff);
-                    blocks += cb * kk * kk;
-                    boxes += cb * sd * sd;
-                }
-                choose_tile(n.d.h, n.d.w, g->batch, max_cols, g->opt_tile_w, blocks / std::max(1.0, boxes), P);
-                build_kblocks(g, E, P);
-                const long long cycles = item_cycles(g, P);
-                for (const TcTile& t : node_tiles(g, P, ni)) tl.push_back({cycles, t});
+        // What can be chosen per plan: the most columns of its tiles (256, 128, 64: variants 0, 1, 2), and the parts of its items.
+        struct Variant { NodePlan P; std::vector<TcTile> tiles; int box_kb = 1, w_slot = 1024, words = 0; long long plain, cycles[2][kMaxW + 1]; };   // of an item; by crowded, slots
+        struct Choice { int v, parts; };
+        std::vector<std::vector<Variant>> variants(members.size());
+        auto variant_of = [&](size_t m, int max_cols) {
+            Variant V;
+            V.P = E->nodes[members[m]];
+            const SrHostNode& n = g->nodes[V.P.node];
+            double blocks = 0, boxes = 0;
+            std::vector<int> in_edges(n.in_edges.begin(), n.in_edges.end());
+            if (V.P.node2 >= 0) in_edges.insert(in_edges.end(), g->nodes[V.P.node2].in_edges.begin(), g->nodes[V.P.node2].in_edges.end());
+            for (int e : in_edges) {
+                const SrHostEdge& he = g->edges[e];
+                const double cb = is_stem(g, he) ? 1.0 : (double)(g->nodes[he.d.src].d.c / block_k(g->nodes[he.d.src].d.c));
+                const int kk = is_stem(g, he) ? 1 : he.k_eff, sd = is_stem(g, he) ? 1 : std::min(he.k_eff, he.stride_eff);
+                blocks += cb * kk * kk;
+                boxes += cb * sd * sd;
             }
-            std::stable_sort(tl.begin(), tl.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
-            return tl;
+            choose_tile(n.d.h, n.d.w, g->batch, max_cols, g->opt_tile_w, blocks / std::max(1.0, boxes), V.P);
+            build_kblocks(g, E, V.P);
+            V.tiles = node_tiles(g, V.P, members[m]);
+            int bk_max = 16;
+            for (const KbHost& kb : V.P.kbs) {
+                V.box_kb = std::max(V.box_kb, kb.ring_kb);
+                bk_max = std::max(bk_max, kb.bk);
+                V.words += 2 * kb.x_load + 1;
+            }
+            V.w_slot = (int)sr_align_up((size_t)std::min(V.P.rows_total(g), 128) * std::max(64, bk_max) * 2, 1024);
+            V.plain = item_cycles(g, V.P, 0.0);
+            for (int w = 2; w <= kMaxW; ++w)
+                for (int crowded = 0; crowded < 2; ++crowded) V.cycles[crowded][w] = item_cycles(g, V.P, ring_cycles(w, crowded != 0));
+            return V;
         };
-        int best_cols = kMaxCols;
-        long long best_span = -1;
-        for (int max_cols = kMaxCols; max_cols >= 64 && !members.empty(); max_cols /= 2) {
-            const auto tl = plan_tiles(max_cols);
-            const long long span = spread_items(tl, tl.size(), (int)std::min<size_t>(tl.size(), (size_t)g->sm_count), nullptr);
-            if (best_span < 0 || span < best_span) {
-                best_span = span;
-                best_cols = max_cols;
-            }
-            if (tl.size() > 8 * (size_t)g->sm_count) break;        // plenty of items: smaller tiles only cost copies
-        }
-        const std::vector<std::pair<long long, TcTile>> tl = plan_tiles(best_cols);
-        // Shared memory: weight slots, the node tables, and the rest for activation boxes, of which two of the largest should
-        // fit.  A launch with several items per CTA is better off with room for a third box (a box read by one tap only lasts
-        // 512 cycles of MMAs, and the one after it has to be on its way before that), one with an item or two per CTA with a
-        // deeper weight ring.  Measured on B200, us per frame with six / five / four slots: six-node network at 256 samples
+        // Shared memory: what the parts of items exchange, the node tables, weight slots, and the rest for activation boxes, of which
+        // two of the largest should fit.  A launch with several items per CTA is better off with room for a third box (a box read by
+        // one tap only lasts 512 cycles of MMAs, and the one after it has to be on its way before that), one with an item or two per
+        // CTA with a deeper weight ring.  Measured on B200, us per frame with six / five / four slots: six-node network at 256 samples
         // 146.3 / 143.0 / 147.8, ten-node at 128 115.1 / 112.7 / 117.9, stress graph at 32 253.9 / 246.2 / 250.7, deep window
         // 100.8 / 100.4 / 103.3; six-node hybrid at 37 samples (one item per CTA) 57.3 / 59.1 / 64.0.
-        int w_slot = 1024, box_kb = 1, n_tab = 0;
-        for (int ni : members) {
-            const NodePlan& P = E->nodes[ni];
-            int n_act = 0, bk_max = 16;
-            for (const KbHost& kb : P.kbs) {
-                box_kb = std::max(box_kb, kb.ring_kb);
-                n_act += kb.x_load;
-                bk_max = std::max(bk_max, kb.bk);
+        auto rings = [&](const std::vector<Choice>& ch, int table_words) {
+            TcEngine::Launch L;
+            int box_kb = 1, words = 0;
+            size_t items = 0;
+            bool widest = true;
+            for (size_t m = 0; m < members.size(); ++m) {
+                const Variant& V = variants[m][ch[m].v];
+                box_kb = std::max(box_kb, V.box_kb);
+                L.w_slot = std::max(L.w_slot, V.w_slot);
+                words = std::max(words, V.words / ch[m].parts + 16);
+                if (ch[m].parts > 1) L.exch = std::max(L.exch, (ch[m].parts - 1) * part_chunks(V.P, ch[m].parts) * 8192);
+                items += V.tiles.size();
+                widest = widest && ch[m].v == 0;
             }
-            w_slot = std::max(w_slot, (int)sr_align_up((size_t)std::min(P.rows_total(g), 128) * std::max(64, bk_max) * 2, 1024));
-            build_groups(E->nodes[ni]);
-            n_tab = std::max(n_tab, 2 * count_bursts(P) + n_act);
+            L.table_bytes = (int)sizeof(TcNode) + (table_words ? table_words : words) * 16;
+            const int sums = L.exch;
+            for (;;) {
+                const int avail = kSmemBudget - 1024 - kTables * L.table_bytes - L.exch;
+                L.n_w = g->opt_b_units > 0 ? std::min(kMaxW, std::max(2, g->opt_b_units)) : widest && items > 2 * (size_t)g->sm_count ? 5 : kMaxW;
+                while (g->opt_b_units == 0 && L.n_w > 6 && (avail - L.n_w * L.w_slot) / 1024 < 3 * box_kb) --L.n_w;
+                while (L.n_w > 3 && (avail - L.n_w * L.w_slot) / 1024 < 2 * box_kb) --L.n_w;
+                while (L.n_w > 2 && (avail - L.n_w * L.w_slot) / 1024 < box_kb) --L.n_w;
+                L.ring_kb = (avail - L.n_w * L.w_slot) / 1024;
+                L.fits = avail > 0 && L.ring_kb >= box_kb && box_kb <= 255;
+                if (L.exch == 0 || (L.fits && L.n_w >= 6)) break;
+                L.exch = 0;                                        // no room of its own: in the rings
+            }
+            if (sums > 0 && L.exch == 0 && sums > L.n_w * L.w_slot + L.ring_kb * 1024) L.fits = false;
+            return L;
+        };
+        // cycles and lists of a choice; tail: the epilogue of the widest tile, which no other item hides (13 cycles a column)
+        struct Bound { long long longest = 0, total = 0, tail = 0; size_t parts = 0, at = 0; };
+        auto crowded_by = [&](const std::vector<Choice>& ch) {
+            size_t parts = 0;
+            for (size_t m = 0; m < members.size(); ++m) parts += variants[m][ch[m].v].tiles.size() * ch[m].parts;
+            return parts > (size_t)g->sm_count;
+        };
+        auto cycles_of = [&](const Variant& V, int parts, const TcEngine::Launch& L, bool few, bool crowded) {
+            return few ? part_cycles(V.P, V.cycles[crowded][L.n_w], parts, L.exch == 0) : V.plain;
+        };
+        auto bound_of = [&](const std::vector<Choice>& ch, const TcEngine::Launch& L, bool few) {
+            const bool crowded = crowded_by(ch);
+            Bound b;
+            for (size_t m = 0; m < members.size(); ++m) {
+                const Variant& V = variants[m][ch[m].v];
+                const long long c = cycles_of(V, ch[m].parts, L, few, crowded);
+                b.total += c * ch[m].parts * (long long)V.tiles.size();
+                b.parts += V.tiles.size() * ch[m].parts;
+                b.tail = std::max(b.tail, 13ll * V.P.nl * V.P.lane_cols / ch[m].parts);
+                if (c > b.longest) { b.longest = c; b.at = m; }
+            }
+            return b;
+        };
+        auto work_of = [&](const std::vector<Choice>& ch, const TcEngine::Launch& L, bool few, bool tiles) {
+            const bool crowded = crowded_by(ch);
+            std::vector<TcWork> work;
+            for (size_t m = 0; m < members.size(); ++m) {
+                const Variant& V = variants[m][ch[m].v];
+                const long long c = cycles_of(V, ch[m].parts, L, few, crowded);
+                for (const TcTile& t : V.tiles) work.push_back(TcWork{c, ch[m].parts, tiles ? t : TcTile{}});
+            }
+            std::stable_sort(work.begin(), work.end(), [](const TcWork& a, const TcWork& b) { return a.cycles > b.cycles; });
+            return work;
+        };
+        // A launch with many items per SM takes the widest tiles (fewest copies per MMA).  For one with few, the split that ends first
+        // by the estimate is sought: from 256, 128 or 64 columns for every plan, the plan whose items take longest gets narrower
+        // tiles or has its items cut into twice as many parts, whichever leaves the shorter bound, again and again.  The line lies at
+        // three items of the widest tiles per SM: at 2.8 (stress graph at 4 samples) the search still gains 8 %, from 3.5 on
+        // (six-node network at 64 samples, ten-node at 48) nothing.
+        std::vector<Choice> best;
+        int best_cluster = 1, best_grid = 0;
+        long long best_cost = -1;
+        size_t widest_items = 0;
+        for (size_t m = 0; m < members.size(); ++m) {
+            for (int cols = kMaxCols; cols >= 64; cols /= 2) variants[m].push_back(variant_of(m, cols));
+            widest_items += variants[m][0].tiles.size();
         }
-        const int table_bytes = (int)sizeof(TcNode) + n_tab * 16;
-        const int avail = kSmemBudget - 1024 - kTables * table_bytes;
-        int n_w = g->opt_b_units > 0 ? std::min(kMaxW, std::max(2, g->opt_b_units)) : (best_cols == kMaxCols && tl.size() > 2 * (size_t)g->sm_count ? 5 : 6);
-        while (n_w > 3 && (avail - n_w * w_slot) / 1024 < 2 * box_kb) --n_w;
-        while (n_w > 2 && (avail - n_w * w_slot) / 1024 < box_kb) --n_w;
-        const int ring_kb = (avail - n_w * w_slot) / 1024;
-        if (!members.empty() && (ring_kb < box_kb || box_kb > 255)) return SR_ERR_UNSUPPORTED;
-        // Work lists: the items go, longest first, to the CTA with the least work so far; CTA c walks column c of a
-        // matrix with one row per round (entries of node -1 pad the shorter columns).  Unless the lists are asked to be
-        // static, the smallest items - a fifth of the work, if the launch has more than two items per CTA - stay out of
-        // the matrix and follow it as one shared list (see the kernel).
-        const int grid = (int)std::min<size_t>(tl.size(), (size_t)g->sm_count);
-        std::vector<std::vector<TcTile>> lists(std::max(grid, 1));
-        size_t n_matrix = tl.size();
-        if (g->opt_tc_lists == 0 && tl.size() > 2 * (size_t)grid) {
-            long long total = 0, tail = 0;
-            for (auto& it : tl) total += it.first;
-            while (n_matrix > (size_t)grid && (tail + tl[n_matrix - 1].first) * 5 <= total) tail += tl[--n_matrix].first;
+        const bool few = g->opt_b_units == 0 && g->opt_tile_w == 0 && widest_items <= 3 * (size_t)g->sm_count;
+        for (int start = 0; start < 3 && !members.empty(); ++start) {
+            size_t items = 0;
+            for (size_t m = 0; m < members.size(); ++m) items += variants[m][start].tiles.size();
+            for (int cluster = 1; cluster <= (few ? kMaxParts : 1); cluster *= 2)
+                // all SMs, or half of them: then the next launch starts up on the others
+                for (int half = 0; half < (few ? 2 : 1); ++half) {
+                    const int ctas = (half ? std::min(held[cluster], g->sm_count / 2 / cluster) : held[cluster]) * cluster;
+                    std::vector<Choice> ch(members.size(), Choice{start, 1});
+                    for (;;) {
+                        const TcEngine::Launch L = rings(ch, 0);
+                        const Bound b = bound_of(ch, L, few);
+                        const int grid = (int)std::min<size_t>((b.parts + cluster - 1) / cluster * cluster, ctas);
+                        const long long fixed = (few ? b.tail : 0) + (grid > g->sm_count / 2 ? kLateStart : 0) + (cluster > 1 ? kClusterStart : 0);
+                        if (L.fits && (best_cost < 0 || std::max(b.longest, b.total / grid) + fixed < best_cost)) {
+                            const std::vector<TcWork> work = work_of(ch, L, few, false);
+                            const long long span = cluster > 1 ? spread_split(work, grid, cluster, nullptr) : spread_items(work, work.size(), grid, nullptr);
+                            if (span >= 0 && (best_cost < 0 || span + fixed < best_cost)) {
+                                best_cost = span + fixed;
+                                best = ch;
+                                best_cluster = cluster;
+                                best_grid = grid;
+                            }
+                        }
+                        if (!few) break;
+                        const Choice now = ch[b.at];
+                        const std::vector<Variant>& of = variants[b.at];
+                        Choice ways[2] = {Choice{now.v, now.parts * 2}, Choice{now.v + 1, now.parts}};
+                        while (ways[1].v < 2 && of[ways[1].v].tiles.size() == of[now.v].tiles.size()) ++ways[1].v;
+                        int way = -1;
+                        long long shortest = 0;
+                        for (int w = 0; w < 2; ++w) {
+                            if (w == 0 && (ways[0].parts > cluster || (int)of[now.v].P.kbs.size() < 2 * ways[0].parts)) continue;
+                            if (w == 1 && (ways[1].v > 2 || of[ways[1].v].tiles.size() == of[now.v].tiles.size())) continue;
+                            ch[b.at] = ways[w];
+                            const Bound c = bound_of(ch, rings(ch, 0), few);
+                            const long long t = std::max(c.longest, c.total / ctas) + c.tail;
+                            if (way < 0 || t < shortest) { way = w; shortest = t; }
+                        }
+                        if (way < 0) break;
+                        ch[b.at] = ways[way];
+                    }
+                }
+            if (items > 8 * (size_t)g->sm_count) break;            // plenty of items: smaller tiles only cost copies
         }
-        if (grid > 0) {
-            spread_items(tl, n_matrix, grid, &lists);
-            size_t n_rows = 0;
+        TcEngine::Launch L;
+        if (!members.empty()) {
+            if (best_cost < 0) return SR_ERR_UNSUPPORTED;
+            int words = 1;
+            for (size_t m = 0; m < members.size(); ++m) {
+                NodePlan& P = E->nodes[members[m]];
+                P = variants[m][best[m].v].P;
+                P.n_parts = best[m].parts;
+                build_groups(g, P);
+                for (const NodePlan::Part& q : P.parts) {
+                    int n_act = 0;
+                    for (const KbHost& kb : q.kbs) n_act += kb.x_load;
+                    words = std::max(words, 2 * count_bursts(q) + n_act);
+                }
+            }
+            L = rings(best, words);
+            if (!L.fits) return SR_ERR_UNSUPPORTED;
+            // Work lists: the items go, longest first, to the CTA with the least work so far; CTA c walks column c of a
+            // matrix with one row per round (entries of node -1 pad the shorter columns).  Unless the lists are asked to be
+            // static, the smallest items - a fifth of the work, if the launch has more than two items per CTA - stay out of
+            // the matrix and follow it as one shared list (see the kernel).
+            const std::vector<TcWork> work = work_of(best, L, few, true);
+            std::vector<std::vector<TcTile>> lists;
+            size_t n_matrix = work.size(), n_rows = 0;
+            if (best_cluster > 1) {
+                spread_split(work, best_grid, best_cluster, &lists);
+                while (std::all_of(lists.end() - best_cluster, lists.end(), [](const auto& l) { return l.empty(); })) lists.resize(lists.size() - best_cluster);
+                L.cluster = best_cluster;
+            } else {
+                if (g->opt_tc_lists == 0 && work.size() > 2 * (size_t)best_grid) {
+                    long long total = 0, tail = 0;
+                    for (auto& it : work) total += it.cycles;
+                    while (n_matrix > (size_t)best_grid && (tail + work[n_matrix - 1].cycles) * 5 <= total) tail += work[--n_matrix].cycles;
+                }
+                spread_items(work, n_matrix, best_grid, &lists);
+            }
             for (auto& l : lists) n_rows = std::max(n_rows, l.size());
             for (size_t r = 0; r < n_rows; ++r)
-                for (int c = 0; c < grid; ++c)
-                    E->group_tiles[gi].push_back(r < lists[c].size() ? lists[c][r] : TcTile{-1, 0, 0, 0, 0, 0, 0, 0});
+                for (auto& l : lists) E->group_tiles[gi].push_back(r < l.size() ? l[r] : TcTile{-1, 0, 0, 0, 0, 0, 0, 0});
+            L.grid = (int)lists.size();
+            L.n_own = (int)E->group_tiles[gi].size();
+            for (size_t i = n_matrix; i < work.size(); ++i) E->group_tiles[gi].push_back(work[i].tile);
         }
-        E->group_n_own.push_back((int)E->group_tiles[gi].size());
-        for (size_t i = n_matrix; i < tl.size(); ++i) E->group_tiles[gi].push_back(tl[i].second);
-        E->group_grid.push_back(grid);
-        E->group_tile_offset.push_back(n_tiles);
+        L.first_tile = n_tiles;
         n_tiles += (int)E->group_tiles[gi].size();
-        E->group_n_w.push_back(n_w);
-        E->group_w_slot.push_back(w_slot);
-        E->group_ring_kb.push_back(ring_kb);
-        E->group_table_bytes.push_back(table_bytes);
+        E->launches.push_back(L);
     }
     int n_kbs = 0;
     for (NodePlan& P : E->nodes) {
@@ -1388,7 +1737,9 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
     E->n_kbs = n_kbs;
     // upper bound on distinct tensor maps: two parities per K-block plus one weight map per (node, bk)
     E->r_maps = take(sizeof(CUtensorMap) * (size_t)(4 * n_kbs + 1));
-    E->r_tables = take(48 * (size_t)n_kbs + sizeof(TcNode) * E->nodes.size());
+    size_t n_entries = 0;
+    for (const NodePlan& P : E->nodes) n_entries += P.parts.size();
+    E->r_tables = take(48 * (size_t)n_kbs + sizeof(TcNode) * n_entries);
     E->r_tiles = take(sizeof(TcTile) * (size_t)std::max(1, n_tiles));
     return SR_OK;
 }
@@ -1399,12 +1750,12 @@ sr_status sr_tc_bind(sr_graph* g)
     if (!E) return SR_OK;
     EncodeTiledFn encode = encode_fn();
     if (!encode) return SR_ERR_CUDA;
-    if (cudaFuncSetAttribute(sr_tc_group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget) != cudaSuccess)
-        return SR_ERR_CUDA;
     // Always the largest shared-memory partition: otherwise the SM is configured with the smallest partition that holds
     // this kernel's CTA, which can leave a few hundred bytes, and the frame's other kernels cannot run beside it.
-    if (cudaFuncSetAttribute(sr_tc_group_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess)
-        return SR_ERR_CUDA;
+    for (auto kernel : {sr_tc_group_kernel<false>, sr_tc_group_kernel<true>})
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget) != cudaSuccess ||
+            cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess)
+            return SR_ERR_CUDA;
     char* ws = g->ws;
     std::vector<CUtensorMap> maps;
     std::map<std::tuple<uintptr_t, int, int, int, int, int, int, int, int>, int> cache;
@@ -1446,14 +1797,13 @@ sr_status sr_tc_bind(sr_graph* g)
         d.tw = P.tw; d.th = P.th; d.tb = P.tb; d.sep = P.sep;
         d.nl = P.nl;
         d.lane_cols = P.lane_cols;
-        std::vector<TcAct> da;
-        struct KbIssue { uint32_t x_off16, x_hi, w_hi; };
-        std::vector<KbIssue> dm;                      // per K-block of this node: what its MMAs need
+        d.n_parts = P.n_parts;
+        d.part_chunks = part_chunks(P, P.n_parts);
         const int rows128 = std::min(P.rows_total(g), 128);
-        if (P.k_total > 65535 || (int)P.runs.size() > kMaxRuns || P.wgroups.size() > 32 * sizeof(d.pairs) / sizeof(d.pairs[0])) return SR_ERR_UNSUPPORTED;
+        if (P.k_total > 65535 || (int)P.runs.size() > kMaxRuns) return SR_ERR_UNSUPPORTED;
         // one 3-D view per run: (channels of a block, output channels, blocks of the run); a box of two blocks lands in
         // shared memory block after block, each an ordinary K-major swizzled tile
-        d.n_runs = (int)P.runs.size();
+        std::vector<TcRun> runs;
         for (size_t r = 0; r < P.runs.size(); ++r) {
             const WRun& R = P.runs[r];
             int map_of[2] = {0, -1};
@@ -1472,95 +1822,111 @@ sr_status sr_tc_bind(sr_graph* g)
                 map_of[nb - 1] = (int)maps.size() - 1;
             }
             if (maps.size() > 65535) return SR_ERR_UNSUPPORTED;
-            d.runs[r].map1 = (uint16_t)map_of[0];
-            d.runs[r].map2 = (uint16_t)(map_of[1] < 0 ? map_of[0] : map_of[1]);   // equal: no group of two blocks
-            d.runs[r].bytes16 = (uint16_t)((size_t)rows128 * R.bk * 2 >> 4);
+            TcRun t{};
+            t.map1 = (uint16_t)map_of[0];
+            t.map2 = (uint16_t)(map_of[1] < 0 ? map_of[0] : map_of[1]);   // equal: no group of two blocks
+            t.bytes16 = (uint16_t)((size_t)rows128 * R.bk * 2 >> 4);
+            runs.push_back(t);
         }
-        for (size_t gi = 0; gi < P.wgroups.size(); ++gi) {
-            d.runs[P.wgroups[gi].run].n_groups += 1;
-            if (P.wgroups[gi].n == 2) d.pairs[gi / 32] |= 1u << (gi % 32);
-        }
-        for (size_t i = 0; i < P.kbs.size(); ++i) {
-            const KbHost& kb = P.kbs[i];
-            const SrHostEdge& he = g->edges[kb.edge];
-            const SrHostNode& s = g->nodes[he.d.src];
-            TcAct kl{};
-            KbIssue km{};
-            int map0 = -1, map1 = -1, qxv = 0, qyv = 0;
-            kl.flags = (uint8_t)(he.R ? 1 : 0);
-            km.w_hi = desc_hi_of(kb.bk);
-            const size_t x_bytes = (size_t)kb.bk * 2 * kb.x_width * kb.x_rows * P.tb;
-            const size_t sbo_bytes = (size_t)(P.flat ? 8 : kb.x_width) * kb.bk * 2;
-            if ((x_bytes >> 4) > 65535 || (sbo_bytes >> 4) > 0x3FFF) return SR_ERR_UNSUPPORTED;
-            kl.x_bytes16 = (uint16_t)(x_bytes >> 4);
-            kl.ring_kb = (uint16_t)kb.ring_kb;
-            km.x_hi = (km.w_hi & ~0x3FFFu) | (uint32_t)(sbo_bytes >> 4);
-            km.x_off16 = (uint32_t)(((size_t)kb.x_shift * kb.bk * 2) >> 4);
-            if (km.x_off16 + 4 > 65535) return SR_ERR_UNSUPPORTED;
-            dm.push_back(km);
-            if (!kb.x_load) continue;                // reads the box the first tap of its class loads
-            if (kb.stem) {
-                const StemPlan& S = E->stems[kb.stem_index];
-                for (int par = 0; par < 2; ++par)
-                    (par ? map1 : map0) = act_map(ws + S.buf[par].offset, S.Kp, n.d.w, n.d.h, (size_t)S.Kp * 2,
-                                                  (size_t)n.d.w * S.Kp * 2, (size_t)n.d.h * n.d.w * S.Kp * 2, kb.bk, kb.x_width, kb.x_rows, P.tb);
-            } else {
-                // input pixel = stride * (output pixel + q) + r, q = floor((tap - pad) / stride), r the residue:
-                // the residue-class view of the source makes the tap a dense box starting at (w0 + qx, h0 + qy)
-                const int st = he.stride_eff;
-                const int ry = kb.box_ry, rx = kb.box_rx;
-                const int Hv = (s.d.h - ry + st - 1) / st, Wv = (s.d.w - rx + st - 1) / st;
-                if (Hv <= 0 || Wv <= 0) return SR_ERR_UNSUPPORTED;
-                for (int par = 0; par < 2; ++par) {
-                    char* base = ws + s.state[par].offset + ((size_t)ry * s.d.w + rx) * s.d.c * 2;
-                    (par ? map1 : map0) = act_map(base, s.d.c, Wv, Hv, (size_t)st * s.d.c * 2, (size_t)st * s.d.w * s.d.c * 2,
-                                                  (size_t)s.d.h * s.d.w * s.d.c * 2, kb.bk, kb.x_width, kb.x_rows, P.tb);
+        for (NodePlan::Part& q : P.parts) {
+            TcNode e = d;
+            e.part = (int)(&q - P.parts.data());
+            if (q.wgroups.size() > 32 * sizeof(e.pairs) / sizeof(e.pairs[0])) return SR_ERR_UNSUPPORTED;
+            int run = -1;
+            for (size_t gi = 0; gi < q.wgroups.size(); ++gi) {
+                const WGroup& wg = q.wgroups[gi];
+                if (wg.run != run) {
+                    run = wg.run;
+                    e.runs[e.n_runs] = runs[run];
+                    e.runs[e.n_runs++].blk0 = (uint16_t)wg.blk;
                 }
-                qxv = kb.box_qx; qyv = kb.box_qy;
+                e.runs[e.n_runs - 1].n_groups += 1;
+                if (wg.n == 2) e.pairs[gi / 32] |= 1u << (gi % 32);
             }
-            if (map0 < 0 || map1 < 0) return SR_ERR_CUDA;
-            if (map0 > 65535 || map1 > 65535 || qxv < -128 || qxv > 127 || qyv < -128 || qyv > 127 || kb.c0 / 16 > 255) return SR_ERR_UNSUPPORTED;
-            kl.x_map0 = (uint16_t)map0; kl.x_map1 = (uint16_t)map1;
-            kl.qx = (int8_t)qxv; kl.qy = (int8_t)qyv;
-            kl.c0_16 = (uint8_t)(kb.c0 / 16);
-            da.push_back(kl);
-        }
-        // Bursts: two consecutive weight groups if their K-blocks are equally wide, else one.
-        std::vector<TcBurst> db;
-        for (size_t gi = 0; gi < P.wgroups.size();) {
-            const int i0 = P.wgroups[gi].first_kb, bk = P.kbs[i0].bk;
-            const bool two = one_burst(P, gi);
-            TcBurst b{};
-            b.w_hi = dm[i0].w_hi;
-            b.l1_off16 = (uint16_t)(8 * bk * 2 >> 4);                          // a lane's window lies 8 pixels after the one before
-            b.w1_off16 = (uint16_t)(bk == 64 ? 4 : rows128 * bk * 2 >> 4);     // a block of 64 channels is two segments, a narrower one is one
-            b.flags = (two ? kBuTwo : 0) | (bk == 16 ? kBuK16 : 0);
-            for (int half = 0; half < (two ? 2 : 1); ++half) {
-                const WGroup& wg = P.wgroups[gi + half];
-                const KbHost& kb0 = P.kbs[wg.first_kb];
-                b.x_hi[half] = dm[wg.first_kb].x_hi;
-                if (kb0.x_load) {
-                    b.flags |= half ? kBuNew1 : kBuNew0;
-                    b.size[half] = (uint8_t)kb0.ring_kb;
+            std::vector<TcAct> da;
+            struct KbIssue { uint32_t x_off16, x_hi, w_hi; };
+            std::vector<KbIssue> dm;                      // per K-block: what its MMAs need
+            for (const KbHost& kb : q.kbs) {
+                const SrHostEdge& he = g->edges[kb.edge];
+                const SrHostNode& s = g->nodes[he.d.src];
+                TcAct kl{};
+                KbIssue km{};
+                int map0 = -1, map1 = -1, qxv = 0, qyv = 0;
+                kl.flags = (uint8_t)(he.R ? 1 : 0);
+                km.w_hi = desc_hi_of(kb.bk);
+                const size_t x_bytes = (size_t)kb.bk * 2 * kb.x_width * kb.x_rows * P.tb;
+                const size_t sbo_bytes = (size_t)(P.flat ? 8 : kb.x_width) * kb.bk * 2;
+                if ((x_bytes >> 4) > 65535 || (sbo_bytes >> 4) > 0x3FFF) return SR_ERR_UNSUPPORTED;
+                kl.x_bytes16 = (uint16_t)(x_bytes >> 4);
+                kl.ring_kb = (uint16_t)kb.ring_kb;
+                km.x_hi = (km.w_hi & ~0x3FFFu) | (uint32_t)(sbo_bytes >> 4);
+                km.x_off16 = (uint32_t)(((size_t)kb.x_shift * kb.bk * 2) >> 4);
+                if (km.x_off16 + 4 > 65535) return SR_ERR_UNSUPPORTED;
+                dm.push_back(km);
+                if (!kb.x_load) continue;                // reads the box the first tap of its class loads
+                if (kb.stem) {
+                    const StemPlan& S = E->stems[kb.stem_index];
+                    for (int par = 0; par < 2; ++par)
+                        (par ? map1 : map0) = act_map(ws + S.buf[par].offset, S.Kp, n.d.w, n.d.h, (size_t)S.Kp * 2,
+                                                      (size_t)n.d.w * S.Kp * 2, (size_t)n.d.h * n.d.w * S.Kp * 2, kb.bk, kb.x_width, kb.x_rows, P.tb);
+                } else {
+                    // input pixel = stride * (output pixel + q) + r, q = floor((tap - pad) / stride), r the residue:
+                    // the residue-class view of the source makes the tap a dense box starting at (w0 + qx, h0 + qy)
+                    const int st = he.stride_eff;
+                    const int ry = kb.box_ry, rx = kb.box_rx;
+                    const int Hv = (s.d.h - ry + st - 1) / st, Wv = (s.d.w - rx + st - 1) / st;
+                    if (Hv <= 0 || Wv <= 0) return SR_ERR_UNSUPPORTED;
+                    for (int par = 0; par < 2; ++par) {
+                        char* base = ws + s.state[par].offset + ((size_t)ry * s.d.w + rx) * s.d.c * 2;
+                        (par ? map1 : map0) = act_map(base, s.d.c, Wv, Hv, (size_t)st * s.d.c * 2, (size_t)st * s.d.w * s.d.c * 2,
+                                                      (size_t)s.d.h * s.d.w * s.d.c * 2, kb.bk, kb.x_width, kb.x_rows, P.tb);
+                    }
+                    qxv = kb.box_qx; qyv = kb.box_qy;
                 }
-                if (P.kbs[wg.first_kb + wg.n - 1].x_release) b.flags |= half ? kBuLast1 : kBuLast0;
-                for (int sg = 0; sg < (bk == 64 ? 2 : wg.n); ++sg) {
-                    b.x_off16[half * 2 + sg] = (uint16_t)(bk == 64 ? dm[wg.first_kb].x_off16 + 4 * sg : dm[wg.first_kb + sg].x_off16);
-                    b.flags |= 1u << (half * 2 + sg);
-                }
+                if (map0 < 0 || map1 < 0) return SR_ERR_CUDA;
+                if (map0 > 65535 || map1 > 65535 || qxv < -128 || qxv > 127 || qyv < -128 || qyv > 127 || kb.c0 / 16 > 255) return SR_ERR_UNSUPPORTED;
+                kl.x_map0 = (uint16_t)map0; kl.x_map1 = (uint16_t)map1;
+                kl.qx = (int8_t)qxv; kl.qy = (int8_t)qyv;
+                kl.c0_16 = (uint8_t)(kb.c0 / 16);
+                da.push_back(kl);
             }
-            db.push_back(b);
-            gi += two ? 2 : 1;
+            // Bursts: two consecutive weight groups if their K-blocks are equally wide, else one.
+            std::vector<TcBurst> db;
+            for (size_t gi = 0; gi < q.wgroups.size();) {
+                const int i0 = q.wgroups[gi].first_kb, bk = q.kbs[i0].bk;
+                const bool two = one_burst(q, gi);
+                TcBurst b{};
+                b.w_hi = dm[i0].w_hi;
+                b.l1_off16 = (uint16_t)(8 * bk * 2 >> 4);                          // a lane's window lies 8 pixels after the one before
+                b.w1_off16 = (uint16_t)(bk == 64 ? 4 : rows128 * bk * 2 >> 4);     // a block of 64 channels is two segments, a narrower one is one
+                b.flags = (two ? kBuTwo : 0) | (bk == 16 ? kBuK16 : 0);
+                for (int half = 0; half < (two ? 2 : 1); ++half) {
+                    const WGroup& wg = q.wgroups[gi + half];
+                    const KbHost& kb0 = q.kbs[wg.first_kb];
+                    b.x_hi[half] = dm[wg.first_kb].x_hi;
+                    if (kb0.x_load) {
+                        b.flags |= half ? kBuNew1 : kBuNew0;
+                        b.size[half] = (uint8_t)kb0.ring_kb;
+                    }
+                    if (q.kbs[wg.first_kb + wg.n - 1].x_release) b.flags |= half ? kBuLast1 : kBuLast0;
+                    for (int sg = 0; sg < (bk == 64 ? 2 : wg.n); ++sg) {
+                        b.x_off16[half * 2 + sg] = (uint16_t)(bk == 64 ? dm[wg.first_kb].x_off16 + 4 * sg : dm[wg.first_kb + sg].x_off16);
+                        b.flags |= 1u << (half * 2 + sg);
+                    }
+                }
+                db.push_back(b);
+                gi += two ? 2 : 1;
+            }
+            e.n_bu = (int)db.size();
+            e.n_act = (int)da.size();
+            const size_t at = dt.size(), words = sizeof(TcNode) / 16;
+            q.table_off = (int)at;
+            q.table_words = (int)(words + 2 * db.size() + da.size());
+            dt.resize(at + q.table_words);
+            std::memcpy(dt.data() + at, &e, sizeof(e));
+            std::memcpy(dt.data() + at + words, db.data(), db.size() * sizeof(TcBurst));
+            std::memcpy(dt.data() + at + words + 2 * db.size(), da.data(), da.size() * sizeof(TcAct));
         }
-        d.n_bu = (int)db.size();
-        d.n_act = (int)da.size();
-        const size_t at = dt.size(), words = sizeof(TcNode) / 16;
-        P.table_off = (int)at;
-        P.table_words = (int)(words + 2 * db.size() + da.size());
-        dt.resize(at + P.table_words);
-        std::memcpy(dt.data() + at, &d, sizeof(d));
-        std::memcpy(dt.data() + at + words, db.data(), db.size() * sizeof(TcBurst));
-        std::memcpy(dt.data() + at + words + 2 * db.size(), da.data(), da.size() * sizeof(TcAct));
     }
     if (maps.size() * sizeof(CUtensorMap) > E->r_maps.bytes || dt.size() * sizeof(uint4) > E->r_tables.bytes) return SR_ERR_UNSUPPORTED;
     E->n_maps = (int)maps.size();
@@ -1568,9 +1934,9 @@ sr_status sr_tc_bind(sr_graph* g)
     for (auto& v : E->group_tiles) tiles.insert(tiles.end(), v.begin(), v.end());
     for (TcTile& t : tiles)
         if (t.node >= 0) {
-            const NodePlan& P = E->nodes[t.node];
-            t.node = P.table_off;
-            t.words = P.table_words;
+            const NodePlan::Part& q = E->nodes[t.node].parts[t.words];
+            t.node = q.table_off;
+            t.words = q.table_words;
         }
     g->stems.clear();
     for (const StemPlan& S : E->stems) {
@@ -1652,7 +2018,7 @@ int sr_tc_launch_group(sr_graph* g, int group, SrFollow how, cudaStream_t s)
 {
     TcEngine* E = eng(g);
     if (!E || E->group_tiles[group].empty()) return 0;
-    const size_t smem = (size_t)E->group_n_w[group] * E->group_w_slot[group] + (size_t)E->group_ring_kb[group] * 1024 + (size_t)kTables * E->group_table_bytes[group] + 1024;
+    const TcEngine::Launch& L = E->launches[group];
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     bool timed = g->opt_time_tc != 0 && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
     if (timed) {
@@ -1671,20 +2037,27 @@ int sr_tc_launch_group(sr_graph* g, int group, SrFollow how, cudaStream_t s)
     TcParams P{};
     P.maps = reinterpret_cast<const CUtensorMap*>(g->ws + E->r_maps.offset);
     P.tables = reinterpret_cast<const uint4*>(g->ws + E->r_tables.offset);
-    P.tiles = reinterpret_cast<const TcTile*>(g->ws + E->r_tiles.offset) + E->group_tile_offset[group];
+    P.tiles = reinterpret_cast<const TcTile*>(g->ws + E->r_tiles.offset) + L.first_tile;
     P.fr = g->frame;
     P.error = reinterpret_cast<int*>(g->ws + g->r_flags.offset);
     P.sched = g->opt_tc_lists == 0 ? P.error + 16 : nullptr;
     P.wait_limit = (long long)g->opt_wait_ms * 2000000LL;
     P.n_tiles = (int)E->group_tiles[group].size();
-    P.n_own = E->group_n_own[group];
+    P.n_own = L.n_own;
     P.B = g->batch;
-    P.table_bytes = E->group_table_bytes[group];
-    P.n_w = E->group_n_w[group];
-    P.w_slot = E->group_w_slot[group];
-    P.ring_kb = E->group_ring_kb[group];
+    P.table_bytes = L.table_bytes;
+    P.n_w = L.n_w;
+    P.w_slot = L.w_slot;
+    P.ring_kb = L.ring_kb;
+    P.exch_off = L.exch_off();
     P.follow = how.flags();
-    sr_launch(sr_tc_group_kernel, E->group_grid[group], kThreads, smem, s, how.early && !timed, P);
+    if (L.cluster) {
+        cudaLaunchAttribute at[2];
+        const cudaLaunchConfig_t cfg = cluster_config(L.grid, L.cluster, L.smem(), s, how.early && !timed, at);
+        cudaLaunchKernelEx(&cfg, sr_tc_group_kernel<true>, P);
+    } else {
+        sr_launch(sr_tc_group_kernel<false>, L.grid, kThreads, L.smem(), s, how.early && !timed, P);
+    }
     if (timed) {
         cudaEventRecord(E->ev[E->ev_used + 1], s);
         E->ev_used += 2;

@@ -232,3 +232,23 @@ def test_the_wait_limit_does_not_count_the_run_before(name, kw):
         G.step([x[t]], out[t - 1])
         G.sync_status()
     assert parity.rel_err(out.cpu().numpy()[:, samples].reshape(want[o][1:].shape), want[o][1:]) <= parity.TOL["bf16"]
+
+
+@pytest.mark.parametrize("cin,c,k,stride,size,batch", [
+    (256, 256, 3, 1, 8, 1),        # two edges of 36 K-blocks on one tile of 64 pixels
+    (256, 128, 3, 1, 8, 5),
+    (48, 96, 3, 1, 7, 2),          # 16-channel K-blocks, channels and pixels that fill no tile
+    (64, 512, 3, 4, 16, 1),        # a box per tap; 16 pixels: parts without columns of their own
+    (128, 64, 3, 2, 28, 37),       # wide tiles, their sums in the rings
+    (64, 128, 1, 1, 12, 1),        # one K-block per edge: nothing to cut
+])
+def test_long_reductions_of_few_pixels(cin, c, k, stride, size, batch):
+    # launches with fewer items than SMs, whose items are cut along K over the CTAs of a cluster
+    out = size // stride
+    g = tiny("split", [Node("in", size, size, cin, IDENTITY), Node("a", out, out, c), Node("b", out, out, c), Node("o", 1, 1, 4, IDENTITY)],
+             [Edge(0, 1, CONV, k, stride), Edge(1, 1, CONV, k, 1), Edge(1, 2, CONV, k, 1), Edge(2, 2, CONV, 3, 1), Edge(2, 3, GAP_DENSE)],
+             batch=batch, frames=3)
+    samples = list(range(min(batch, 4))) + ([batch - 1] if batch > 4 else [])
+    parity.check_stepwise(g, "p", samples=samples, zero_bias=False)
+    g.patterns["q"] = [0, 1, 0, 1, 0]
+    parity.check_stepwise(g, "q", samples=samples, zero_bias=False)
