@@ -225,23 +225,39 @@ int enqueue_frames(sr_graph* g, const SrFrameArgs& fr, int frames, cudaStream_t 
         return how;
     };
     g->frame = fr;
+    const int last = (int)g->groups.size() - 1;
+    // The input of a further frame may go beside the last group of the frame before it: it takes the buffers of the frame before
+    // that, which only edges that bridge a frame (R = 1) still read.
+    bool ahead = g->input_feeds_same_frame && overlap && chain;
+    for (const SrHostEdge& e : g->edges)
+        if (g->nodes[e.d.src].is_input && e.R == 1 && g->nodes[e.d.tgt].level == last + 1) ahead = false;
+    bool there = false;                                          // the input of this frame has been queued
     for (int f = 0; f < frames; ++f, ++g->frame.off) {
         // The frame input: ahead of the first group if the update reads it (with its heads, where they can read the caller's
-        // frame themselves), else beside the first group.
+        // frame themselves; for all frames of a call but the first, beside the last group of the frame before: sequential rollouts
+        // of the six-node and ten-node networks at one sample 38.5 -> 35.1 and 67.0 -> 63.2 us per frame), else beside the first group.
         const bool feeds = g->input_feeds_same_frame;
         for (int gi = 0; gi < (int)g->groups.size(); ++gi) {
             // up to four independent launches: one of them leads, the others run beside it
             const bool has_heads = !g->group_head_nodes[gi].empty(), has_items = g->group_item_count[gi] > 0, has_tc = sr_tc_group_has_work(g, gi);
             const bool heads_lead = !has_tc && !has_items;
             const bool merged = gi == 0 && has_heads && (heads_lead || !feeds) && sr_heads_take_input(g, gi, g->frame, copies, stems_R);
-            if (gi == 0 && feeds && !merged) launches += sr_launch_input(g, g->frame, copies, stems_R, follow(false, false), nullptr, s);
+            if (merged) ahead = false;
+            if (gi == 0 && feeds && !merged && !there) launches += sr_launch_input(g, g->frame, copies, stems_R, follow(false, false), nullptr, s);
             const bool input_beside = gi == 0 && !feeds && !merged;
-            const bool late = overlap && (input_beside || (has_tc + has_items + has_heads > 1));
+            const bool next_input = ahead && gi == last && f + 1 < frames;
+            const bool late = overlap && (input_beside || next_input || (has_tc + has_items + has_heads > 1));
             if (has_tc) launches += sr_tc_launch_group(g, gi, follow(false, late), s);
             if (has_items) launches += sr_launch_direct_group(g, gi, follow(overlap && has_tc, late && !has_tc), s);
             if (input_beside && !heads_lead) launches += sr_launch_input(g, g->frame, copies, stems_R, follow(overlap, false), nullptr, s);
             if (has_heads) launches += sr_launch_heads(g, gi, merged, copies, stems_R, follow(overlap && !heads_lead, late && heads_lead), s);
             if (input_beside && heads_lead) launches += sr_launch_input(g, g->frame, copies, stems_R, follow(overlap, false), nullptr, s);
+            there = next_input;
+            if (next_input) {
+                ++g->frame.off;
+                launches += sr_launch_input(g, g->frame, copies, stems_R, follow(true, false), nullptr, s);
+                --g->frame.off;
+            }
         }
     }
     return launches;

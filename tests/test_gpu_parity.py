@@ -432,3 +432,28 @@ def test_infinite_weights_leave_pixels_alone_whose_window_they_miss(batch, size,
     inside[:, 0] = inside[:, :, 0] = False
     assert parity.rel_err(got[inside], want[inside]) <= parity.TOL[dtype]
     del recorded
+
+
+@pytest.mark.parametrize("name,pattern", [("mini", "sequential"), ("mini", "mixed_input"), ("mini", "hybrid"), ("c3", "sequential"),
+                                          ("c3", "hybrid"), ("dsr2", "sequential"), ("sink", "sequential")])
+@pytest.mark.parametrize("graph_frames", [0, 2])
+def test_frames_of_one_call_equal_calls_of_one_frame(name, pattern, graph_frames):
+    # the input of a further frame of a call is queued beside the frame before it, where the pattern allows; every value is the same
+    import torch
+    spec = graphs.build(name, batch=2, frames=5)
+    X, W, Bi = data.make_inputs(spec), data.make_weights(spec), data.make_biases(spec, zero=False)
+    got = []
+    for whole in (True, False):
+        G = parity.make_graph(spec, pattern, "auto", graph_frames if whole else 0, W, Bi, resident=False)
+        dev = {v: parity.to_device(spec, X[v]) for v in G.input_nodes}
+        G.reset([dev[v][0] for v in G.input_nodes])
+        out = torch.empty((5,) + tuple(G.out_shape()), dtype=torch.float32, device="cuda:0")
+        if whole:
+            G.run([dev[v][1:6] for v in G.input_nodes], out)
+        else:
+            for t in range(5):
+                G.step([dev[v][t + 1] for v in G.input_nodes], out[t])
+        G.sync_status()
+        got.append([out] + [G.get_state(v) for v in range(len(spec.nodes))])
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
