@@ -29,7 +29,7 @@
 // none of whose edges shares a box (1 x 1 filters, strides above the filter size) takes "flat" tiles of any width
 // instead, whose pixels are consecutive.
 //
-// Work items.  An item is one pixel tile of one plan (a node, or two narrow nodes fused, see TcNode).  CTAs are
+// Work items.  An item is one pixel tile of one plan (a node, or up to four narrow nodes fused, see TcNode).  CTAs are
 // persistent, one per SM.
 //
 // Warp roles in a CTA of 384 threads: warp 2 = keeper (finds the items, copies the K-loop tables of their nodes into shared
@@ -65,6 +65,7 @@ constexpr int kTables = 3;                            // node tables in shared m
 // the SM's shared-memory partition is left (a 117 us frame then takes 170 us).
 constexpr int kSmemBudget = 204 * 1024;
 constexpr int kMaxNodeKb = 128;                       // K-blocks per node
+constexpr int kMaxFused = 4;                          // nodes of a plan
 constexpr int kMaxParts = 8;                          // parts of an item's reduction
 
 // A run of equally wide K-blocks of a node's reduction as the weight producer sees it: n_groups weight groups (one copy
@@ -112,16 +113,16 @@ constexpr uint32_t kBuLast0 = 1u << 10, kBuLast1 = 1u << 11;  // the first / sec
 constexpr uint32_t kBuTwo = 1u << 12;                         // the burst has a second half
 constexpr uint32_t kBuK16 = 1u << 13;                         // segments of one MMA
 
-// A plan can cover TWO nodes of at most 64 channels each that have the same shape: an M = 128 instruction on a
-// 64-channel node is half empty, so the second node's weights take rows 64..127 and every K-block of a source both
-// read (same filter geometry, same frame) serves both.  TMEM lanes 64..127 then belong to the second node.  Nodes are
-// paired if they share a source, or if one of them has next to no reduction of its own.
+// A plan can cover SEVERAL nodes of 32 or 64 channels that have the same shape: an M = 128 instruction on a 64-channel node is half
+// empty, on a 32-channel node three quarters, so the weights of up to two or four nodes take the rows one after the other, and
+// every K-block of a source that several of them read (same filter geometry, same frame) serves them all.  TMEM lanes
+// rows * q .. belong to the plan's node q.  Nodes are joined if they share a source, or if one of them has next to no reduction of
+// its own; of all joins the one that saves most K-blocks comes first.  (Deepest CIFAR10 network: 29 K-blocks for the four nodes of
+// its first block, where two plans of two had 11 and 27, and 72 for those of the second instead of 81.)
 struct alignas(16) TcNode {
-    void* state[2];
-    void* state2[2];                // the second node of a fused plan (fused != 0)
-    const float* bias;
-    const float* bias2;
-    int32_t act, act2, fused, C;
+    void* state[kMaxFused][2];
+    const float* bias[kMaxFused];
+    int32_t relu, rows, n_nodes, C; // relu: a bit per node; rows: rows of the weight matrix per node (0: the plan has one node)
     int32_t H, W;
     int32_t tw, th, tb, sep;        // geometry of the tile (see the file comment): tw = columns of a lane
     int32_t nl, lane_cols;          // lanes, TMEM columns of each (N of the MMA)
@@ -791,18 +792,19 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                 break;
             }
             const uint32_t acc = (uint32_t)it & 1u;
-            const int fused = nd->fused, C = nd->C;
-            const bool second = fused && quarter >= 2;              // this warp's TMEM lanes belong to the plan's second node
-            __nv_bfloat16* out = static_cast<__nv_bfloat16*>(second ? nd->state2[cur] : nd->state[cur]);
-            const int co_w = fused ? (quarter & 1) * 32 : tl.m0 + quarter * 32;   // first channel of this warp
+            const int rows = nd->rows, C = nd->C;
+            const int which = rows == 32 ? quarter : rows == 64 ? quarter >> 1 : 0;       // the plan's node that this warp's TMEM lanes belong to
+            const bool there = which < nd->n_nodes;
+            __nv_bfloat16* out = static_cast<__nv_bfloat16*>(nd->state[which][cur]);
+            const int co_w = rows ? (quarter * 32) & (rows - 1) : tl.m0 + quarter * 32;   // first channel of this warp
             float bias[4];                                          // of channels co_w + lane / 4 + 0, 8, 16, 24
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int co = co_w + (lane >> 2) + 8 * q;
-                bias[q] = co < C ? __ldg((second ? nd->bias2 : nd->bias) + co) : 0.f;
+                bias[q] = there && co < C ? __ldg(nd->bias[which] + co) : 0.f;
             }
-            const int act = second ? nd->act2 : nd->act;
-            const bool gvalid = co_w + (lane & 3) * 8 < C;          // this thread's group of 8 channels exists
+            const bool relu = (nd->relu >> which) & 1;
+            const bool gvalid = there && co_w + (lane & 3) * 8 < C;          // this thread's group of 8 channels exists
             ok = mbar_wait(bar_tfull + 8 * acc, ((uint32_t)it >> 1) & 1u, abortp, wait_limit);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) continue;                                      // to the joint decision at the next barrier
@@ -823,7 +825,7 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                     for (int cb = 0; cb < 4; ++cb) {
                         const uint32_t* r = (cb < 2 ? lo : hi) + pb * 4 + (cb & 1) * 2;
                         __nv_bfloat162 z = __floats2bfloat162_rn(__uint_as_float(r[0]) + bias[cb], __uint_as_float(r[1]) + bias[cb]);
-                        if (act == 1) z = __hmax2(z, __floats2bfloat162_rn(0.f, 0.f));
+                        if (relu) z = __hmax2(z, __floats2bfloat162_rn(0.f, 0.f));
                         h[pb][cb] = *reinterpret_cast<const uint32_t*>(&z);
                     }
                 fetch_next();
@@ -944,8 +946,8 @@ struct KbHost {
     int blk = 0;
     int w_off = 0;     // byte offset of this block's weights inside the group's slot
     int ring_kb = 0;   // KiB the box takes in the activation ring
-    int row_off = 0;         // first row of `edge`'s weights in the plan's weight matrix (64: the second node of a fused plan)
-    int edge2 = -1;          // fused plan: the second node's edge that shares this block (its weights take rows 64..127)
+    std::vector<std::pair<int, int>> users;   // the edges that this block serves (of different nodes of the plan, the first is `edge`), and
+                                              // the first row of their weights in the plan's weight matrix
 };
 
 // Consecutive K-blocks of equal channel-block width: one 3-D view (channels of a block, output channels, blocks) of
@@ -955,8 +957,14 @@ struct WGroup { int run, blk, n, first_kb; };
 
 struct NodePlan {
     int node;
-    int node2 = -1;                 // the second node of a fused plan
-    int rows_total(const sr_graph* g) const { return node2 >= 0 ? 128 : g->nodes[node].d.c; }   // rows of the weight matrix
+    std::vector<int> nodes;         // the nodes of the plan, `node` first
+    int rows_total(const sr_graph* g) const { return (int)nodes.size() * g->nodes[node].d.c; }   // rows of the weight matrix
+    std::vector<int> in_edges(const sr_graph* g) const
+    {
+        std::vector<int> all;
+        for (int v : nodes) all.insert(all.end(), g->nodes[v].in_edges.begin(), g->nodes[v].in_edges.end());
+        return all;
+    }
     int sep, span;                  // rows / columns the taps that share one activation box are apart at most
     int tw, th, tb, nl, lane_cols;  // tile geometry (see the file comment)
     bool flat;
@@ -1106,24 +1114,83 @@ bool same_source(const sr_graph* g, int e1, int e2)
            !is_stem(g, a) && !is_stem(g, b);
 }
 
+// The incoming edges of a plan's nodes: an edge of a further node that reads the same source through the same filter geometry in
+// the same frame shares the K-blocks of an earlier node's.  edges: (edge, place of its node in the plan).
+struct SharedEdge { std::vector<std::pair<int, int>> edges; };
+std::vector<SharedEdge> shared_edges(const sr_graph* g, const std::vector<int>& nodes)
+{
+    std::vector<SharedEdge> out;
+    for (int q = 0; q < (int)nodes.size(); ++q)
+        for (int e : g->nodes[nodes[q]].in_edges) {
+            SharedEdge* with = nullptr;
+            for (SharedEdge& s : out)
+                if (!with && s.edges.back().second < q && same_source(g, s.edges[0].first, e)) with = &s;
+            if (with) with->edges.push_back({e, q});
+            else out.push_back(SharedEdge{{{e, q}}});
+        }
+    return out;
+}
+int edge_blocks(const sr_graph* g, int e)
+{
+    const SrHostEdge& he = g->edges[e];
+    const int cs = g->nodes[he.d.src].d.c;
+    return is_stem(g, he) ? 2 : he.k_eff * he.k_eff * (cs / block_k(cs));
+}
+int plan_blocks(const sr_graph* g, const std::vector<int>& nodes)
+{
+    int n = 0;
+    for (const SharedEdge& s : shared_edges(g, nodes)) n += edge_blocks(g, s.edges[0].first);
+    return n;
+}
+
+// The plans of a launch group's nodes, of up to `most` nodes each (see TcNode).
+std::vector<std::vector<int>> join_nodes(const sr_graph* g, const std::vector<int>& group, size_t most)
+{
+    std::vector<std::vector<int>> of;
+    for (int v : group)
+        if (g->nodes[v].use_tc) of.push_back({v});
+    for (bool more = most > 1; more;) {
+        int a = -1, b = -1, best = -1;
+        for (size_t i = 0; i < of.size(); ++i)
+            for (size_t j = i + 1; j < of.size(); ++j) {
+                const sr_node_desc &x = g->nodes[of[i][0]].d, &y = g->nodes[of[j][0]].d;
+                const size_t n_nodes = of[i].size() + of[j].size();
+                if ((x.c != 32 && x.c != 64) || y.c != x.c || y.h != x.h || y.w != x.w || n_nodes * x.c > 128 || n_nodes > most) continue;
+                std::vector<int> both = of[i];
+                both.insert(both.end(), of[j].begin(), of[j].end());
+                std::sort(both.begin(), both.end());
+                const int bi = plan_blocks(g, of[i]), bj = plan_blocks(g, of[j]), n = plan_blocks(g, both);
+                // without a shared source the joint plan issues as many MMAs as the two; it still pays when one of them has next
+                // to no reduction (a node fed by a staged edge only): its tiles are all epilogue, which then runs beside the
+                // other's MMAs
+                const int saved = bi + bj - n;
+                if ((saved > 0 || std::min(bi, bj) <= 2) && n <= kMaxNodeKb && saved > best) {
+                    a = (int)i;
+                    b = (int)j;
+                    best = saved;
+                }
+            }
+        more = a >= 0;
+        if (!more) break;
+        of[a].insert(of[a].end(), of[b].begin(), of[b].end());
+        std::sort(of[a].begin(), of[a].end());
+        of.erase(of.begin() + b);
+    }
+    return of;
+}
+
 // The K-blocks of a plan for its tile geometry (the stems' staging buffers exist already).
 void build_kblocks(const sr_graph* g, const TcEngine* E, NodePlan& P)
 {
     const SrHostNode& n = g->nodes[P.node];
     P.kbs.clear();
-    // the incoming edges of the plan: of its node and, fused, of its second node; an edge of the second node that
-    // reads the same source through the same filter geometry in the same frame shares the first node's K-blocks
-    struct Ent { int e, e2, row_off; };
+    struct Ent { int e; std::vector<std::pair<int, int>> users; };
     std::vector<Ent> ents;
-    for (int e : n.in_edges) ents.push_back(Ent{e, -1, 0});
-    if (P.node2 >= 0)
-        for (int e2 : g->nodes[P.node2].in_edges) {
-            int m = -1;
-            for (size_t i = 0; i < ents.size() && m < 0; ++i)
-                if (ents[i].row_off == 0 && ents[i].e2 < 0 && same_source(g, ents[i].e, e2)) m = (int)i;
-            if (m >= 0) ents[m].e2 = e2;
-            else ents.push_back(Ent{e2, -1, 64});
-        }
+    for (const SharedEdge& sh : shared_edges(g, P.nodes)) {
+        Ent en{sh.edges[0].first, {}};
+        for (const auto& u : sh.edges) en.users.push_back({u.first, u.second * n.d.c});
+        ents.push_back(en);
+    }
     // The order of the reduction is free (a sum): edges with wider channel blocks come first, so that K-blocks of
     // equal width form one run each and a run's weights are one 3-D tensor.
     auto width_of = [&](int e) {
@@ -1149,7 +1216,7 @@ void build_kblocks(const sr_graph* g, const TcEngine* E, NodePlan& P)
             for (int c0 = 0; c0 < Kp; c0 += bk) {
                 KbHost kb{e, true, si, 0, 0, c0, bk, 0, true, 0, cols, P.th + (P.tb > 1 ? P.sep : 0), true};
                 kb.src_col = c0;
-                kb.row_off = en.row_off;
+                kb.users = en.users;
                 kb.ring_kb = ring_kb(kb, 0);
                 P.kbs.push_back(kb);
             }
@@ -1185,8 +1252,7 @@ void build_kblocks(const sr_graph* g, const TcEngine* E, NodePlan& P)
                                   i == 0, (t.qy - qy0) * bw + (t.qx - qx0), bw, bh, i + 1 == taps.size()};
                         max_shift = std::max(max_shift, kb.x_shift);
                         kb.src_col = (t.ky * k + t.kx) * s.d.c + c0;
-                        kb.row_off = en.row_off;
-                        kb.edge2 = en.e2;
+                        kb.users = en.users;
                         kb.box_qy = qy0;
                         kb.box_qx = qx0;
                         kb.box_ry = cl.first.first;
@@ -1431,70 +1497,29 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
         off = sr_align_up(off + bytes, 1024);
         return r;
     };
-    // Fused plans: two nodes of one launch group with the same shape and at most 64 channels (a multiple of 32) each,
-    // which share at least one source or of which one is fed by next to nothing (see TcNode).
-    std::vector<int> partner(g->nodes.size(), -1), leader(g->nodes.size(), -1);
-    if (g->opt_tc_fuse)
-        for (const std::vector<int>& grp : g->groups)
-            for (size_t i = 0; i < grp.size(); ++i) {
-                const int a = grp[i];
-                const SrHostNode& na = g->nodes[a];
-                if (!na.use_tc || partner[a] >= 0 || leader[a] >= 0 || na.d.c > 64 || na.d.c % 32 != 0) continue;
-                for (size_t j = i + 1; j < grp.size() && partner[a] < 0; ++j) {
-                    const int b = grp[j];
-                    const SrHostNode& nb = g->nodes[b];
-                    if (!nb.use_tc || partner[b] >= 0 || leader[b] >= 0 || nb.d.c != na.d.c || nb.d.h != na.d.h || nb.d.w != na.d.w) continue;
-                    int shared = 0, blocks = 0, blocks_a = 0, blocks_b = 0;
-                    for (int ea : na.in_edges) {
-                        const SrHostEdge& he = g->edges[ea];
-                        blocks_a += is_stem(g, he) ? 2 : he.k_eff * he.k_eff * (g->nodes[he.d.src].d.c / block_k(g->nodes[he.d.src].d.c));
-                    }
-                    blocks = blocks_a;
-                    for (int eb : nb.in_edges) {
-                        const SrHostEdge& he = g->edges[eb];
-                        bool sh = false;
-                        for (int ea : na.in_edges) sh |= same_source(g, ea, eb);
-                        const int nb_e = is_stem(g, he) ? 2 : he.k_eff * he.k_eff * (g->nodes[he.d.src].d.c / block_k(g->nodes[he.d.src].d.c));
-                        blocks_b += nb_e;
-                        if (sh) ++shared;
-                        else blocks += nb_e;
-                    }
-                    // without a shared source the fused plan issues as many MMAs as the two nodes; it still pays when one
-                    // of them has next to no reduction (a node fed by a staged edge only): its tiles are all epilogue,
-                    // which then runs beside the other node's MMAs
-                    const bool tiny = std::min(blocks_a, blocks_b) <= 2;
-                    if ((shared > 0 || tiny) && blocks <= kMaxNodeKb) {
-                        partner[a] = b;
-                        leader[b] = a;
-                    }
-                }
-            }
-    // tile geometry and staging buffers
-    for (size_t v = 0; v < g->nodes.size(); ++v) {
-        const SrHostNode& n = g->nodes[v];
-        if (!n.use_tc) continue;
-        if (leader[v] >= 0) continue;                     // the second node of a fused plan: its leader's plan covers it
+    // staging buffers
+    for (size_t e = 0; e < g->edges.size(); ++e) {
+        const SrHostNode& t = g->nodes[g->edges[e].d.tgt];
+        if (!t.use_tc || !is_stem(g, g->edges[e])) continue;
+        StemPlan S;
+        S.edge = (int)e;
+        S.Kp = stem_kp(g->edges[e].K);
+        const size_t bytes = (size_t)g->batch * t.d.h * t.d.w * S.Kp * 2;
+        S.buf[0] = take(bytes);
+        S.buf[1] = take(bytes);
+        E->stem_of_edge[e] = (int)E->stems.size();
+        E->stems.push_back(S);
+    }
+    auto plan_of = [&](const std::vector<int>& nodes) {
         NodePlan P{};
-        P.node = (int)v;
-        P.node2 = partner[v];
+        P.nodes = nodes;
+        P.node = nodes[0];
         // sep / span: how many image rows / columns the taps that share one activation box are apart at most
         P.sep = 0;
         P.span = 0;
-        std::vector<int> in_edges(n.in_edges.begin(), n.in_edges.end());
-        if (P.node2 >= 0) in_edges.insert(in_edges.end(), g->nodes[P.node2].in_edges.begin(), g->nodes[P.node2].in_edges.end());
-        for (int e : in_edges) {
+        for (int e : P.in_edges(g)) {
             const SrHostEdge& he = g->edges[e];
-            if (is_stem(g, he)) {
-                StemPlan S;
-                S.edge = e;
-                S.Kp = stem_kp(he.K);
-                const size_t bytes = (size_t)g->batch * n.d.h * n.d.w * S.Kp * 2;
-                S.buf[0] = take(bytes);
-                S.buf[1] = take(bytes);
-                E->stem_of_edge[e] = (int)E->stems.size();
-                E->stems.push_back(S);
-                continue;
-            }
+            if (is_stem(g, he)) continue;
             for (int r0 = 0; r0 < he.stride_eff; ++r0) {
                 int lo = 1 << 20, hi = -(1 << 20);
                 for (int t = 0; t < he.k_eff; ++t) {
@@ -1505,11 +1530,8 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
                 if (hi >= lo) P.sep = P.span = std::max(P.sep, hi - lo);
             }
         }
-        E->node_of[v] = (int)E->nodes.size();
-        E->nodes.push_back(P);
-    }
-    for (size_t v = 0; v < g->nodes.size(); ++v)
-        if (leader[v] >= 0) E->node_of[v] = E->node_of[leader[v]];
+        return P;
+    };
     std::map<int, int> held;
     held[1] = g->sm_count;
     for (int cluster = 2; cluster <= kMaxParts; cluster *= 2) held[cluster] = clusters_held(g, cluster);
@@ -1517,21 +1539,18 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
     E->group_tiles.assign(g->groups.size(), {});
     int n_tiles = 0;
     for (size_t gi = 0; gi < g->groups.size(); ++gi) {
+        const size_t first_plan = E->nodes.size();
         std::vector<int> members;
-        for (int v : g->groups[gi])
-            if (E->node_of[v] >= 0 && leader[v] < 0) members.push_back(E->node_of[v]);
         // What can be chosen per plan: the most columns of its tiles (256, 128, 64: variants 0, 1, 2), and the parts of its items.
         struct Variant { NodePlan P; std::vector<TcTile> tiles; int box_kb = 1, w_slot = 1024, words = 0; long long plain, cycles[2][kMaxW + 1]; };   // of an item; by crowded, slots
         struct Choice { int v, parts; };
-        std::vector<std::vector<Variant>> variants(members.size());
+        std::vector<std::vector<Variant>> variants;
         auto variant_of = [&](size_t m, int max_cols) {
             Variant V;
             V.P = E->nodes[members[m]];
             const SrHostNode& n = g->nodes[V.P.node];
             double blocks = 0, boxes = 0;
-            std::vector<int> in_edges(n.in_edges.begin(), n.in_edges.end());
-            if (V.P.node2 >= 0) in_edges.insert(in_edges.end(), g->nodes[V.P.node2].in_edges.begin(), g->nodes[V.P.node2].in_edges.end());
-            for (int e : in_edges) {
+            for (int e : V.P.in_edges(g)) {
                 const SrHostEdge& he = g->edges[e];
                 const double cb = is_stem(g, he) ? 1.0 : (double)(g->nodes[he.d.src].d.c / block_k(g->nodes[he.d.src].d.c));
                 const int kk = is_stem(g, he) ? 1 : he.k_eff, sd = is_stem(g, he) ? 1 : std::min(he.k_eff, he.stride_eff);
@@ -1631,56 +1650,79 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
         std::vector<Choice> best;
         int best_cluster = 1, best_grid = 0;
         long long best_cost = -1;
-        size_t widest_items = 0;
-        for (size_t m = 0; m < members.size(); ++m) {
-            for (int cols = kMaxCols; cols >= 64; cols /= 2) variants[m].push_back(variant_of(m, cols));
-            widest_items += variants[m][0].tiles.size();
-        }
-        const bool few = g->opt_b_units == 0 && g->opt_tile_w == 0 && widest_items <= 3 * (size_t)g->sm_count;
-        for (int start = 0; start < 3 && !members.empty(); ++start) {
-            size_t items = 0;
-            for (size_t m = 0; m < members.size(); ++m) items += variants[m][start].tiles.size();
-            for (int cluster = 1; cluster <= (few ? kMaxParts : 1); cluster *= 2)
-                // all SMs, or half of them: then the next launch starts up on the others
-                for (int half = 0; half < (few ? 2 : 1); ++half) {
-                    const int ctas = (half ? std::min(held[cluster], g->sm_count / 2 / cluster) : held[cluster]) * cluster;
-                    std::vector<Choice> ch(members.size(), Choice{start, 1});
-                    for (;;) {
-                        const TcEngine::Launch L = rings(ch, 0);
-                        const Bound b = bound_of(ch, L, few);
-                        const int grid = (int)std::min<size_t>((b.parts + cluster - 1) / cluster * cluster, ctas);
-                        const long long fixed = (few ? b.tail : 0) + (grid > g->sm_count / 2 ? kLateStart : 0) + (cluster > 1 ? kClusterStart : 0);
-                        if (L.fits && (best_cost < 0 || std::max(b.longest, b.total / grid) + fixed < best_cost)) {
-                            const std::vector<TcWork> work = work_of(ch, L, few, false);
-                            const long long span = cluster > 1 ? spread_split(work, grid, cluster, nullptr) : spread_items(work, work.size(), grid, nullptr);
-                            if (span >= 0 && (best_cost < 0 || span + fixed < best_cost)) {
-                                best_cost = span + fixed;
-                                best = ch;
-                                best_cluster = cluster;
-                                best_grid = grid;
+        bool few = false;
+        auto search = [&](const std::vector<std::vector<int>>& plans) {
+            E->nodes.resize(first_plan);
+            members.clear();
+            for (const std::vector<int>& nodes : plans) {
+                members.push_back((int)E->nodes.size());
+                E->nodes.push_back(plan_of(nodes));
+            }
+            variants.assign(members.size(), {});
+            best_cost = -1;
+            size_t widest_items = 0;
+            for (size_t m = 0; m < members.size(); ++m) {
+                for (int cols = kMaxCols; cols >= 64; cols /= 2) variants[m].push_back(variant_of(m, cols));
+                widest_items += variants[m][0].tiles.size();
+            }
+            few = g->opt_b_units == 0 && g->opt_tile_w == 0 && widest_items <= 3 * (size_t)g->sm_count;
+            for (int start = 0; start < 3 && !members.empty(); ++start) {
+                size_t items = 0;
+                for (size_t m = 0; m < members.size(); ++m) items += variants[m][start].tiles.size();
+                for (int cluster = 1; cluster <= (few ? kMaxParts : 1); cluster *= 2)
+                    // all SMs, or half of them: then the next launch starts up on the others
+                    for (int half = 0; half < (few ? 2 : 1); ++half) {
+                        const int ctas = (half ? std::min(held[cluster], g->sm_count / 2 / cluster) : held[cluster]) * cluster;
+                        std::vector<Choice> ch(members.size(), Choice{start, 1});
+                        for (;;) {
+                            const TcEngine::Launch L = rings(ch, 0);
+                            const Bound b = bound_of(ch, L, few);
+                            const int grid = (int)std::min<size_t>((b.parts + cluster - 1) / cluster * cluster, ctas);
+                            const long long fixed = (few ? b.tail : 0) + (grid > g->sm_count / 2 ? kLateStart : 0) + (cluster > 1 ? kClusterStart : 0);
+                            if (L.fits && (best_cost < 0 || std::max(b.longest, b.total / grid) + fixed < best_cost)) {
+                                const std::vector<TcWork> work = work_of(ch, L, few, false);
+                                const long long span = cluster > 1 ? spread_split(work, grid, cluster, nullptr) : spread_items(work, work.size(), grid, nullptr);
+                                if (span >= 0 && (best_cost < 0 || span + fixed < best_cost)) {
+                                    best_cost = span + fixed;
+                                    best = ch;
+                                    best_cluster = cluster;
+                                    best_grid = grid;
+                                }
                             }
+                            if (!few) break;
+                            const Choice now = ch[b.at];
+                            const std::vector<Variant>& of = variants[b.at];
+                            Choice ways[2] = {Choice{now.v, now.parts * 2}, Choice{now.v + 1, now.parts}};
+                            while (ways[1].v < 2 && of[ways[1].v].tiles.size() == of[now.v].tiles.size()) ++ways[1].v;
+                            int way = -1;
+                            long long shortest = 0;
+                            for (int w = 0; w < 2; ++w) {
+                                if (w == 0 && (ways[0].parts > cluster || (int)of[now.v].P.kbs.size() < 2 * ways[0].parts)) continue;
+                                if (w == 1 && (ways[1].v > 2 || of[ways[1].v].tiles.size() == of[now.v].tiles.size())) continue;
+                                ch[b.at] = ways[w];
+                                const Bound c = bound_of(ch, rings(ch, 0), few);
+                                const long long t = std::max(c.longest, c.total / ctas) + c.tail;
+                                if (way < 0 || t < shortest) { way = w; shortest = t; }
+                            }
+                            if (way < 0) break;
+                            ch[b.at] = ways[way];
                         }
-                        if (!few) break;
-                        const Choice now = ch[b.at];
-                        const std::vector<Variant>& of = variants[b.at];
-                        Choice ways[2] = {Choice{now.v, now.parts * 2}, Choice{now.v + 1, now.parts}};
-                        while (ways[1].v < 2 && of[ways[1].v].tiles.size() == of[now.v].tiles.size()) ++ways[1].v;
-                        int way = -1;
-                        long long shortest = 0;
-                        for (int w = 0; w < 2; ++w) {
-                            if (w == 0 && (ways[0].parts > cluster || (int)of[now.v].P.kbs.size() < 2 * ways[0].parts)) continue;
-                            if (w == 1 && (ways[1].v > 2 || of[ways[1].v].tiles.size() == of[now.v].tiles.size())) continue;
-                            ch[b.at] = ways[w];
-                            const Bound c = bound_of(ch, rings(ch, 0), few);
-                            const long long t = std::max(c.longest, c.total / ctas) + c.tail;
-                            if (way < 0 || t < shortest) { way = w; shortest = t; }
-                        }
-                        if (way < 0) break;
-                        ch[b.at] = ways[way];
                     }
-                }
-            if (items > 8 * (size_t)g->sm_count) break;            // plenty of items: smaller tiles only cost copies
+                if (items > 8 * (size_t)g->sm_count) break;            // plenty of items: smaller tiles only cost copies
+            }
+        };
+        // Joined as far as they go, or in twos: the launch that ends first (with few tiles, more and shorter items may; joined where it
+        // is 3 % ahead).  Deepest CIFAR10 network, us per frame in twos / joined: 13.2 / 13.1, 19.0 / 24.0, 43.7 / 44.8, 74.0 / 66.9 at 4,
+        // 16, 64, 128 samples; with four added layers 17.0 / 12.4, 36.6 / 34.2, 108 / 95 at 8, 64, 256.
+        const auto joined = join_nodes(g, g->groups[gi], g->opt_tc_fuse ? kMaxFused : 1), twos = join_nodes(g, g->groups[gi], g->opt_tc_fuse ? 2 : 1);
+        search(joined);
+        if (joined != twos) {
+            const long long cost = best_cost;
+            search(twos);
+            if (best_cost < 0 || (cost >= 0 && cost * 103 <= best_cost * 100)) search(joined);
         }
+        for (int ni : members)
+            for (int v : E->nodes[ni].nodes) E->node_of[v] = ni;
         TcEngine::Launch L;
         if (!members.empty()) {
             if (best_cost < 0) return SR_ERR_UNSUPPORTED;
@@ -1782,17 +1824,14 @@ sr_status sr_tc_bind(sr_graph* g)
     for (NodePlan& P : E->nodes) {
         const SrHostNode& n = g->nodes[P.node];
         TcNode d{};
-        d.state[0] = ws + n.state[0].offset;
-        d.state[1] = ws + n.state[1].offset;
-        d.bias = reinterpret_cast<const float*>(ws + n.bias.offset);
-        d.H = n.d.h; d.W = n.d.w; d.C = n.d.c; d.act = n.d.act;
-        if (P.node2 >= 0) {
-            const SrHostNode& n2 = g->nodes[P.node2];
-            d.state2[0] = ws + n2.state[0].offset;
-            d.state2[1] = ws + n2.state[1].offset;
-            d.bias2 = reinterpret_cast<const float*>(ws + n2.bias.offset);
-            d.act2 = n2.d.act;
-            d.fused = 1;
+        d.H = n.d.h; d.W = n.d.w; d.C = n.d.c;
+        d.n_nodes = (int)P.nodes.size();
+        d.rows = d.n_nodes > 1 ? n.d.c : 0;
+        for (int q = 0; q < d.n_nodes; ++q) {
+            const SrHostNode& nq = g->nodes[P.nodes[q]];
+            for (int par = 0; par < 2; ++par) d.state[q][par] = ws + nq.state[par].offset;
+            d.bias[q] = reinterpret_cast<const float*>(ws + nq.bias.offset);
+            if (nq.d.act == 1) d.relu |= 1 << q;
         }
         d.tw = P.tw; d.th = P.th; d.tb = P.tb; d.sep = P.sep;
         d.nl = P.nl;
@@ -1976,11 +2015,17 @@ sr_status sr_tc_set_weights(sr_graph* g, int edge, const float* w_eff)
     // (K-blocks of an edge that follow one another go in one copy)
     bool any = false;
     std::vector<uint16_t> h;
+    auto row_of = [&](const KbHost& kb) {
+        for (const auto& u : kb.users)
+            if (u.first == edge) return u.second;
+        return -1;
+    };
     for (size_t i = 0; i < P.kbs.size();) {
-        if (P.kbs[i].edge != edge && P.kbs[i].edge2 != edge) { ++i; continue; }
+        const int row_off = row_of(P.kbs[i]);
+        if (row_off < 0) { ++i; continue; }
         size_t end = i;
         int width = 0;
-        while (end < P.kbs.size() && P.kbs[end].edge == P.kbs[i].edge) width += P.kbs[end++].bk;
+        while (end < P.kbs.size() && row_of(P.kbs[end]) == row_off) width += P.kbs[end++].bk;
         h.assign((size_t)t.d.c * width, 0);
         int col = 0;
         for (size_t j = i; j < end; ++j) {
@@ -1998,7 +2043,6 @@ sr_status sr_tc_set_weights(sr_graph* g, int edge, const float* w_eff)
             }
             col += kb.bk;
         }
-        const int row_off = P.kbs[i].edge == edge ? P.kbs[i].row_off : 64;
         char* dst = g->ws + P.wcat.offset + ((size_t)row_off * P.k_total + P.kbs[i].k_off) * 2;
         if (cudaMemcpy2D(dst, (size_t)P.k_total * 2, h.data(), (size_t)width * 2, (size_t)width * 2, t.d.c, cudaMemcpyHostToDevice) != cudaSuccess)
             return SR_ERR_CUDA;

@@ -252,3 +252,15 @@ def test_long_reductions_of_few_pixels(cin, c, k, stride, size, batch):
     parity.check_stepwise(g, "p", samples=samples, zero_bias=False)
     g.patterns["q"] = [0, 1, 0, 1, 0]
     parity.check_stepwise(g, "q", samples=samples, zero_bias=False)
+
+
+@pytest.mark.parametrize("c,n", [(32, 3), (32, 4), (32, 5), (64, 3)])
+def test_several_narrow_nodes_that_share_sources(c, n):
+    # a block in which every earlier node feeds every later one, as in the paper's CIFAR10 networks: up to 128 channels run as one
+    # plan; the nodes' activations and biases stay their own, the last plan may be part empty
+    nodes = [Node("in", 12, 20, 3, IDENTITY)] + [Node("n%d" % i, 12, 20, c, IDENTITY if i == 1 else RELU) for i in range(n)]
+    edges = [Edge(0, 1, CONV, 5, 1), Edge(1, 1, CONV, 3, 1)] + [Edge(i, j, CONV, 3, 1) for i in range(1, n + 1) for j in range(i + 1, n + 1)]
+    g = tiny("block", nodes + [Node("o", 1, 1, 4, IDENTITY)], edges + [Edge(i, n + 1, GAP_DENSE) for i in range(1, n + 1)], batch=3, frames=4)
+    for fuse in (1, 0):
+        parity.check_stepwise(g, "p", zero_bias=False, tc_fuse=fuse)
+    parity.check_stepwise(g, "p", zero_bias=False, tc_lists=1, weight_ring_units=2, tile_width=16)
