@@ -299,7 +299,7 @@ void refresh_staging(sr_graph* g, cudaStream_t s)
 // them: windows exist only for patterns in which every edge that bridges a frame leaves an input node.)
 void leave_window(sr_graph* g) { g->in_window.assign(g->in_window.size(), 0); }
 
-// The dense resident kernel fetches input frames in 16-byte words.
+// The dense resident kernel fetches input frames in words of four values (the states lie on larger boundaries).
 bool dense_resident_takes(const sr_graph* g, const void* const* in_dev)
 {
     if (!sr_dn_available(g)) return false;
@@ -675,7 +675,7 @@ sr_status sr_graph_reset(sr_graph* g, const void* const* in0_dev, void* stream)
     SrFrameCtl c{};
     c.t = -1;                                                    // "the input of frame 0"
     for (size_t i = 0; i < g->input_nodes.size(); ++i) c.in_base[i] = in0_dev[i];
-    const bool resident = sr_rs_available(g);                    // a resident run does not read staged edges
+    const bool resident = sr_rs_available(g) || sr_dn_available(g);      // a resident run does not read staged edges
     g->launches += sr_launch_input(g, by_value(c), ~0u, resident ? 0u : 2u, SrFollow(), &g->r_clear, s);
     g->stage_dirty = resident;
     return cuda_ok(cudaGetLastError()) ? SR_OK : SR_ERR_CUDA;
@@ -698,6 +698,7 @@ try {
         st = sr_dn_launch(g, 1, make_ctl(g, in_next_dev, false, out_dev), s);
         if (st != SR_OK) return st;
         g->launches += 1;
+        g->stage_dirty = true;
     } else {
         refresh_staging(g, s);
         g->launches += enqueue_frames(g, by_value(make_ctl(g, in_next_dev, false, out_dev)), 1, s);
@@ -737,6 +738,7 @@ try {
         if (st != SR_OK) return st;
         g->launches += 1;
         g->t += T;
+        g->stage_dirty = true;
         return cuda_ok(cudaGetLastError()) ? SR_OK : SR_ERR_CUDA;
     }
     refresh_staging(g, s);

@@ -1,5 +1,6 @@
-// Dense resident engine: the frame update  x_v = sigma(b_v + sum_e W_e x_src(e))  (paper Sec. A1.2) of a small network
-// whose edges are all dense, in fp32, for all T frames of a run in ONE launch.
+// Dense resident engine: the frame update  x_v = sigma(b_v + sum_e f_e(theta_e, x_src(e)))  (paper Sec. A1.2) of a small network
+// whose edges are dense, or small convolutions, for all T frames of a run in ONE launch.  Arithmetic is fp32; bf16 states are
+// rounded when they are stored and lie in shared memory as fp32.
 //
 // Such a network (the paper's H2 / O layers, a tiny MLP) moves a few hundred kilobytes of weights per frame and does a
 // million multiply-adds: launched frame by frame it is pure launch latency.  Here a cluster of eight or sixteen CTAs
@@ -24,7 +25,15 @@
 // sequences per cluster, sixteen warps, scalar multiply-adds and a cluster barrier per frame, 656 us (2.49) with the packed
 // multiply-adds and the counted stores, whose shared-memory loads per step stayed the same, and take 388 us (1.45) with two
 // sequences per cluster.
+// Convolutions (a few thousand weights, the paper's H1 of the MNIST networks): every CTA keeps all weights of the edge, [K][C].  A work
+// unit is eight quads (a pixel and four neighbouring channels each) for up to four sequences; a lane takes a quad and a quarter of the
+// reduction, taps outside the image left out, and after a sum over the quarters writes four channels of one sequence.  A rank computes
+// a run of quads; the sequences lie quad by quad side by side (and an unused one, against bank conflicts), so what a rank has computed
+// is one piece, which goes to every other CTA as one bulk copy when its last unit is done.  MNIST network SR, fp32, 100 sequences, us
+// per frame: 15.4 launched, 8.1 here (sequential 27.0 and 9.3).  Bound by the instructions around the multiply-adds with two warps
+// per scheduler; walked tap by tap instead of row by row it took 11.2.
 // The sums run in a fixed order, so results are reproducible bit for bit.
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -33,6 +42,7 @@
 #include <vector>
 
 #include "sr_dense.h"
+#include "sr_resident.h"
 
 namespace {
 
@@ -42,12 +52,15 @@ constexpr int kDnMoreThanHalf = 120 * 1024;   // of an SM's shared memory, bytes
 constexpr int kDnMaxCluster = 16;      // CTAs per cluster: 8, or 16 (a non-portable size) for rollouts with one level per frame
 constexpr int kDnWarps = 8;            // 256 threads: a work unit keeps 64 registers of packed accumulators and its operands
 constexpr int kDnRows = 4;             // output rows per work unit
-constexpr int kDnSmemMax = 220 * 1024;
+constexpr int kDnHeld = 8;             // vectors of the next bf16 input frame that a fetching thread holds in registers
+constexpr int kDnConvWork = 1 << 18;   // multiply-adds per sample and frame of all convolutions, most
+constexpr int kDnSmemMax = 226 * 1024;
 
 struct DnNode {
-    float* gstate[2];                  // state buffers in global memory, [B][C], by frame parity
+    void* gstate[2];                   // state buffers in global memory, [B][C], by frame parity
     const float* bias;
-    int32_t C, Cpad, act, is_input, input_slot, is_output;
+    int32_t C, Cpad, act, is_input, input_slot, is_output;   // C: values of a sample
+    int32_t n_bias, step, seq;         // in shared memory: floats from one vector of four values to the next, from one sequence to the next
     int32_t buf[3];                    // float offsets of the shared-memory state buffers: frame f lives in buf[f % 3] (input
                                        // nodes) or buf[f & 1] (others)
     int32_t bias_off;                  // float offset of the node's bias copy in shared memory
@@ -58,23 +71,38 @@ struct DnEdge { int32_t src, tgt, R, Kpad; };
 // One incoming edge of a work unit, ready to use (32 bytes): where the unit's weight rows start (floats from the
 // rank's first weight), the padded reduction length = row pitch of the weights, the row pitch of the source state,
 // the frames the edge looks back (Eq. 2), and the source's shared-memory buffers (three for an input node).
-struct DnTerm { int32_t w_off, Kpad, xp, R, n_buf, buf[3]; };
+struct DnTerm { int32_t w_off, Kpad, xp, R, n_buf, buf[3]; };   // n_buf: also, << 8, floats from one vector of four to the next
 static_assert(sizeof(DnTerm) == 32, "read as two 16-byte words");
 
-// Up to four rows of a node with everything a warp needs (48 bytes).  nrows = 0: no unit (a gap in a warp's list).
+// The second term of an edge of a convolution unit; there Kpad = k | stride << 8 | pad << 16.
+struct DnConv { int32_t Hs, Ws, Cs, pad_[5]; };
+static_assert(sizeof(DnConv) == sizeof(DnTerm), "lies among the terms");
+
+// Up to four rows of a node with everything a warp needs (48 bytes).  nrows = 0: no unit (a gap in a warp's list).  A convolution unit:
+// nrows = quads, row0 = the first of them, Cpad = floats from one to the next, channels, width, first = channels and width of the node,
+// first sequence.
 struct DnUnit {
     int32_t nrows, row0, term0, n_terms;
-    int32_t bias_off, Cpad, C, flags;                        // flags: 1 = ReLU, 2 = the output node
-    int32_t buf[2], pad_[2];                                 // the node's two shared-memory buffers by frame parity
+    int32_t bias_off, Cpad, C, flags;                        // flags: 1 = ReLU, 2 = the output node, 4 = a convolution
+    int32_t buf[2];                                          // the node's two shared-memory buffers by frame parity
+    int16_t channels, width, first, pad_;
 };
 static_assert(sizeof(DnUnit) == 48, "read as three 16-byte words");
 
 constexpr int kDnMaxTerms = 256;
+constexpr int kDnMaxSlices = kDnMaxNodes;
+
+// What a rank computes of a convolution node: in both buffers of the node, the same place in every CTA's copy.
+struct DnSlice { int32_t off[2], bytes, pad_; };
 
 struct DnBlobHdr {                     // head of a rank's blob; the rank's weight slices follow
     int32_t n_units, fetch_mask, idle, pad_;                 // fetch_mask: warps that fetch input frames; idle: the rank has no unit
     int32_t level_begin[kDnMaxLevels + 1];                   // units of level l: [level_begin[l-1], level_begin[l]); warp w
     int32_t pad2_[3];                                        // takes entries w, w + kDnWarps, ... of a level
+    int32_t level_bytes[kDnMaxLevels];                       // bytes of a level's new states that arrive from elsewhere (or are
+                                                             // sent to the rank itself)
+    int32_t conv_units[kDnMaxLevels], first_slice[kDnMaxLevels + 4];      // convolution units of a level, and slices
+    DnSlice slices[kDnMaxSlices];
     DnUnit units[kDnMaxUnits];
     DnTerm terms[kDnMaxTerms];
 };
@@ -84,7 +112,6 @@ static_assert(offsetof(DnBlobHdr, units) % 16 == 0 && offsetof(DnBlobHdr, terms)
 struct DnParams {
     int32_t n_nodes, n_edges, n_levels, B;
     int32_t blob_bytes, hdr_floats, total_floats, n_idle;    // n_idle: ranks without a unit
-    int32_t level_bytes[kDnMaxLevels];                       // bytes that a level's new states are, in one CTA's copy
     int32_t* error;                                          // device-side error code
     long long wait_limit;                                    // cycles after which a wait gives up
     const unsigned char* blobs;        // one blob of blob_bytes per rank of the cluster
@@ -180,10 +207,15 @@ __device__ __forceinline__ void dn_halve(float (&out)[R][N / 2], const float (&v
         }
 }
 
+// A value as a state of type T holds it.
+template <typename T>
+__device__ __forceinline__ float dn_rounded(float v) { return sizeof(T) == 2 ? __bfloat162float(__float2bfloat16_rn(v)) : v; }
+
 // One work unit: up to R rows of a node for the S sequences of the cluster, relative frame f -> f + 1.
 // The loads of a reduction step are issued ahead of the multiply-adds that use them: the weights and the first four
 // sequences of step i + 1 while the last four sequences of step i are still being multiplied.
-template <int R, int CL, int S>
+// (MIXED: a source may be a convolution, whose vectors of four lie further apart.)
+template <int R, int CL, int S, typename T, bool MIXED>
 __device__ __forceinline__ void dn_unit(const DnBlobHdr* H, const DnUnit& un, float* dn_mem, const float* wsm,
                                         const SrFrameCtl& init, int f, int lane, int b0, int nb, long long run0, uint32_t bar)
 {
@@ -195,8 +227,8 @@ __device__ __forceinline__ void dn_unit(const DnBlobHdr* H, const DnUnit& un, fl
     for (int ti = un.term0; ti < un.term0 + un.n_terms; ++ti) {
         const DnTerm tm = H->terms[ti];
         const int sf = f + 1 - tm.R;                                  // Eq. 2: the source frame
-        const int bi = tm.n_buf == 3 ? sf % 3 : (sf & 1);
-        const float* xs = dn_mem + (bi == 0 ? tm.buf[0] : (bi == 1 ? tm.buf[1] : tm.buf[2])) + lane * 4;
+        const int bi = (tm.n_buf & 0xFF) == 3 ? sf % 3 : (sf & 1), step = MIXED ? tm.n_buf >> 8 : 4;
+        const float* xs = dn_mem + (bi == 0 ? tm.buf[0] : (bi == 1 ? tm.buf[1] : tm.buf[2])) + lane * step;
         const float* w0 = wsm + tm.w_off + lane * 4;
         int ro[R];                                                    // rows the unit does not have repeat row 0 (their sums are dropped)
 #pragma unroll
@@ -209,23 +241,24 @@ __device__ __forceinline__ void dn_unit(const DnBlobHdr* H, const DnUnit& un, fl
         for (int r = 0; r < R; ++r) a[r] = *reinterpret_cast<const ulonglong2*>(w0 + ro[r]);
 #pragma unroll
         for (int b = 0; b < G; ++b) xa[b] = *reinterpret_cast<const ulonglong2*>(xs + b * xp);
-        for (int k = 0; k < n_k; k += 128) {
+        for (int k = 0, x = 0; k < n_k; k += 128, x += 32 * step) {
             ulonglong2 an[R], xb[G];
             const int kn = k + 128 < n_k ? k + 128 : k;               // the last step re-reads itself (no branch)
+            const int xn = MIXED ? (k + 128 < n_k ? x + 32 * step : x) : kn;
             if (S > G) {
 #pragma unroll
-                for (int b = 0; b < G; ++b) xb[b] = *reinterpret_cast<const ulonglong2*>(xs + (b + G) * xp + k);
+                for (int b = 0; b < G; ++b) xb[b] = *reinterpret_cast<const ulonglong2*>(xs + (b + G) * xp + (MIXED ? x : k));
                 dn_fma<R, S, G>(acc2, a, xa, 0);
 #pragma unroll
                 for (int r = 0; r < R; ++r) an[r] = *reinterpret_cast<const ulonglong2*>(w0 + ro[r] + kn);
 #pragma unroll
-                for (int b = 0; b < G; ++b) xa[b] = *reinterpret_cast<const ulonglong2*>(xs + b * xp + kn);
+                for (int b = 0; b < G; ++b) xa[b] = *reinterpret_cast<const ulonglong2*>(xs + b * xp + xn);
                 dn_fma<R, S, G>(acc2, a, xb, S - G);
             } else {
 #pragma unroll
                 for (int r = 0; r < R; ++r) an[r] = *reinterpret_cast<const ulonglong2*>(w0 + ro[r] + kn);
 #pragma unroll
-                for (int b = 0; b < G; ++b) xb[b] = *reinterpret_cast<const ulonglong2*>(xs + b * xp + kn);
+                for (int b = 0; b < G; ++b) xb[b] = *reinterpret_cast<const ulonglong2*>(xs + b * xp + xn);
                 dn_fma<R, S, G>(acc2, a, xa, 0);
 #pragma unroll
                 for (int b = 0; b < G; ++b) xa[b] = xb[b];
@@ -272,13 +305,16 @@ __device__ __forceinline__ void dn_unit(const DnBlobHdr* H, const DnUnit& un, fl
         z[r] += dn_mem[un.bias_off + un.row0 + (r < un.nrows ? r : 0)];
         if (un.flags & 1) z[r] = fmaxf(z[r], 0.f);
     }
+    float y[R];                                                       // as the state holds them
+#pragma unroll
+    for (int r = 0; r < R; ++r) y[r] = dn_rounded<T>(z[r]);
     const uint32_t cell = dn_smem(dn_mem + (((f + 1) & 1) ? un.buf[1] : un.buf[0]) + b * un.Cpad + un.row0);
     constexpr uint32_t kPerLane = CL > kLanes ? CL / kLanes : 1;      // ranks that each of them serves
     const uint32_t q = (uint32_t)(lane % kLanes) * kPerLane;
     if (q >= CL) {
         // (more lanes than ranks: nothing to send)
     } else if (R == 4 && un.nrows == 4 && (un.row0 & 3) == 0) {
-        const float z4[4] = {z[0], z[1], z[2 % R], z[3 % R]};
+        const float z4[4] = {y[0], y[1], y[2 % R], y[3 % R]};
 #pragma unroll
         for (uint32_t i = 0; i < kPerLane; ++i) dn_st_async4(cell, bar, q + i, z4);
     } else {
@@ -286,7 +322,7 @@ __device__ __forceinline__ void dn_unit(const DnBlobHdr* H, const DnUnit& un, fl
         for (int r = 0; r < R; ++r)
             if (r < un.nrows) {
 #pragma unroll
-                for (uint32_t i = 0; i < kPerLane; ++i) dn_st_async(cell + 4 * r, bar, q + i, z[r]);
+                for (uint32_t i = 0; i < kPerLane; ++i) dn_st_async(cell + 4 * r, bar, q + i, y[r]);
             }
     }
     if ((un.flags & 2) && init.out_base && lane % kLanes == 0 && b < nb) {
@@ -297,18 +333,176 @@ __device__ __forceinline__ void dn_unit(const DnBlobHdr* H, const DnUnit& un, fl
     }
 }
 
-template <int CL, int S>
+// A convolution unit (see the file comment): eight quads, four slices of the reduction (lane / 8), N sequences.
+template <int CL, int N, typename T>
+__device__ __forceinline__ void dn_conv_unit(const DnBlobHdr* H, const DnUnit& un, float* dn_mem, const float* wsm,
+                                             const SrFrameCtl& init, int f, int lane, int b0, int nb, long long run0, uint32_t bar,
+                                             int level, uint32_t rank, int* done)
+{
+    const int slice = lane >> 3, at = min(lane & 7, un.nrows - 1);
+    const int quads = un.channels >> 2, idx = un.row0 + at, C = un.channels;
+    const int px = idx / quads, ch = (idx - px * quads) * 4, oy = px / un.width, ox = px - oy * un.width;
+    unsigned long long acc[N][2];
+#pragma unroll
+    for (int s = 0; s < N; ++s) acc[s][0] = acc[s][1] = 0ull;
+    auto pair = [](float v) {
+        unsigned long long r;
+        asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+        return r;
+    };
+    for (int ti = un.term0; ti < un.term0 + 2 * un.n_terms; ti += 2) {
+        const DnTerm tm = H->terms[ti];
+        const DnConv cv = *reinterpret_cast<const DnConv*>(&H->terms[ti + 1]);
+        const int k = tm.Kpad & 0xFF, stride = (tm.Kpad >> 8) & 0xFF, pad = tm.Kpad >> 16, Cs = cv.Cs, xp = tm.xp;
+        const int sf = f + 1 - tm.R;                                  // Eq. 2: the source frame
+        const int bi = (tm.n_buf & 0xFF) == 3 ? sf % 3 : (sf & 1), step = tm.n_buf >> 8;
+        const int y0 = oy * stride - pad, x0 = ox * stride - pad;
+        const float* xs = dn_mem + (bi == 0 ? tm.buf[0] : (bi == 1 ? tm.buf[1] : tm.buf[2])) + un.first * xp;
+        const int origin = (y0 * cv.Ws + x0) * Cs;
+        const float* w0 = wsm + tm.w_off + ch;
+        // a filter row is one run of values; the slices take its values (in fours where the source has whole vectors) in turn
+        const int kx0 = max(0, -x0), kx1 = min(k, cv.Ws - x0);
+        for (int ky = max(0, -y0); ky < min(k, cv.Hs - y0); ++ky) {
+            const int at0 = origin + ky * cv.Ws * Cs;
+            const float* w = w0 + ky * k * Cs * C;
+            if ((Cs & 3) == 0) {
+                const int e0 = kx0 * Cs >> 2, e1 = kx1 * Cs >> 2;
+                int e = e0 + ((slice - e0) & 3);
+                const float* x = xs + ((at0 >> 2) + e) * step;
+                const float* wp = w + 4 * e * C;
+#pragma unroll 2
+                for (; e < e1; e += 4, x += 4 * step, wp += 16 * C) {
+                    float4 v[N];
+                    ulonglong2 wv[4];
+#pragma unroll
+                    for (int s = 0; s < N; ++s) v[s] = *reinterpret_cast<const float4*>(x + s * xp);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) wv[q] = *reinterpret_cast<const ulonglong2*>(wp + q * C);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+#pragma unroll
+                        for (int s = 0; s < N; ++s) {
+                            const unsigned long long xx = pair(q == 0 ? v[s].x : q == 1 ? v[s].y : q == 2 ? v[s].z : v[s].w);
+                            dn_fma2(acc[s][0], wv[q].x, xx);
+                            dn_fma2(acc[s][1], wv[q].y, xx);
+                        }
+                }
+            } else {
+                const int e0 = kx0 * Cs, e1 = kx1 * Cs;
+                int e = e0 + ((slice - e0) & 3);
+                const float* x = xs + at0 + e;
+                const float* wp = w + e * C;
+#pragma unroll 2
+                for (; e < e1; e += 4, x += 4, wp += 4 * C) {
+                    const ulonglong2 wv = *reinterpret_cast<const ulonglong2*>(wp);
+#pragma unroll
+                    for (int s = 0; s < N; ++s) {
+                        const unsigned long long xx = pair(x[s * xp]);
+                        dn_fma2(acc[s][0], wv.x, xx);
+                        dn_fma2(acc[s][1], wv.y, xx);
+                    }
+                }
+            }
+        }
+    }
+    __syncwarp();
+    // Sum over the slices: halving steps until a lane holds the four channels of one sequence (N = 4: sequence `slice`; N = 2: sequence
+    // slice / 2, in two lanes).
+    float a[4][N], z[4];
+#pragma unroll
+    for (int s = 0; s < N; ++s) {
+        a[0][s] = __uint_as_float((uint32_t)acc[s][0]); a[1][s] = __uint_as_float((uint32_t)(acc[s][0] >> 32));
+        a[2][s] = __uint_as_float((uint32_t)acc[s][1]); a[3][s] = __uint_as_float((uint32_t)(acc[s][1] >> 32));
+    }
+    float h[4][N / 2];
+    dn_halve<4, N, 16>(h, a, lane);
+    if constexpr (N == 4) {
+        float h1[4][1];
+        dn_halve<4, 2, 8>(h1, h, lane);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) z[i] = h1[i][0];
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) z[i] = h[i][0] + __shfl_xor_sync(0xffffffffu, h[i][0], 8);
+    }
+    const int b = un.first + (N == 4 ? slice : slice >> 1);
+    const float4 bias = *reinterpret_cast<const float4*>(dn_mem + un.bias_off + ch);
+    z[0] += bias.x; z[1] += bias.y; z[2] += bias.z; z[3] += bias.w;
+    if (un.flags & 1)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) z[i] = fmaxf(z[i], 0.f);
+    if ((lane & 7) < un.nrows) {
+        if ((un.flags & 2) && init.out_base && b < nb && (N == 4 || (slice & 1) == 0)) {
+            float* o = init.out_base + (run0 + f) * init.out_stride + (long long)(b0 + b) * un.C + idx * 4;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) o[i] = z[i];
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) z[i] = dn_rounded<T>(z[i]);
+        if (N == 4 || (slice & 1) == 0)
+            *reinterpret_cast<float4*>(dn_mem + (((f + 1) & 1) ? un.buf[1] : un.buf[0]) + idx * un.Cpad + b * 4) = make_float4(z[0], z[1], z[2], z[3]);
+    }
+    // the unit that is the rank's last of its level sends what the rank has computed
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __threadfence_block();
+    __syncwarp();
+    int last = 0;
+    if (lane == 0) last = atomicAdd(done, 1) == H->conv_units[level] - 1;
+    if (__shfl_sync(0xffffffffu, last, 0)) {
+        __threadfence_block();
+        if (lane == 0) {
+            *done = 0;
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        if (lane < CL && lane != (int)rank)
+            for (int i = H->first_slice[level]; i < H->first_slice[level + 1]; ++i) {
+                const uint32_t src = dn_smem(dn_mem + H->slices[i].off[(f + 1) & 1]);
+                asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                             ::"r"(dn_map_rank(src, (uint32_t)lane)), "r"(src), "r"(H->slices[i].bytes), "r"(dn_map_rank(bar, (uint32_t)lane)) : "memory");
+            }
+    }
+    __syncwarp();
+}
+
+// `n` values (a multiple of 4) of a state in global memory into shared memory, as fp32.
+__device__ __forceinline__ void dn_load(float* dst, const float* src, int n, int tid, int nthr) { dn_fetch(dst, src, n, tid, nthr); }
+__device__ __forceinline__ void dn_load(float* dst, const __nv_bfloat16* src, int n, int tid, int nthr)
+{
+#pragma unroll 4
+    for (int i = tid * 4; i < n; i += nthr * 4) {
+        const uint2 q = *reinterpret_cast<const uint2*>(src + i);
+        *reinterpret_cast<float4*>(dst + i) = make_float4(__uint_as_float(q.x << 16), __uint_as_float(q.x & 0xFFFF0000u),
+                                                          __uint_as_float(q.y << 16), __uint_as_float(q.y & 0xFFFF0000u));
+    }
+}
+__device__ __forceinline__ float4 dn_widen(uint2 q)
+{
+    return make_float4(__uint_as_float(q.x << 16), __uint_as_float(q.x & 0xFFFF0000u), __uint_as_float(q.y << 16), __uint_as_float(q.y & 0xFFFF0000u));
+}
+__device__ __forceinline__ float dn_value(float v) { return v; }
+__device__ __forceinline__ float dn_value(__nv_bfloat16 v) { return __bfloat162float(v); }
+__device__ __forceinline__ void dn_store(float* p, float v) { *p = v; }
+__device__ __forceinline__ void dn_store(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
+__device__ __forceinline__ void dn_store4(float* p, const float* v) { *reinterpret_cast<float4*>(p) = *reinterpret_cast<const float4*>(v); }
+__device__ __forceinline__ void dn_store4(__nv_bfloat16* p, const float* v)
+{
+    const __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
+    *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+}
+
+template <int CL, int S, typename T, bool CONV>
 __global__ void __launch_bounds__(kDnWarps * 32, 1)
-sr_dense_kernel(const DnParams P, const SrFrameCtl init, int T)
+sr_dense_kernel(const DnParams P, const SrFrameCtl init, int n_frames)
 {
     extern __shared__ __align__(16) float dn_mem[];
     // the input nodes as the fetching warps need them: first float of this cluster's sequences in the caller's frame 0
     // of the run, floats from one frame to the next, floats per frame, the three shared-memory buffers
-    __shared__ const float* in_src[SR_MAX_INPUTS];
+    __shared__ const T* in_src[SR_MAX_INPUTS];
     __shared__ long long in_step[SR_MAX_INPUTS];
     __shared__ int in_len[SR_MAX_INPUTS], in_buf[SR_MAX_INPUTS][3], n_in;
     __shared__ uint64_t bars[kDnMaxLevels][2];               // per level and frame parity: the level's new states have arrived
-    __shared__ int gave_up;
+    __shared__ int gave_up, conv_done;
     const int tid = threadIdx.x, nthr = blockDim.x, warp = tid >> 5, lane = tid & 31;
     sr_let_successor_start();
     uint32_t rank;
@@ -323,16 +517,21 @@ sr_dense_kernel(const DnParams P, const SrFrameCtl init, int T)
         const float* blob = reinterpret_cast<const float*>(P.blobs + (size_t)rank * P.blob_bytes);
         dn_fetch(dn_mem, blob, P.blob_bytes / 4, tid, nthr);
         for (int i = P.blob_bytes / 4 + tid; i < P.total_floats; i += nthr) dn_mem[i] = 0.f;
+        __syncthreads();
+        for (int v = 0; v < P.n_nodes; ++v)                  // (biases, like weights, are the host's)
+            if (!P.nodes[v].is_input)
+                for (int i = tid; i < P.nodes[v].n_bias; i += nthr) dn_mem[P.nodes[v].bias_off + i] = P.nodes[v].bias[i];
     }
     const long long t0 = init.t, run0 = init.run_t;
     if (tid == 0) {
         gave_up = 0;
+        conv_done = 0;
         int n = 0;
         for (int v = 0; v < P.n_nodes; ++v) {
             const DnNode& nd = P.nodes[v];
             if (!nd.is_input) continue;
-            in_src[n] = reinterpret_cast<const float*>(static_cast<const char*>(init.in_base[nd.input_slot]) + run0 * init.in_stride_bytes[nd.input_slot]) + (size_t)b0 * nd.C;
-            in_step[n] = init.in_stride_bytes[nd.input_slot] / 4;
+            in_src[n] = reinterpret_cast<const T*>(static_cast<const char*>(init.in_base[nd.input_slot]) + run0 * init.in_stride_bytes[nd.input_slot]) + (size_t)b0 * nd.C;
+            in_step[n] = init.in_stride_bytes[nd.input_slot] / (long long)sizeof(T);
             in_len[n] = nb * nd.C;                           // input nodes have Cpad == C
             for (int i = 0; i < 3; ++i) in_buf[n][i] = nd.buf[i];
             ++n;
@@ -343,47 +542,74 @@ sr_dense_kernel(const DnParams P, const SrFrameCtl init, int T)
     __syncthreads();
     if (tid < 2 * P.n_levels) {
         // one arrival announces the bytes; in the last level every fetching thread arrives when its copies have landed, and
-        // every rank that sends no states does once per frame
-        const int l = tid >> 1, n_arrive = 1 + (l == P.n_levels - 1 ? 32 * __popc(H->fetch_mask) + P.n_idle : 0);
+        // every rank that sends no states does once per frame; in a level with convolutions, what this rank computes is complete
+        const int l = tid >> 1, n_arrive = 1 + (H->conv_units[l] > 0) + (l == P.n_levels - 1 ? 32 * __popc(H->fetch_mask) + P.n_idle : 0);
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(dn_smem(&bars[l][tid & 1])), "r"(n_arrive) : "memory");
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    // The other CTAs may store into this one from here on: its barriers stand, the buffers of frame 1 are zeroed, and those of frame 0,
+    // filled below, are stored into again only once this CTA has sent its part of frame 1.
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     // (Weights and tables do not depend on the kernel before this one; states and input frames do.)
     sr_wait_for_predecessor();
     // frame t of every node from the state buffers in global memory (relative frame 0)
     const int par0 = (int)(t0 & 1);
     for (int v = 0; v < P.n_nodes; ++v) {
         const DnNode& nd = P.nodes[v];
-        const float* gsrc = nd.gstate[par0] + (size_t)b0 * nd.C;
+        const T* gsrc = static_cast<const T*>(nd.gstate[par0]) + (size_t)b0 * nd.C;
         float* dst = dn_mem + nd.buf[0];
-        if (nd.Cpad == nd.C) dn_fetch(dst, gsrc, nb * nd.C, tid, nthr);                  // rows are contiguous: 16-byte copies
+        if (CONV && nd.step != 4)
+            for (int i = tid; i < nb * (nd.C / 4); i += nthr) {
+                const int b = i / (nd.C / 4), v = i - b * (nd.C / 4);
+                dn_load(dst + v * nd.step + b * nd.seq, gsrc + 4 * i, 4, 0, 1);
+            }
+        else if (nd.Cpad == nd.C) dn_load(dst, gsrc, nb * nd.C, tid, nthr);              // rows are contiguous: four values at a time
         else
-            for (int i = tid; i < nb * nd.C; i += nthr) dst[(i / nd.C) * nd.Cpad + (i % nd.C)] = gsrc[i];
-        if (!nd.is_input)
-            for (int i = tid; i < nd.C; i += nthr) dn_mem[nd.bias_off + i] = nd.bias[i];
+            for (int i = tid; i < nb * nd.C; i += nthr) dst[(i / nd.C) * nd.Cpad + (i % nd.C)] = dn_value(gsrc[i]);
     }
     // Input frame k of the run (relative frame k) -> buffer k % 3, by the warps of fetch_mask.
     const int f_nthr = 32 * __popc(H->fetch_mask);
     const int f_tid = (H->fetch_mask >> warp) & 1 ? 32 * __popc(H->fetch_mask & ((1 << warp) - 1)) + lane : -1;
     auto fetch_inputs = [&](int k) {
         if (f_tid < 0) return;
-        for (int i = 0; i < n_in; ++i) dn_fetch(dn_mem + in_buf[i][k % 3], in_src[i] + (k - 1) * in_step[i], in_len[i], f_tid, f_nthr);
+        for (int i = 0; i < n_in; ++i) dn_load(dn_mem + in_buf[i][k % 3], in_src[i] + (k - 1) * in_step[i], in_len[i], f_tid, f_nthr);
     };
     fetch_inputs(1);
+    // Vector v (four values) of input frame k: where it lies and where it goes; null beyond the last.
+    uint2 held[kDnHeld];
+    auto input_vector = [&](int v, int k, const T*& src) -> float* {
+        for (int i = 0; i < n_in; ++i) {
+            if (v * 4 < in_len[i]) {
+                src = in_src[i] + (k - 1) * in_step[i] + v * 4;
+                return dn_mem + in_buf[i][k % 3] + v * 4;
+            }
+            v -= in_len[i] / 4;
+        }
+        return nullptr;
+    };
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-    dn_cluster_sync();                                       // every CTA of the cluster has its buffers in place before remote writes start
+    __syncthreads();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 
-    for (int f = 0; f < T && !*(volatile int*)&gave_up; ++f) {                // relative frame f -> f + 1
+    for (int f = 0; f < n_frames && !*(volatile int*)&gave_up; ++f) {                // relative frame f -> f + 1
         // the input frame after the next one is on its way during this update; it has landed when the last level's barrier
         // completes
         const int par = (f + 1) & 1;
         const uint32_t phase = (uint32_t)(f >> 1) & 1u;
-        if (f + 1 < T) fetch_inputs(f + 2);
-        if (f_tid >= 0) asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(dn_smem(&bars[P.n_levels - 1][par])) : "memory");
+        if (sizeof(T) == 4) {
+            if (f + 1 < n_frames) fetch_inputs(f + 2);
+        } else if (f_tid >= 0 && f + 1 < n_frames) {
+#pragma unroll
+            for (int r = 0; r < kDnHeld; ++r) {
+                const T* src;
+                if (input_vector(f_tid + r * f_nthr, f + 2, src)) held[r] = *reinterpret_cast<const uint2*>(src);
+            }
+        }
+        if (sizeof(T) == 4 && f_tid >= 0) asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(dn_smem(&bars[P.n_levels - 1][par])) : "memory");
         for (int l = 1; l <= P.n_levels; ++l) {
             const uint32_t bar = dn_smem(&bars[l - 1][par]);
             if (tid == 0)
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(P.level_bytes[l - 1]) : "memory");
+                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(H->level_bytes[l - 1]) : "memory");
             // Nobody runs more than a frame ahead of a rank, because a level needs the states of every rank with a unit in it;
             // a rank without any says so instead.
             if (H->idle && l == P.n_levels && tid < CL)
@@ -391,31 +617,54 @@ sr_dense_kernel(const DnParams P, const SrFrameCtl init, int T)
             for (int u = H->level_begin[l - 1] + warp; u < H->level_begin[l]; u += kDnWarps) {
                 const DnUnit un = H->units[u];
                 if (un.nrows == 0) continue;
-                if (un.nrows > 2) dn_unit<4, CL, S>(H, un, dn_mem, wsm, init, f, lane, b0, nb, run0, bar);
-                else dn_unit<2, CL, S>(H, un, dn_mem, wsm, init, f, lane, b0, nb, run0, bar);
+                if (CONV && (un.flags & 4)) dn_conv_unit<CL, S < 4 ? 2 : 4, T>(H, un, dn_mem, wsm, init, f, lane, b0, nb, run0, bar, l - 1, rank, &conv_done);
+                else if (un.nrows > 2) dn_unit<4, CL, S, T, CONV>(H, un, dn_mem, wsm, init, f, lane, b0, nb, run0, bar);
+                else dn_unit<2, CL, S, T, CONV>(H, un, dn_mem, wsm, init, f, lane, b0, nb, run0, bar);
+            }
+            if (sizeof(T) == 2 && l == P.n_levels && f_tid >= 0) {   // the next input frame, loaded ahead of the update, goes into its buffer
+                if (f + 1 < n_frames) {
+                    const T* src;
+#pragma unroll
+                    for (int r = 0; r < kDnHeld; ++r)
+                        if (float* dst = input_vector(f_tid + r * f_nthr, f + 2, src)) *reinterpret_cast<float4*>(dst) = dn_widen(held[r]);
+                    for (int v = f_tid + kDnHeld * f_nthr;; v += f_nthr) {
+                        float* dst = input_vector(v, f + 2, src);
+                        if (!dst) break;
+                        *reinterpret_cast<float4*>(dst) = dn_widen(*reinterpret_cast<const uint2*>(src));
+                    }
+                }
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
             }
             if (!dn_wait(bar, phase, &gave_up, P.wait_limit)) break;    // the level is complete in this CTA's copy
         }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
-    if (*(volatile int*)&gave_up) __nanosleep(100000);       // stores on their way to this CTA land before it leaves
+    // Whatever the others send to this CTA counts on a barrier that it has waited for, so it may leave: unless it gave up (then what
+    // is on its way lands first), or another one still copies out of its shared memory (convolutions).
+    __syncthreads();
+    if (*(volatile int*)&gave_up) __nanosleep(100000);
     __syncwarp();
-    dn_cluster_sync();                                       // no CTA leaves while another one may still store into it
+    if (CONV || *(volatile int*)&gave_up) dn_cluster_sync();
     if (tid == 0 && gave_up) atomicExch(P.error, 1);
 
-    // relative frame T back to the state buffers in global memory (parity of t + T); every rank holds a full copy and
+    // the last frame back to the state buffers in global memory (parity of t + T); every rank holds a full copy and
     // writes its share of it
     {
-        const int parT = (int)((t0 + T) & 1);
+        const int parT = (int)((t0 + n_frames) & 1);
         const int gtid = (int)rank * nthr + tid, gthr = CL * nthr;
         for (int v = 0; v < P.n_nodes; ++v) {
             const DnNode& nd = P.nodes[v];
-            const float* src = dn_mem + (nd.is_input ? nd.buf[T % 3] : nd.buf[T & 1]);
-            float* gdst = nd.gstate[parT] + (size_t)b0 * nd.C;
-            if (nd.Cpad == nd.C)
-                for (int i = gtid * 4; i < nb * nd.C; i += gthr * 4) *reinterpret_cast<float4*>(gdst + i) = *reinterpret_cast<const float4*>(src + i);
+            const float* src = dn_mem + (nd.is_input ? nd.buf[n_frames % 3] : nd.buf[n_frames & 1]);
+            T* gdst = static_cast<T*>(nd.gstate[parT]) + (size_t)b0 * nd.C;
+            if (CONV && nd.step != 4)
+                for (int i = gtid; i < nb * (nd.C / 4); i += gthr) {
+                    const int b = i / (nd.C / 4), v = i - b * (nd.C / 4);
+                    dn_store4(gdst + 4 * i, src + v * nd.step + b * nd.seq);
+                }
+            else if (nd.Cpad == nd.C)
+                for (int i = gtid * 4; i < nb * nd.C; i += gthr * 4) dn_store4(gdst + i, src + i);
             else
-                for (int i = gtid; i < nb * nd.C; i += gthr) gdst[i] = src[(i / nd.C) * nd.Cpad + (i % nd.C)];
+                for (int i = gtid; i < nb * nd.C; i += gthr) dn_store(gdst + i, src[(i / nd.C) * nd.Cpad + (i % nd.C)]);
         }
     }
 }
@@ -449,17 +698,29 @@ bool dn_prepare(DnKernel kernel, int cluster)
     return true;
 }
 
+int dn_values(const sr_graph* g, int v) { return g->nodes[v].d.h * g->nodes[v].d.w * g->nodes[v].d.c; }
+bool dn_is_conv(const sr_graph* g, int v) { return !g->nodes[v].is_input && !g->nodes[v].dense_target; }
+
+template <typename T, bool CONV>
 DnKernel dn_kernel_of(int cluster, int samples)
 {
-    if (cluster == 16) return samples == 8 ? sr_dense_kernel<16, 8> : samples == 4 ? sr_dense_kernel<16, 4> : sr_dense_kernel<16, 2>;
-    return samples == 8 ? sr_dense_kernel<8, 8> : samples == 4 ? sr_dense_kernel<8, 4> : sr_dense_kernel<8, 2>;
+    if (cluster == 16)
+        return samples == 8 ? sr_dense_kernel<16, 8, T, CONV> : samples == 4 ? sr_dense_kernel<16, 4, T, CONV> : sr_dense_kernel<16, 2, T, CONV>;
+    return samples == 8 ? sr_dense_kernel<8, 8, T, CONV> : samples == 4 ? sr_dense_kernel<8, 4, T, CONV> : sr_dense_kernel<8, 2, T, CONV>;
+}
+DnKernel dn_kernel_of(const sr_graph* g, int cluster, int samples)
+{
+    bool conv = false;
+    for (size_t v = 0; v < g->nodes.size(); ++v) conv = conv || dn_is_conv(g, (int)v);
+    if (g->dtype == SR_DTYPE_BF16) return conv ? dn_kernel_of<__nv_bfloat16, true>(cluster, samples) : dn_kernel_of<__nv_bfloat16, false>(cluster, samples);
+    return conv ? dn_kernel_of<float, true>(cluster, samples) : dn_kernel_of<float, false>(cluster, samples);
 }
 
 // Clusters of this size and shared-memory footprint that the device holds at once with one CTA per SM (0: none): two CTAs on an SM
 // share its shared-memory pipe, so a second one there gains little over a second wave.
-int dn_clusters_held(int cluster, int samples, int smem_bytes)
+int dn_clusters_held(const sr_graph* g, int cluster, int samples, int smem_bytes)
 {
-    DnKernel kernel = dn_kernel_of(cluster, samples);
+    DnKernel kernel = dn_kernel_of(g, cluster, samples);
     if (!dn_prepare(kernel, cluster)) { cudaGetLastError(); return 0; }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)cluster);
@@ -492,12 +753,14 @@ DnEngine* dn_build(const sr_graph* g, int CL, int S)
     // edges sorted by target
     E->edge_of_host.assign(n_edges, -1);
     int pos = 0;
+    const SrHostEdge* host_edge[kDnMaxEdges] = {};
     for (int v = 0; v < n_nodes; ++v) {
         P.first_edge[v] = pos;
         for (int e : g->nodes[v].in_edges) {
             const SrHostEdge& he = g->edges[e];
-            const int Kpad = (g->nodes[he.d.src].d.c + 3) / 4 * 4;
+            const int Kpad = (dn_values(g, he.d.src) + 3) / 4 * 4;
             P.edges[pos] = DnEdge{he.d.src, he.d.tgt, he.R, Kpad};
+            host_edge[pos] = &he;
             E->edge_of_host[e] = pos++;
         }
     }
@@ -507,15 +770,17 @@ DnEngine* dn_build(const sr_graph* g, int CL, int S)
     E->w_off.assign(CL, std::vector<int>(kDnMaxEdges, 0));
     int max_w = 0;
     for (int v = 0; v < n_nodes; ++v)
-        for (int r = 0; r <= CL; ++r) E->row_lo[(size_t)v * (CL + 1) + r] = g->nodes[v].d.c * r / CL;
+        for (int r = 0; r <= CL; ++r) E->row_lo[(size_t)v * (CL + 1) + r] = dn_is_conv(g, v) ? 0 : dn_values(g, v) * r / CL;
     for (int r = 0; r < CL; ++r) {
         int w = 0;
-        for (int e = 0; e < n_edges; ++e) {
-            const int v = P.edges[e].tgt;
-            const int rows = E->row_lo[(size_t)v * (CL + 1) + r + 1] - E->row_lo[(size_t)v * (CL + 1) + r];
-            E->w_off[r][e] = w;
-            w += rows * P.edges[e].Kpad;
-        }
+        for (bool conv : {true, false})                          // (convolutions first: at the same place in every rank)
+            for (int e = 0; e < n_edges; ++e) {
+                const int v = P.edges[e].tgt;
+                if (dn_is_conv(g, v) != conv) continue;
+                const int rows = E->row_lo[(size_t)v * (CL + 1) + r + 1] - E->row_lo[(size_t)v * (CL + 1) + r];
+                E->w_off[r][e] = w;
+                w += conv ? host_edge[e]->K * g->nodes[v].d.c : rows * P.edges[e].Kpad;
+            }
         max_w = std::max(max_w, w);
     }
     // shared-memory layout in floats: header, weights, state buffers
@@ -526,24 +791,25 @@ DnEngine* dn_build(const sr_graph* g, int CL, int S)
     for (int v = 0; v < n_nodes; ++v) {
         const SrHostNode& n = g->nodes[v];
         DnNode& d = P.nodes[v];
-        d.C = n.d.c;
-        d.Cpad = (n.d.c + 3) / 4 * 4;
+        d.C = dn_values(g, v);
+        d.Cpad = (d.C + 3) / 4 * 4;
+        d.n_bias = n.d.c;
         d.act = n.d.act;
         d.is_input = n.is_input ? 1 : 0;
         d.input_slot = n.input_slot;
         d.is_output = v == g->info.output_node ? 1 : 0;
+        // (a convolution's sequences lie side by side, vector by vector)
+        const bool conv = dn_is_conv(g, v);
+        d.step = conv ? 4 * (S + 1) : 4;
+        d.seq = conv ? 4 : d.Cpad;
         for (int i = 0; i < (n.is_input ? 3 : 2); ++i) {
             d.buf[i] = off;
-            off += S * d.Cpad;
+            off += conv ? d.C / 4 * d.step : S * d.Cpad;
         }
         d.bias_off = off;
-        if (!n.is_input) off += d.Cpad;
+        if (!n.is_input) off += (n.d.c + 3) / 4 * 4;
     }
     P.total_floats = off;
-    for (int l = 0; l < P.n_levels; ++l) {
-        P.level_bytes[l] = 0;
-        for (int v : g->groups[l]) P.level_bytes[l] += g->nodes[v].d.c * S * 4;
-    }
     E->smem_bytes = off * 4;
     if (E->smem_bytes > kDnSmemMax) {
         delete E;
@@ -557,15 +823,62 @@ DnEngine* dn_build(const sr_graph* g, int CL, int S)
     for (int r = 0; r < CL; ++r) {
         DnBlobHdr& h = hdrs[r];
         std::memset(&h, 0, sizeof(h));
-        int n_units = 0, n_terms = 0;
+        int n_units = 0, n_terms = 0, n_slices = 0;
         bool fits = true;
         for (int l = 1; l <= P.n_levels && fits; ++l) {
             std::vector<std::pair<long long, DnUnit>> lv;
+            h.first_slice[l - 1] = n_slices;
             for (int v : g->groups[l - 1]) {
                 const DnNode& d = P.nodes[v];
+                if (!dn_is_conv(g, v)) h.level_bytes[l - 1] += d.C * S * 4;
                 long long K = 0;
                 for (int e = P.first_edge[v]; e < P.first_edge[v + 1]; ++e) K += P.edges[e].Kpad;
                 const int lo = E->row_lo[(size_t)v * (CL + 1) + r], hi = E->row_lo[(size_t)v * (CL + 1) + r + 1];
+                // a convolution: a run of its blocks of eight quads
+                const int quads = d.C / 4, blocks = dn_is_conv(g, v) ? (quads + 7) / 8 : 0, seqs = std::min(S, 4);
+                const int first = blocks * r / CL, end = blocks * (r + 1) / CL;
+                if (blocks > 0) {
+                    const int q0 = std::min(quads, first * 8), q1 = std::min(quads, end * 8);
+                    h.level_bytes[l - 1] += (quads - (q1 - q0)) * d.step * 4;
+                    h.conv_units[l - 1] += (end - first) * (S / seqs);
+                    if (q1 > q0) h.slices[n_slices++] = DnSlice{{d.buf[0] + q0 * d.step, d.buf[1] + q0 * d.step}, (q1 - q0) * d.step * 4, 0};
+                }
+                for (int i = 0; i < (end - first) * (S / seqs) && fits; ++i) {
+                    const int n_e = P.first_edge[v + 1] - P.first_edge[v];
+                    if (n_terms + 2 * n_e > kDnMaxTerms) { fits = false; break; }
+                    DnUnit u{};
+                    u.row0 = (first + i % (end - first)) * 8;
+                    u.nrows = std::min(8, quads - u.row0);
+                    u.first = (int16_t)(i / (end - first) * seqs);
+                    u.term0 = n_terms;
+                    u.n_terms = n_e;
+                    u.bias_off = d.bias_off;
+                    u.Cpad = d.step;
+                    u.C = d.C;
+                    u.flags = (d.act == 1 ? 1 : 0) | (d.is_output ? 2 : 0) | 4;
+                    u.buf[0] = d.buf[0];
+                    u.buf[1] = d.buf[1];
+                    u.channels = (int16_t)g->nodes[v].d.c;
+                    u.width = (int16_t)g->nodes[v].d.w;
+                    long long steps = 0;
+                    for (int e = P.first_edge[v]; e < P.first_edge[v + 1]; ++e) {
+                        const SrHostEdge& he = *host_edge[e];
+                        const DnNode& sn = P.nodes[P.edges[e].src];
+                        const sr_node_desc& sd = g->nodes[he.d.src].d;
+                        DnTerm& tm = h.terms[n_terms++];
+                        tm.w_off = E->w_off[r][e];
+                        tm.Kpad = he.k_eff | he.stride_eff << 8 | he.pad_eff << 16;
+                        tm.xp = sn.seq;
+                        tm.R = P.edges[e].R;
+                        tm.n_buf = (sn.is_input ? 3 : 2) | sn.step << 8;
+                        for (int q = 0; q < 3; ++q) tm.buf[q] = sn.buf[q < (tm.n_buf & 0xFF) ? q : 0];
+                        DnConv cv{};
+                        cv.Hs = sd.h; cv.Ws = sd.w; cv.Cs = sd.c;
+                        std::memcpy(&h.terms[n_terms++], &cv, sizeof(cv));
+                        steps += he.K * (sd.c % 4 == 0 ? 1 : 2);
+                    }
+                    lv.push_back({steps * 16 + 256, u});
+                }
                 for (int row = lo; row < hi && fits; row += kDnRows) {
                     const int nr = std::min(kDnRows, hi - row), n_e = P.first_edge[v + 1] - P.first_edge[v];
                     if (n_terms + n_e > kDnMaxTerms) { fits = false; break; }
@@ -585,10 +898,10 @@ DnEngine* dn_build(const sr_graph* g, int CL, int S)
                         DnTerm& tm = h.terms[n_terms++];
                         tm.w_off = E->w_off[r][e] + (row - lo) * P.edges[e].Kpad;
                         tm.Kpad = P.edges[e].Kpad;
-                        tm.xp = sn.Cpad;
+                        tm.xp = sn.seq;
                         tm.R = P.edges[e].R;
-                        tm.n_buf = sn.is_input ? 3 : 2;
-                        for (int i = 0; i < 3; ++i) tm.buf[i] = sn.buf[i < tm.n_buf ? i : 0];
+                        tm.n_buf = (sn.is_input ? 3 : 2) | sn.step << 8;
+                        for (int i = 0; i < 3; ++i) tm.buf[i] = sn.buf[i < (tm.n_buf & 0xFF) ? i : 0];
                     }
                     lv.push_back({K * (4 + (nr > 2 ? 4 : 2)) + 256, u});     // loads per step + reduction and stores
                 }
@@ -623,6 +936,7 @@ DnEngine* dn_build(const sr_graph* g, int CL, int S)
             }
         }
         for (int l = P.n_levels + 1; l <= kDnMaxLevels; ++l) h.level_begin[l] = n_units;
+        for (int l = P.n_levels; l <= kDnMaxLevels; ++l) h.first_slice[l] = n_slices;
         h.n_units = n_units;
         h.idle = 1;
         for (int u = 0; u < n_units; ++u)
@@ -656,21 +970,34 @@ void sr_dn_describe(const sr_graph* g, int* cluster_size, int* smem_bytes)
     *smem_bytes = E ? E->smem_bytes : 0;
 }
 
-// The engine applies to fp32 graphs in which every node is a vector (h = w = 1) and every edge dense, small enough for
-// the shared memory of a cluster.  Rows of every node are split evenly over the ranks.
+// The engine applies to graphs whose edges are dense, or convolutions of a quarter of a million multiply-adds per sample at most, small enough
+// for the shared memory of a cluster.  Rows of every dense node are split evenly over the ranks.
 sr_status sr_dn_plan(sr_graph* g, size_t& offset)
 {
     sr_dn_destroy(g);
-    if (!g->opt_resident || g->opt_engine != 0 || g->dtype != SR_DTYPE_F32) return SR_OK;
+    if (!g->opt_resident || g->opt_engine != 0) return SR_OK;
     const int n_nodes = (int)g->nodes.size(), n_edges = (int)g->edges.size();
     if (n_nodes > kDnMaxNodes || n_edges > kDnMaxEdges || (int)g->groups.size() > kDnMaxLevels || g->groups.empty()) return SR_OK;
     if ((int)g->input_nodes.size() > SR_MAX_INPUTS) return SR_OK;
-    for (const SrHostNode& n : g->nodes) {
-        if (n.d.h != 1 || n.d.w != 1) return SR_OK;
-        if (n.is_input && n.d.c % 4 != 0) return SR_OK;
+    // (the other resident engine's, where it applies)
+    if (sr_rs_available(g)) return SR_OK;
+    double work = 0;                                         // of the convolutions
+    for (int v = 0; v < n_nodes; ++v) {
+        const SrHostNode& n = g->nodes[v];
+        if ((double)n.d.h * n.d.w * n.d.c > kDnSmemMax / 4) return SR_OK;
+        if (n.is_input && dn_values(g, v) % 4 != 0) return SR_OK;
+        if (dn_is_conv(g, v) && (n.d.c % 4 != 0 || n.d.c > 1024 || n.d.w > 1024)) return SR_OK;
     }
-    for (const SrHostEdge& e : g->edges)
-        if (e.d.kind == SR_EDGE_CONV) return SR_OK;
+    for (const SrHostEdge& e : g->edges) {
+        const sr_node_desc &s = g->nodes[e.d.src].d, &t = g->nodes[e.d.tgt].d;
+        if (e.d.kind == SR_EDGE_CONV) {
+            if (e.k_eff > 32 || e.stride_eff > 255 || e.pad_eff > 255) return SR_OK;
+            work += (double)e.K * t.h * t.w * t.c;
+        } else if (e.d.kind == SR_EDGE_MEAN_DENSE && s.h * s.w != 1) {
+            return SR_OK;
+        }
+    }
+    if (work > kDnConvWork) return SR_OK;
     // With one level per frame (the streaming rollout) a frame is one round of work units and one exchange: sixteen CTAs (a
     // non-portable cluster size) halve the units of each CTA, while with several levels per frame the costlier exchange of the
     // larger cluster outweighs that.  Measured on the 784-128-128-10 network, four clusters of two sequences, per frame: streaming
@@ -680,7 +1007,7 @@ sr_status sr_dn_plan(sr_graph* g, size_t& offset)
     DnEngine* E = nullptr;
     if (g->groups.size() == 1) {
         E = dn_build(g, kDnMaxCluster, kDnMaxSamples);
-        if (E && (g->batch + kDnMaxSamples - 1) / kDnMaxSamples > dn_clusters_held(kDnMaxCluster, kDnMaxSamples, E->smem_bytes)) {
+        if (E && (g->batch + kDnMaxSamples - 1) / kDnMaxSamples > dn_clusters_held(g, kDnMaxCluster, kDnMaxSamples, E->smem_bytes)) {
             delete E;
             E = nullptr;
         }
@@ -697,7 +1024,7 @@ sr_status sr_dn_plan(sr_graph* g, size_t& offset)
         for (int S = kDnMaxSamples; S >= 2; S /= 2) {
             DnEngine* F = S == kDnMaxSamples ? E : dn_build(g, cl, S);
             if (!F) continue;
-            const int clusters = (g->batch + S - 1) / S, held = std::max(dn_clusters_held(cl, S, F->smem_bytes), 1);
+            const int clusters = (g->batch + S - 1) / S, held = std::max(dn_clusters_held(g, cl, S, F->smem_bytes), 1);
             const int waves = (clusters + held - 1) / held;
             const double cost = waves * (S == 8 ? 1.0 : S == 4 ? 0.76 : 0.6);
             if (F != E) delete F;
@@ -708,6 +1035,14 @@ sr_status sr_dn_plan(sr_graph* g, size_t& offset)
             E = dn_build(g, cl, best_s);
         }
         if (E) E->one_wave = best_waves == 1;
+        // In bf16 a convolution has the tensor cores, and the launch path takes no longer for many sequences than for one: there the
+        // engine is for what goes out at once, and for frames of one level with up to four sequences per cluster.  MNIST network SR, us
+        // per frame launched / resident: bf16 at 8 / 64 / 256 samples 7.0 / 4.1, 8.4 / 8.9, 16.7 / 27.7, sequential at 128 (two waves)
+        // 19.8 / 26.4; fp32 at 1 / 100 / 128 11.5 / 4.0, 15.4 / 8.1, 18.2 / 16.6, sequential at 8 / 100 19.0 / 6.1, 27.0 / 9.3.
+        if (E && work > 0 && g->dtype == SR_DTYPE_BF16 && (!E->one_wave || (g->groups.size() == 1 && E->samples > 4))) {
+            delete E;
+            E = nullptr;
+        }
     }
     if (!E) return SR_OK;
     const int CL = E->cluster;
@@ -732,15 +1067,13 @@ sr_status sr_dn_bind(sr_graph* g)
     P.blobs = reinterpret_cast<const unsigned char*>(ws + E->r_blobs.offset);
     for (int v = 0; v < P.n_nodes; ++v) {
         const SrHostNode& n = g->nodes[v];
-        P.nodes[v].gstate[0] = reinterpret_cast<float*>(ws + n.state[0].offset);
-        P.nodes[v].gstate[1] = reinterpret_cast<float*>(ws + n.state[1].offset);
+        P.nodes[v].gstate[0] = ws + n.state[0].offset;
+        P.nodes[v].gstate[1] = ws + n.state[1].offset;
         P.nodes[v].bias = reinterpret_cast<const float*>(ws + n.bias.offset);
     }
     // the workspace was zeroed by the caller of bind: weights start at zero, headers go in now
-    for (int r = 0; r < CL; ++r)
-        if (cudaMemcpy(ws + E->r_blobs.offset + (size_t)r * P.blob_bytes, g->dn_headers.data() + (size_t)r * sizeof(DnBlobHdr),
-                       sizeof(DnBlobHdr), cudaMemcpyHostToDevice) != cudaSuccess)
-            return SR_ERR_CUDA;
+    if (cudaMemcpy2D(ws + E->r_blobs.offset, P.blob_bytes, g->dn_headers.data(), sizeof(DnBlobHdr), sizeof(DnBlobHdr), CL, cudaMemcpyHostToDevice) != cudaSuccess)
+        return SR_ERR_CUDA;
     return SR_OK;
 }
 
@@ -753,14 +1086,33 @@ sr_status sr_dn_set_weights(sr_graph* g, int edge, const float* w)
     const int e = E->edge_of_host[edge];
     const SrHostEdge& he = g->edges[edge];
     const int v = he.d.tgt, K = he.K, Kpad = P.edges[e].Kpad;
-    for (int r = 0; r < CL; ++r) {
-        const int lo = E->row_lo[(size_t)v * (CL + 1) + r], hi = E->row_lo[(size_t)v * (CL + 1) + r + 1];
-        if (hi <= lo) continue;
-        std::vector<float> h((size_t)(hi - lo) * Kpad, 0.f);
-        for (int row = lo; row < hi; ++row)
-            std::memcpy(&h[(size_t)(row - lo) * Kpad], w + (size_t)row * K, sizeof(float) * K);
+    if (dn_is_conv(g, v)) {                                  // [C_out][K] -> [K][C_out], the same for every rank
+        const int C = g->nodes[v].d.c;
+        const size_t n = (size_t)K * C;
+        std::vector<float> h(n * CL);
+        for (int co = 0; co < C; ++co)
+            for (int kk = 0; kk < K; ++kk) h[(size_t)kk * C + co] = w[(size_t)co * K + kk];
+        for (int r = 1; r < CL; ++r) std::copy_n(h.begin(), n, h.begin() + n * r);
+        // one copy for all ranks where the edge lies at the same place in each
+        bool same = true;
+        for (int r = 1; r < CL; ++r) same = same && E->w_off[r][e] == E->w_off[0][e];
+        for (int r = 0; r < (same ? 1 : CL); ++r) {
+            char* dst = g->ws + E->r_blobs.offset + (size_t)r * P.blob_bytes + sizeof(DnBlobHdr) + (size_t)E->w_off[r][e] * 4;
+            if (cudaMemcpy2D(dst, P.blob_bytes, h.data(), n * 4, n * 4, same ? CL : 1, cudaMemcpyHostToDevice) != cudaSuccess) return SR_ERR_CUDA;
+        }
+        return SR_OK;
+    }
+    const int rows = dn_values(g, v);
+    std::vector<float> h((size_t)rows * Kpad, 0.f);
+    for (int row = 0; row < rows; ++row) std::memcpy(&h[(size_t)row * Kpad], w + (size_t)row * K, sizeof(float) * K);
+    const int* lo = &E->row_lo[(size_t)v * (CL + 1)];
+    bool same = true;
+    for (int r = 1; r < CL; ++r) same = same && E->w_off[r][e] == E->w_off[0][e] && lo[r + 1] - lo[r] == lo[1] - lo[0];
+    for (int r = 0; r < (same ? 1 : CL); ++r) {
+        const size_t bytes = (size_t)(lo[r + 1] - lo[r]) * Kpad * sizeof(float);
+        if (bytes == 0) continue;
         char* dst = g->ws + E->r_blobs.offset + (size_t)r * P.blob_bytes + sizeof(DnBlobHdr) + (size_t)E->w_off[r][e] * 4;
-        if (cudaMemcpy(dst, h.data(), h.size() * sizeof(float), cudaMemcpyHostToDevice) != cudaSuccess) return SR_ERR_CUDA;
+        if (cudaMemcpy2D(dst, P.blob_bytes, &h[(size_t)lo[r] * Kpad], bytes, bytes, same ? CL : 1, cudaMemcpyHostToDevice) != cudaSuccess) return SR_ERR_CUDA;
     }
     return SR_OK;
 }
@@ -771,7 +1123,7 @@ sr_status sr_dn_launch(sr_graph* g, int T, const SrFrameCtl& init, cudaStream_t 
     if (!E) return SR_ERR_STATE;
     const int CL = E->cluster;
     const int S = E->samples;
-    auto kernel = dn_kernel_of(CL, S);
+    auto kernel = dn_kernel_of(g, CL, S);
     if (!E->attr_set) {
         if (!dn_prepare(kernel, CL)) return SR_ERR_CUDA;
         E->attr_set = true;

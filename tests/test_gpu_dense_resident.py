@@ -6,7 +6,7 @@ import pytest
 
 from tests import parity
 from workloads import data, graphs
-from workloads.graphs import DENSE, GAP_DENSE, IDENTITY, RELU, Edge, GraphSpec, Node, sequential_pattern, streaming_pattern
+from workloads.graphs import CONV, DENSE, GAP_DENSE, IDENTITY, RELU, Edge, GraphSpec, Node, sequential_pattern, streaming_pattern
 
 pytestmark = pytest.mark.gpu
 
@@ -133,3 +133,61 @@ def test_a_smaller_network_leaves_a_larger_one_runnable(pattern, batch):
         assert parity.rel_err(out.cpu().numpy()[:, samples].reshape(want[o][1:].shape), want[o][1:]) <= 1e-4
         parity.check_run(small, pattern, samples=samples)
         parity.check_stepwise(small, pattern, samples=samples)
+
+
+def small_cnn(batch, frames, dtype, cin=1, size=(12, 10), c=12, seed=41):
+    """input -> a (5x5, stride 2, recurrent) -> b (3x3), both -> h (dense) -> out, skips a -> out, input -> b (1x1, stride 2)."""
+    h, w = size
+    nodes = [Node("in", h, w, cin, IDENTITY), Node("a", h // 2, w // 2, c, RELU), Node("b", h // 2, w // 2, 8, RELU), Node("h", 1, 1, 22, RELU),
+             Node("out", 1, 1, 7, IDENTITY)]
+    edges = [Edge(0, 1, CONV, 5, 2), Edge(1, 1, CONV, 3, 1), Edge(1, 2, CONV, 3, 1), Edge(0, 2, CONV, 1, 2), Edge(1, 3, DENSE), Edge(2, 3, DENSE),
+             Edge(3, 4, DENSE), Edge(1, 4, DENSE), Edge(3, 3, DENSE)]
+    g = GraphSpec("small_cnn", nodes, edges, batch=batch, frames=frames, dtype=dtype, seed=seed, weight_gain=1.0)
+    g.patterns = {"streaming": streaming_pattern(g), "sequential": sequential_pattern(g), "hybrid": [0, 1, 1, 0, 0, 1, 0, 1, 1]}
+    return g
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("batch,cin,size,c", [(1, 1, (12, 10), 12), (3, 3, (12, 8), 4), (8, 4, (6, 10), 32), (11, 1, (14, 14), 16), (41, 2, (8, 8), 20)])
+def test_small_convolutions(dtype, batch, cin, size, c):
+    # blocks of eight quads that are not full, sources of one to many channels, ragged clusters; sixteen-bit states are rounded as the
+    # launch path rounds them
+    g = small_cnn(batch, 6, dtype, cin, size, c)
+    for p in g.patterns:
+        parity.check_run(g, p)
+        parity.check_run(g, p, frames=1)
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+def test_small_networks_run_on_the_engine_in_both_types(dtype):
+    g = mlp(5, 4)
+    g.dtype = dtype
+    for p in g.patterns:
+        parity.check_run(g, p, expect_resident=CLUSTER[p])
+        parity.check_stepwise(g, p, zero_bias=False)
+    g = small_cnn(5, 5, dtype)
+    for p in g.patterns:
+        parity.check_run(g, p, expect_resident=CLUSTER[p])
+        parity.check_stepwise(g, p, zero_bias=False)
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+def test_convolutions_hand_over_to_the_launch_path_and_back(dtype):
+    import torch
+    from oracle import frame_update as fu
+    g = small_cnn(5, 12, dtype)
+    X, W, Bi = data.make_inputs(g), data.make_weights(g), data.make_biases(g, zero=False)
+    want = fu.rollout_spec(g, "sequential", X, W, Bi)
+    G = parity.make_graph(g, "sequential", "auto", 0, W, Bi)
+    x = parity.to_device(g, X[0])
+    shifted = torch.empty(x[5:7].numel() + 1, dtype=x.dtype, device="cuda:0")[1:].view(x[5:7].shape)   # not on a 16-byte boundary:
+    shifted.copy_(x[5:7])                                                                               # the launch path takes it
+    out = torch.empty((11, 5, 7), dtype=torch.float32, device="cuda:0")
+    G.reset([x[0]])
+    G.run([x[1:5]], out[:4])
+    G.run([shifted], out[4:6])
+    G.run([x[7:12]], out[6:])
+    G.sync_status()
+    assert parity.rel_err(out.cpu().numpy(), want[4][1:12].reshape(11, 5, 7)) <= parity.TOL[dtype]
+    for v in range(5):
+        assert parity.rel_err(G.get_state(v).float().cpu().numpy(), want[v][11]) <= parity.TOL[dtype]
