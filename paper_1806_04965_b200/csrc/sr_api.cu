@@ -141,6 +141,7 @@ sr_status plan(sr_graph* g)
     g->items.clear();
     g->group_item_offset.clear();
     g->group_item_count.clear();
+    g->group_sliced.clear();
     g->group_head_nodes.assign(g->groups.size(), {});
     const int dco = sr_direct_dense_outputs_per_block(),
               dsb = sr_direct_dense_samples_per_block();
@@ -169,6 +170,9 @@ sr_status plan(sr_graph* g)
         std::stable_sort(g->items.begin() + g->group_item_offset.back(), g->items.end(),
                          [&](const SrDirectItem& a, const SrDirectItem& b) { return work(a) > work(b); });
         g->group_item_count.push_back((int)g->items.size() - g->group_item_offset.back());
+        g->group_sliced.push_back(0);
+        for (size_t i = g->group_item_offset.back(); i < g->items.size(); ++i)
+            if (!g->nodes[g->items[i].node].dense_target && sr_direct_sliced(g->items[i])) g->group_sliced.back() = 1;
     }
     g->r_items = take(off, sizeof(SrDirectItem) * std::max<size_t>(1, g->items.size()));
     sr_status st = sr_tc_plan(g, off);

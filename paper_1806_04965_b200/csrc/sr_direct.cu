@@ -61,6 +61,7 @@ __device__ __forceinline__ void store4(__nv_bfloat16* p, const float (&v)[4])
     *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
 }
 
+constexpr int kItemSlices = 1 << 30;   // SrDirectItem::pad_: the block's warps share the pixels and take slices of the reduction
 constexpr int kPix = 4;            // pixels per warp (conv nodes)
 constexpr int kWarps = 4;          // warps per block
 constexpr int kDenseB = 8;         // samples per warp (dense nodes)
@@ -77,9 +78,9 @@ __device__ void conv_item(const SrDevNode& nd, const SrDevEdge* edges, const SrD
     const int HW = nd.H * nd.W;
     int b = it.b0, n_pix = kWarps * kPix, c_first = 0, c_end = nd.C;
     if (ANY_ITEM && nd.untiled == (sizeof(T) == 2 ? 2 : 4)) {                                                       // conv_tile's items: pixels and channels of their own
-        const int qlog = it.pad_ >> 24;
+        const int qlog = (it.pad_ >> 24) & 15;
         b = it.b0 < 0 ? ~it.b0 : it.b0;
-        n_pix = (kWarps * 32 >> qlog) * (it.b0 < 0 ? 4 : 1);
+        n_pix = ((it.pad_ & kItemSlices ? 32 : kWarps * 32) >> qlog) * (it.b0 < 0 ? 4 : 1);
         c_first = it.pad_ & 0xFFFFFF;
         c_end = min(nd.C, c_first + (4 << qlog));
     }
@@ -163,14 +164,21 @@ __device__ void conv_item(const SrDevNode& nd, const SrDevEdge* edges, const SrD
 // inside the window, filter row and column): no branch per tap, so the loads of several steps are in flight together.  What
 // bounds it is the latency of those loads for a small node and the load / store unit for a large one; PX = 4 loads a weight
 // vector once for four pixels and is taken when that still leaves threads enough (see sr_direct_conv_items).
+// SLICES: the warps of a block take the same 32 threads' worth of outputs and every fourth step of the reduction each, and the first one
+// adds the sums, in order: a quarter of the chain of dependent loads, and four times the blocks.  Small CNN, fp32, us per frame before /
+// now: at 1 / 16 / 64 / 128 samples 26.0 / 11.1, 42.6 / 24.0, 78.7 / 52.5, 113 / 95.2 (sequential at 1 / 64 / 128 56.6 / 28.3, 125 / 73,
+// 176 / 117).
 // Measured on B200 (was: a warp per four pixels, lanes over channels, a branch per tap), fp32, us per frame: MNIST net SR at 100
 // samples 49 -> 17.5, at one 34 -> 12.6; small CNN at 128 samples 260 -> 114, at one 80 -> 27.
 constexpr int kTab = 512;          // table entries at a time
-template <typename T, int PX>
+constexpr int kTabSliced = (kWarps - 1) * 32 * 16 * 4 / (int)sizeof(int2);   // its place, where the sums of the slices go as well
+template <typename T, int PX, bool SLICES>
 __device__ void conv_tile(const SrDevNode& nd, const SrDevEdge* edges, const SrDirectItem& it, int prev, int cur, float* out_f32, int2* tab)
 {
-    const int qlog = it.pad_ >> 24, c = (it.pad_ & 0xFFFFFF) + 4 * ((int)threadIdx.x & ((1 << qlog) - 1));
-    const int HW = nd.H * nd.W, C = nd.C, p_first = it.p0 + ((int)threadIdx.x >> qlog) * PX;
+    constexpr int kStep = SLICES ? kWarps : 1;
+    const int place = SLICES ? (int)threadIdx.x & 31 : (int)threadIdx.x, slice = SLICES ? (int)threadIdx.x >> 5 : 0;
+    const int qlog = (it.pad_ >> 24) & 15, c = (it.pad_ & 0xFFFFFF) + 4 * (place & ((1 << qlog) - 1));
+    const int HW = nd.H * nd.W, C = nd.C, p_first = it.p0 + (place >> qlog) * PX;
     const bool cv = c < C;
     int oy[PX], ox[PX];
     float acc[PX][4];
@@ -205,7 +213,7 @@ __device__ void conv_tile(const SrDevNode& nd, const SrDevEdge* edges, const SrD
             __syncthreads();
             if (vec == 4) {
 #pragma unroll 2
-                for (int i = 0; i < m; ++i) {
+                for (int i = slice; i < m; i += kStep) {
                     const int2 t = tab[i];
                     const int dy = t.y >> 16, dx = t.y & 0xFFFF;
                     float4 wv[4];
@@ -227,7 +235,7 @@ __device__ void conv_tile(const SrDevNode& nd, const SrDevEdge* edges, const SrD
                 }
             } else {
 #pragma unroll 8
-                for (int i = 0; i < m; ++i) {
+                for (int i = slice; i < m; i += kStep) {
                     const int2 t = tab[i];
                     const int dy = t.y >> 16, dx = t.y & 0xFFFF;
                     const float4 wv = __ldg(reinterpret_cast<const float4*>(w + (size_t)(e0 + i) * C));
@@ -241,6 +249,24 @@ __device__ void conv_tile(const SrDevNode& nd, const SrDevEdge* edges, const SrD
                 }
             }
         }
+    }
+    if (SLICES) {
+        // (in the table's place: 32 threads x 4 * PX sums per warp but the first)
+        static_assert(kTabSliced >= kTab, "the sums of the slices take the table's place");
+        float4* sums = reinterpret_cast<float4*>(tab);
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < PX; ++j)
+            if (slice > 0) sums[((slice - 1) * PX + j) * 32 + place] = make_float4(acc[j][0], acc[j][1], acc[j][2], acc[j][3]);
+        __syncthreads();
+        if (slice > 0) return;
+#pragma unroll
+        for (int q = 0; q < kWarps - 1; ++q)
+#pragma unroll
+            for (int j = 0; j < PX; ++j) {
+                const float4 a = sums[(q * PX + j) * 32 + place];
+                acc[j][0] += a.x; acc[j][1] += a.y; acc[j][2] += a.z; acc[j][3] += a.w;
+            }
     }
     if (!cv) return;
     const float4 b = *reinterpret_cast<const float4*>(nd.bias + c);
@@ -675,10 +701,11 @@ struct DirectParams {
 // convolutions change with everything beside them (32 -> 32 channels of 32 x 32, 64 samples: 570 us for eight frames, 626 in the
 // kernel that takes both); bf16 is as fast either way.  A launch that a caller recorded before the weight came keeps its kernel, and
 // its tiles.
-template <typename T, bool NON_FINITE>
+// SLICED: a kernel of its own, too, for launches with such items.
+template <typename T, bool NON_FINITE, bool SLICED>
 __global__ void __launch_bounds__(kWarps * 32) sr_direct_group_kernel(const __grid_constant__ DirectParams P)
 {
-    __shared__ int2 tab[kTab];
+    __shared__ __align__(16) int2 tab[SLICED ? kTabSliced : kTab];
     sr_begin(P.follow);
     sr_drop_old_lines(P.follow);
     const SrDirectItem it = P.items[blockIdx.x];
@@ -690,11 +717,13 @@ __global__ void __launch_bounds__(kWarps * 32) sr_direct_group_kernel(const __gr
     // (As two tests joined by ||, or a mark in the item, this took the compiler from 96 registers to 128, and 3 -> 32 channels of
     // 32 x 32 at 64 samples, fp32, from 171 us for eight frames to 202.)
     else if ((nd.C | nd.untiled | (NON_FINITE && sizeof(T) == 4 ? nd.untiled >> 2 : 0)) % 4 != 0) conv_item<T, NON_FINITE>(nd, P.edges, it, prev, cur, out);
-    else if (it.b0 >= 0) conv_tile<T, 1>(nd, P.edges, it, prev, cur, out, tab);
+    else if (SLICED && it.b0 >= 0 && (it.pad_ & kItemSlices)) conv_tile<T, 1, true>(nd, P.edges, it, prev, cur, out, tab);
+    else if (it.b0 >= 0) conv_tile<T, 1, false>(nd, P.edges, it, prev, cur, out, tab);
     else {
         SrDirectItem four = it;
         four.b0 = ~it.b0;
-        conv_tile<T, 4>(nd, P.edges, four, prev, cur, out, tab);
+        if (SLICED && (it.pad_ & kItemSlices)) conv_tile<T, 4, true>(nd, P.edges, four, prev, cur, out, tab);
+        else conv_tile<T, 4, false>(nd, P.edges, four, prev, cur, out, tab);
     }
     sr_end(P.follow);
 }
@@ -714,9 +743,11 @@ int sr_launch_direct_group(const sr_graph* g, int group, SrFollow how, cudaStrea
     P.follow = how.flags();
     bool finite = true;
     for (int v : g->groups[group]) finite = finite && g->nodes[v].w_finite;
-    sr_launch(g->dtype == SR_DTYPE_BF16 ? sr_direct_group_kernel<__nv_bfloat16, true>
-                                        : finite ? sr_direct_group_kernel<float, false> : sr_direct_group_kernel<float, true>,
-              n, kWarps * 32, 0, s, how.early, P);
+    auto kernel = [&](auto sliced) {
+        return g->dtype == SR_DTYPE_BF16 ? sr_direct_group_kernel<__nv_bfloat16, true, sliced>
+                                         : finite ? sr_direct_group_kernel<float, false, sliced> : sr_direct_group_kernel<float, true, sliced>;
+    };
+    sr_launch(g->group_sliced[group] ? kernel(std::true_type()) : kernel(std::false_type()), n, kWarps * 32, 0, s, how.early, P);
     return 1;
 }
 
@@ -870,12 +901,19 @@ void sr_direct_conv_items(const sr_graph* g, int v, std::vector<SrDirectItem>& i
     // Four pixels per thread once that still gives every SM 256 threads; marked by the complement of the sample.  Measured on
     // B200, fp32, us per frame with one / four pixels everywhere: small CNN (28 x 28 x 32, 14 x 14 x 32, 7 x 7 x 64) at 128
     // samples 161 / 133 (this rule: 114), at 32 samples (sequential) 90 / 144, at one 27 / 51; MNIST net at 256 samples 35 / 53.
-    const bool four = (size_t)g->batch * HW * (d.c / 4) / 4 >= (size_t)g->sm_count * 256;
-    const int px = (kWarps * 32 >> qlog) * (four ? 4 : 1);
+    // Slices of a reduction of 128 steps or more until there are 512 threads per SM without them (256: sequential at 128 samples 146
+    // instead of 117 us a frame); with four pixels per thread where a pixel per thread would make 64 threads per SM (256: 29.8 instead
+    // of 24.0 us at 16 samples, 49.2 instead of 39.9 at 48; never: 27.0 and 62.1).
+    const size_t quads = (size_t)g->batch * HW * (d.c / 4), sms = (size_t)g->sm_count;
+    int K = 0;
+    for (int e : g->nodes[v].in_edges) K += g->edges[e].K;
+    const bool slices = K >= 128 && quads / 4 < sms * 512, four = quads / 4 >= sms * 256 || (slices && quads >= sms * 64);
+    const int px = ((slices ? 32 : kWarps * 32) >> qlog) * (four ? 4 : 1);
     for (int b = 0; b < g->batch; ++b)
         for (int p0 = 0; p0 < HW; p0 += px)
-            for (int c0 = 0; c0 < d.c; c0 += 4 << qlog) items.push_back(SrDirectItem{v, four ? ~b : b, p0, c0 | qlog << 24});
+            for (int c0 = 0; c0 < d.c; c0 += 4 << qlog) items.push_back(SrDirectItem{v, four ? ~b : b, p0, c0 | qlog << 24 | (slices ? kItemSlices : 0)});
 }
+bool sr_direct_sliced(const SrDirectItem& it) { return (it.pad_ & kItemSlices) != 0; }
 int sr_direct_dense_outputs_per_block() { return kWarps; }
 int sr_direct_dense_samples_per_block() { return kDenseB; }
 
@@ -949,5 +987,5 @@ bool sr_direct_share_sm()
                ask(sr_mean_head_kernel<__nv_bfloat16, beside>);
     };
     return heads(std::false_type()) && heads(std::true_type()) && ask(sr_wide_head_kernel<__nv_bfloat16, 1>) &&
-           ask(sr_wide_head_kernel<__nv_bfloat16, kWideQ>) && ask(sr_direct_group_kernel<__nv_bfloat16, true>);
+           ask(sr_wide_head_kernel<__nv_bfloat16, kWideQ>) && ask(sr_direct_group_kernel<__nv_bfloat16, true, false>) && ask(sr_direct_group_kernel<__nv_bfloat16, true, true>);
 }

@@ -251,6 +251,7 @@ struct sr_graph {
     std::vector<int> group_item_count;             // per group
     std::vector<SrDirectItem> items;
     std::vector<int> group_item_offset;
+    std::vector<char> group_sliced;                // per group: some item's reduction is cut into slices
     std::vector<std::vector<int>> group_head_nodes;       // per group: nodes of the head kernels
     std::vector<std::vector<SrHeadNode>> group_heads;     // and what they need to know about them (filled when a workspace is bound)
     std::vector<std::vector<SrWideNode>> group_wide;

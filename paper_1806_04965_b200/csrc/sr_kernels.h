@@ -10,6 +10,7 @@ void sr_launch_set_ctl(const sr_graph* g, const SrFrameCtl& v, cudaStream_t s);
 void sr_launch_advance(const sr_graph* g, int n, cudaStream_t s);
 bool sr_direct_untiled(const sr_graph* g, int v);
 void sr_direct_conv_items(const sr_graph* g, int v, std::vector<SrDirectItem>& items);
+bool sr_direct_sliced(const SrDirectItem& it);
 int sr_direct_dense_outputs_per_block();
 int sr_direct_dense_samples_per_block();
 int sr_head_class(const sr_graph* g, int v);

@@ -457,3 +457,11 @@ def test_frames_of_one_call_equal_calls_of_one_frame(name, pattern, graph_frames
         got.append([out] + [G.get_state(v) for v in range(len(spec.nodes))])
     for a, b in zip(*got):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("batch,size,cin,c", [(1, 6, 16, 4), (20, 12, 16, 36), (40, 7, 24, 132), (3, 13, 14, 20)])
+def test_cuda_core_convolutions_in_slices(batch, size, cin, c, dtype):
+    # reductions of 128 steps and more whose steps the warps of a block share: one and four pixels per thread, quads and pixels that do
+    # not fill a block, several channel blocks, a source read value by value
+    test_cuda_core_convolutions_at_the_edges_of_their_tiles(batch, size, cin, c, dtype)
