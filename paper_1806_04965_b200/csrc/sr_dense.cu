@@ -1044,6 +1044,13 @@ sr_status sr_dn_plan(sr_graph* g, size_t& offset)
             E = nullptr;
         }
     }
+    // A graph that fits the built-in workspace without this engine keeps fitting (fp32 networks of dense edges only have always had
+    // its tables counted).
+    if (E && (work > 0 || g->dtype == SR_DTYPE_BF16) && offset - g->r_items.bytes <= (size_t)SR_STATIC_WORKSPACE_BYTES &&
+        offset - g->r_items.bytes + (size_t)E->cluster * E->P.blob_bytes + 256 > (size_t)SR_STATIC_WORKSPACE_BYTES) {
+        delete E;
+        E = nullptr;
+    }
     if (!E) return SR_OK;
     const int CL = E->cluster;
     DnParams& P = E->P;

@@ -9,6 +9,7 @@ import pytest
 
 from oracle import rollout_theory as rt
 from paper_1806_04965_b200 import Graph, SrError, load_library
+from paper_1806_04965_b200.binding import _EdgeDesc, _NodeDesc
 from workloads import graphs
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -178,3 +179,22 @@ print("ok")
 """ % ROOT
     out = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
     assert out.returncode == 0 and out.stdout.strip() == "ok", (out.returncode, out.stderr[-500:])
+
+
+@pytest.mark.parametrize("batch", [3926, 7695, 7852])
+def test_resident_tables_keep_a_graph_in_the_built_in_workspace(batch):
+    # the dense engine's tables (0.7 MB) of a bf16 dense network count only where the sum stays within the built-in workspace's 32 MiB
+    lib = load_library()
+    g = graphs.build("c1", batch=1, frames=2)
+    n = (_NodeDesc * len(g.nodes))(*[_NodeDesc(v.h, v.w, v.c, v.act) for v in g.nodes])
+    e = (_EdgeDesc * len(g.edges))(*[_EdgeDesc(x.src, x.tgt, x.kind, x.k, x.stride, x.pool) for x in g.edges])
+    sizes = []
+    for resident in (0, 1):
+        h, size = ctypes.c_void_p(), ctypes.c_size_t()
+        assert lib.sr_graph_create(n, len(g.nodes), e, len(g.edges), (ctypes.c_uint8 * len(g.edges))(*g.patterns["streaming"]), batch, 1,
+                                   ctypes.byref(h)) == 0
+        assert lib.sr_graph_set_option(h, 6, resident) == 0 and lib.sr_graph_workspace_bytes(h, ctypes.byref(size)) == 0
+        lib.sr_graph_destroy(h)
+        sizes.append(size.value)
+    assert sizes[0] <= 32 << 20 and sizes[1] <= 32 << 20
+    assert (sizes[1] > sizes[0]) == (batch == 3926)
