@@ -66,6 +66,11 @@ constexpr int kTables = 3;                            // node tables in shared m
 constexpr int kSmemBudget = 204 * 1024;
 constexpr int kMaxNodeKb = 128;                       // K-blocks per node
 constexpr int kMaxFused = 4;                          // nodes of a plan
+// The most columns of a tile that are tried.  160: two 8 x 8 images with the gap between them (144 columns), which took either 256
+// columns for three images or 64 for one.  Us per frame without / with it: ten-node network at 8 / 16 samples 18.6 / 17.0, 25.9 / 25.0,
+// sequential at 20 / 32 / 128 105.9 / 97.8, 111.2 / 106.1, 197.5 / 186.5, six-node sequential at 256 212 / 203, hybrid at 20 samples 41.4 / 37.0.
+constexpr int kTileCols[] = {256, 160, 128, 64};
+constexpr int kVariants = sizeof(kTileCols) / sizeof(int);
 constexpr int kMaxParts = 8;                          // parts of an item's reduction
 
 // A run of equally wide K-blocks of a node's reduction as the weight producer sees it: n_groups weight groups (one copy
@@ -1085,7 +1090,7 @@ void choose_tile(int H, int W, int B, int max_cols, int forced_tw, double per_bo
     for (int nl = 1; nl <= 8; nl *= 2) {
         if (nl > 1 && 8 * (nl / 2) >= W) break;
         if (forced_tw > 0 && nl != forced_tw / 8 && !(8 * nl >= W && forced_tw > 8 * nl)) continue;
-        const int lane_max = max_cols / nl, rows = lane_max / 8;
+        const int lane_max = max_cols / nl / 16 * 16, rows = lane_max / 8;       // (whole steps of an instruction's N)
         if (rows < 1) break;
         if (rows >= H) {
             const int tb = std::max(1, std::min(B, (lane_max + P.sep * 8) / ((H + P.sep) * 8)));
@@ -1374,10 +1379,12 @@ long long spread_items(const std::vector<TcWork>& work, size_t n, int grid, std:
 int part_chunks(const NodePlan& P, int parts) { return (P.nl * P.lane_cols / 16 + parts - 1) / parts; }
 
 // Estimated cycles of one of the parts of an item of `cycles`: K-blocks and start, and what it sends to the others (8 KiB a chunk).
+// Sums that have no room of their own go where the rings were, each part's once these have run dry there: 1200 cycles a part (by a
+// constant instead, ten-node sequential at 16 samples 88.9 -> 93.1 us per frame, six-node at 4 samples 10.3 -> 11.4).
 long long part_cycles(const NodePlan& P, long long cycles, int parts, bool in_rings)
 {
     if (parts <= 1) return cycles;
-    return 1500 + (cycles - 1500) / parts + 1200 + (in_rings ? 1200 : 0) + 320 * (P.nl * P.lane_cols / 16 - part_chunks(P, parts));
+    return 1500 + (cycles - 1500) / parts + 1200 + (in_rings ? 1200 * (parts - 1) : 0) + 320 * (P.nl * P.lane_cols / 16 - part_chunks(P, parts));
 }
 
 // Items (sorted, longest first) onto `grid` CTAs in clusters: an item of p > 1 parts goes to p neighbouring CTAs of one cluster that
@@ -1541,7 +1548,7 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
     for (size_t gi = 0; gi < g->groups.size(); ++gi) {
         const size_t first_plan = E->nodes.size();
         std::vector<int> members;
-        // What can be chosen per plan: the most columns of its tiles (256, 128, 64: variants 0, 1, 2), and the parts of its items.
+        // What can be chosen per plan: the most columns of its tiles (variants, as in kTileCols), and the parts of its items.
         struct Variant { NodePlan P; std::vector<TcTile> tiles; int box_kb = 1, w_slot = 1024, words = 0; long long plain, cycles[2][kMaxW + 1]; };   // of an item; by crowded, slots
         struct Choice { int v, parts; };
         std::vector<std::vector<Variant>> variants;
@@ -1590,7 +1597,7 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
                 words = std::max(words, V.words / ch[m].parts + 16);
                 if (ch[m].parts > 1) L.exch = std::max(L.exch, (ch[m].parts - 1) * part_chunks(V.P, ch[m].parts) * 8192);
                 items += V.tiles.size();
-                widest = widest && ch[m].v == 0;
+                widest = widest && ch[m].v <= 1;
             }
             L.table_bytes = (int)sizeof(TcNode) + (table_words ? table_words : words) * 16;
             const int sums = L.exch;
@@ -1610,10 +1617,13 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
         };
         // cycles and lists of a choice; tail: the epilogue of the widest tile, which no other item hides (13 cycles a column)
         struct Bound { long long longest = 0, total = 0, tail = 0; size_t parts = 0, at = 0; };
+        // A launch with more parts than CTAs is crowded; one of half the SMs has fewer of them (counted as if it had all, six-node
+        // hybrid at 10 samples 32.8 -> 35.5 us per frame).
+        int ctas_now = g->sm_count;
         auto crowded_by = [&](const std::vector<Choice>& ch) {
             size_t parts = 0;
             for (size_t m = 0; m < members.size(); ++m) parts += variants[m][ch[m].v].tiles.size() * ch[m].parts;
-            return parts > (size_t)g->sm_count;
+            return parts > (size_t)ctas_now;
         };
         auto cycles_of = [&](const Variant& V, int parts, const TcEngine::Launch& L, bool few, bool crowded) {
             return few ? part_cycles(V.P, V.cycles[crowded][L.n_w], parts, L.exch == 0) : V.plain;
@@ -1643,8 +1653,9 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
             return work;
         };
         // A launch with many items per SM takes the widest tiles (fewest copies per MMA).  For one with few, the split that ends first
-        // by the estimate is sought: from 256, 128 or 64 columns for every plan, the plan whose items take longest gets narrower
-        // tiles or has its items cut into twice as many parts, whichever leaves the shorter bound, again and again.  The line lies at
+        // by the estimate is sought: from the same columns for every plan, the plan whose items take longest gets narrower
+        // tiles (of the next or the second next width) or has its items cut into twice as many parts, whichever leaves the shortest
+        // bound, again and again.  The line lies at
         // three items of the widest tiles per SM: at 2.8 (stress graph at 4 samples) the search still gains 8 %, from 3.5 on
         // (six-node network at 64 samples, ten-node at 48) nothing.
         std::vector<Choice> best;
@@ -1662,17 +1673,19 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
             best_cost = -1;
             size_t widest_items = 0;
             for (size_t m = 0; m < members.size(); ++m) {
-                for (int cols = kMaxCols; cols >= 64; cols /= 2) variants[m].push_back(variant_of(m, cols));
+                for (int cols : kTileCols) variants[m].push_back(variant_of(m, cols));
                 widest_items += variants[m][0].tiles.size();
             }
             few = g->opt_b_units == 0 && g->opt_tile_w == 0 && widest_items <= 3 * (size_t)g->sm_count;
-            for (int start = 0; start < 3 && !members.empty(); ++start) {
+            for (int start = 0; start < kVariants && !members.empty(); ++start) {
+                if (start == 1 && !few) continue;              // (ten-node windows of 8 frames, 128 samples: 1842 -> 1905 us per pass with them)
                 size_t items = 0;
                 for (size_t m = 0; m < members.size(); ++m) items += variants[m][start].tiles.size();
                 for (int cluster = 1; cluster <= (few ? kMaxParts : 1); cluster *= 2)
                     // all SMs, or half of them: then the next launch starts up on the others
                     for (int half = 0; half < (few ? 2 : 1); ++half) {
                         const int ctas = (half ? std::min(held[cluster], g->sm_count / 2 / cluster) : held[cluster]) * cluster;
+                        ctas_now = half ? ctas : g->sm_count;
                         std::vector<Choice> ch(members.size(), Choice{start, 1});
                         for (;;) {
                             const TcEngine::Launch L = rings(ch, 0);
@@ -1692,13 +1705,14 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
                             if (!few) break;
                             const Choice now = ch[b.at];
                             const std::vector<Variant>& of = variants[b.at];
-                            Choice ways[2] = {Choice{now.v, now.parts * 2}, Choice{now.v + 1, now.parts}};
-                            while (ways[1].v < 2 && of[ways[1].v].tiles.size() == of[now.v].tiles.size()) ++ways[1].v;
+                            Choice ways[3] = {Choice{now.v, now.parts * 2}, Choice{now.v + 1, now.parts}, Choice{now.v + 2, now.parts}};
+                            while (ways[1].v < kVariants - 1 && of[ways[1].v].tiles.size() == of[now.v].tiles.size()) ++ways[1].v;
+                            ways[2].v = ways[1].v + 1;
                             int way = -1;
                             long long shortest = 0;
-                            for (int w = 0; w < 2; ++w) {
+                            for (int w = 0; w < 3; ++w) {
                                 if (w == 0 && (ways[0].parts > cluster || (int)of[now.v].P.kbs.size() < 2 * ways[0].parts)) continue;
-                                if (w == 1 && (ways[1].v > 2 || of[ways[1].v].tiles.size() == of[now.v].tiles.size())) continue;
+                                if (w > 0 && (ways[w].v >= kVariants || of[ways[w].v].tiles.size() == of[now.v].tiles.size())) continue;
                                 ch[b.at] = ways[w];
                                 const Bound c = bound_of(ch, rings(ch, 0), few);
                                 const long long t = std::max(c.longest, c.total / ctas) + c.tail;
@@ -1744,6 +1758,7 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
             // matrix with one row per round (entries of node -1 pad the shorter columns).  Unless the lists are asked to be
             // static, the smallest items - a fifth of the work, if the launch has more than two items per CTA - stay out of
             // the matrix and follow it as one shared list (see the kernel).
+            ctas_now = best_grid > g->sm_count / 2 ? g->sm_count : best_grid;
             const std::vector<TcWork> work = work_of(best, L, few, true);
             std::vector<std::vector<TcTile>> lists;
             size_t n_matrix = work.size(), n_rows = 0;

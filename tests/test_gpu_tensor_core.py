@@ -254,6 +254,19 @@ def test_long_reductions_of_few_pixels(cin, c, k, stride, size, batch):
     parity.check_stepwise(g, "q", samples=samples, zero_bias=False)
 
 
+@pytest.mark.parametrize("c,size,batch", [
+    (256, 8, 127),                 # two images to a tile, the last one alone
+    (256, 8, 25),                  # the same with the reduction cut: nine chunks of columns do not divide by the parts
+    (256, 5, 60),                  # three images, all 160 columns; the parts' sums in the rings
+])
+def test_tiles_of_a_few_small_images(c, size, batch):
+    g = tiny("pair", [Node("in", size, size, 64, IDENTITY), Node("a", size, size, c), Node("b", size, size, c), Node("o", 1, 1, 4, IDENTITY)],
+             [Edge(0, 1, CONV, 3, 1), Edge(1, 1, CONV, 3, 1), Edge(1, 2, CONV, 3, 1), Edge(2, 3, GAP_DENSE)], batch=batch, frames=3)
+    g.patterns["q"] = [0, 1, 0, 0]
+    for pattern in ("p", "q"):
+        parity.check_stepwise(g, pattern, samples=[0, 1, 2, batch // 2, batch - 2, batch - 1], zero_bias=False)
+
+
 @pytest.mark.parametrize("c,n", [(32, 3), (32, 4), (32, 5), (64, 3)])
 def test_several_narrow_nodes_that_share_sources(c, n):
     # a block in which every earlier node feeds every later one, as in the paper's CIFAR10 networks: up to 128 channels run as one
