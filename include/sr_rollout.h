@@ -200,12 +200,13 @@ sr_status sr_graph_set_node_bias(sr_graph* g, int node, const float* bias_host);
  *                  CTA, balanced on the host by estimated cost; 0 (default) = the same for the larger items, while
  *                  the smallest ones (a fifth of the work of a launch with many items) form one shared list that
  *                  every CTA takes from when its own list is done (a device-wide counter).
- *           key 14 "fused nodes": 1 (default) = two convolutional nodes of one launch group that have the same shape,
- *                  at most 64 channels (a multiple of 32) each and an incoming edge from the same source with the
+ *           key 14 "fused nodes": 1 (default) = up to four convolutional nodes of one launch group that have the same shape,
+ *                  32 or 64 channels each (128 together at most) and incoming edges from the same source with the
  *                  same filter geometry and the same R (or of which one has two K-blocks of reduction at most)
- *                  run as ONE tensor-core work item per pixel tile: the second
- *                  node's weights fill the otherwise empty rows 64..127 of the M = 128 instruction, and the shared
- *                  source is read and multiplied once for both.  0 = every node on its own.  Results are identical.
+ *                  run as ONE tensor-core work item per pixel tile: their weights fill the otherwise empty rows of the
+ *                  M = 128 instruction, and a shared source is read and multiplied once for all.  0 = every node on its
+ *                  own.  Every value sums the same products either way, in an order that may differ; a node is not
+ *                  touched by what it does not read, infinities and NaNs included.
  * Must be set before sr_graph_workspace_bytes / sr_graph_bind_workspace (engine, weight ring, tile width, tile pairs,
  * staged boxes, work lists, fused nodes, resident keys) / before the first run (graphs). */
 sr_status sr_graph_set_option(sr_graph* g, int key, int value);

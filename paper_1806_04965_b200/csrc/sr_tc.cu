@@ -46,6 +46,7 @@
 #include <cstring>
 #include <map>
 #include <tuple>
+#include <type_traits>
 #include <vector>
 
 #include "sr_tc.h"
@@ -117,13 +118,20 @@ constexpr uint32_t kBuNew0 = 1u << 8, kBuNew1 = 1u << 9;      // the first / sec
 constexpr uint32_t kBuLast0 = 1u << 10, kBuLast1 = 1u << 11;  // the first / second half is the last reader of its box
 constexpr uint32_t kBuTwo = 1u << 12;                         // the burst has a second half
 constexpr uint32_t kBuK16 = 1u << 13;                         // segments of one MMA
+constexpr uint32_t kBuFirst0 = 1u << 14, kBuFirst1 = 1u << 15;   // the first MMA of the half (per lane of the tile) overwrites
+constexpr int kBuOff = 16, kBuMix = 24;                       // from these bits on, four for each half: quarters of the TMEM lanes that the half leaves
+                                                              // alone (nodes of the plan that do not read its source); that it writes first, where
+                                                              // others that it writes have sums already
 
 // A plan can cover SEVERAL nodes of 32 or 64 channels that have the same shape: an M = 128 instruction on a 64-channel node is half
 // empty, on a 32-channel node three quarters, so the weights of up to two or four nodes take the rows one after the other, and
 // every K-block of a source that several of them read (same filter geometry, same frame) serves them all.  TMEM lanes
 // rows * q .. belong to the plan's node q.  Nodes are joined if they share a source, or if one of them has next to no reduction of
 // its own; of all joins the one that saves most K-blocks comes first.  (Deepest CIFAR10 network: 29 K-blocks for the four nodes of
-// its first block, where two plans of two had 11 and 27, and 72 for those of the second instead of 81.)
+// its first block, where two plans of two had 11 and 27, and 72 for those of the second instead of 81.)  The MMAs of a K-block leave the
+// lanes of a node that does not read its source alone (an output-lane mask): rows of zero weights there would turn an infinity in that
+// source into a NaN.  Without / with the masks, us per pass: deepest CIFAR10 network 1140 / 1149, six-node at 256 samples 3216 / 3226,
+// ten-node 8365 / 8435, which has more of them (a mask is four more operands for the issuing thread).
 struct alignas(16) TcNode {
     void* state[kMaxFused][2];
     const float* bias[kMaxFused];
@@ -132,7 +140,7 @@ struct alignas(16) TcNode {
     int32_t tw, th, tb, sep;        // geometry of the tile (see the file comment): tw = columns of a lane
     int32_t nl, lane_cols;          // lanes, TMEM columns of each (N of the MMA)
     int32_t n_runs, n_act, n_bu;    // lengths of the node's tables
-    int32_t pad_;
+    uint32_t part_lanes;            // bit 4 * p + q: part p of a split item has K-blocks for quarter q of the TMEM lanes
     uint32_t pairs[4];              // bit i: weight group i of the node has two blocks
     TcRun runs[kMaxRuns];
     int32_t part, n_parts, part_chunks;     // of a split item (see the kernel); part_chunks: 16-column chunks per part
@@ -270,6 +278,24 @@ __device__ __forceinline__ void tc_mma_bf16_lohi(uint32_t d_tmem, uint32_t a_lo,
         "mov.b64 db, {%3, %4};\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}"
         ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate) : "memory");
+}
+// Words of ones: TMEM lanes that an MMA does not write (four words of 32 lanes).
+struct TcLanes { uint32_t w[4]; };
+__device__ __forceinline__ TcLanes tc_lanes(uint32_t quarters)
+{
+    return TcLanes{{0u - (quarters & 1u), 0u - ((quarters >> 1) & 1u), 0u - ((quarters >> 2) & 1u), 0u - ((quarters >> 3) & 1u)}};
+}
+__device__ __forceinline__ void tc_mma_bf16_lohi(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, uint32_t idesc,
+                                                 uint32_t accumulate, const TcLanes& off)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "mov.b64 da, {%1, %2};\n\t"
+        "mov.b64 db, {%3, %4};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, {%7, %8, %9, %10}, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate), "r"(off.w[0]), "r"(off.w[1]), "r"(off.w[2]), "r"(off.w[3])
+        : "memory");
 }
 __device__ __forceinline__ void tc_commit_if(uint32_t bar, uint32_t cond)
 {
@@ -675,7 +701,6 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                 if (!ok) break;
                 tc_fence_after();                                     // the accumulator was just handed back
                 uint32_t ready = mbar_test_wait(c.bw0, c.pw0) & mbar_test_wait(c.bw1, c.pw1) & mbar_test_wait(c.ba0, c.pa0) & mbar_test_wait(c.ba1, c.pa1);
-                uint32_t more = 0;                                    // the first MMA of an item overwrites the accumulator
                 uint32_t p_fl = 0, p_w1 = 0, p_a1 = 0;                // commits owed for the second half of the burst before
                 auto pay = [&](uint32_t cond) {
                     tc_commit_if(p_w1, cond);
@@ -687,37 +712,52 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                     const uint4 o = tab[2 * nx], r = tab[2 * nx + 1];
                     Burst n = c;
                     if (!ready) ready = mbar_test_wait(c.bw0, c.pw0) & mbar_test_wait(c.bw1, c.pw1) & mbar_test_wait(c.ba0, c.pa0) & mbar_test_wait(c.ba1, c.pa1);
-                    if (ready && (c.fl & (15u | kBuK16)) == 15u && nl <= 2) {
+                    // The common kind; `masked`: with lanes that it leaves alone.
+                    auto common = [&](auto masked) {
+                        const TcLanes off0 = tc_lanes(c.fl >> kBuOff), off1 = tc_lanes(c.fl >> (kBuOff + 4));
+                        const uint32_t sum0 = c.fl & kBuFirst0 ? 0u : 1u, sum1 = decltype(masked)::value && (c.fl & kBuFirst1) ? 0u : 1u;
+                        auto mma0 = [&](uint32_t d, uint32_t w, uint32_t x, uint32_t sum) {
+                            if constexpr (decltype(masked)::value) tc_mma_bf16_lohi(d, w, c.wh, x, c.xh0, idesc, sum, off0);
+                            else tc_mma_bf16_lohi(d, w, c.wh, x, c.xh0, idesc, sum);
+                        };
+                        auto mma1 = [&](uint32_t d, uint32_t w, uint32_t x, uint32_t sum) {
+                            if constexpr (decltype(masked)::value) tc_mma_bf16_lohi(d, w, c.wh, x, c.xh1, idesc, sum, off1);
+                            else tc_mma_bf16_lohi(d, w, c.wh, x, c.xh1, idesc, sum);
+                        };
                         // a K = 16 step moves both operands 32 bytes along K: +2 in the descriptors' address field
-                        tc_mma_bf16_lohi(d0, c.v0, c.wh, c.x0, c.xh0, idesc, more);
+                        mma0(d0, c.v0, c.x0, sum0);
                         pay(owed);
-                        tc_mma_bf16_lohi(d0, c.v0 + 2, c.wh, c.x0 + 2, c.xh0, idesc, 1u);
+                        mma0(d0, c.v0 + 2, c.x0 + 2, 1u);
                         if (bu + 1 < n_bu) decode(o, r, n);
-                        tc_mma_bf16_lohi(d0, c.v1, c.wh, c.x1, c.xh0, idesc, 1u);
-                        tc_mma_bf16_lohi(d0, c.v1 + 2, c.wh, c.x1 + 2, c.xh0, idesc, 1u);
+                        mma0(d0, c.v1, c.x1, 1u);
+                        mma0(d0, c.v1 + 2, c.x1 + 2, 1u);
                         if (nl == 2) {
-                            tc_mma_bf16_lohi(d1, c.v0, c.wh, c.x0 + c.l1, c.xh0, idesc, more);
-                            tc_mma_bf16_lohi(d1, c.v0 + 2, c.wh, c.x0 + c.l1 + 2, c.xh0, idesc, 1u);
-                            tc_mma_bf16_lohi(d1, c.v1, c.wh, c.x1 + c.l1, c.xh0, idesc, 1u);
-                            tc_mma_bf16_lohi(d1, c.v1 + 2, c.wh, c.x1 + c.l1 + 2, c.xh0, idesc, 1u);
+                            mma0(d1, c.v0, c.x0 + c.l1, sum0);
+                            mma0(d1, c.v0 + 2, c.x0 + c.l1 + 2, 1u);
+                            mma0(d1, c.v1, c.x1 + c.l1, 1u);
+                            mma0(d1, c.v1 + 2, c.x1 + c.l1 + 2, 1u);
                         }
-                        tc_mma_bf16_lohi(d0, c.v2, c.wh, c.x2, c.xh1, idesc, 1u);
+                        mma1(d0, c.v2, c.x2, sum1);
                         tc_commit(c.bw0 + 8 * kMaxW);
                         tc_commit_if(c.ba0 + 8 * kBoxes, c.fl & kBuLast0);
-                        tc_mma_bf16_lohi(d0, c.v2 + 2, c.wh, c.x2 + 2, c.xh1, idesc, 1u);
+                        mma1(d0, c.v2 + 2, c.x2 + 2, 1u);
                         ready = mbar_test_wait(n.bw0, n.pw0) & mbar_test_wait(n.ba0, n.pa0);
-                        tc_mma_bf16_lohi(d0, c.v3, c.wh, c.x3, c.xh1, idesc, 1u);
+                        mma1(d0, c.v3, c.x3, 1u);
                         ready &= mbar_test_wait(n.bw1, n.pw1) & mbar_test_wait(n.ba1, n.pa1);
-                        tc_mma_bf16_lohi(d0, c.v3 + 2, c.wh, c.x3 + 2, c.xh1, idesc, 1u);
+                        mma1(d0, c.v3 + 2, c.x3 + 2, 1u);
                         if (nl == 2) {
-                            tc_mma_bf16_lohi(d1, c.v2, c.wh, c.x2 + c.l1, c.xh1, idesc, 1u);
-                            tc_mma_bf16_lohi(d1, c.v2 + 2, c.wh, c.x2 + c.l1 + 2, c.xh1, idesc, 1u);
-                            tc_mma_bf16_lohi(d1, c.v3, c.wh, c.x3 + c.l1, c.xh1, idesc, 1u);
-                            tc_mma_bf16_lohi(d1, c.v3 + 2, c.wh, c.x3 + c.l1 + 2, c.xh1, idesc, 1u);
+                            mma1(d1, c.v2, c.x2 + c.l1, sum1);
+                            mma1(d1, c.v2 + 2, c.x2 + c.l1 + 2, 1u);
+                            mma1(d1, c.v3, c.x3 + c.l1, 1u);
+                            mma1(d1, c.v3 + 2, c.x3 + c.l1 + 2, 1u);
                         }
                         p_fl = c.fl; p_w1 = c.bw1 + 8 * kMaxW; p_a1 = c.ba1 + 8 * kBoxes;
                         owed = 1;
-                    } else {
+                    };
+                    // A burst whose operands are not there, or of another kind: half by half.  (One copy for all bursts, and the masked copy of
+                    // the common kind out of the way: launches of an item or two per CTA fetch this code from L2.  With two copies
+                    // of both the deepest CIFAR10 network took 1174 us per pass instead of 1149, the six-node hybrid 485 instead of 477.)
+                    auto plain = [&] {
                         pay(owed);
                         owed = 0;
 #pragma unroll
@@ -725,26 +765,37 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                             if (h == 1 && !(c.fl & kBuTwo)) break;
                             ok = mbar_wait(h ? c.bw1 : c.bw0, h ? c.pw1 : c.pw0, abortp, wait_limit) && mbar_wait(h ? c.ba1 : c.ba0, h ? c.pa1 : c.pa0, abortp, wait_limit);
                             if (!ok) break;
+                            const uint32_t off = (c.fl >> (kBuOff + 4 * h)) & 15u, mix = (c.fl >> (kBuMix + 4 * h)) & 15u;
+                            const uint32_t sum = c.fl & (h ? kBuFirst1 : kBuFirst0) ? 0u : 1u;
                             for (uint32_t l = 0; l < nl; ++l) {
                                 const uint32_t d = d0 + l * lane_cols, xl = l * c.l1, xh = h ? c.xh1 : c.xh0;
                                 const uint32_t xa = (h ? c.x2 : c.x0) + xl, xb = (h ? c.x3 : c.x1) + xl, va = h ? c.v2 : c.v0, vb = h ? c.v3 : c.v1;
-                                tc_mma_bf16_lohi(d, va, c.wh, xa, xh, idesc, h ? 1u : more);
-                                if (!(c.fl & kBuK16)) tc_mma_bf16_lohi(d, va + 2, c.wh, xa + 2, xh, idesc, 1u);
+                                auto mma = [&](uint32_t w, uint32_t x, uint32_t sum, uint32_t off) {
+                                    tc_mma_bf16_lohi(d, w, c.wh, x, xh, idesc, sum, tc_lanes(off));
+                                };
+                                if (mix) mma(va, xa, 0u, ~mix);
+                                mma(va, xa, sum, off | mix);
+                                if (!(c.fl & kBuK16)) mma(va + 2, xa + 2, 1u, off);
                                 if (c.fl & (h ? 8u : 2u)) {
-                                    tc_mma_bf16_lohi(d, vb, c.wh, xb, xh, idesc, 1u);
-                                    if (!(c.fl & kBuK16)) tc_mma_bf16_lohi(d, vb + 2, c.wh, xb + 2, xh, idesc, 1u);
+                                    mma(vb, xb, 1u, off);
+                                    if (!(c.fl & kBuK16)) mma(vb + 2, xb + 2, 1u, off);
                                 }
                             }
                             tc_commit((h ? c.bw1 : c.bw0) + 8 * kMaxW);
                             tc_commit_if((h ? c.ba1 : c.ba0) + 8 * kBoxes, c.fl & (h ? kBuLast1 : kBuLast0));
                         }
-                        if (!ok) break;
-                        if (bu + 1 < n_bu) {
+                        if (ok && bu + 1 < n_bu) {
                             decode(o, r, n);
                             ready = mbar_test_wait(n.bw0, n.pw0) & mbar_test_wait(n.bw1, n.pw1) & mbar_test_wait(n.ba0, n.pa0) & mbar_test_wait(n.ba1, n.pa1);
                         }
+                    };
+                    if (ready && (c.fl & (15u | kBuK16)) == 15u && nl <= 2 && (c.fl >> kBuMix) == 0) {
+                        if (__builtin_expect((c.fl >> kBuOff) == 0, 1)) common(std::false_type());
+                        else common(std::true_type());
+                    } else {
+                        plain();
+                        if (!ok) break;
                     }
-                    more = 1u;
                     c = n;
                 }
                 if (!ok) break;
@@ -882,14 +933,21 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) continue;
                 owed_sums = false;
+                // (a part without K-blocks for these lanes has no sums for them)
+                const uint32_t have = nd->part_lanes >> quarter;
                 for (int c = own0 + ((own0 ^ half) & 1); c < own1; c += 2) {
                     fetch(c * 16);
                     tc_wait_ld();
+                    if (!((have >> (4 * me)) & 1u)) {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) lo[i] = hi[i] = 0u;
+                    }
                     for (int p = 0; p + 1 < n_parts; ++p) {
+                        const bool has = (have >> (4 * (p < me ? p : p + 1))) & 1u;
                         const uint4* x = reinterpret_cast<const uint4*>(smem_raw + (mine - smem_u32(smem_raw)) + (size_t)(p * per + c - own0) * 8192u);
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
-                            const uint4 v = x[q * 32];
+                            const uint4 v = has ? x[q * 32] : make_uint4(0u, 0u, 0u, 0u);
                             uint32_t* r = (q < 2 ? lo : hi) + (q & 1) * 4;
                             r[0] = __float_as_uint(__uint_as_float(r[0]) + __uint_as_float(v.x));
                             r[1] = __float_as_uint(__uint_as_float(r[1]) + __uint_as_float(v.y));
@@ -974,6 +1032,15 @@ struct NodePlan {
     int tw, th, tb, nl, lane_cols;  // tile geometry (see the file comment)
     bool flat;
     int k_total;                    // columns of the concatenated weight matrix
+    // Quarters of the TMEM lanes whose nodes a K-block serves (those that no node has are served by all).
+    uint32_t quarters_of(const sr_graph* g, const KbHost& kb) const
+    {
+        if (nodes.size() == 1) return 15u;
+        const int per = g->nodes[node].d.c / 32;
+        uint32_t used = (15u << per * nodes.size()) & 15u;
+        for (const auto& u : kb.users) used |= ((1u << per) - 1u) << u.second / 32;
+        return used;
+    }
     std::vector<KbHost> kbs;
     std::vector<WRun> runs;
     int n_parts = 1;                // parts of an item's reduction
@@ -1946,6 +2013,7 @@ sr_status sr_tc_bind(sr_graph* g)
             }
             // Bursts: two consecutive weight groups if their K-blocks are equally wide, else one.
             std::vector<TcBurst> db;
+            uint32_t begun = 0;                           // quarters of the lanes that an earlier K-block of the part writes
             for (size_t gi = 0; gi < q.wgroups.size();) {
                 const int i0 = q.wgroups[gi].first_kb, bk = q.kbs[i0].bk;
                 const bool two = one_burst(q, gi);
@@ -1963,6 +2031,11 @@ sr_status sr_tc_bind(sr_graph* g)
                         b.size[half] = (uint8_t)kb0.ring_kb;
                     }
                     if (q.kbs[wg.first_kb + wg.n - 1].x_release) b.flags |= half ? kBuLast1 : kBuLast0;
+                    const uint32_t used = P.quarters_of(g, kb0), first = used & ~begun;
+                    b.flags |= (~used & 15u) << (kBuOff + 4 * half);
+                    if (first == used) b.flags |= half ? kBuFirst1 : kBuFirst0;
+                    else b.flags |= first << (kBuMix + 4 * half);
+                    begun |= used;
                     for (int sg = 0; sg < (bk == 64 ? 2 : wg.n); ++sg) {
                         b.x_off16[half * 2 + sg] = (uint16_t)(bk == 64 ? dm[wg.first_kb].x_off16 + 4 * sg : dm[wg.first_kb + sg].x_off16);
                         b.flags |= 1u << (half * 2 + sg);
@@ -1973,6 +2046,8 @@ sr_status sr_tc_bind(sr_graph* g)
             }
             e.n_bu = (int)db.size();
             e.n_act = (int)da.size();
+            for (const NodePlan::Part& other : P.parts)
+                for (const KbHost& kb : other.kbs) e.part_lanes |= P.quarters_of(g, kb) << 4 * (&other - P.parts.data());
             const size_t at = dt.size(), words = sizeof(TcNode) / 16;
             q.table_off = (int)at;
             q.table_words = (int)(words + 2 * db.size() + da.size());

@@ -277,3 +277,41 @@ def test_several_narrow_nodes_that_share_sources(c, n):
     for fuse in (1, 0):
         parity.check_stepwise(g, "p", zero_bias=False, tc_fuse=fuse)
     parity.check_stepwise(g, "p", zero_bias=False, tc_lists=1, weight_ring_units=2, tile_width=16)
+
+
+@pytest.mark.parametrize("c,n,cin,size,batch", [
+    (32, 4, 64, 12, 2),            # few items: the reduction is cut, parts without K-blocks for some of the nodes
+    (32, 4, 64, 16, 160),          # many items
+    (32, 3, 16, 12, 40),           # rows without a node; K-blocks of 16 channels
+    (64, 2, 32, 16, 3),
+    (64, 2, 128, 28, 37),
+])
+def test_an_infinity_stays_with_the_nodes_that_read_it(c, n, cin, size, batch):
+    # nodes that share a source run as one plan; what only one of them reads must not reach the others, at any pixel, whether the first
+    # K-blocks of the plan serve all nodes or not
+    import numpy as np
+    import torch
+    from oracle import frame_update as fu
+    from workloads import data
+    nodes = [Node("x", size, size, 48, IDENTITY), Node("y", size, size, cin, IDENTITY)]
+    nodes += [Node("n%d" % i, size, size, c, RELU if i else IDENTITY) for i in range(n)] + [Node("o", 1, 1, 4, IDENTITY)]
+    edges = [Edge(0, 2 + i, CONV, 3, 1) for i in range(n)] + [Edge(1, 2, CONV, 3, 1)]
+    edges += [Edge(2 + i, 2 + i, CONV, 3, 1) for i in range(n)] + [Edge(1 + n, 2 + n, GAP_DENSE)]
+    g = tiny("inf", nodes, edges, batch=batch, frames=3)
+    samples = [0, batch // 2, batch - 1]
+    X, W, Bi = data.make_inputs(g), data.make_weights(g), data.make_biases(g, zero=False)
+    X[1][0, :, 1, 1, :] = np.inf
+    X[1][1, :, size - 1, 2, 0] = -np.inf
+    want = fu.rollout_spec(g, "p", X, W, Bi, samples=samples)
+    for options in ({}, {"tile_width": 32, "weight_ring_units": 2}, {"tile_width": 8}):
+        G = parity.make_graph(g, "p", "auto", 0, W, Bi, **options)
+        dev = [parity.to_device(g, X[v]) for v in (0, 1)]
+        G.reset([d[0] for d in dev])
+        for t in range(1, 4):
+            G.step([d[t] for d in dev], None)
+            for v in range(2, 2 + n):
+                got = G.get_state(v).float().cpu().numpy()[samples]
+                finite = np.isfinite(want[v][t])
+                assert finite.all() == (v > 2)
+                assert np.abs(got[finite] - want[v][t][finite]).max() <= parity.TOL["bf16"] * np.abs(want[v][t][finite]).max(), (options, v, t)
+        G.sync_status()
