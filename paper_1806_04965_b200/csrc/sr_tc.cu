@@ -50,6 +50,7 @@
 #include <vector>
 
 #include "sr_tc.h"
+#include "sr_tc_lists.h"
 
 namespace {
 
@@ -146,11 +147,6 @@ struct alignas(16) TcNode {
     int32_t part, n_parts, part_chunks;     // of a split item (see the kernel); part_chunks: 16-column chunks per part
 };
 static_assert(sizeof(TcNode) % 16 == 0, "copied as 16-byte words");
-
-// node: where its table begins, in 16-byte words from the start of the table area (on the host, until a workspace is bound: its plan):
-// a TcNode, bursts, activation boxes; words: how many it has (until then: the part of a split item).  m0: first output channel; slot:
-// of the table in shared memory (set by the keeper); rank0: the cluster rank that has part 0 of a split item
-struct alignas(16) TcTile { int32_t node, b0, h0, w0, m0, slot, words, rank0; };
 
 struct TcParams {
     const CUtensorMap* maps;
@@ -1419,29 +1415,6 @@ long long item_cycles(const sr_graph* g, const NodePlan& P, double ring_cycles)
     return (long long)c;
 }
 
-// An item as the work lists see it: cycles of one of its parts (estimated), parts, what the kernel reads.
-struct TcWork { long long cycles; int parts; TcTile tile; };
-
-// Longest processing time first: items (sorted, longest first) onto the least loaded of `grid` lists.  Returns the longest list's load.
-long long spread_items(const std::vector<TcWork>& work, size_t n, int grid, std::vector<std::vector<TcTile>>* lists)
-{
-    std::vector<std::pair<long long, int>> heap;             // (-load, cta): the standard heap keeps the largest on top
-    for (int c = 0; c < grid; ++c) heap.push_back({0, -c});
-    std::make_heap(heap.begin(), heap.end());
-    if (lists) lists->assign(grid, {});
-    long long longest = 0;
-    for (size_t i = 0; i < n; ++i) {
-        std::pop_heap(heap.begin(), heap.end());
-        std::pair<long long, int> top = heap.back();
-        if (lists) (*lists)[-top.second].push_back(work[i].tile);
-        top.first -= work[i].cycles;
-        longest = std::max(longest, -top.first);
-        heap.back() = top;
-        std::push_heap(heap.begin(), heap.end());
-    }
-    return longest;
-}
-
 // 16-column chunks of the accumulator that one of an item's parts sums.
 int part_chunks(const NodePlan& P, int parts) { return (P.nl * P.lane_cols / 16 + parts - 1) / parts; }
 
@@ -1452,48 +1425,6 @@ long long part_cycles(const NodePlan& P, long long cycles, int parts, bool in_ri
 {
     if (parts <= 1) return cycles;
     return 1500 + (cycles - 1500) / parts + 1200 + (in_rings ? 1200 * (parts - 1) : 0) + 320 * (P.nl * P.lane_cols / 16 - part_chunks(P, parts));
-}
-
-// Items (sorted, longest first) onto `grid` CTAs in clusters: an item of p > 1 parts goes to p neighbouring CTAs of one cluster that
-// have no part yet, behind what else they have; whole items to the least loaded CTAs.  Returns the longest list's load, or -1 if
-// the parts do not find room.
-long long spread_split(const std::vector<TcWork>& work, int grid, int cluster, std::vector<std::vector<TcTile>>* lists)
-{
-    std::vector<long long> load(grid, 0);
-    std::vector<char> taken(grid, 0);
-    std::vector<TcTile> part(grid);
-    if (lists) lists->assign(grid, {});
-    for (const TcWork& w : work) {
-        const int n = w.parts;
-        int at = -1;
-        long long least = 0;
-        for (int c = 0; c + n <= grid; c += n) {
-            long long l = 0;
-            bool room = true;
-            for (int q = 0; q < n; ++q) {
-                l = std::max(l, load[c + q]);
-                room = room && (n == 1 || !taken[c + q]);
-            }
-            if (room && (at < 0 || l < least)) { at = c; least = l; }
-        }
-        if (at < 0) return -1;
-        for (int q = 0; q < n; ++q) {
-            load[at + q] += w.cycles;
-            TcTile t = w.tile;
-            t.words = q;
-            t.rank0 = at % cluster;
-            if (n > 1) {
-                part[at + q] = t;
-                taken[at + q] = 1;
-            } else if (lists) {
-                (*lists)[at].push_back(t);
-            }
-        }
-    }
-    if (lists)
-        for (int c = 0; c < grid; ++c)
-            if (taken[c]) (*lists)[c].push_back(part[c]);
-    return *std::max_element(load.begin(), load.end());
 }
 
 cudaLaunchConfig_t cluster_config(int grid, int cluster, size_t smem, cudaStream_t stream, bool early, cudaLaunchAttribute (&at)[2])
@@ -1830,7 +1761,7 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
             std::vector<std::vector<TcTile>> lists;
             size_t n_matrix = work.size(), n_rows = 0;
             if (best_cluster > 1) {
-                spread_split(work, best_grid, best_cluster, &lists);
+                if (!place_split(work, best_grid, best_cluster, lists)) return SR_ERR_UNSUPPORTED;
                 while (std::all_of(lists.end() - best_cluster, lists.end(), [](const auto& l) { return l.empty(); })) lists.resize(lists.size() - best_cluster);
                 L.cluster = best_cluster;
             } else {
