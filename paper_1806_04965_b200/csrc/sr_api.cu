@@ -18,8 +18,8 @@
 
 // Built-in workspace for callers that may not allocate device memory.  In host code the array's name
 // is only a handle: its device address is looked up once per device and that pointer is what the
-// kernels get (through the ordinary bind path).  The work lists of the CUDA-core kernels (16 bytes per 16 pixels and 128 channels, so
-// at most one part in 512 of the states) have room beyond the size that callers know.
+// kernels get (through the ordinary bind path).  The work lists of the CUDA-core kernels have room beyond the size that callers know: 16
+// bytes per 512 values or so (see sr_direct_conv_items; more where images are tiny).
 constexpr size_t kStaticBytes = SR_STATIC_WORKSPACE_BYTES + SR_STATIC_WORKSPACE_BYTES / 256;
 static __device__ __align__(256) unsigned char sr_static_workspace[kStaticBytes];
 
@@ -92,11 +92,13 @@ SrRegion take(size_t& off, size_t bytes)
     return r;
 }
 
-// Decide the engine of every node, lay out the workspace and build the block work lists.
-sr_status plan(sr_graph* g)
+// Whether the built-in workspace takes a graph of this size.
+bool fits_built_in(const sr_graph* g, size_t need) { return need - g->r_items.bytes <= (size_t)SR_STATIC_WORKSPACE_BYTES && need <= kStaticBytes; }
+
+// Decide the engine of every node, lay out the workspace and build the block work lists.  Sets *least: bytes that the graph needs
+// however it is planned.
+sr_status lay_out(sr_graph* g, size_t* least)
 {
-    if (g->batch <= 0) return SR_ERR_STATE;
-    if (g->planned) return SR_OK;                                // asking for the size and binding share one plan
     const int n_nodes = (int)g->nodes.size(), n_edges = (int)g->edges.size();
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0) g->sm_count = sms;
@@ -134,6 +136,9 @@ sr_status plan(sr_graph* g)
         he.w_direct = SrRegion();
         if (!t.use_tc) he.w_direct = take(off, (size_t)he.K * t.d.c * sizeof(float));
     }
+    *least = off;
+    for (const SrHostEdge& he : g->edges)
+        if (g->nodes[he.d.tgt].use_tc) *least += (size_t)he.K * g->nodes[he.d.tgt].d.c * g->elem;
     g->r_nodes = take(off, sizeof(SrDevNode) * n_nodes);
     g->r_edges = take(off, sizeof(SrDevEdge) * n_edges);
     g->r_ctl = take(off, sizeof(SrFrameCtl));
@@ -193,8 +198,29 @@ sr_status plan(sr_graph* g)
         sr_dn_describe(g, &g->info.resident_cluster, &g->info.resident_smem_bytes);
         g->info.resident_heads_on_chip = 1;
     }
-    g->planned = true;
     return SR_OK;
+}
+
+// Launches planned for speed may have longer lists (items cut into slices or parts, narrow tiles) and weight matrices with more zero
+// rows (joined nodes) than a graph needs.  One that the built-in workspace takes only without them is planned without: lists
+// and tables first, then joins.
+sr_status plan(sr_graph* g)
+{
+    if (g->batch <= 0) return SR_ERR_STATE;
+    if (g->planned) return SR_OK;                                // asking for the size and binding share one plan
+    size_t least = 0;
+    g->compact = 0;
+    sr_status st = lay_out(g, &least);
+    if (st == SR_OK && !fits_built_in(g, g->ws_bytes) && least <= (size_t)SR_STATIC_WORKSPACE_BYTES) {
+        for (g->compact = 1; g->compact <= 2; ++g->compact)
+            if (lay_out(g, &least) == SR_OK && fits_built_in(g, g->ws_bytes)) break;
+        if (g->compact > 2) {
+            g->compact = 0;
+            st = lay_out(g, &least);
+        }
+    }
+    g->planned = st == SR_OK;
+    return st;
 }
 
 bool cuda_ok(cudaError_t e) { return e == cudaSuccess; }
@@ -558,7 +584,7 @@ sr_status sr_graph_bind_static_workspace(sr_graph* g)
     size_t need = 0;
     sr_status st = sr_graph_workspace_bytes(g, &need);
     if (st != SR_OK) return st;
-    if (need - g->r_items.bytes > (size_t)SR_STATIC_WORKSPACE_BYTES || need > kStaticBytes) return SR_ERR_TOO_LARGE;
+    if (!fits_built_in(g, need)) return SR_ERR_TOO_LARGE;
     int dev = -1;
     if (!cuda_ok(cudaGetDevice(&dev)) || dev < 0 || dev >= 64) return SR_ERR_CUDA;
     std::lock_guard<std::mutex> lock(static_mutex);

@@ -907,7 +907,7 @@ void sr_direct_conv_items(const sr_graph* g, int v, std::vector<SrDirectItem>& i
     const size_t quads = (size_t)g->batch * HW * (d.c / 4), sms = (size_t)g->sm_count;
     int K = 0;
     for (int e : g->nodes[v].in_edges) K += g->edges[e].K;
-    const bool slices = K >= 128 && quads / 4 < sms * 512, four = quads / 4 >= sms * 256 || (slices && quads >= sms * 64);
+    const bool slices = K >= 128 && quads / 4 < sms * 512 && g->compact == 0, four = quads / 4 >= sms * 256 || (slices && quads >= sms * 64);
     const int px = ((slices ? 32 : kWarps * 32) >> qlog) * (four ? 4 : 1);
     for (int b = 0; b < g->batch; ++b)
         for (int p0 = 0; p0 < HW; p0 += px)

@@ -38,7 +38,7 @@ struct SrDirectItem {
     int32_t node;        // index into the SrDevNode table
     int32_t b0;          // first sample (dense nodes: sample chunk); its complement: four pixels per thread (conv_tile)
     int32_t p0;          // first pixel (conv nodes) or first output channel (dense nodes)
-    int32_t pad_;        // conv nodes on conv_tile: first channel | log2(channel quads per block) << 24
+    int32_t pad_;        // conv nodes on conv_tile: first channel | log2(channel quads per block) << 24 | 1 << 30 (slices of the reduction)
 };
 
 // Dense / mean-dense nodes as the head kernels see them: passed as kernel parameters.
@@ -240,6 +240,7 @@ struct sr_graph {
     // workspace
     size_t ws_bytes = 0;
     bool planned = false;                          // the workspace layout stands for the current options
+    int compact = 0;                               // 0: launches planned for speed; 1, 2: for small tables, for small weights too (see plan)
     char* ws = nullptr;
     SrRegion r_nodes, r_edges, r_ctl, r_items;
     SrRegion r_clear;                              // what a reset zeroes: the flags, then the non-input nodes' parity-0 states

@@ -1068,7 +1068,7 @@ struct TcEngine {
     };
     std::vector<Launch> launches;
     SrRegion r_maps, r_tables, r_tiles;
-    int n_maps = 0, n_kbs = 0, n_tiles = 0;
+    int n_maps = 0, n_tiles = 0;
     // optional timing of the group launches with CUDA events on the launching stream
     std::vector<cudaEvent_t> ev;             // pairs: start, stop
     size_t ev_used = 0;
@@ -1674,7 +1674,7 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
                 for (int cols : kTileCols) variants[m].push_back(variant_of(m, cols));
                 widest_items += variants[m][0].tiles.size();
             }
-            few = g->opt_b_units == 0 && g->opt_tile_w == 0 && widest_items <= 3 * (size_t)g->sm_count;
+            few = g->opt_b_units == 0 && g->opt_tile_w == 0 && g->compact == 0 && widest_items <= 3 * (size_t)g->sm_count;
             for (int start = 0; start < kVariants && !members.empty(); ++start) {
                 if (start == 1 && !few) continue;              // (ten-node windows of 8 frames, 128 samples: 1842 -> 1905 us per pass with them)
                 size_t items = 0;
@@ -1726,7 +1726,8 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
         // Joined as far as they go, or in twos: the launch that ends first (with few tiles, more and shorter items may; joined where it
         // is 3 % ahead).  Deepest CIFAR10 network, us per frame in twos / joined: 13.2 / 13.1, 19.0 / 24.0, 43.7 / 44.8, 74.0 / 66.9 at 4,
         // 16, 64, 128 samples; with four added layers 17.0 / 12.4, 36.6 / 34.2, 108 / 95 at 8, 64, 256.
-        const auto joined = join_nodes(g, g->groups[gi], g->opt_tc_fuse ? kMaxFused : 1), twos = join_nodes(g, g->groups[gi], g->opt_tc_fuse ? 2 : 1);
+        const int most = !g->opt_tc_fuse || g->compact > 1 ? 1 : g->compact > 0 ? 2 : kMaxFused;
+        const auto joined = join_nodes(g, g->groups[gi], most), twos = join_nodes(g, g->groups[gi], std::min(most, 2));
         search(joined);
         if (joined != twos) {
             const long long cost = best_cost;
@@ -1783,18 +1784,20 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
         n_tiles += (int)E->group_tiles[gi].size();
         E->launches.push_back(L);
     }
-    int n_kbs = 0;
-    for (NodePlan& P : E->nodes) {
-        n_kbs += (int)P.kbs.size();
-        P.wcat = take((size_t)P.rows_total(g) * P.k_total * 2);
-    }
+    for (NodePlan& P : E->nodes) P.wcat = take((size_t)P.rows_total(g) * P.k_total * 2);
     E->n_tiles = n_tiles;
-    E->n_kbs = n_kbs;
-    // upper bound on distinct tensor maps: two parities per K-block plus one weight map per (node, bk)
-    E->r_maps = take(sizeof(CUtensorMap) * (size_t)(4 * n_kbs + 1));
-    size_t n_entries = 0;
-    for (const NodePlan& P : E->nodes) n_entries += P.parts.size();
-    E->r_tables = take(48 * (size_t)n_kbs + sizeof(TcNode) * n_entries);
+    // tensor maps, as many as there can be: two parities per activation box, two widths per run of weights
+    size_t n_maps = 1, n_words = 0;
+    for (const NodePlan& P : E->nodes) {
+        n_maps += 2 * P.runs.size();
+        for (const NodePlan::Part& q : P.parts) {
+            const size_t boxes = std::count_if(q.kbs.begin(), q.kbs.end(), [](const KbHost& kb) { return kb.x_load; });
+            n_maps += 2 * boxes;
+            n_words += sizeof(TcNode) / 16 + 2 * count_bursts(q) + boxes;
+        }
+    }
+    E->r_maps = take(sizeof(CUtensorMap) * n_maps);
+    E->r_tables = take(16 * n_words);
     E->r_tiles = take(sizeof(TcTile) * (size_t)std::max(1, n_tiles));
     return SR_OK;
 }

@@ -198,3 +198,30 @@ def test_resident_tables_keep_a_graph_in_the_built_in_workspace(batch):
         sizes.append(size.value)
     assert sizes[0] <= 32 << 20 and sizes[1] <= 32 << 20
     assert (sizes[1] > sizes[0]) == (batch == 3926)
+
+
+C, M = 0, 2                    # convolution, mean-dense
+NEAR_THE_LIMIT = {
+    # work lists: 101 fp32 nodes whose reductions the warps of a block would share, at one sample
+    "fp32_chain": (0, 1, [(16, 128, 0)] + 101 * [(16, 128, 1)] + [(1, 4, 0)], [(i, i + 1, C, 1) for i in range(101)] + [(101, 102, M, 1)], [1] * 102),
+    # the same with channels that the tensor-core kernel does not take
+    "bf16_40_channels": (1, 34, [(28, 128, 0), (28, 40, 0), (28, 40, 0), (28, 40, 1), (28, 40, 0), (28, 8, 0), (1, 10, 0)],
+                         [(0, 1, C, 3), (1, 2, C, 7), (2, 3, C, 7), (0, 4, C, 7), (3, 4, C, 5), (1, 5, C, 7), (4, 5, C, 1), (5, 5, C, 1), (5, 6, M, 1)],
+                         [0, 1, 0, 1, 0, 0, 0, 1, 1]),
+    # tables of the tensor-core kernel
+    "bf16_two_nodes": (1, 1251, [(5, 8, 0), (5, 64, 0), (5, 64, 0), (1, 10, 0)], [(0, 1, C, 3), (1, 2, C, 7), (2, 3, M, 1)], [0, 0, 1]),
+}
+
+
+@pytest.mark.parametrize("name", sorted(NEAR_THE_LIMIT))
+def test_lists_and_tables_keep_a_graph_in_the_built_in_workspace(name):
+    # graphs whose states and weights all but fill the 32 MiB: what a launch planned for speed wants beyond them is left out
+    lib = load_library()
+    dtype, batch, nodes, edges, R = NEAR_THE_LIMIT[name]
+    n = (_NodeDesc * len(nodes))(*[_NodeDesc(s, s, c, act) for s, c, act in nodes])
+    e = (_EdgeDesc * len(edges))(*[_EdgeDesc(s, t, kind, k, 1, 0) for s, t, kind, k in edges])
+    h = ctypes.c_void_p()
+    assert lib.sr_graph_create(n, len(nodes), e, len(edges), (ctypes.c_uint8 * len(R))(*R), batch, dtype, ctypes.byref(h)) == 0
+    status = lib.sr_graph_bind_static_workspace(h)
+    lib.sr_graph_destroy(h)
+    assert status in (0, 6)                                     # bound, or no GPU to bind on; not SR_ERR_TOO_LARGE
