@@ -146,15 +146,19 @@ __device__ __forceinline__ void dn_st_async4(uint32_t cell, uint32_t bar, uint32
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
                  ::"r"(dn_map_rank(cell, rank)), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"(dn_map_rank(bar, rank)) : "memory");
 }
+__device__ __forceinline__ bool dn_try_wait(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.b32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
 // Bounded wait for a phase of a barrier that other CTAs' stores complete.
 __device__ __forceinline__ bool dn_wait(uint32_t bar, uint32_t parity, volatile int* gave_up, long long limit)
 {
     long long t0 = 0;
     for (int i = 0;; ++i) {
-        uint32_t ok;
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.b32 %0, 1, 0, p;\n\t}"
-                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-        if (ok) return true;
+        if (dn_try_wait(bar, parity)) return true;
         if ((i & 31) == 31) {
             const long long t = clock64();
             if (t0 == 0) t0 = t;
@@ -547,6 +551,7 @@ sr_dense_kernel(const DnParams P, const SrFrameCtl init, int n_frames)
         asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(dn_smem(&bars[l][tid & 1])), "r"(n_arrive) : "memory");
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");      // (their bulk copies go where this thread has stored zeros)
     // The other CTAs may store into this one from here on: its barriers stand, the buffers of frame 1 are zeroed, and those of frame 0,
     // filled below, are stored into again only once this CTA has sent its part of frame 1.
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
@@ -591,7 +596,8 @@ sr_dense_kernel(const DnParams P, const SrFrameCtl init, int n_frames)
     __syncthreads();
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 
-    for (int f = 0; f < n_frames && !*(volatile int*)&gave_up; ++f) {                // relative frame f -> f + 1
+    int f = 0;
+    for (; f < n_frames && !*(volatile int*)&gave_up; ++f) {                         // relative frame f -> f + 1
         // the input frame after the next one is on its way during this update; it has landed when the last level's barrier
         // completes
         const int par = (f + 1) & 1;
@@ -639,12 +645,21 @@ sr_dense_kernel(const DnParams P, const SrFrameCtl init, int n_frames)
         }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
-    // Whatever the others send to this CTA counts on a barrier that it has waited for, so it may leave: unless it gave up (then what
-    // is on its way lands first), or another one still copies out of its shared memory (convolutions).
+    // Whatever the others send to this CTA counts on a barrier that it has waited for, so it may leave: unless it gave up, or another
+    // one still copies out of its shared memory (convolutions).
     __syncthreads();
-    if (*(volatile int*)&gave_up) __nanosleep(100000);
-    __syncwarp();
     if (CONV || *(volatile int*)&gave_up) dn_cluster_sync();
+    if (*(volatile int*)&gave_up) {
+        // Nobody starts a store any more.  What is on its way lands first: all that can be is of the frame in which the wait expired or
+        // of the next; what will not come, because its sender gave up too, ends with the limit.
+        if (tid == 0) {
+            const long long begin = clock64();
+            for (int g = max(f - 1, 0); g <= f && g < n_frames; ++g)
+                for (int l = 0; l < P.n_levels; ++l)
+                    while (!dn_try_wait(dn_smem(&bars[l][(g + 1) & 1]), (uint32_t)(g >> 1) & 1u) && clock64() - begin <= P.wait_limit) {}
+        }
+        __syncthreads();
+    }
     if (tid == 0 && gave_up) atomicExch(P.error, 1);
 
     // the last frame back to the state buffers in global memory (parity of t + T); every rank holds a full copy and

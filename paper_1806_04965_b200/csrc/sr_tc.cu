@@ -179,14 +179,23 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+// PEERS: what completes the barrier was written by other CTAs of the cluster.
+template <bool PEERS = false>
 __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity)
 {
     uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.b32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    if (PEERS)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.b32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    else
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.b32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok;
 }
 // Non-blocking probe.
@@ -213,13 +222,14 @@ __device__ __forceinline__ bool elect_one()
 // Bounded wait.  Returns false if the limit expired or another role already gave up.  A launch may start early, while a run of many
 // frames before it is still on; the limit must not count that time, so every role waits for the predecessor ahead of its first
 // bounded wait that depends, through whatever other role, on the predecessor.
+template <bool PEERS>
 __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long limit)
 {
     const long long t0 = clock64();
     for (;;) {
 #pragma unroll 1
         for (int i = 0; i < 32; ++i)
-            if (mbar_try_wait(bar, parity)) return true;
+            if (mbar_try_wait<PEERS>(bar, parity)) return true;
         if (*abort_flag) return false;
         if (clock64() - t0 > limit) {
             *abort_flag = 1;
@@ -227,10 +237,11 @@ __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volat
         }
     }
 }
+template <bool PEERS = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, long long limit)
 {
-    if (mbar_try_wait(bar, parity)) return true;
-    return mbar_wait_slow(bar, parity, abort_flag, limit);
+    if (mbar_try_wait<PEERS>(bar, parity)) return true;
+    return mbar_wait_slow<PEERS>(bar, parity, abort_flag, limit);
 }
 // Wait for a copy this thread started itself, before the CTA gives up its shared memory.  It has its own limit and
 // does not look at the abort flag: after another role gave up, the copies in flight still have to land.
@@ -909,7 +920,7 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                         for (int p = 0; p < n_parts; ++p)
                             if (p != me) st_async_v4(map_rank(smem_u32(&clear_words[me]), tl.rank0 + p), map_rank(bar_clear, tl.rank0 + p), 1u, 1u, 1u, 1u);
                     }
-                    ok = mbar_wait(bar_clear, 0, abortp, wait_limit);
+                    ok = mbar_wait<true>(bar_clear, 0, abortp, wait_limit);
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) continue;
                 }
@@ -925,7 +936,7 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                     st_async_v4(dst + 1024, bar, hi[0], hi[1], hi[2], hi[3]);
                     st_async_v4(dst + 1536, bar, hi[4], hi[5], hi[6], hi[7]);
                 }
-                ok = mbar_wait(bar_sums, 0, abortp, wait_limit);
+                ok = mbar_wait<true>(bar_sums, 0, abortp, wait_limit);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) continue;
                 owed_sums = false;
@@ -970,7 +981,9 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
     __syncwarp();
     tc_fence_before();
     __syncthreads();
-    if (SPLIT && abort_flag) cluster_sync();               // (given up: those that have not left may still write to this CTA)
+    // Given up: those that have not left may still write to this CTA.  (What they have sent has landed when they arrive here: a part that
+    // sends then waits, or drains, for a sum from this CTA that does not come, as long as a wait may last.)
+    if (SPLIT && abort_flag) cluster_sync();
     if (threadIdx.x == 0 && abort_flag) atomicExch(P.error, 1);
     if (threadIdx.x == 0 && P.sched && P.n_own < P.n_tiles) {
         // the CTA that leaves last (none takes an item any more) puts the counters back for the next launch
