@@ -131,8 +131,8 @@ constexpr int kBuOff = 16, kBuMix = 24;                       // from these bits
 // its own; of all joins the one that saves most K-blocks comes first.  (Deepest CIFAR10 network: 29 K-blocks for the four nodes of
 // its first block, where two plans of two had 11 and 27, and 72 for those of the second instead of 81.)  The MMAs of a K-block leave the
 // lanes of a node that does not read its source alone (an output-lane mask): rows of zero weights there would turn an infinity in that
-// source into a NaN.  Without / with the masks, us per pass: deepest CIFAR10 network 1140 / 1149, six-node at 256 samples 3216 / 3226,
-// ten-node 8365 / 8435, which has more of them (a mask is four more operands for the issuing thread).
+// source into a NaN.  Without / with the masks, us per pass: deepest CIFAR10 network 1139 / 1143, six-node at 256 samples 3216 / 3226,
+// ten-node 8297 / 8339 (at 4 samples 195.6 / 198.6), which has more of them (a mask is four more operands for the issuing thread).
 struct alignas(16) TcNode {
     void* state[kMaxFused][2];
     const float* bias[kMaxFused];
@@ -369,7 +369,9 @@ constexpr int kAhead = 3;
 // start weight copies in turn (deepest CIFAR10 network at 16 samples 18.8 -> 22.5, at 128 73.8 -> 77.6); two issuing threads with an
 // accumulator each for tiles of up to 128 columns (8.8 -> 9.6); launches of half an SM's shared memory, so that the next one
 // sets up beside them (14.9 -> 22 before the split: the ring is too shallow).
-template <bool SPLIT>
+// MASKED: some K-block of the launch leaves lanes alone (see TcNode).  A kernel of its own, because a launch of an item or two per CTA
+// fetches its code from L2: with the masks in every launch the ten-node network, sequential at 16 samples, took 1421 us per pass, so 1379.
+template <bool SPLIT, bool MASKED>
 __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_constant__ TcParams P)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -761,9 +763,9 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                         p_fl = c.fl; p_w1 = c.bw1 + 8 * kMaxW; p_a1 = c.ba1 + 8 * kBoxes;
                         owed = 1;
                     };
-                    // A burst whose operands are not there, or of another kind: half by half.  (One copy for all bursts, and the masked copy of
-                    // the common kind out of the way: launches of an item or two per CTA fetch this code from L2.  With two copies
-                    // of both the deepest CIFAR10 network took 1174 us per pass instead of 1149, the six-node hybrid 485 instead of 477.)
+                    // A burst whose operands are not there, or of another kind: half by half.  (One copy for all bursts of a
+                    // kernel, and the masked copy of the common kind out of the way: with two copies of both the deepest CIFAR10 network
+                    // took 1174 us per pass instead of 1149.)
                     auto plain = [&] {
                         pay(owed);
                         owed = 0;
@@ -778,9 +780,10 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                                 const uint32_t d = d0 + l * lane_cols, xl = l * c.l1, xh = h ? c.xh1 : c.xh0;
                                 const uint32_t xa = (h ? c.x2 : c.x0) + xl, xb = (h ? c.x3 : c.x1) + xl, va = h ? c.v2 : c.v0, vb = h ? c.v3 : c.v1;
                                 auto mma = [&](uint32_t w, uint32_t x, uint32_t sum, uint32_t off) {
-                                    tc_mma_bf16_lohi(d, w, c.wh, x, xh, idesc, sum, tc_lanes(off));
+                                    if constexpr (MASKED) tc_mma_bf16_lohi(d, w, c.wh, x, xh, idesc, sum, tc_lanes(off));
+                                    else tc_mma_bf16_lohi(d, w, c.wh, x, xh, idesc, sum);
                                 };
-                                if (mix) mma(va, xa, 0u, ~mix);
+                                if (MASKED && mix) mma(va, xa, 0u, ~mix);
                                 mma(va, xa, sum, off | mix);
                                 if (!(c.fl & kBuK16)) mma(va + 2, xa + 2, 1u, off);
                                 if (c.fl & (h ? 8u : 2u)) {
@@ -796,9 +799,9 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                             ready = mbar_test_wait(n.bw0, n.pw0) & mbar_test_wait(n.bw1, n.pw1) & mbar_test_wait(n.ba0, n.pa0) & mbar_test_wait(n.ba1, n.pa1);
                         }
                     };
-                    if (ready && (c.fl & (15u | kBuK16)) == 15u && nl <= 2 && (c.fl >> kBuMix) == 0) {
-                        if (__builtin_expect((c.fl >> kBuOff) == 0, 1)) common(std::false_type());
-                        else common(std::true_type());
+                    if (ready && (c.fl & (15u | kBuK16)) == 15u && nl <= 2 && (!MASKED || (c.fl >> kBuMix) == 0)) {
+                        if (!MASKED || __builtin_expect((c.fl >> kBuOff) == 0, 1)) common(std::false_type());
+                        else common(std::bool_constant<MASKED>());
                     } else {
                         plain();
                         if (!ok) break;
@@ -945,12 +948,12 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
                 for (int c = own0 + ((own0 ^ half) & 1); c < own1; c += 2) {
                     fetch(c * 16);
                     tc_wait_ld();
-                    if (!((have >> (4 * me)) & 1u)) {
+                    if (MASKED && !((have >> (4 * me)) & 1u)) {
 #pragma unroll
                         for (int i = 0; i < 8; ++i) lo[i] = hi[i] = 0u;
                     }
                     for (int p = 0; p + 1 < n_parts; ++p) {
-                        const bool has = (have >> (4 * (p < me ? p : p + 1))) & 1u;
+                        const bool has = !MASKED || ((have >> (4 * (p < me ? p : p + 1))) & 1u);
                         const uint4* x = reinterpret_cast<const uint4*>(smem_raw + (mine - smem_u32(smem_raw)) + (size_t)(p * per + c - own0) * 8192u);
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
@@ -1074,7 +1077,7 @@ struct TcEngine {
     struct Launch {
         int first_tile = 0, n_own = 0, grid = 0, cluster = 0;
         int n_w = 2, w_slot = 1024, ring_kb = 0, table_bytes = 0, exch = 0;      // exch: bytes for what the other parts of an item send
-        bool fits = false;
+        bool fits = false, masked = false;                                       // masked: some K-block of a plan does not serve all of its lanes
         int rings() const { return n_w * w_slot + ring_kb * 1024 + kTables * table_bytes; }
         int exch_off() const { return exch ? rings() : 0; }                      // 0: in the rings
         size_t smem() const { return (size_t)rings() + exch + 1024; }
@@ -1463,8 +1466,8 @@ int clusters_held(const sr_graph* g, int cluster)
     cudaLaunchAttribute at[2];
     const cudaLaunchConfig_t cfg = cluster_config(cluster, cluster, kSmemBudget, nullptr, false, at);
     int held = 0;
-    if (cudaFuncSetAttribute(sr_tc_group_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget) == cudaSuccess &&
-        cudaOccupancyMaxActiveClusters(&held, sr_tc_group_kernel<true>, &cfg) == cudaSuccess && held > 0)
+    if (cudaFuncSetAttribute(sr_tc_group_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&held, sr_tc_group_kernel<true, true>, &cfg) == cudaSuccess && held > 0)
         return std::min(held, g->sm_count / cluster);
     cudaGetLastError();
     return std::max(1, g->sm_count / cluster);
@@ -1790,6 +1793,8 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
             for (size_t r = 0; r < n_rows; ++r)
                 for (auto& l : lists) E->group_tiles[gi].push_back(r < l.size() ? l[r] : TcTile{-1, 0, 0, 0, 0, 0, 0, 0});
             L.grid = (int)lists.size();
+            for (int ni : members)
+                for (const KbHost& kb : E->nodes[ni].kbs) L.masked = L.masked || E->nodes[ni].quarters_of(g, kb) != 15u;
             L.n_own = (int)E->group_tiles[gi].size();
             for (size_t i = n_matrix; i < work.size(); ++i) E->group_tiles[gi].push_back(work[i].tile);
         }
@@ -1823,7 +1828,7 @@ sr_status sr_tc_bind(sr_graph* g)
     if (!encode) return SR_ERR_CUDA;
     // Always the largest shared-memory partition: otherwise the SM is configured with the smallest partition that holds
     // this kernel's CTA, which can leave a few hundred bytes, and the frame's other kernels cannot run beside it.
-    for (auto kernel : {sr_tc_group_kernel<false>, sr_tc_group_kernel<true>})
+    for (auto kernel : {sr_tc_group_kernel<false, false>, sr_tc_group_kernel<false, true>, sr_tc_group_kernel<true, false>, sr_tc_group_kernel<true, true>})
         if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget) != cudaSuccess ||
             cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess)
             return SR_ERR_CUDA;
@@ -2135,9 +2140,9 @@ int sr_tc_launch_group(sr_graph* g, int group, SrFollow how, cudaStream_t s)
     if (L.cluster) {
         cudaLaunchAttribute at[2];
         const cudaLaunchConfig_t cfg = cluster_config(L.grid, L.cluster, L.smem(), s, how.early && !timed, at);
-        cudaLaunchKernelEx(&cfg, sr_tc_group_kernel<true>, P);
+        cudaLaunchKernelEx(&cfg, L.masked ? sr_tc_group_kernel<true, true> : sr_tc_group_kernel<true, false>, P);
     } else {
-        sr_launch(sr_tc_group_kernel<false>, L.grid, kThreads, L.smem(), s, how.early && !timed, P);
+        sr_launch(L.masked ? sr_tc_group_kernel<false, true> : sr_tc_group_kernel<false, false>, L.grid, kThreads, L.smem(), s, how.early && !timed, P);
     }
     if (timed) {
         cudaEventRecord(E->ev[E->ev_used + 1], s);
