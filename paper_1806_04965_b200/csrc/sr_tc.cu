@@ -371,8 +371,12 @@ constexpr int kAhead = 3;
 // sets up beside them (14.9 -> 22 before the split: the ring is too shallow).
 // MASKED: some K-block of the launch leaves lanes alone (see TcNode).  A kernel of its own, because a launch of an item or two per CTA
 // fetches its code from L2: with the masks in every launch the ten-node network, sequential at 16 samples, took 1421 us per pass, so 1379.
+// Registers: 80 at most, so that an SM has room for a block of the heads (128 registers x 256 threads) or three of the frame input
+// beside a CTA.  (SPLIT is bound to them; unbound, with the sums of all parts in flight, it took 114, and the deepest CIFAR10 network at
+// 16 samples, whose heads then waited for the launch to end, 18.6 us per frame, so 17.0.  Without SPLIT the compiler needs 77, and
+// being held to 80 costs the ten-node network 2 %.)
 template <bool SPLIT, bool MASKED>
-__global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_constant__ TcParams P)
+__global__ void __launch_bounds__(kThreads, SPLIT ? 2 : 1) sr_tc_group_kernel(const __grid_constant__ TcParams P)
 {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t bars[2 * kBoxes + 2 * kMaxW + 4 + kItems + 2];
@@ -952,6 +956,7 @@ __global__ void __launch_bounds__(kThreads, 1) sr_tc_group_kernel(const __grid_c
 #pragma unroll
                         for (int i = 0; i < 8; ++i) lo[i] = hi[i] = 0u;
                     }
+#pragma unroll 1
                     for (int p = 0; p + 1 < n_parts; ++p) {
                         const bool has = !MASKED || ((have >> (4 * (p < me ? p : p + 1))) & 1u);
                         const uint4* x = reinterpret_cast<const uint4*>(smem_raw + (mine - smem_u32(smem_raw)) + (size_t)(p * per + c - own0) * 8192u);
