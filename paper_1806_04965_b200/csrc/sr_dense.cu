@@ -52,7 +52,7 @@ constexpr int kDnMoreThanHalf = 120 * 1024;   // of an SM's shared memory, bytes
 constexpr int kDnMaxCluster = 16;      // CTAs per cluster: 8, or 16 (a non-portable size) for rollouts with one level per frame
 constexpr int kDnWarps = 8;            // 256 threads: a work unit keeps 64 registers of packed accumulators and its operands
 constexpr int kDnRows = 4;             // output rows per work unit
-constexpr int kDnHeld = 8;             // vectors of the next bf16 input frame that a fetching thread holds in registers
+constexpr int kDnHeld = 8;             // vectors of a bf16 input frame that a fetching thread has on their way at a time
 constexpr int kDnConvWork = 1 << 18;   // multiply-adds per sample and frame of all convolutions, most
 constexpr int kDnSmemMax = 226 * 1024;
 
@@ -504,7 +504,7 @@ sr_dense_kernel(const DnParams P, const SrFrameCtl init, int n_frames)
     // of the run, floats from one frame to the next, floats per frame, the three shared-memory buffers
     __shared__ const T* in_src[SR_MAX_INPUTS];
     __shared__ long long in_step[SR_MAX_INPUTS];
-    __shared__ int in_len[SR_MAX_INPUTS], in_buf[SR_MAX_INPUTS][3], n_in;
+    __shared__ int in_len[SR_MAX_INPUTS], in_buf[SR_MAX_INPUTS][3], n_in, n_vectors;   // n_vectors: of four values, in a frame of all inputs
     __shared__ uint64_t bars[kDnMaxLevels][2];               // per level and frame parity: the level's new states have arrived
     __shared__ int gave_up, conv_done;
     const int tid = threadIdx.x, nthr = blockDim.x, warp = tid >> 5, lane = tid & 31;
@@ -531,12 +531,14 @@ sr_dense_kernel(const DnParams P, const SrFrameCtl init, int n_frames)
         gave_up = 0;
         conv_done = 0;
         int n = 0;
+        n_vectors = 0;
         for (int v = 0; v < P.n_nodes; ++v) {
             const DnNode& nd = P.nodes[v];
             if (!nd.is_input) continue;
             in_src[n] = reinterpret_cast<const T*>(static_cast<const char*>(init.in_base[nd.input_slot]) + run0 * init.in_stride_bytes[nd.input_slot]) + (size_t)b0 * nd.C;
             in_step[n] = init.in_stride_bytes[nd.input_slot] / (long long)sizeof(T);
             in_len[n] = nb * nd.C;                           // input nodes have Cpad == C
+            n_vectors += nb * nd.C / 4;
             for (int i = 0; i < 3; ++i) in_buf[n][i] = nd.buf[i];
             ++n;
         }
@@ -580,18 +582,29 @@ sr_dense_kernel(const DnParams P, const SrFrameCtl init, int n_frames)
         for (int i = 0; i < n_in; ++i) dn_load(dn_mem + in_buf[i][k % 3], in_src[i] + (k - 1) * in_step[i], in_len[i], f_tid, f_nthr);
     };
     fetch_inputs(1);
-    // Vector v (four values) of input frame k: where it lies and where it goes; null beyond the last.
+    // What a fetching thread takes of input frame k: vectors of four values f_nthr apart, through all inputs, kDnHeld of them from its
+    // `first` on.  (Where a vector lies is worked out from the one before, and what exceeds kDnHeld goes in as many at a time.  With a
+    // search per vector and the rest one by one these few warps were what the frame waited for: 784-128-128-10 network in bf16, us per
+    // frame at 8 / 32 / 64 / 256 sequences 2.60 / 5.24 / 5.24 / 15.2, so 2.01 / 3.65 / 4.53 / 13.1; with 12 or 16 the same.)
     uint2 held[kDnHeld];
-    auto input_vector = [&](int v, int k, const T*& src) -> float* {
-        for (int i = 0; i < n_in; ++i) {
-            if (v * 4 < in_len[i]) {
-                src = in_src[i] + (k - 1) * in_step[i] + v * 4;
-                return dn_mem + in_buf[i][k % 3] + v * 4;
+    auto each_vector = [&](int first, int k, auto&& take) {
+        int i = -1, len = 0, v = f_tid + first * f_nthr;
+        const T* src = nullptr;
+        float* dst = nullptr;
+#pragma unroll
+        for (int r = 0; r < kDnHeld; ++r, v += f_nthr) {
+            while (v * 4 >= len) {
+                v -= len / 4;
+                if (++i >= n_in) return;
+                len = in_len[i];
+                src = in_src[i] + (k - 1) * in_step[i];
+                dst = dn_mem + in_buf[i][k % 3];
             }
-            v -= in_len[i] / 4;
+            take(r, src + v * 4, dst + v * 4);
         }
-        return nullptr;
     };
+    auto hold_vectors = [&](int first, int k) { each_vector(first, k, [&](int r, const T* src, float*) { held[r] = *reinterpret_cast<const uint2*>(src); }); };
+    auto store_vectors = [&](int first, int k) { each_vector(first, k, [&](int r, const T*, float* dst) { *reinterpret_cast<float4*>(dst) = dn_widen(held[r]); }); };
     asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -605,11 +618,7 @@ sr_dense_kernel(const DnParams P, const SrFrameCtl init, int n_frames)
         if (sizeof(T) == 4) {
             if (f + 1 < n_frames) fetch_inputs(f + 2);
         } else if (f_tid >= 0 && f + 1 < n_frames) {
-#pragma unroll
-            for (int r = 0; r < kDnHeld; ++r) {
-                const T* src;
-                if (input_vector(f_tid + r * f_nthr, f + 2, src)) held[r] = *reinterpret_cast<const uint2*>(src);
-            }
+            hold_vectors(0, f + 2);
         }
         if (sizeof(T) == 4 && f_tid >= 0) asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(dn_smem(&bars[P.n_levels - 1][par])) : "memory");
         for (int l = 1; l <= P.n_levels; ++l) {
@@ -627,16 +636,14 @@ sr_dense_kernel(const DnParams P, const SrFrameCtl init, int n_frames)
                 else if (un.nrows > 2) dn_unit<4, CL, S, T, CONV>(H, un, dn_mem, wsm, init, f, lane, b0, nb, run0, bar);
                 else dn_unit<2, CL, S, T, CONV>(H, un, dn_mem, wsm, init, f, lane, b0, nb, run0, bar);
             }
-            if (sizeof(T) == 2 && l == P.n_levels && f_tid >= 0) {   // the next input frame, loaded ahead of the update, goes into its buffer
+            // The next input frame, loaded ahead of the update, goes into its buffer; what is more than the threads hold follows, as many
+            // vectors on their way as they hold.
+            if (sizeof(T) == 2 && l == P.n_levels && f_tid >= 0) {
                 if (f + 1 < n_frames) {
-                    const T* src;
-#pragma unroll
-                    for (int r = 0; r < kDnHeld; ++r)
-                        if (float* dst = input_vector(f_tid + r * f_nthr, f + 2, src)) *reinterpret_cast<float4*>(dst) = dn_widen(held[r]);
-                    for (int v = f_tid + kDnHeld * f_nthr;; v += f_nthr) {
-                        float* dst = input_vector(v, f + 2, src);
-                        if (!dst) break;
-                        *reinterpret_cast<float4*>(dst) = dn_widen(*reinterpret_cast<const uint2*>(src));
+                    store_vectors(0, f + 2);
+                    for (int first = kDnHeld; f_tid + first * f_nthr < n_vectors; first += kDnHeld) {
+                        hold_vectors(first, f + 2);
+                        store_vectors(first, f + 2);
                     }
                 }
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");

@@ -191,3 +191,15 @@ def test_convolutions_hand_over_to_the_launch_path_and_back(dtype):
     assert parity.rel_err(out.cpu().numpy(), want[4][1:12].reshape(11, 5, 7)) <= parity.TOL[dtype]
     for v in range(5):
         assert parity.rel_err(G.get_state(v).float().cpu().numpy(), want[v][11]) <= parity.TOL[dtype]
+
+
+@pytest.mark.parametrize("pattern", ["streaming", "sequential"])
+@pytest.mark.parametrize("batch,width", [(72, 784), (67, 1000), (9, 4)])
+def test_bf16_input_frames_of_more_vectors_than_the_fetching_threads_hold(pattern, batch, width):
+    # with eight sequences per cluster a frame of the 784-wide input is up to 17 vectors for each of 96 fetching threads, which have
+    # eight on their way at a time; the last cluster is not full
+    g = mlp(batch, 5, (width, 128, 128, 10))
+    g.dtype = "bf16"
+    samples = sorted({0, 7, batch // 2, batch - 1})
+    parity.check_run(g, pattern, samples=samples, expect_resident=CLUSTER[pattern] if batch == 9 else 8)
+    parity.check_run(g, pattern, samples=samples, frames=2)
