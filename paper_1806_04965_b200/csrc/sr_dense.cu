@@ -53,7 +53,10 @@ constexpr int kDnMaxCluster = 16;      // CTAs per cluster: 8, or 16 (a non-port
 constexpr int kDnWarps = 8;            // 256 threads: a work unit keeps 64 registers of packed accumulators and its operands
 constexpr int kDnRows = 4;             // output rows per work unit
 constexpr int kDnHeld = 8;             // vectors of a bf16 input frame that a fetching thread has on their way at a time
-constexpr int kDnConvWork = 1 << 18;   // multiply-adds per sample and frame of all convolutions, most
+// Multiply-adds per sample and frame of all convolutions, most.  Of the networks measured (28 x 28 x 1 to 7 x 7 x 16..108, 14 x 14 x 4 to a
+// recurrent 7 x 7 x 8..40) those with more did not fit the shared memory, but for one of 296 thousand at up to 16 sequences (launched /
+// here 6.8 / 3.5 us per frame at one); at 211 thousand it is 6.4 / 3.6, 11.7 / 8.2 at 64.
+constexpr int kDnConvWork = 1 << 18;
 constexpr int kDnSmemMax = 226 * 1024;
 
 struct DnNode {
@@ -1057,11 +1060,17 @@ sr_status sr_dn_plan(sr_graph* g, size_t& offset)
             E = dn_build(g, cl, best_s);
         }
         if (E) E->one_wave = best_waves == 1;
-        // In bf16 a convolution has the tensor cores, and the launch path takes no longer for many sequences than for one: there the
-        // engine is for what goes out at once, and for frames of one level with up to four sequences per cluster.  MNIST network SR, us
-        // per frame launched / resident: bf16 at 8 / 64 / 256 samples 7.0 / 4.1, 8.4 / 8.9, 16.7 / 27.7, sequential at 128 (two waves)
-        // 19.8 / 26.4; fp32 at 1 / 100 / 128 11.5 / 4.0, 15.4 / 8.1, 18.2 / 16.6, sequential at 8 / 100 19.0 / 6.1, 27.0 / 9.3.
-        if (E && work > 0 && g->dtype == SR_DTYPE_BF16 && (!E->one_wave || (g->groups.size() == 1 && E->samples > 4))) {
+        // A frame of a convolutional network takes the launch path little longer for many sequences than for one, and this engine as much
+        // longer as there are waves.  So it is for what goes out at once, in fp32 also for two waves of frames of several levels (launches);
+        // in bf16, where the tensor cores do the convolutions, frames of one level only with up to four sequences per cluster.  us per frame
+        // launched / resident (MNIST network SR; 14 x 14 x 4 to a recurrent 7 x 7 x 16):
+        //   fp32, one level, 100 samples (one wave) 12.1 / 8.1; 9.4 / 6.6 at 64; 128 (two) 13.3 / 15.7; 10.7 / 13.0; 256 (three) 20.1 / 23.5; 14.2 / 19.4
+        //   fp32, sequential, 100 19.2 / 9.3; 14.4 / 7.5; 128 19.8 / 18.0; 15.7 / 14.7; 256 25.8 / 27.0; 19.1 / 22.1
+        //   bf16, one level, 8 7.1 / 4.2; 64 (eight sequences a cluster) 8.4 / 8.9; sequential, 64 13.0 / 12.7; 12.5 / 11.7; 128 (two) 19.8 / 26.4
+        // (Of 48 sizes and networks the former rule, any number of waves in fp32, had 13 up to 49 % slower than launches; this one
+        // has a 14 x 14 x 4 to 7 x 7 x 8 at 128 samples launched, 10.8, that the engine would take 8.5 for, and four up to 6 %.)
+        const int most_waves = g->dtype == SR_DTYPE_F32 && g->groups.size() > 1 ? 2 : 1;
+        if (E && work > 0 && (best_waves > most_waves || (g->dtype == SR_DTYPE_BF16 && g->groups.size() == 1 && E->samples > 4))) {
             delete E;
             E = nullptr;
         }

@@ -203,3 +203,16 @@ def test_bf16_input_frames_of_more_vectors_than_the_fetching_threads_hold(patter
     samples = sorted({0, 7, batch // 2, batch - 1})
     parity.check_run(g, pattern, samples=samples, expect_resident=CLUSTER[pattern] if batch == 9 else 8)
     parity.check_run(g, pattern, samples=samples, frames=2)
+
+
+@pytest.mark.parametrize("dtype,pattern,batch,resident", [
+    ("fp32", "streaming", 32, True), ("fp32", "streaming", 400, False), ("fp32", "sequential", 32, True), ("fp32", "sequential", 800, False),
+    ("bf16", "streaming", 2, True), ("bf16", "streaming", 400, False), ("bf16", "sequential", 400, False),
+])
+def test_convolutions_in_more_waves_than_pay_are_launched(dtype, pattern, batch, resident):
+    # one wave of clusters, in fp32 two where a frame is several launches; a device holds 18 clusters of eight CTAs at most
+    g = small_cnn(batch, 3, dtype)
+    G = parity.make_graph(g, pattern, "auto", 0, data.make_weights(g), data.make_biases(g))
+    assert (G.info["resident_cluster"] > 0) == resident, G.info
+    samples = sorted({0, batch // 2, batch - 1})
+    parity.check_run(g, pattern, samples=samples)
