@@ -1674,9 +1674,11 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
         // A launch with many items per SM takes the widest tiles (fewest copies per MMA).  For one with few, the split that ends first
         // by the estimate is sought: from the same columns for every plan, the plan whose items take longest gets narrower
         // tiles (of the next or the second next width) or has its items cut into twice as many parts, whichever leaves the shortest
-        // bound, again and again.  The line lies at
-        // three items of the widest tiles per SM: at 2.8 (stress graph at 4 samples) the search still gains 8 %, from 3.5 on
-        // (six-node network at 64 samples, ten-node at 48) nothing.
+        // bound, again and again.  The line lies at four items of the widest tiles per SM.  At three of them launches of joined nodes had
+        // items too long to share out: networks of the CIFAR10 kind with six / four added layers, us per pass of 16 frames with the line at
+        // three / four / five, at 40 samples 605 / 447 / 448, at 64 721 / 659 / 755 (in twos 658), at 96 857 / 857 / 906; at 48 542 / 479 / 480, at 72
+        // 637 / 605 / 631; stress graph at 6 1012 / 891 / 895; two added layers at 80 485 / 498 / 498; six-node at 48 to 80, ten-node at 40 to 64 samples
+        // equal.
         std::vector<Choice> best;
         int best_cluster = 1, best_grid = 0;
         long long best_cost = -1;
@@ -1695,7 +1697,7 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
                 for (int cols : kTileCols) variants[m].push_back(variant_of(m, cols));
                 widest_items += variants[m][0].tiles.size();
             }
-            few = g->opt_b_units == 0 && g->opt_tile_w == 0 && g->compact == 0 && widest_items <= 3 * (size_t)g->sm_count;
+            few = g->opt_b_units == 0 && g->opt_tile_w == 0 && g->compact == 0 && widest_items <= 4 * (size_t)g->sm_count;
             for (int start = 0; start < kVariants && !members.empty(); ++start) {
                 if (start == 1 && !few) continue;              // (ten-node windows of 8 frames, 128 samples: 1842 -> 1905 us per pass with them)
                 size_t items = 0;
@@ -1744,9 +1746,10 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
                 if (items > 8 * (size_t)g->sm_count) break;            // plenty of items: smaller tiles only cost copies
             }
         };
-        // Joined as far as they go, or in twos: the launch that ends first (with few tiles, more and shorter items may; joined where it
-        // is 3 % ahead).  Deepest CIFAR10 network, us per frame in twos / joined: 13.2 / 13.1, 19.0 / 24.0, 43.7 / 44.8, 74.0 / 66.9 at 4,
-        // 16, 64, 128 samples; with four added layers 17.0 / 12.4, 36.6 / 34.2, 108 / 95 at 8, 64, 256.
+        // Joined as far as they go, or in twos: the launch that ends first by the estimate (with few tiles, more and shorter items may; joined
+        // where it is 3 % ahead).  Networks of the CIFAR10 kind with six added layers, us per pass of 16 frames in twos / joined: at 4
+        // samples 181 / 216, 8 248 / 233, 16 277 / 384, 32 528 / 431, 64 658 / 719, 96 940 / 857, 128 1271 / 1120, 256 2506 / 2204; with four: 1 120 / 133,
+        // 8 347 / 214, 24 348 / 321, 64 578 / 542, 128 967 / 856.
         const int most = !g->opt_tc_fuse || g->compact > 1 ? 1 : g->compact > 0 ? 2 : kMaxFused;
         const auto joined = join_nodes(g, g->groups[gi], most), twos = join_nodes(g, g->groups[gi], std::min(most, 2));
         search(joined);
