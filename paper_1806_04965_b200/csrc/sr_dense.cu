@@ -1045,21 +1045,23 @@ sr_status sr_dn_plan(sr_graph* g, size_t& offset)
     if (E) {
         const int cl = E->cluster;
         double best = 0.0;
-        int best_s = 0, best_waves = 0;
+        int best_waves = 0;
         for (int S = kDnMaxSamples; S >= 2; S /= 2) {
-            DnEngine* F = S == kDnMaxSamples ? E : dn_build(g, cl, S);
+            DnEngine* F = S == E->samples ? E : dn_build(g, cl, S);       // (the first is the one there is)
             if (!F) continue;
             const int clusters = (g->batch + S - 1) / S, held = std::max(dn_clusters_held(g, cl, S, F->smem_bytes), 1);
             const int waves = (clusters + held - 1) / held;
             const double cost = waves * (S == 8 ? 1.0 : S == 4 ? 0.76 : 0.6);
-            if (F != E) delete F;
-            if (best_s == 0 || cost < best) { best = cost; best_s = S; best_waves = waves; }
+            if (best_waves == 0 || cost < best) {
+                best = cost;
+                best_waves = waves;
+                if (F != E) delete E;
+                E = F;
+            } else {
+                delete F;
+            }
         }
-        if (best_s != E->samples) {
-            delete E;
-            E = dn_build(g, cl, best_s);
-        }
-        if (E) E->one_wave = best_waves == 1;
+        E->one_wave = best_waves == 1;
         // A frame of a convolutional network takes the launch path little longer for many sequences than for one, and this engine as much
         // longer as there are waves.  So it is for what goes out at once, in fp32 also for two waves of frames of several levels (launches);
         // in bf16, where the tensor cores do the convolutions, frames of one level only with up to four sequences per cluster.  us per frame

@@ -132,7 +132,8 @@ constexpr int kBuOff = 16, kBuMix = 24;                       // from these bits
 // its first block, where two plans of two had 11 and 27, and 72 for those of the second instead of 81.)  The MMAs of a K-block leave the
 // lanes of a node that does not read its source alone (an output-lane mask): rows of zero weights there would turn an infinity in that
 // source into a NaN.  Without / with the masks, us per pass: deepest CIFAR10 network 1139 / 1143, six-node at 256 samples 3216 / 3226,
-// ten-node 8297 / 8339 (at 4 samples 195.6 / 198.6), which has more of them (a mask is four more operands for the issuing thread).
+// ten-node 8297 / 8339; launches of fewer items lose more, six-node at 20 samples 293 / 316, ten-node at 48 846 / 873.  (The masked MMAs
+// themselves seem to take longer: constant masks, which the issuing thread gets for nothing, took as long.)
 struct alignas(16) TcNode {
     void* state[kMaxFused][2];
     const float* bias[kMaxFused];
@@ -1690,16 +1691,20 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
                 members.push_back((int)E->nodes.size());
                 E->nodes.push_back(plan_of(nodes));
             }
-            variants.assign(members.size(), {});
+            variants.assign(members.size(), std::vector<Variant>(kVariants));
             best_cost = -1;
+            // (the widths that are looked at)
+            auto make = [&](int v) {
+                for (size_t m = 0; m < members.size(); ++m) variants[m][v] = variant_of(m, kTileCols[v]);
+            };
+            make(0);
             size_t widest_items = 0;
-            for (size_t m = 0; m < members.size(); ++m) {
-                for (int cols : kTileCols) variants[m].push_back(variant_of(m, cols));
-                widest_items += variants[m][0].tiles.size();
-            }
+            for (size_t m = 0; m < members.size(); ++m) widest_items += variants[m][0].tiles.size();
             few = g->opt_b_units == 0 && g->opt_tile_w == 0 && g->compact == 0 && widest_items <= 4 * (size_t)g->sm_count;
+            for (int v = 1; v < kVariants && few; ++v) make(v);
             for (int start = 0; start < kVariants && !members.empty(); ++start) {
                 if (start == 1 && !few) continue;              // (ten-node windows of 8 frames, 128 samples: 1842 -> 1905 us per pass with them)
+                if (start > 0 && !few) make(start);
                 size_t items = 0;
                 for (size_t m = 0; m < members.size(); ++m) items += variants[m][start].tiles.size();
                 for (int cluster = 1; cluster <= (few ? kMaxParts : 1); cluster *= 2)
@@ -1754,9 +1759,15 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
         const auto joined = join_nodes(g, g->groups[gi], most), twos = join_nodes(g, g->groups[gi], std::min(most, 2));
         search(joined);
         if (joined != twos) {
-            const long long cost = best_cost;
+            const std::vector<NodePlan> plans(E->nodes.begin() + first_plan, E->nodes.end());
+            auto kept = std::make_tuple(std::move(members), std::move(variants), best, best_cluster, best_grid, best_cost, few);
             search(twos);
-            if (best_cost < 0 || (cost >= 0 && cost * 103 <= best_cost * 100)) search(joined);
+            const long long cost = std::get<5>(kept);
+            if (best_cost < 0 || (cost >= 0 && cost * 103 <= best_cost * 100)) {
+                E->nodes.resize(first_plan);
+                E->nodes.insert(E->nodes.end(), plans.begin(), plans.end());
+                std::tie(members, variants, best, best_cluster, best_grid, best_cost, few) = std::move(kept);
+            }
         }
         for (int ni : members)
             for (int v : E->nodes[ni].nodes) E->node_of[v] = ni;
