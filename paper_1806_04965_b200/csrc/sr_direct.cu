@@ -85,13 +85,14 @@ __device__ void conv_item(const SrDevNode& nd, const SrDevEdge* edges, const SrD
         c_end = min(nd.C, c_first + (4 << qlog));
     }
     T* dst = static_cast<T*>(nd.state[cur]) + (size_t)b * HW * nd.C;
-    for (int pbase = it.p0 + warp * kPix; pbase < min(HW, it.p0 + n_pix); pbase += kWarps * kPix) {
+    const int p_end = min(HW, it.p0 + n_pix);
+    for (int pbase = it.p0 + warp * kPix; pbase < p_end; pbase += kWarps * kPix) {
         int oy[kPix], ox[kPix];
         bool pv[kPix];
 #pragma unroll
         for (int j = 0; j < kPix; ++j) {
             const int p = pbase + j;
-            pv[j] = p < HW;
+            pv[j] = p < p_end;
             oy[j] = pv[j] ? p / nd.W : 0;
             ox[j] = pv[j] ? p % nd.W : 0;
         }
@@ -901,7 +902,7 @@ void sr_direct_conv_items(const sr_graph* g, int v, std::vector<SrDirectItem>& i
     // Four pixels per thread once that still gives every SM 256 threads; marked by the complement of the sample.  Measured on
     // B200, fp32, us per frame with one / four pixels everywhere: small CNN (28 x 28 x 32, 14 x 14 x 32, 7 x 7 x 64) at 128
     // samples 161 / 133 (this rule: 114), at 32 samples (sequential) 90 / 144, at one 27 / 51; MNIST net at 256 samples 35 / 53.
-    // Slices of a reduction of 128 steps or more until there are 512 threads per SM without them (256: sequential at 128 samples 146
+    // Slices of a reduction of 128 values or more (32 steps where the source's channels come in fours) until there are 512 threads per SM without them (256: sequential at 128 samples 146
     // instead of 117 us a frame); with four pixels per thread where a pixel per thread would make 64 threads per SM (256: 29.8 instead
     // of 24.0 us at 16 samples, 49.2 instead of 39.9 at 48; never: 27.0 and 62.1).
     const size_t quads = (size_t)g->batch * HW * (d.c / 4), sms = (size_t)g->sm_count;
