@@ -268,6 +268,16 @@ sr_status sr_graph_set_state(sr_graph* g, int node, const void* src_dev, void* s
 sr_status sr_graph_frame(const sr_graph* g, int64_t* t);
 /* Kernels launched by this graph so far (counts launches inside replayed CUDA graphs as well). */
 sr_status sr_graph_launch_count(const sr_graph* g, int64_t* n);
+/* How launch group `group` (0 .. n_groups - 1) is planned on the tensor cores: what a test looks at to know the path that it takes.
+ * All zero for a group without tensor-core nodes.  Errors: INVALID_ARG, STATE (not planned yet: ask for the workspace size first). */
+typedef struct {
+    int32_t items, ctas;      /* work items; CTAs of the launch */
+    int32_t cluster, parts;   /* CTAs of a cluster (1: none); most parts that the reduction of an item is cut into */
+    int32_t sums_in_rings;    /* 1: the parts hand their sums over in the memory of the rings */
+    int32_t columns, joined;  /* most TMEM columns of a tile; most nodes of an item */
+    int32_t masked;           /* 1: some K-block of an item does not serve all its nodes */
+} sr_launch_plan;
+sr_status sr_graph_launch_plan(const sr_graph* g, int group, sr_launch_plan* out);
 /* Sum of the event-timed durations (milliseconds) and the number of tensor-core group launches and resident
  * launches since the previous call (option key 5); waits for those launches to finish. */
 sr_status sr_graph_kernel_time(sr_graph* g, double* ms, int64_t* launches);

@@ -43,6 +43,10 @@ class _Info(ctypes.Structure):
                  "n_tensor_core_nodes", "n_direct_nodes", "resident_cluster", "resident_smem_bytes", "resident_heads_on_chip")]
 
 
+class _LaunchPlan(ctypes.Structure):
+    _fields_ = [(n, ctypes.c_int32) for n in ("items", "ctas", "cluster", "parts", "sums_in_rings", "columns", "joined", "masked")]
+
+
 def load_library(path: Optional[str] = None):
     """Load the C-ABI library; build it first if the file is missing and nvcc is present."""
     global _lib
@@ -77,6 +81,8 @@ def load_library(path: Optional[str] = None):
     lib.sr_graph_sync_status.argtypes = [vp, vp]
     lib.sr_graph_kernel_time.argtypes = [vp, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_int64)]
     lib.sr_graph_kernel_time.restype = ctypes.c_int
+    lib.sr_graph_launch_plan.argtypes = [vp, ip, ctypes.POINTER(_LaunchPlan)]
+    lib.sr_graph_launch_plan.restype = ctypes.c_int
     lib.sr_graph_window_tableau.argtypes = [vp, ip, ctypes.POINTER(ctypes.c_int32)]
     lib.sr_graph_window_workspace_bytes.argtypes = [vp, ip, ctypes.POINTER(ctypes.c_size_t)]
     lib.sr_graph_bind_window.argtypes = [vp, ip, vp, ctypes.c_size_t]
@@ -275,6 +281,12 @@ class Graph:
         v = ctypes.c_int64()
         _check(self._lib.sr_graph_launch_count(self._h, ctypes.byref(v)), "sr_graph_launch_count")
         return v.value
+
+    def launch_plan(self, group: int = 0) -> dict:
+        """How a launch group is planned on the tensor cores."""
+        p = _LaunchPlan()
+        _check(self._lib.sr_graph_launch_plan(self._h, group, ctypes.byref(p)), "sr_graph_launch_plan")
+        return {n: getattr(p, n) for (n, _) in _LaunchPlan._fields_}
 
     def set_option(self, key: int, value: int):
         _check(self._lib.sr_graph_set_option(self._h, key, value), "sr_graph_set_option")

@@ -986,6 +986,14 @@ sr_status sr_graph_launch_count(const sr_graph* g, int64_t* n)
     return SR_OK;
 }
 
+sr_status sr_graph_launch_plan(const sr_graph* g, int group, sr_launch_plan* out)
+{
+    if (!g || !out || group < 0 || group >= (int)g->groups.size()) return SR_ERR_INVALID_ARG;
+    if (!g->planned) return SR_ERR_STATE;
+    sr_tc_describe(g, group, out);
+    return SR_OK;
+}
+
 sr_status sr_graph_kernel_time(sr_graph* g, double* ms, int64_t* launches)
 {
     if (!g || !ms || !launches) return SR_ERR_INVALID_ARG;

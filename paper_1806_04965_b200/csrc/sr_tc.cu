@@ -2170,6 +2170,26 @@ int sr_tc_launch_group(sr_graph* g, int group, SrFollow how, cudaStream_t s)
     return 1;
 }
 
+void sr_tc_describe(const sr_graph* g, int group, sr_launch_plan* out)
+{
+    *out = sr_launch_plan{};
+    const TcEngine* E = eng(g);
+    if (!E || E->group_tiles[group].empty()) return;
+    const TcEngine::Launch& L = E->launches[group];
+    for (const TcTile& t : E->group_tiles[group]) {
+        if (t.node < 0) continue;
+        const NodePlan& P = E->nodes[t.node];
+        out->items += t.words == 0;
+        out->parts = std::max(out->parts, P.n_parts);
+        out->columns = std::max(out->columns, P.nl * P.lane_cols);
+        out->joined = std::max(out->joined, (int)P.nodes.size());
+    }
+    out->ctas = L.grid;
+    out->cluster = std::max(1, L.cluster);
+    out->sums_in_rings = out->parts > 1 && L.exch == 0;
+    out->masked = L.masked;
+}
+
 // Sum of the event-timed durations of the tensor-core group launches since the last call (synchronises).
 sr_status sr_tc_timing(sr_graph* g, double* ms, long long* launches)
 {

@@ -154,8 +154,10 @@ def test_small_convolutions(dtype, batch, cin, size, c):
     # launch path rounds them
     g = small_cnn(batch, 6, dtype, cin, size, c)
     for p in g.patterns:
-        parity.check_run(g, p)
-        parity.check_run(g, p, frames=1)
+        # (in bf16 with more than four sequences per cluster, which 41 take, frames of one level are launched)
+        on_chip = 0 if dtype == "bf16" and p == "streaming" and batch == 41 else CLUSTER[p]
+        parity.check_run(g, p, expect_resident=on_chip)
+        parity.check_run(g, p, frames=1, expect_resident=on_chip)
 
 
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])
@@ -216,3 +218,41 @@ def test_convolutions_in_more_waves_than_pay_are_launched(dtype, pattern, batch,
     assert (G.info["resident_cluster"] > 0) == resident, G.info
     samples = sorted({0, batch // 2, batch - 1})
     parity.check_run(g, pattern, samples=samples)
+
+
+def test_staged_copies_are_brought_up_to_date_behind_the_engine():
+    # a few-channel input edge that the launch path reads through staged copies of the frame before, which neither a reset nor the engine
+    # writes: frames from a buffer that is not on a 16-byte boundary, which the engine does not take, follow each of them
+    import torch
+    from oracle import frame_update as fu
+    g = small_cnn(5, 14, "bf16", 3, (12, 12), 16)
+    X, W, Bi = data.make_inputs(g), data.make_weights(g), data.make_biases(g, zero=False)
+    want = fu.rollout_spec(g, "streaming", X, W, Bi)
+    G = parity.make_graph(g, "streaming", "auto", 0, W, Bi)
+    assert G.info["resident_cluster"] == CLUSTER["streaming"] and G.info["n_tensor_core_nodes"] == 1
+    x = parity.to_device(g, X[0])
+
+    def shifted(a):
+        y = torch.empty(a.numel() + 1, dtype=a.dtype, device="cuda:0")[1:].view(a.shape)
+        return y.copy_(a)
+
+    def check(t):
+        G.sync_status()
+        for v in range(5):
+            assert parity.rel_err(G.get_state(v).float().cpu().numpy(), want[v][t]) <= parity.TOL["bf16"], (v, t)
+
+    G.reset([x[0]])
+    G.run([shifted(x[1:3])])             # a reset, then launches
+    check(2)
+    G.run([x[3:6]])
+    G.run([shifted(x[6:8])])             # a run of the engine, then launches
+    check(7)
+    G.step([x[8]])
+    G.step([shifted(x[9])])              # a step of the engine, then a launched one
+    check(9)
+    G.step([x[10]])
+    G.run([shifted(x[11:13])])
+    check(12)
+    G.reset([x[0]])
+    G.step([shifted(x[1])])
+    check(1)
