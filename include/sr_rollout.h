@@ -177,10 +177,10 @@ sr_status sr_graph_set_node_bias(sr_graph* g, int node, const float* bias_host);
  *                  sr_graph_kernel_time.
  *           key 6 "resident": 1 (default) lets sr_rollout_run use a resident kernel when the network qualifies: all T
  *                  frames in one launch with weights and states in the shared memory of thread-block clusters.
- *                  bfloat16 networks of convolutions with dense heads: one cluster per sequence.  networks of dense
- *                  edges, and the smallest convolutional ones beside those: one cluster per two, four or eight
- *                  sequences, if every input frame starts on a 16-byte boundary; sr_rollout_step uses that one too while the device holds all clusters of the batch at
- *                  once.  0 = always the per-frame launch path.
+ *                  bfloat16 networks of convolutions with dense heads: one cluster per sequence.  Networks of dense
+ *                  edges, and those with small convolutions while few waves of clusters hold the batch: one cluster
+ *                  per two, four or eight sequences, if every input frame starts on a 16-byte boundary; sr_rollout_step
+ *                  uses that one too while the device holds all clusters of the batch at once.  0 = always the per-frame launch path.
  *           key 7 "resident cluster size": CTAs per sequence of the bfloat16 kernel, 1, 2 or 4; 0 (default) = chosen by the
  *                  library.
  *           key 8 "resident warps": warps per CTA of the bfloat16 kernel, 4..32; 0 = default.

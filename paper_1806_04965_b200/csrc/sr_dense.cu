@@ -30,7 +30,7 @@
 // reduction, taps outside the image left out, and after a sum over the quarters writes four channels of one sequence.  A rank computes
 // a run of quads; the sequences lie quad by quad side by side (and an unused one, against bank conflicts), so what a rank has computed
 // is one piece, which goes to every other CTA as one bulk copy when its last unit is done.  MNIST network SR, fp32, 100 sequences, us
-// per frame: 15.4 launched, 8.1 here (sequential 27.0 and 9.3).  Bound by the instructions around the multiply-adds with two warps
+// per frame: 12.1 launched, 8.1 here (sequential 19.2 and 9.3).  Bound by the instructions around the multiply-adds with two warps
 // per scheduler; walked tap by tap instead of row by row it took 11.2.
 // The sums run in a fixed order, so results are reproducible bit for bit.
 #include <cuda_bf16.h>

@@ -233,7 +233,7 @@ struct sr_graph {
     std::vector<std::vector<int>> groups;          // groups[l-1] = nodes of level l
     // options
     int opt_engine = 0, opt_graph_frames = 0, opt_b_units = 0, opt_tile_w = 0, opt_overlap = 1, opt_time_tc = 0;
-    int opt_tc_fuse = 1;                           // two nodes of at most 64 channels that share a source run as one 128-row plan
+    int opt_tc_fuse = 1;                           // nodes of at most 64 channels that share a source run as one 128-row plan
     int opt_tc_lists = 0;                          // tensor-core work items: 1 = a list per CTA made on the host, 0 = the same plus a shared list of the smallest items
     int opt_wait_ms = 1000;                        // limit of every device-side wait; 0 = expire at once (test hook)
     int opt_resident = 1, opt_rs_cluster = 0, opt_rs_warps = 0, opt_rs_split = 0;   // 16-channel work units: 0 never, 1 always, 2 by cost

@@ -363,9 +363,9 @@ constexpr int kAhead = 3;
 // split item at most, the last of its list, so the room for what others send is used once, and one barrier, on which those bytes
 // count, is all there is between the CTAs.  Where that room would cost the weight ring its depth, it lies in the rings, which are
 // idle by then, and the parts tell each other first that they are (half a microsecond more).  Everything that others write into a
-// CTA it has waited for when it leaves.  Measured on B200, us per frame before / now: six-node network at one sample 14.3 / 8.8
-// (sequential 52.0 / 38.5), ten-node at 1 / 4 / 16 samples 22.5 / 9.8, 23.4 / 12.7, 32.5 / 26.4 (sequential at 16 110 / 94), stress graph
-// at 1 / 4 samples 34.1 / 18.9, 46.9 / 43.3 (sequential at 4 241 / 156), deepest CIFAR10 network at 1 / 16 19.8 / 7.9, 29.2 / 18.8.
+// CTA it has waited for when it leaves.  Measured on B200, us per pass of 16 frames without / with it: six-node network at one
+// sample 246 / 143 (sequential 862 / 567), ten-node at 1 / 8 / 20 samples 387 / 166, 403 / 276, 581 / 413 (sequential at 1 / 8 1601 / 940, 1680 / 1178),
+// stress graph at 1 / 4 samples 547 / 284, 757 / 671, deepest CIFAR10 network at 1 / 16 352 / 162, 463 / 277.
 // Alternatives that lost: a cluster barrier at the end and the sums always in the rings (8.8 -> 10.5 with both); two threads that
 // start weight copies in turn (deepest CIFAR10 network at 16 samples 18.8 -> 22.5, at 128 73.8 -> 77.6); two issuing threads with an
 // accumulator each for tiles of up to 128 columns (8.8 -> 9.6); launches of half an SM's shared memory, so that the next one
@@ -1569,7 +1569,7 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
         const size_t first_plan = E->nodes.size();
         std::vector<int> members;
         // What can be chosen per plan: the most columns of its tiles (variants, as in kTileCols), and the parts of its items.
-        struct Variant { NodePlan P; std::vector<TcTile> tiles; int box_kb = 1, w_slot = 1024, words = 0; long long plain, cycles[2][kMaxW + 1]; };   // of an item; by crowded, slots
+        struct Variant { NodePlan P; std::vector<TcTile> tiles; int box_kb = 1, w_slot = 1024, words = 0; long long plain = 0; mutable long long cycles[2][kMaxW + 1] = {}; };   // of an item; by crowded, slots (when they are asked for)
         struct Choice { int v, parts; };
         std::vector<std::vector<Variant>> variants;
         auto variant_of = [&](size_t m, int max_cols) {
@@ -1595,8 +1595,6 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
             }
             V.w_slot = (int)sr_align_up((size_t)std::min(V.P.rows_total(g), 128) * std::max(64, bk_max) * 2, 1024);
             V.plain = item_cycles(g, V.P, 0.0);
-            for (int w = 2; w <= kMaxW; ++w)
-                for (int crowded = 0; crowded < 2; ++crowded) V.cycles[crowded][w] = item_cycles(g, V.P, ring_cycles(w, crowded != 0));
             return V;
         };
         // Shared memory: what the parts of items exchange, the node tables, weight slots, and the rest for activation boxes, of which
@@ -1646,7 +1644,10 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
             return parts > (size_t)ctas_now;
         };
         auto cycles_of = [&](const Variant& V, int parts, const TcEngine::Launch& L, bool few, bool crowded) {
-            return few ? part_cycles(V.P, V.cycles[crowded][L.n_w], parts, L.exch == 0) : V.plain;
+            if (!few) return V.plain;
+            long long& cycles = V.cycles[crowded][L.n_w];
+            if (cycles == 0) cycles = item_cycles(g, V.P, ring_cycles(L.n_w, crowded));
+            return part_cycles(V.P, cycles, parts, L.exch == 0);
         };
         auto bound_of = [&](const std::vector<Choice>& ch, const TcEngine::Launch& L, bool few) {
             const bool crowded = crowded_by(ch);

@@ -16,6 +16,7 @@ struct TcWork { long long cycles; int parts; TcTile tile; };
 // Longest processing time first: items (sorted, longest first) onto the least loaded of `grid` lists.  Returns the longest list's load.
 inline long long spread_items(const std::vector<TcWork>& work, size_t n, int grid, std::vector<std::vector<TcTile>>* lists)
 {
+    if (!lists && n <= (size_t)grid) return n > 0 ? work[0].cycles : 0;
     std::vector<std::pair<long long, int>> heap;             // (-load, cta): the standard heap keeps the largest on top
     for (int c = 0; c < grid; ++c) heap.push_back({0, -c});
     std::make_heap(heap.begin(), heap.end());
@@ -46,12 +47,13 @@ inline long long spread_split(const std::vector<TcWork>& work, int grid, int clu
         const int n = w.parts;
         int at = -1;
         long long least = 0;
-        for (int c = 0; c + n <= grid; c += n) {
+        if (n == 1) at = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+        for (int c = 0; n > 1 && c + n <= grid; c += n) {
             long long l = 0;
             bool room = true;
             for (int q = 0; q < n; ++q) {
                 l = std::max(l, load[c + q]);
-                room = room && (n == 1 || !taken[c + q]);
+                room = room && !taken[c + q];
             }
             if (room && (at < 0 || l < least)) { at = c; least = l; }
         }

@@ -1,5 +1,5 @@
-"""GPU parity of the dense resident engine (small all-dense fp32 networks: weights and states in the shared memory of
-one thread-block cluster, all frames of a run in one launch) against the oracle, and its hand-over to the per-frame
+"""GPU parity of the dense resident engine (small networks of dense edges and small convolutions: weights and states in the shared
+memory of one thread-block cluster, all frames of a run in one launch) against the oracle, and its hand-over to the per-frame
 launch path: states left in global memory, frame counter, resumed runs."""
 import numpy as np
 import pytest
