@@ -211,7 +211,7 @@ sr_status plan(sr_graph* g)
     size_t least = 0;
     g->compact = 0;
     sr_status st = lay_out(g, &least);
-    if (st == SR_OK && !fits_built_in(g, g->ws_bytes) && least <= (size_t)SR_STATIC_WORKSPACE_BYTES) {
+    if (st == SR_OK && !g->is_window && !fits_built_in(g, g->ws_bytes) && least <= (size_t)SR_STATIC_WORKSPACE_BYTES) {
         for (g->compact = 1; g->compact <= 2; ++g->compact)
             if (lay_out(g, &least) == SR_OK && fits_built_in(g, g->ws_bytes)) break;
         if (g->compact > 2) {
@@ -866,6 +866,7 @@ try {
         sr_graph* w = nullptr;
         const sr_status st = sr_graph_create(nd.data(), (int)nd.size(), ed.data(), (int)ed.size(), R.data(), g->batch * W, g->dtype, &w);
         if (st != SR_OK) return st;
+        w->is_window = true;
         w->opt_engine = g->opt_engine;
         w->opt_b_units = g->opt_b_units;
         w->opt_tile_w = g->opt_tile_w;

@@ -269,6 +269,7 @@ struct sr_graph {
     bool input_feeds_same_frame = false;           // some edge that leaves an input node has R = 0
     // deep-window mode: a second graph of the same network whose batch holds the W frames of a window side by side
     sr_graph* window = nullptr;
+    bool is_window = false;                        // of another graph: never in the built-in workspace
     int window_frames = 0;
     std::vector<char> in_window;                   // per node: its current state is the last frame of the window's states
     std::vector<std::vector<float>> kept_weights;  // the parameters as the caller set them (host copies), for that graph

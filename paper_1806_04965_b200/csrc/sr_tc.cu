@@ -132,8 +132,9 @@ constexpr int kBuOff = 16, kBuMix = 24;                       // from these bits
 // its first block, where two plans of two had 11 and 27, and 72 for those of the second instead of 81.)  The MMAs of a K-block leave the
 // lanes of a node that does not read its source alone (an output-lane mask): rows of zero weights there would turn an infinity in that
 // source into a NaN.  Without / with the masks, us per pass: deepest CIFAR10 network 1139 / 1143, six-node at 256 samples 3216 / 3226,
-// ten-node 8297 / 8339; launches of fewer items lose more, six-node at 20 samples 293 / 316, ten-node at 48 846 / 873.  (The masked MMAs
-// themselves seem to take longer: constant masks, which the issuing thread gets for nothing, took as long.)
+// ten-node 8297 / 8339; launches of fewer items lose more, six-node at 20 samples 293 / 316, ten-node at 48 846 / 873.  (It is the kernel
+// compiled with masks rather than the masked MMAs: constant masks, an order of the K-blocks that leaves a tenth of them masked, one copy
+// of a burst less or more, all took as long or longer.)
 struct alignas(16) TcNode {
     void* state[kMaxFused][2];
     const float* bias[kMaxFused];
