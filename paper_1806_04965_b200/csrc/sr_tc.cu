@@ -132,9 +132,9 @@ constexpr int kBuOff = 16, kBuMix = 24;                       // from these bits
 // its first block, where two plans of two had 11 and 27, and 72 for those of the second instead of 81.)  The MMAs of a K-block leave the
 // lanes of a node that does not read its source alone (an output-lane mask): rows of zero weights there would turn an infinity in that
 // source into a NaN.  Without / with the masks, us per pass: deepest CIFAR10 network 1139 / 1143, six-node at 256 samples 3216 / 3226,
-// ten-node 8297 / 8339; launches of fewer items lose more, six-node at 20 samples 293 / 316, ten-node at 48 846 / 873.  (It is the kernel
-// compiled with masks rather than the masked MMAs: constant masks, an order of the K-blocks that leaves a tenth of them masked, one copy
-// of a burst less or more, all took as long or longer.)
+// ten-node 8297 / 8339; launches of fewer items lose more, six-node at 20 samples 292 / 297, ten-node at 8 / 20 / 48 264 / 272, 393 / 411, 846 / 874.  (It is the kernel
+// compiled with masks rather than the masked MMAs: constant masks and an order of the K-blocks that leaves a tenth of them masked
+// took as long; where the copies of a burst lie does matter, see the issuer.)
 struct alignas(16) TcNode {
     void* state[kMaxFused][2];
     const float* bias[kMaxFused];
@@ -769,10 +769,8 @@ __global__ void __launch_bounds__(kThreads, SPLIT ? 2 : 1) sr_tc_group_kernel(co
                         p_fl = c.fl; p_w1 = c.bw1 + 8 * kMaxW; p_a1 = c.ba1 + 8 * kBoxes;
                         owed = 1;
                     };
-                    // A burst whose operands are not there, or of another kind: half by half.  (One copy for all bursts of a
-                    // kernel, and the masked copy of the common kind out of the way: with two copies of both the deepest CIFAR10 network
-                    // took 1174 us per pass instead of 1149.)
-                    auto plain = [&] {
+                    // A burst whose operands are not there, or of another kind: half by half.
+                    auto plain = [&](auto masked) {
                         pay(owed);
                         owed = 0;
 #pragma unroll
@@ -786,10 +784,10 @@ __global__ void __launch_bounds__(kThreads, SPLIT ? 2 : 1) sr_tc_group_kernel(co
                                 const uint32_t d = d0 + l * lane_cols, xl = l * c.l1, xh = h ? c.xh1 : c.xh0;
                                 const uint32_t xa = (h ? c.x2 : c.x0) + xl, xb = (h ? c.x3 : c.x1) + xl, va = h ? c.v2 : c.v0, vb = h ? c.v3 : c.v1;
                                 auto mma = [&](uint32_t w, uint32_t x, uint32_t sum, uint32_t off) {
-                                    if constexpr (MASKED) tc_mma_bf16_lohi(d, w, c.wh, x, xh, idesc, sum, tc_lanes(off));
+                                    if constexpr (decltype(masked)::value) tc_mma_bf16_lohi(d, w, c.wh, x, xh, idesc, sum, tc_lanes(off));
                                     else tc_mma_bf16_lohi(d, w, c.wh, x, xh, idesc, sum);
                                 };
-                                if (MASKED && mix) mma(va, xa, 0u, ~mix);
+                                if (decltype(masked)::value && mix) mma(va, xa, 0u, ~mix);
                                 mma(va, xa, sum, off | mix);
                                 if (!(c.fl & kBuK16)) mma(va + 2, xa + 2, 1u, off);
                                 if (c.fl & (h ? 8u : 2u)) {
@@ -805,11 +803,26 @@ __global__ void __launch_bounds__(kThreads, SPLIT ? 2 : 1) sr_tc_group_kernel(co
                             ready = mbar_test_wait(n.bw0, n.pw0) & mbar_test_wait(n.bw1, n.pw1) & mbar_test_wait(n.ba0, n.pa0) & mbar_test_wait(n.ba1, n.pa1);
                         }
                     };
-                    if (ready && (c.fl & (15u | kBuK16)) == 15u && nl <= 2 && (!MASKED || (c.fl >> kBuMix) == 0)) {
+                    // Where the copies for bursts with masks lie matters as much as what they do.  A launch of cut items, which fetches its
+                    // code from L2, has copies of both kinds for bursts without masks and both for those with, out of the way (six-node
+                    // network at 20 samples 316 us per pass with one copy of the plain kind, so 297; ten-node at 8 280 / 272).  One of many
+                    // items has the masked copy of the common kind out of the way and one of the plain kind (with two the deepest
+                    // CIFAR10 network took 1150 us instead of 1080, the six-node at 48 samples 571 instead of 562).
+                    if constexpr (MASKED && SPLIT) {
+                        const bool usual = ready && (c.fl & (15u | kBuK16)) == 15u && nl <= 2 && (c.fl >> kBuMix) == 0;
+                        if (__builtin_expect((c.fl >> kBuOff) == 0, 1)) {
+                            if (usual) common(std::false_type());
+                            else plain(std::false_type());
+                        } else {
+                            if (usual) common(std::true_type());
+                            else plain(std::true_type());
+                        }
+                        if (!ok) break;
+                    } else if (ready && (c.fl & (15u | kBuK16)) == 15u && nl <= 2 && (!MASKED || (c.fl >> kBuMix) == 0)) {
                         if (!MASKED || __builtin_expect((c.fl >> kBuOff) == 0, 1)) common(std::false_type());
                         else common(std::bool_constant<MASKED>());
                     } else {
-                        plain();
+                        plain(std::bool_constant<MASKED>());
                         if (!ok) break;
                     }
                     c = n;
