@@ -154,10 +154,8 @@ def test_small_convolutions(dtype, batch, cin, size, c):
     # launch path rounds them
     g = small_cnn(batch, 6, dtype, cin, size, c)
     for p in g.patterns:
-        # (in bf16 with more than four sequences per cluster, which 41 take, frames of one level are launched)
-        on_chip = 0 if dtype == "bf16" and p == "streaming" and batch == 41 else CLUSTER[p]
-        parity.check_run(g, p, expect_resident=on_chip)
-        parity.check_run(g, p, frames=1, expect_resident=on_chip)
+        parity.check_run(g, p)
+        parity.check_run(g, p, frames=1)
 
 
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])
@@ -256,3 +254,14 @@ def test_staged_copies_are_brought_up_to_date_behind_the_engine():
     G.reset([x[0]])
     G.step([shifted(x[1])])
     check(1)
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("batch,cin,size,c", [(1, 1, (12, 10), 12), (3, 3, (12, 8), 4), (8, 4, (6, 10), 32), (11, 1, (14, 14), 16), (41, 2, (8, 8), 20)])
+def test_small_convolutions_take_the_engine(dtype, batch, cin, size, c):
+    # (in bf16 with more than four sequences per cluster, which 41 take, frames of one level are launched)
+    g = small_cnn(batch, 6, dtype, cin, size, c)
+    for p in g.patterns:
+        on_chip = 0 if dtype == "bf16" and p == "streaming" and batch == 41 else CLUSTER[p]
+        G = parity.make_graph(g, p, "auto", 0, data.make_weights(g), data.make_biases(g))
+        assert G.info["resident_cluster"] == on_chip, (p, G.info)

@@ -385,11 +385,10 @@ def test_cuda_core_convolution_of_a_sample_beyond_32_bit_offsets():
 
 
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])
-@pytest.mark.parametrize("batch,size,cin,c", [(2, 5, 3, 4), (2, 7, 8, 132), (130, 16, 4, 64), (2, 7, 16, 132), (40, 7, 24, 132)])
+@pytest.mark.parametrize("batch,size,cin,c", [(2, 5, 3, 4), (2, 7, 8, 132), (130, 16, 4, 64)])
 def test_infinite_weights_leave_pixels_alone_whose_window_they_miss(batch, size, cin, c, dtype):
     # the weight of a corner tap is infinite: the first row and column, for which that tap lies outside the image, stay finite, with one
-    # and (the third and the last case) four pixels per thread, and (the last two) with items whose reduction the warps of a block share;
-    # finite weights afterwards bring the usual results back
+    # and (the last case) four pixels per thread; finite weights afterwards bring the usual results back
     import torch
     from oracle import frame_update as fu
     from workloads.graphs import CONV, GAP_DENSE, IDENTITY, Edge, GraphSpec, Node, check_shapes
@@ -466,3 +465,10 @@ def test_cuda_core_convolutions_in_slices(batch, size, cin, c, dtype):
     # reductions of 128 values and more, which the warps of a block share: one and four pixels per thread, quads and pixels that do
     # not fill a block, several channel blocks, a source read value by value
     test_cuda_core_convolutions_at_the_edges_of_their_tiles(batch, size, cin, c, dtype)
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("batch,size,cin,c", [(2, 7, 16, 132), (40, 7, 24, 132)])
+def test_infinite_weights_on_items_whose_reduction_is_shared(batch, size, cin, c, dtype):
+    # the warps of a block share the reduction; one and four pixels per thread
+    test_infinite_weights_leave_pixels_alone_whose_window_they_miss(batch, size, cin, c, dtype)

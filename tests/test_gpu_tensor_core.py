@@ -234,6 +234,51 @@ def test_the_wait_limit_does_not_count_the_run_before(name, kw):
     assert parity.rel_err(out.cpu().numpy()[:, samples].reshape(want[o][1:].shape), want[o][1:]) <= parity.TOL["bf16"]
 
 
+@pytest.mark.parametrize("cin,c,k,stride,size,batch", [
+    (256, 256, 3, 1, 8, 1),        # two edges of 36 K-blocks on one tile of 64 pixels
+    (256, 128, 3, 1, 8, 5),
+    (48, 96, 3, 1, 7, 2),          # 16-channel K-blocks, channels and pixels that fill no tile
+    (64, 512, 3, 4, 16, 1),        # a box per tap; 16 pixels: parts without columns of their own
+    (128, 64, 3, 2, 28, 37),       # wide tiles, their sums in the rings
+    (64, 128, 1, 1, 12, 1),        # one K-block per edge: nothing to cut
+])
+def test_long_reductions_of_few_pixels(cin, c, k, stride, size, batch):
+    # launches with fewer items than SMs, whose items are cut along K over the CTAs of a cluster
+    out = size // stride
+    g = tiny("split", [Node("in", size, size, cin, IDENTITY), Node("a", out, out, c), Node("b", out, out, c), Node("o", 1, 1, 4, IDENTITY)],
+             [Edge(0, 1, CONV, k, stride), Edge(1, 1, CONV, k, 1), Edge(1, 2, CONV, k, 1), Edge(2, 2, CONV, 3, 1), Edge(2, 3, GAP_DENSE)],
+             batch=batch, frames=3)
+    samples = list(range(min(batch, 4))) + ([batch - 1] if batch > 4 else [])
+    parity.check_stepwise(g, "p", samples=samples, zero_bias=False)
+    g.patterns["q"] = [0, 1, 0, 1, 0]
+    parity.check_stepwise(g, "q", samples=samples, zero_bias=False)
+
+
+@pytest.mark.parametrize("c,size,batch", [
+    (256, 8, 127),                 # two images to a tile, the last one alone
+    (256, 8, 25),                  # the same with the reduction cut: nine chunks of columns do not divide by the parts
+    (256, 5, 60),                  # three images, all 160 columns; the parts' sums in the rings
+])
+def test_tiles_of_a_few_small_images(c, size, batch):
+    g = tiny("pair", [Node("in", size, size, 64, IDENTITY), Node("a", size, size, c), Node("b", size, size, c), Node("o", 1, 1, 4, IDENTITY)],
+             [Edge(0, 1, CONV, 3, 1), Edge(1, 1, CONV, 3, 1), Edge(1, 2, CONV, 3, 1), Edge(2, 3, GAP_DENSE)], batch=batch, frames=3)
+    g.patterns["q"] = [0, 1, 0, 0]
+    for pattern in ("p", "q"):
+        parity.check_stepwise(g, pattern, samples=[0, 1, 2, batch // 2, batch - 2, batch - 1], zero_bias=False)
+
+
+@pytest.mark.parametrize("c,n", [(32, 3), (32, 4), (32, 5), (64, 3)])
+def test_several_narrow_nodes_that_share_sources(c, n):
+    # a block in which every earlier node feeds every later one, as in the paper's CIFAR10 networks: up to 128 channels run as one
+    # plan; the nodes' activations and biases stay their own, the last plan may be part empty
+    nodes = [Node("in", 12, 20, 3, IDENTITY)] + [Node("n%d" % i, 12, 20, c, IDENTITY if i == 1 else RELU) for i in range(n)]
+    edges = [Edge(0, 1, CONV, 5, 1), Edge(1, 1, CONV, 3, 1)] + [Edge(i, j, CONV, 3, 1) for i in range(1, n + 1) for j in range(i + 1, n + 1)]
+    g = tiny("block", nodes + [Node("o", 1, 1, 4, IDENTITY)], edges + [Edge(i, n + 1, GAP_DENSE) for i in range(1, n + 1)], batch=3, frames=4)
+    for fuse in (1, 0):
+        parity.check_stepwise(g, "p", zero_bias=False, tc_fuse=fuse)
+    parity.check_stepwise(g, "p", zero_bias=False, tc_lists=1, weight_ring_units=2, tile_width=16)
+
+
 def plans(g, pattern, **options):
     """How the launch groups of a pattern are planned: the path that a case means to take."""
     from paper_1806_04965_b200 import Graph
@@ -242,57 +287,48 @@ def plans(g, pattern, **options):
 
 
 @pytest.mark.parametrize("cin,c,k,stride,size,batch,parts,rings,columns", [
-    (256, 256, 3, 1, 8, 1, 8, 0, 64),          # two edges of 36 K-blocks on one tile of 64 pixels
+    (256, 256, 3, 1, 8, 1, 8, 0, 64),
     (256, 128, 3, 1, 8, 5, 8, 0, 64),
-    (48, 96, 3, 1, 7, 2, 8, 0, 64),            # 16-channel K-blocks, channels and pixels that fill no tile
-    (64, 512, 3, 4, 16, 1, 8, 0, 32),          # a box per tap; 16 pixels, two chunks of columns: parts without columns of their own
+    (48, 96, 3, 1, 7, 2, 8, 0, 64),
+    (64, 512, 3, 4, 16, 1, 8, 0, 32),          # two chunks of columns: parts without columns of their own
     (128, 64, 3, 2, 28, 37, 2, 0, 112),        # two nodes to a plan
     (128, 256, 3, 1, 8, 12, 4, 1, 144),        # sums in the rings, nine chunks of columns over four parts
     (64, 256, 3, 1, 16, 20, 2, 1, 256),        # sums in the rings, the widest tile
     (64, 128, 1, 1, 12, 1, 8, 0, 64),          # one K-block per 1 x 1 edge (in the second pattern a launch with nothing to cut)
 ])
-def test_long_reductions_of_few_pixels(cin, c, k, stride, size, batch, parts, rings, columns):
-    # launches with fewer items than SMs, whose items are cut along K over the CTAs of a cluster
+def test_long_reductions_take_the_path_that_is_meant(cin, c, k, stride, size, batch, parts, rings, columns):
     out = size // stride
     g = tiny("split", [Node("in", size, size, cin, IDENTITY), Node("a", out, out, c), Node("b", out, out, c), Node("o", 1, 1, 4, IDENTITY)],
              [Edge(0, 1, CONV, k, stride), Edge(1, 1, CONV, k, 1), Edge(1, 2, CONV, k, 1), Edge(2, 2, CONV, 3, 1), Edge(2, 3, GAP_DENSE)],
              batch=batch, frames=3)
-    samples = list(range(min(batch, 4))) + ([batch - 1] if batch > 4 else [])
     plan = plans(g, "p")[0]
     assert (plan["parts"], plan["sums_in_rings"], plan["columns"]) == (parts, rings, columns), plan
-    parity.check_stepwise(g, "p", samples=samples, zero_bias=False)
-    g.patterns["q"] = [0, 1, 0, 1, 0]
     if k == 1:
+        g.patterns["q"] = [0, 1, 0, 1, 0]
         assert plans(g, "q")[0]["parts"] == 1
-    parity.check_stepwise(g, "q", samples=samples, zero_bias=False)
+    if rings:
+        test_long_reductions_of_few_pixels(cin, c, k, stride, size, batch)
 
 
 @pytest.mark.parametrize("c,size,batch,parts,rings,columns", [
-    (256, 8, 127, 1, 0, 144),      # two images to a tile, the last one alone
-    (256, 8, 25, 2, 0, 144),       # the same with the reduction cut: nine chunks of columns do not divide by the parts
-    (256, 5, 60, 2, 1, 208),       # four images to a tile; the parts' sums in the rings
+    (256, 8, 127, 1, 0, 144),
+    (256, 8, 25, 2, 0, 144),
+    (256, 5, 60, 2, 1, 208),       # four images to a tile
 ])
-def test_tiles_of_a_few_small_images(c, size, batch, parts, rings, columns):
+def test_tiles_of_a_few_small_images_take_the_path_that_is_meant(c, size, batch, parts, rings, columns):
     g = tiny("pair", [Node("in", size, size, 64, IDENTITY), Node("a", size, size, c), Node("b", size, size, c), Node("o", 1, 1, 4, IDENTITY)],
              [Edge(0, 1, CONV, 3, 1), Edge(1, 1, CONV, 3, 1), Edge(1, 2, CONV, 3, 1), Edge(2, 3, GAP_DENSE)], batch=batch, frames=3)
-    g.patterns["q"] = [0, 1, 0, 0]
     plan = plans(g, "p")[0]
     assert (plan["parts"], plan["sums_in_rings"], plan["columns"]) == (parts, rings, columns), plan
-    for pattern in ("p", "q"):
-        parity.check_stepwise(g, pattern, samples=[0, 1, 2, batch // 2, batch - 2, batch - 1], zero_bias=False)
 
 
 @pytest.mark.parametrize("c,n,joined", [(32, 3, 2), (32, 4, 4), (32, 5, 2), (64, 3, 2)])
-def test_several_narrow_nodes_that_share_sources(c, n, joined):
-    # a block in which every earlier node feeds every later one, as in the paper's CIFAR10 networks: up to 128 channels run as one
-    # plan; the nodes' activations and biases stay their own, the last plan may be part empty
+def test_narrow_nodes_that_share_sources_are_joined(c, n, joined):
     nodes = [Node("in", 12, 20, 3, IDENTITY)] + [Node("n%d" % i, 12, 20, c, IDENTITY if i == 1 else RELU) for i in range(n)]
     edges = [Edge(0, 1, CONV, 5, 1), Edge(1, 1, CONV, 3, 1)] + [Edge(i, j, CONV, 3, 1) for i in range(1, n + 1) for j in range(i + 1, n + 1)]
     g = tiny("block", nodes + [Node("o", 1, 1, 4, IDENTITY)], edges + [Edge(i, n + 1, GAP_DENSE) for i in range(1, n + 1)], batch=3, frames=4)
     for fuse in (1, 0):
         assert plans(g, "p", tc_fuse=fuse)[0]["joined"] == (joined if fuse else 1)
-        parity.check_stepwise(g, "p", zero_bias=False, tc_fuse=fuse)
-    parity.check_stepwise(g, "p", zero_bias=False, tc_lists=1, weight_ring_units=2, tile_width=16)
 
 
 @pytest.mark.parametrize("c,n,cin,size,batch,joined,parts", [
