@@ -1678,13 +1678,19 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
         };
         auto work_of = [&](const std::vector<Choice>& ch, const TcEngine::Launch& L, bool few, bool tiles) {
             const bool crowded = crowded_by(ch);
-            std::vector<TcWork> work;
+            // longest first; all items of a plan are as long
+            std::vector<std::pair<long long, size_t>> order;
+            size_t n = 0;
             for (size_t m = 0; m < members.size(); ++m) {
                 const Variant& V = variants[m][ch[m].v];
-                const long long c = cycles_of(V, ch[m].parts, L, few, crowded);
-                for (const TcTile& t : V.tiles) work.push_back(TcWork{c, ch[m].parts, tiles ? t : TcTile{}});
+                order.push_back({-cycles_of(V, ch[m].parts, L, few, crowded), m});
+                n += V.tiles.size();
             }
-            std::stable_sort(work.begin(), work.end(), [](const TcWork& a, const TcWork& b) { return a.cycles > b.cycles; });
+            std::sort(order.begin(), order.end());
+            std::vector<TcWork> work;
+            work.reserve(n);
+            for (const auto& [c, m] : order)
+                for (const TcTile& t : variants[m][ch[m].v].tiles) work.push_back(TcWork{-c, ch[m].parts, tiles ? t : TcTile{}});
             return work;
         };
         // A launch with many items per SM takes the widest tiles (fewest copies per MMA).  For one with few, the split that ends first
@@ -1735,7 +1741,8 @@ sr_status sr_tc_plan(sr_graph* g, size_t& off)
                             const long long fixed = (few ? b.tail : 0) + (grid > g->sm_count / 2 ? kLateStart : 0) + (cluster > 1 ? kClusterStart : 0);
                             if (L.fits && (best_cost < 0 || std::max(b.longest, b.total / grid) + fixed < best_cost)) {
                                 const std::vector<TcWork> work = work_of(ch, L, few, false);
-                                const long long span = cluster > 1 ? spread_split(work, grid, cluster, nullptr) : spread_items(work, work.size(), grid, nullptr);
+                                const long long limit = best_cost < 0 ? kAnyLoad : best_cost - fixed;
+                                const long long span = cluster > 1 ? spread_split(work, grid, cluster, nullptr, limit) : spread_items(work, work.size(), grid, nullptr, limit);
                                 if (span >= 0 && (best_cost < 0 || span + fixed < best_cost)) {
                                     best_cost = span + fixed;
                                     best = ch;

@@ -2,6 +2,8 @@
 #pragma once
 #include <algorithm>
 #include <cstdint>
+#include <functional>
+#include <queue>
 #include <utility>
 #include <vector>
 
@@ -13,8 +15,11 @@ struct alignas(16) TcTile { int32_t node, b0, h0, w0, m0, slot, words, rank0; };
 // An item as the work lists see it: cycles of one of its parts (estimated), parts, what the kernel reads.
 struct TcWork { long long cycles; int parts; TcTile tile; };
 
-// Longest processing time first: items (sorted, longest first) onto the least loaded of `grid` lists.  Returns the longest list's load.
-inline long long spread_items(const std::vector<TcWork>& work, size_t n, int grid, std::vector<std::vector<TcTile>>* lists)
+constexpr long long kAnyLoad = INT64_MAX;
+
+// Longest processing time first: items (sorted, longest first) onto the least loaded of `grid` lists.  Returns the longest list's load, or
+// -1 as soon as one reaches `limit`.
+inline long long spread_items(const std::vector<TcWork>& work, size_t n, int grid, std::vector<std::vector<TcTile>>* lists, long long limit = kAnyLoad)
 {
     if (!lists && n <= (size_t)grid) return n > 0 ? work[0].cycles : 0;
     std::vector<std::pair<long long, int>> heap;             // (-load, cta): the standard heap keeps the largest on top
@@ -28,6 +33,7 @@ inline long long spread_items(const std::vector<TcWork>& work, size_t n, int gri
         if (lists) (*lists)[-top.second].push_back(work[i].tile);
         top.first -= work[i].cycles;
         longest = std::max(longest, -top.first);
+        if (longest >= limit) return -1;
         heap.back() = top;
         std::push_heap(heap.begin(), heap.end());
     }
@@ -36,9 +42,13 @@ inline long long spread_items(const std::vector<TcWork>& work, size_t n, int gri
 
 // Items (sorted, longest first) onto `grid` CTAs in clusters: an item of p > 1 parts goes to p neighbouring CTAs of one cluster that
 // have no part yet, behind what else they have; whole items to the least loaded CTAs.  Returns the longest list's load, or -1 if
-// the parts do not find room in this order.
-inline long long spread_split(const std::vector<TcWork>& work, int grid, int cluster, std::vector<std::vector<TcTile>>* lists)
+// the parts do not find room in this order, or as soon as a list reaches `limit`.
+inline long long spread_split(const std::vector<TcWork>& work, int grid, int cluster, std::vector<std::vector<TcTile>>* lists, long long limit = kAnyLoad)
 {
+    // least loaded first: an entry per CTA and change of its load, those that its load has left behind are dropped when they come up
+    using Entry = std::pair<long long, int>;
+    std::priority_queue<Entry, std::vector<Entry>, std::greater<Entry>> order;
+    for (int c = 0; c < grid; ++c) order.push({0, c});
     std::vector<long long> load(grid, 0);
     std::vector<char> taken(grid, 0);
     std::vector<TcTile> part(grid);
@@ -47,7 +57,11 @@ inline long long spread_split(const std::vector<TcWork>& work, int grid, int clu
         const int n = w.parts;
         int at = -1;
         long long least = 0;
-        if (n == 1) at = (int)(std::min_element(load.begin(), load.end()) - load.begin());
+        if (n == 1) {
+            while (order.top().first != load[order.top().second]) order.pop();
+            at = order.top().second;
+            order.pop();
+        }
         for (int c = 0; n > 1 && c + n <= grid; c += n) {
             long long l = 0;
             bool room = true;
@@ -63,6 +77,11 @@ inline long long spread_split(const std::vector<TcWork>& work, int grid, int clu
         }
         for (int q = 0; q < n; ++q) {
             load[at + q] += w.cycles;
+            if (load[at + q] >= limit) {
+                if (lists) lists->clear();
+                return -1;
+            }
+            order.push({load[at + q], at + q});
             TcTile t = w.tile;
             t.words = q;
             t.rank0 = at % cluster;
