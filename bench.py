@@ -43,9 +43,9 @@ PAPER_NETS = {"dsr0": dict(batch=128, frames=16), "dsr6": dict(batch=128, frames
 # the kernel source it was taken from; the number is reported only while that source is unchanged, else null.
 TRAFFIC = {
     # workload: (bytes per launch, kernel source file, sha256[:12] of that file at capture time, summary under profiles/)
-    "c5": (605.5e6, "sr_tc.cu", "59398ad47452", "profiles/sr_tc_group_kernel_counters.md"),
-    "c3": (247.4e6, "sr_tc.cu", "59398ad47452", "profiles/sr_tc_group_kernel_counters.md"),
-    "c4": (163.0e6, "sr_tc.cu", "59398ad47452", "profiles/sr_tc_group_kernel_counters.md"),
+    "c5": (604.5e6, "sr_tc.cu", "675aa86d3cf8", "profiles/sr_tc_group_kernel_counters.md"),
+    "c3": (245.9e6, "sr_tc.cu", "675aa86d3cf8", "profiles/sr_tc_group_kernel_counters.md"),
+    "c4": (163.7e6, "sr_tc.cu", "675aa86d3cf8", "profiles/sr_tc_group_kernel_counters.md"),
     "c2": (8.0e6, "sr_resident.cu", "5c35ac653b6d", "profiles/sr_resident_kernel_c2.md"),     # one launch = all 32 frames
     "c1": (1.31e6, "sr_dense.cu", "511807f5ca04", "profiles/sr_dense_kernel_c1.md"),           # one launch = all 16 frames
 }

@@ -132,7 +132,8 @@ constexpr int kBuOff = 16, kBuMix = 24;                       // from these bits
 // its first block, where two plans of two had 11 and 27, and 72 for those of the second instead of 81.)  The MMAs of a K-block leave the
 // lanes of a node that does not read its source alone (an output-lane mask): rows of zero weights there would turn an infinity in that
 // source into a NaN.  Without / with the masks, us per pass: deepest CIFAR10 network 1139 / 1143, six-node at 256 samples 3216 / 3226,
-// ten-node 8297 / 8339; launches of fewer items lose more, six-node at 20 samples 292 / 297, ten-node at 8 / 20 / 48 264 / 272, 393 / 411, 846 / 874.  (It is the kernel
+// ten-node 8297 / 8339; launches of fewer items lose more: 1 to 5 % in most, six-node with
+// 16 x 16 images at 33 / 130 samples 236 / 252, 510 / 548, 36 x 36 at 33 674 / 727, ten-node with 16 x 16 at 33 347 / 365.  (It is the kernel
 // compiled with masks rather than the masked MMAs: constant masks and an order of the K-blocks that leaves a tenth of them masked
 // took as long; where the copies of a burst lie does matter, see the issuer.)
 struct alignas(16) TcNode {
